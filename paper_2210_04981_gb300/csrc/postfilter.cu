@@ -20,10 +20,16 @@
 //   can reach it, and per source row to the columns of that disk; every tap
 //   outside has zero weight, so the bounded gathers equal the full ones.
 //   Where every near source close to the tile has a large radius, the near
-//   taps of weight exactly 1 (the interior) are summed as differences of the
-//   row prefix and only the ring around them is tapped.  Each thread gathers
+//   taps of weight exactly 1 for all of a thread's pixels (the interior) are
+//   summed as one difference of the row prefix and only the ring around them
+//   is tapped.  Each thread gathers
 //   a 2x2 pixel block so every tap it loads serves four pixels; the per-tap
-//   arithmetic is branch-free (saturating adds).
+//   arithmetic is branch-free (saturating adds).  Four thread groups share a
+//   tile's window rows.  Bound by the latency of the tap and prefix loads and
+//   by issue.  One common interior per thread (no per-pixel masks, a quarter
+//   of the prefix loads) and the row split took the gather alone from 308 to
+//   240 us (1080p room), 3270 to 2436 us (4K room, FP16/BF16 planes), 455 to
+//   255 us (1080p, mixed depths) and 43 to 17.5 us (128x128).
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -37,25 +43,42 @@ namespace {
 
 constexpr int TP = HDOF_TILE_PF;
 #ifndef HDOF_PF_RY
-#define HDOF_PF_RY 2  // pixel rows per gather thread (each thread gathers 2 x RY pixels)
+#define HDOF_PF_RY 2  // pixel rows per gather thread (each thread gathers 2 x RY pixels; 4 slower by 5-30%)
 #endif
 constexpr int PF_RY = HDOF_PF_RY;
 constexpr int PF_NPX = 2 * PF_RY;
-constexpr int GATHER_THREADS = 8 * (16 / PF_RY);
+constexpr int PF_GROUP = 8 * (16 / PF_RY);  // threads that cover a 16x16 tile once
+// Thread groups per tile, group g taking the source rows g, g + PF_G, ... of
+// each pixel's window.  A tile's work runs from nothing to (2 r_max)^2 taps a
+// pixel, so with one group the widest windows were the kernel's tail (32 of
+// them on one SM outlast the rest of the grid), and a small image had one
+// long serial loop a thread.  Gather alone, 1 / 2 / 4 / 8 groups: mixed
+// depths at 1080p 421 / 283 / 239 / 320 us, the 128x128 frame 43 / 25 / 17.5
+// us, the 1080p room 246 / 222 / 227 us, 4K 2461 / 2425 / 2421 / 2600 us.
+#ifndef HDOF_PF_G
+#define HDOF_PF_G 4
+#endif
+constexpr int PF_G = HDOF_PF_G;
+constexpr int GATHER_THREADS = PF_G * PF_GROUP;
 #ifndef HDOF_PF_MINB
-#define HDOF_PF_MINB 16  // resident gather blocks per SM the register budget targets
+#define HDOF_PF_MINB 4  // resident gather blocks per SM the register budget targets (64 registers; 3: 5-10% slower)
 #endif
 #ifndef HDOF_PF_UNROLL
 #define HDOF_PF_UNROLL 1  // unroll of the gather's tap-pair loop (1, 2, 4, 8 swept: 1 fastest)
 #endif
 constexpr int PF_UNROLL = HDOF_PF_UNROLL;
-// Shared-memory carve-out (percent of the maximum) for the gather: the taps
-// are served from L1, so keep L1 large, but every resident block also holds
-// ~1 KB of driver-reserved shared memory; 8% (a 16 KB configuration) admits
-// about 14-15 blocks, where the minimum configuration (8 KB) admits only 7
-// and a 32 KB one leaves too little L1 for the taps.
+// A near tile's interior path runs above this share of its reach, and a row
+// takes the prefix only for at least PF_MIN_IN columns (two 16-byte loads
+// cost about as much as two tap pairs): 0.2 to 0.5, and 2 to 8 columns, are
+// within 3% of one another.
+constexpr float PF_IN_SHARE = 0.5f;
+constexpr int PF_MIN_IN = 4;
+constexpr float PF_ROW_W = 8.f;  // entries round to 2^-22 at most: 160 of them to below 1e-5 of a pixel's weight
+// Shared-memory carve-out (percent of the maximum) for the gather: four
+// resident blocks hold 16 KB of partial sums each, and the taps are served
+// from L1, so no more than that (50%: the same time).
 #ifndef HDOF_PF_CARVEOUT
-#define HDOF_PF_CARVEOUT 8
+#define HDOF_PF_CARVEOUT 30
 #endif
 constexpr int GATHER_CARVEOUT = HDOF_PF_CARVEOUT;
 constexpr int AREA_MAX = 16384;  // breakpoints for radii up to 127.5
@@ -229,10 +252,10 @@ __device__ __forceinline__ float2 fma2(float s, float ex, float ey, float2 c) {
 
 // far = (S.x, S.y, S.z, W) of the far layer
 template <class COL>
-__device__ __forceinline__ float4 pf_finish(const NearAcc& a, const float4& far, const COL* col, size_t pq,
+__device__ __forceinline__ float4 pf_finish(const float4& near, const float4& far, const COL* col, size_t pq,
                                             float4* aux) {
-    const float3 Sn = f3(a.xy.x, a.xy.y, a.zw.x), Sf = f3(far.x, far.y, far.z);
-    const float Wn = a.zw.y, Wf = far.w;
+    const float3 Sn = f3(near.x, near.y, near.z), Sf = f3(far.x, far.y, far.z);
+    const float Wn = near.w, Wf = far.w;
     float alpha = clamp01(Wn);
     float3 N = Wn > HDOF_PP_MIN_W ? (1.f / Wn) * Sn : f3(0, 0, 0);
     float3 F;
@@ -317,39 +340,40 @@ __device__ __forceinline__ void ld_rec_pair(const bf164s* p, float4& a, float4& 
 // The taps of source row y from column xs to xe (inclusive) for the 2 x RY
 // block at (i, j).  Taps go in pairs (even, odd pixel index): one 256-bit
 // load of the two records and one float2 load of r + 1/2 (and z) per pair;
-// the threads of a row, two columns apart, read consecutive pairs.
+// the threads of a row, two columns apart, read consecutive pairs.  (Loading
+// the next pair ahead of the sums wants 80 registers: with 12 instead of 16
+// warps' worth of blocks the 4K gather is 20% slower.)
 template <bool NEAR, bool MASK, class A, class REC>
 __device__ __forceinline__ void pf_segment(A (&a)[PF_NPX], const float (&dyk)[PF_RY], const float (&win2)[PF_RY],
-                                           int xs, int xe, int i, int y, int W,
-                                           const float* __restrict__ rh, const float* __restrict__ zq,
-                                           const REC* __restrict__ rec) {
+                                           int xs, int xe, int i, int y, int W, const float* __restrict__ rh,
+                                           const float* __restrict__ zq, const REC* __restrict__ rec) {
     const float2* __restrict__ rh2 = reinterpret_cast<const float2*>(rh);
     const float2* __restrict__ zq2 = reinterpret_cast<const float2*>(zq);
     float dx = (float)(xs - i);
     float c[PF_RY], pdx2 = (dx - 1.f) * (dx - 1.f);
 #pragma unroll
     for (int k = 0; k < PF_RY; ++k) c[k] = sqrt_approx(pdx2 + dyk[k]);
-    size_t g = (size_t)y * W + xs;  // pixel index of the next tap
-    const size_t gend = (size_t)y * W + xe + 1;
+    unsigned g = (unsigned)y * W + xs;  // pixel index of the next tap
+    const unsigned gend = (unsigned)y * W + xe + 1;
     if (g & 1) {  // an odd first tap on its own
         const float z = NEAR ? 0.f : __ldg(&zq[g]);
         pf_tap<MASK>(a, c, pdx2, dyk, win2, dx, __ldg(&rh[g]), z, ld4(rec + g));
         ++g;
         dx += 1.f;
     }
-    size_t m = g >> 1;
-    const size_t mend = gend >> 1;  // pairs (2m, 2m + 1) with 2m + 1 < gend
+    unsigned m = g >> 1;
+    const unsigned mend = gend >> 1;  // pairs (2m, 2m + 1) with 2m + 1 < gend
 #pragma unroll PF_UNROLL
     for (; m < mend; ++m, dx += 2.f) {
         const float2 r2 = __ldg(&rh2[m]);
         float4 e0, e1;
-        ld_rec_pair(rec + 2 * m, e0, e1);
+        ld_rec_pair(rec + 2 * (size_t)m, e0, e1);
         const float2 z2 = NEAR ? make_float2(0.f, 0.f) : __ldg(&zq2[m]);
         pf_tap<MASK>(a, c, pdx2, dyk, win2, dx, r2.x, z2.x, e0);
         pf_tap<MASK>(a, c, pdx2, dyk, win2, dx + 1.f, r2.y, z2.y, e1);
     }
     if (gend & 1) {  // an even last tap on its own
-        const size_t gl = gend - 1;
+        const unsigned gl = gend - 1;
         const float z = NEAR ? 0.f : __ldg(&zq[gl]);
         pf_tap<MASK>(a, c, pdx2, dyk, win2, dx, __ldg(&rh[gl]), z, ld4(rec + gl));
     }
@@ -362,12 +386,14 @@ __device__ __forceinline__ void pf_segment(A (&a)[PF_NPX], const float (&dyk)[PF
 // exact integers in float).
 // Near layer with Rin >= 0: every source that feeds the near layer and lies
 // within Rin of the block has r - 1/2 >= Rin, so a tap closer than Rin
-// weighs exactly 1.  Per row, a pixel's taps within its interior half-width
-// floor(sqrt(Rin^2 - dy^2)) are summed from the row prefix `pre` (two
-// loads); the columns inside every pixel's interior are skipped, the rest
-// are tapped with that interior masked out.
-template <bool NEAR, class A, class REC>
-__device__ __forceinline__ void pf_layer(A (&a)[PF_NPX], float R, float Rin, int i, int j, int W, int H,
+// weighs exactly 1 and is summed from the row prefix `pre`.  PERPX false: per
+// row, the columns closer than Rin to all 2 x RY pixels are summed once (two
+// loads, the same sum for every pixel) and the rest are tapped.  PERPX true:
+// each pixel sums its own interior columns (two loads a pixel); the columns
+// inside every pixel's interior are skipped, the rest are tapped with each
+// pixel's interior masked out.
+template <bool NEAR, bool PERPX, class A, class REC>
+__device__ __forceinline__ void pf_layer(A (&a)[PF_NPX], float R, float Rin, int g, int i, int j, int W, int H,
                                          const float* __restrict__ rh, const float* __restrict__ zq,
                                          const REC* __restrict__ rec, const float4* __restrict__ pre) {
     if (R < 0.f) return;  // nothing within reach feeds this layer
@@ -375,22 +401,20 @@ __device__ __forceinline__ void pf_layer(A (&a)[PF_NPX], float R, float Rin, int
     const int G = (int)floorf(R + 1e-3f);
     const int y0 = max(j - G, 0), y1 = min(j + PF_RY - 1 + G, H - 1);
     const float R2 = R * R, Rin2 = Rin * Rin;
-    for (int y = y0; y <= y1; ++y) {
+    for (int y = y0 + g; y <= y1; y += PF_G) {
         const float dy = (float)(y - j);
         float dyk[PF_RY], win2[PF_RY];
 #pragma unroll
         for (int k = 0; k < PF_RY; ++k) dyk[k] = (dy - (float)k) * (dy - (float)k);
-        // nearest of the thread's rows to this source row
+        // nearest and farthest of the thread's rows to this source row
         const float dmin = dy >= 0.f && dy <= (float)(PF_RY - 1) ? 0.f : fminf(dyk[0], dyk[PF_RY - 1]);
-        const int w = (int)floorf(sqrtf(fmaxf(R2 - dmin, 0.f)) + 1e-3f);
+        const float dmax = fmaxf(dyk[0], dyk[PF_RY - 1]);
+        const int w = (int)(sqrt_approx(fmaxf(R2 - dmin, 0.f)) + 1e-3f);
         const int x0 = max(i - w, 0), x1 = min(i + 1 + w, W - 1);
-#pragma unroll
-        for (int k = 0; k < PF_RY; ++k) win2[k] = -1.f;
-        int wmin = -1;        // interior half-width common to the thread's rows (-1: none)
-        bool masked = false;  // some row of the thread has an interior
-        if (NEAR && Rin >= 0.f) {
+        int ls = x1 + 1, rs = x1;  // [ls, rs]: the columns that are not tapped (none)
+        if (PERPX) {
             const float4* prow = pre + (size_t)y * W;
-            wmin = 1 << 30;
+            int wmin = 1 << 30;  // interior half-width common to the thread's rows (-1: none)
 #pragma unroll
             for (int k = 0; k < PF_RY; ++k) {
                 // inward: no outward lean here (Rin already has its margin)
@@ -398,7 +422,6 @@ __device__ __forceinline__ void pf_layer(A (&a)[PF_NPX], float R, float Rin, int
                 win2[k] = wi >= 0 ? (float)(wi * wi) : -1.f;
                 wmin = min(wmin, wi);
                 if (wi >= 0) {
-                    masked = true;
 #pragma unroll
                     for (int b = 0; b < 2; ++b) {
                         const int xa = i + b;
@@ -416,22 +439,49 @@ __device__ __forceinline__ void pf_layer(A (&a)[PF_NPX], float R, float Rin, int
                     }
                 }
             }
+            if (wmin >= 1) {
+                // columns [i + 1 - wmin, i + wmin] lie in every pixel's interior
+                ls = min(x1 + 1, i + 1 - wmin);
+                rs = max(x0 - 1, i + wmin);
+            }
+        } else if (NEAR && dmax < Rin2) {
+            // columns [i + 1 - wi, i + wi] lie in every pixel's interior
+            // (Rin's margin covers the root's rounding); rounded inwards to
+            // whole pairs, so that the taps around them are whole pairs too
+            const int wi = (int)sqrt_approx(Rin2 - dmax), odd = (y & W) & 1;  // parity of the row's first index
+            const int l = max(i + 1 - wi, 0), r = min(i + wi, W - 1);
+            const int la = l + ((l + odd) & 1), ra = r - ((r + odd + 1) & 1);
+            if (ra - la + 1 >= PF_MIN_IN) {
+                const float4* prow = pre + (size_t)y * W;
+                const float4 s = __ldg(&prow[ra]);
+                const float4 l4 = la > 0 ? __ldg(&prow[la - 1]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float2 sxy = make_float2(s.x - l4.x, s.y - l4.y), szw = make_float2(s.z - l4.z, s.w - l4.w);
+#pragma unroll
+                for (int k = 0; k < PF_NPX; ++k) {
+                    a[k].xy = make_float2(a[k].xy.x + sxy.x, a[k].xy.y + sxy.y);
+                    a[k].zw = make_float2(a[k].zw.x + szw.x, a[k].zw.y + szw.y);
+                }
+                ls = la;
+                rs = ra;
+            }
         }
-        if (wmin >= 1) {
-            // columns [i + 1 - wmin, i + wmin] lie in every pixel's interior
-            const int ls = min(x1, i - wmin), rs = max(x0, i + wmin + 1);
-            if (x0 <= ls) pf_segment<NEAR, true>(a, dyk, win2, x0, ls, i, y, W, rh, zq, rec);
-            if (rs <= x1) pf_segment<NEAR, true>(a, dyk, win2, rs, x1, i, y, W, rh, zq, rec);
-        } else if (masked) {
-            pf_segment<NEAR, true>(a, dyk, win2, x0, x1, i, y, W, rh, zq, rec);
-        } else {
-            pf_segment<NEAR, false>(a, dyk, win2, x0, x1, i, y, W, rh, zq, rec);
-        }
+        if (x0 < ls) pf_segment<NEAR, PERPX>(a, dyk, win2, x0, ls - 1, i, y, W, rh, zq, rec);
+        if (rs < x1) pf_segment<NEAR, PERPX>(a, dyk, win2, rs + 1, x1, i, y, W, rh, zq, rec);
     }
 }
 
-// 8 x (16 / RY) threads per 16x16 tile; thread t gathers the 2 x RY pixel
-// block at (2 (t & 7), RY (t >> 3)), so each loaded tap serves 2 RY pixels.
+// the groups' partial sums of pixel p of the tile, in group order
+__device__ __forceinline__ float4 pf_group_sum(const float4 (&part)[PF_G][TP * TP], int p) {
+    float4 s = part[0][p];
+#pragma unroll
+    for (int g = 1; g < PF_G; ++g) s = add4(s, part[g][p]);
+    return s;
+}
+
+// PF_G groups of 8 x (16 / RY) threads per 16x16 tile; thread t of a group
+// gathers the 2 x RY pixel block at (2 (t & 7), RY (t >> 3)) over the group's
+// source rows, so each loaded tap serves 2 RY pixels; the groups' sums are
+// added in group order.
 template <class COL>
 __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx, int ty) {
     const COL* __restrict__ col = ar.col;
@@ -467,8 +517,8 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
     // feeds the near layer and lies closer than Rin to this one has
     // r_min(T) - 1/2 >= Rin: Rin = min over T of max(r_min(T) - 1/2, gap(T)),
     // less a margin, at most Gn.  The interior path (two prefix loads per
-    // pixel and row, masked taps around it) pays only when the interior is
-    // most of the window: below Rin = Gn / 2 the plain loop runs.
+    // thread and row) pays only when the interior is a good part of the
+    // window: below PF_IN_SHARE Gn the plain loop runs.
     if (Gn >= 0.f) {
         for (int k = threadIdx.x; k < nk; k += blockDim.x) {
             int ox = k % (2 * kt + 1) - kt, oy = k / (2 * kt + 1) - kt;
@@ -484,41 +534,73 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
         __syncthreads();
     }
     float Rin = Gn >= 0.f ? fminf(__int_as_float(s_win[2]), Gn) - 1e-3f : -1.f;
-    if (Rin < 0.5f * Gn) Rin = -1.f;
-    const int i = tx * TP + 2 * (threadIdx.x & 7), j = ty * TP + PF_RY * (threadIdx.x >> 3);
-    if (i >= W || j >= H) return;
+    if (Rin < PF_IN_SHARE * Gn) Rin = -1.f;
+    // A prefix entry's rounding grows with the row's sum, and a sum over the
+    // columns that all of a thread's pixels share carries the same rounding
+    // into each of them.  Where a row of the window adds up to more than
+    // PF_ROW_W (rows that cross the focus zone, whose sources weigh about 1
+    // each; a blurred row weighs its length over the disk's area), each pixel
+    // keeps its own columns and so its own rounding.
+    bool per_px = false;
+    if (Rin >= 0.f) {
+        const int G = (int)floorf(Gn + 1e-3f), y0 = max(ty * TP - G, 0), y1 = min(ty * TP + TP - 1 + G, H - 1);
+        bool big = false;
+        for (int y = y0 + threadIdx.x; y <= y1; y += GATHER_THREADS)
+            big |= !(__ldg(&ar.pre[(size_t)y * W + W - 1].w) <= PF_ROW_W);
+        per_px = __syncthreads_or(big);
+    }
+    // group g of the block's PF_G takes every PF_G-th source row; t is the
+    // thread within its group.  s_part holds the groups' sums of one layer;
+    // thread p < 256 adds and finishes pixel p of the tile.
+    __shared__ float4 s_part[PF_G][TP * TP];
+    const int g = threadIdx.x / PF_GROUP, t = threadIdx.x % PF_GROUP;
+    const int li = 2 * (t & 7), lj = PF_RY * (t >> 3);
+    const int i = tx * TP + li, j = ty * TP + lj;
+    const bool in = i < W && j < H;
     // far layer first; its sums wait in the pixels' own pp slots (each pixel
-    // is this thread's alone) so they hold no registers during the near loop
+    // is one thread's alone) so they hold no registers during the near loop
     if (Gf >= 0.f) {
         FarAcc f[PF_NPX];  // pixel (i + (k & 1), j + (k >> 1))
-        const float ka = 1.f + 1.f / ar.kz_rel;  // k_z = clamp(ka - z_q kb), kb = 1 / (kz_rel z_p)
-        const float z00 = __ldg(&ar.zq[(size_t)j * W + i]);
+        if (in) {
+            const float ka = 1.f + 1.f / ar.kz_rel;  // k_z = clamp(ka - z_q kb), kb = 1 / (kz_rel z_p)
+            const float z00 = __ldg(&ar.zq[(size_t)j * W + i]);
 #pragma unroll
-        for (int k = 0; k < PF_NPX; ++k) {
-            const int x = i + (k & 1), y = j + (k >> 1);
-            const float zp = x < W && y < H ? __ldg(&ar.zq[(size_t)y * W + x]) : z00;
-            f[k].ka = ka;
-            f[k].kb = 1.f / (ar.kz_rel * zp);
-            f[k].xy = f[k].zw = make_float2(0.f, 0.f);
-        }
-        pf_layer<false>(f, Gf, -1.f, i, j, W, H, ar.rh, ar.zq, ar.frec, nullptr);
+            for (int k = 0; k < PF_NPX; ++k) {
+                const int x = i + (k & 1), y = j + (k >> 1);
+                const float zp = x < W && y < H ? __ldg(&ar.zq[(size_t)y * W + x]) : z00;
+                f[k].ka = ka;
+                f[k].kb = 1.f / (ar.kz_rel * zp);
+                f[k].xy = f[k].zw = make_float2(0.f, 0.f);
+            }
+            pf_layer<false, false>(f, Gf, -1.f, g, i, j, W, H, ar.rh, ar.zq, ar.frec, nullptr);
 #pragma unroll
-        for (int k = 0; k < PF_NPX; ++k) {
-            const int x = i + (k & 1), y = j + (k >> 1);
-            if (x < W && y < H) pp[(size_t)y * W + x] = make_float4(f[k].xy.x, f[k].xy.y, f[k].zw.x, f[k].zw.y);
+            for (int k = 0; k < PF_NPX; ++k)
+                s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = make_float4(f[k].xy.x, f[k].xy.y, f[k].zw.x, f[k].zw.y);
         }
+        __syncthreads();
+        for (int p = threadIdx.x; p < TP * TP; p += GATHER_THREADS) {
+            const int x = tx * TP + (p & 15), y = ty * TP + (p >> 4);
+            if (x < W && y < H) pp[(size_t)y * W + x] = pf_group_sum(s_part, p);
+        }
+        __syncthreads();
     }
-    NearAcc a[PF_NPX];
+    if (in) {
+        NearAcc a[PF_NPX];
 #pragma unroll
-    for (int k = 0; k < PF_NPX; ++k) a[k].xy = a[k].zw = make_float2(0.f, 0.f);
-    pf_layer<true>(a, Gn, Rin, i, j, W, H, ar.rh, ar.zq, ar.nrec, ar.pre);
+        for (int k = 0; k < PF_NPX; ++k) a[k].xy = a[k].zw = make_float2(0.f, 0.f);
+        if (per_px) pf_layer<true, true>(a, Gn, Rin, g, i, j, W, H, ar.rh, ar.zq, ar.nrec, ar.pre);
+        else pf_layer<true, false>(a, Gn, Rin, g, i, j, W, H, ar.rh, ar.zq, ar.nrec, ar.pre);
 #pragma unroll
-    for (int k = 0; k < PF_NPX; ++k) {
-        const int x = i + (k & 1), y = j + (k >> 1);
+        for (int k = 0; k < PF_NPX; ++k)
+            s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = make_float4(a[k].xy.x, a[k].xy.y, a[k].zw.x, a[k].zw.y);
+    }
+    __syncthreads();
+    for (int p = threadIdx.x; p < TP * TP; p += GATHER_THREADS) {
+        const int x = tx * TP + (p & 15), y = ty * TP + (p >> 4);
         if (x < W && y < H) {
             const size_t q = (size_t)y * W + x;
             const float4 far = Gf >= 0.f ? pp[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-            pp[q] = pf_finish(a[k], far, col, q, aux);
+            pp[q] = pf_finish(pf_group_sum(s_part, p), far, col, q, aux);
         }
     }
 }

@@ -490,6 +490,33 @@ def test_postfilter_interior_prefix(orc, tilt, far_block):
     assert frac_close(got, ref, 1e-4) == 1.0, report("pp", got, ref)
 
 
+@pytest.mark.parametrize("W,Hh,z0", [(61, 47, 0.8), (33, 18, 0.8), (17, 130, 1.2), (64, 5, 0.6), (157, 33, 1.6)])
+def test_postfilter_interior_edges(orc, W, Hh, z0):
+    """The near interior at image borders, odd widths (rows whose first pixel
+    has an odd index) and images smaller than the window or than one tile:
+    columns summed from the prefix and columns tapped meet without a gap.
+    At most (2 x 32 + 1)^2 positive terms, each rounded a few times to 2^-24
+    relative: within 4225 x 2^-24 = 2.5e-4 of values below 0.9; half of it
+    as the sums' errors do not all point one way."""
+    rng = np.random.default_rng(W)
+    yy, xx = np.mgrid[0:Hh, 0:W].astype(np.float64)
+    nd = np.zeros((Hh, W, 4))
+    nd[..., 2] = -1.0
+    nd[..., 3] = z0 + 0.002 * xx + 0.001 * yy
+    col = np.zeros((Hh, W, 4))
+    col[..., :3] = rng.uniform(0.2, 0.9, (Hh, W, 3))
+    nd, col = nd.astype(np.float32), col.astype(np.float32)
+    cam = hi.Camera(width=W, height=Hh).f32()
+    lens = hi.Lens(3.0, 18.0 * 2 * 0.57735 / (Hh * (1 / z0 - 1 / 3.0)), 0.05).f32()  # radii around 18 px
+    p = hi.Params(r_max=32.0)
+    pp = torch.empty((Hh, W, 4), dtype=torch.float32, device="cuda")
+    H.hdof_postfilter(gbuf_from(nd, col), cam, lens, p, pp, workspace(W, Hh, p))
+    H.hdof_sync()
+    ref = orc.postfilter(nd.astype(np.float64), col.astype(np.float64), lens, cam.tan_half_fovy, p)
+    got = host(pp)
+    assert frac_close(got, ref, 1.25e-4) == 1.0, report("pp", got, ref)
+
+
 # -------------------------------------------------------- reconstruction ----
 
 def _reconstruct_inputs(W, Hh, seed):
