@@ -188,10 +188,6 @@ struct RowScanArgsT {
 };
 using RowScanArgs = RowScanArgsT<float4>;
 
-__device__ __forceinline__ float4 add4(float4 a, float4 b) {
-    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
-
 template <class REC>
 __device__ __forceinline__ void pf_rowscan_body(const RowScanArgsT<REC>& a, int y) {
     const int W = a.W, t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -235,20 +231,6 @@ struct FarAcc {
     float2 xy, zw;
     float ka, kb;
 };
-
-// (c.x, c.y) + s (e.x, e.y), each lane rounded once as fmaf would
-__device__ __forceinline__ float2 fma2(float s, float ex, float ey, float2 c) {
-    float2 r;
-    asm("{\n\t.reg .b64 ps, pe, pc, pr;\n\t"
-        "mov.b64 ps, {%2, %2};\n\t"
-        "mov.b64 pe, {%3, %4};\n\t"
-        "mov.b64 pc, {%5, %6};\n\t"
-        "fma.rn.f32x2 pr, ps, pe, pc;\n\t"
-        "mov.b64 {%0, %1}, pr;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(s), "f"(ex), "f"(ey), "f"(c.x), "f"(c.y));
-    return r;
-}
 
 // far = (S.x, S.y, S.z, W) of the far layer
 template <class COL>
@@ -318,23 +300,6 @@ __device__ __forceinline__ void pf_tap(A (&a)[PF_NPX], float (&c)[PF_RY], float&
         c[k] = d0;
     }
     pdx2 = dx2;
-}
-
-// two consecutive records (32 bytes, 32-byte aligned) in one 256-bit load
-__device__ __forceinline__ void ld_rec_pair(const float4* p, float4& a, float4& b) {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
-        : "l"(p));
-}
-// two consecutive BF16 records (16 bytes, 16-byte aligned) in one 128-bit
-// load; a BF16 value is the high half of its FP32 bits
-__device__ __forceinline__ void ld_rec_pair(const bf164s* p, float4& a, float4& b) {
-    unsigned u0, u1, u2, u3;
-    asm("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(u0), "=r"(u1), "=r"(u2), "=r"(u3) : "l"(p));
-    a = make_float4(__uint_as_float(u0 << 16), __uint_as_float(u0 & 0xffff0000u), __uint_as_float(u1 << 16),
-                    __uint_as_float(u1 & 0xffff0000u));
-    b = make_float4(__uint_as_float(u2 << 16), __uint_as_float(u2 & 0xffff0000u), __uint_as_float(u3 << 16),
-                    __uint_as_float(u3 & 0xffff0000u));
 }
 
 // The taps of source row y from column xs to xe (inclusive) for the 2 x RY

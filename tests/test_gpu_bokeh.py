@@ -78,6 +78,33 @@ def test_postfilter_shaped(orc, shape, W, Hh, rmax, A):
     assert np.abs(ref[..., :3] - circ[..., :3]).max() > 1e-3  # the shape changes the filter
 
 
+@pytest.mark.parametrize("W,Hh,rmax", [(131, 37, 0.4), (1, 1, 4.0), (17, 50, 3.0), (97, 33, 8.0), (64, 49, 9.0)])
+@pytest.mark.parametrize("shape", [SHAPES[1], SHAPES[2]])
+def test_postfilter_shaped_small_radii(orc, shape, W, Hh, rmax):
+    """Radii from 0 through 1 (where the radial weight sets in) and 8 (where
+    the area table takes over from the sorted lattice points) on a slanted
+    plane, near and far; caps below 8; images smaller than a tile.  Sums of a
+    few hundred positive terms of values below 0.9: 1e-4 as above; a radius
+    rounded across 1 may take the other weight on single pixels."""
+    rng = np.random.default_rng(W)
+    yy, xx = np.mgrid[0:Hh, 0:W].astype(np.float64)
+    nd, col = np.zeros((Hh, W, 4)), np.zeros((Hh, W, 4))
+    nd[..., 2] = -1.0
+    cam = hi.Camera(width=W, height=Hh).f32()
+    # 1/z - 1/zf linear across the image: signed radii from +9.5 to -9.5
+    c = np.linspace(19.0, -19.0, W)[None, :] * np.ones((Hh, 1)) + 0.01 * yy
+    lens = hi.Lens(3.0, 200.0 * cam.tan_half_fovy / Hh, 0.05).f32()
+    nd[..., 3] = 1.0 / (1.0 / 3.0 + c / 200.0)
+    col[..., :3] = rng.uniform(0.1, 0.9, (Hh, W, 3))
+    nd, col = nd.astype(np.float32), col.astype(np.float32)
+    p = hi.Params(r_max=rmax, **shape)
+    pp = torch.empty((Hh, W, 4), dtype=torch.float32, device="cuda")
+    H.hdof_postfilter(gbuf_from(nd, col), cam, lens, p, pp, workspace(W, Hh, p))
+    H.hdof_sync()
+    ref = orc.postfilter(nd.astype(np.float64), col.astype(np.float64), lens, cam.tan_half_fovy, p)
+    assert frac_close(host(pp), ref, 1e-4) >= 0.999, report("pp", host(pp), ref)
+
+
 def test_shaped_bokeh_frame_and_rejections(orc):
     """A whole frame with a hexagonal, rim-weighted aperture against the
     oracle's; batches and the differentiable path reject shaped apertures."""
