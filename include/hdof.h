@@ -320,7 +320,7 @@ typedef struct hdof_tuning {
     int32_t trace_refill;
     int32_t trace_chunk;   /* queue chunk, 0..16: with packets, packets a warp claims per atomic (0 = 1);
                               ray level, rays per claim in units of 32 (0 = exactly the idle lanes) */
-    int32_t spatial_tile;  /* batched spatial reconstruction's pixel tile: 0 or 8 (8x8), or 16 (16x16) */
+    int32_t spatial_tile;  /* batched spatial reconstruction's pixel tile: 0 or 8 (16x8), or 16 (16x16) */
 } hdof_tuning;
 
 /* Thin-lens distributed ray trace of the masked pixels (Ray Trace section).

@@ -252,6 +252,18 @@ __device__ __forceinline__ float2 fma_x2(f32x2 a, f32x2 b, f32x2 c) {
     return r;
 }
 
+// the same, staying in the pair form
+__device__ __forceinline__ f32x2 ffma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float2 unpk2(f32x2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
 // A ray with its box-test constants in f32x2 form: per axis (1/d, 1/d) and
 // (-cl, -ch), cl and ch being o/d shifted so that the distances to a box's
 // l- and h-plane err outwards; one fma.rn.f32x2 of a box's (l, h) pair on an

@@ -65,30 +65,52 @@ __device__ __forceinline__ void scale(float2& o, float s) {
 __device__ __forceinline__ void zero(float4& o) { o = make_float4(0.f, 0.f, 0.f, 0.f); }
 __device__ __forceinline__ void zero(float2& o) { o = make_float2(0.f, 0.f); }
 
+// The four bilinear taps of a history position: their pixels (the pixel
+// itself for a tap outside the image) and history lengths (0 there).  All
+// four hlen loads are in flight together, and then all of a plane's: with
+// each tap's plane load behind its own hlen test the kernel waited on eight
+// dependent loads per plane (1080p with half the pixels traced: 107 us; so
+// 94).  The sums stay in hist_sample's form, whose bits the mask of the next
+// frame depends on.
+struct HistTaps {
+    unsigned q[4];
+    int hl[4];
+};
+__device__ __forceinline__ HistTaps hist_taps(const TemporalArgs& a, bool valid, float ux, float uy, size_t self) {
+    HistTaps h;
+    const float x0 = floorf(ux), y0 = floorf(uy);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float x = x0 + (k & 1), y = y0 + (k >> 1);
+        const bool in = valid && x >= 0.f && y >= 0.f && x < (float)a.W && y < (float)a.H;
+        h.q[k] = in ? (unsigned)y * (unsigned)a.W + (unsigned)x : (unsigned)self;
+        h.hl[k] = __ldg(&a.hl[h.q[k]]);
+        if (!in) h.hl[k] = 0;
+    }
+    return h;
+}
+template <class T>
+__device__ __forceinline__ void hist_load(const HistTaps& h, const T* __restrict__ plane, T (&v)[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __ldg(&plane[h.q[k]]);
+}
 // bilinear history sample over taps that hold history (hlen > 0), renormalised;
 // invalid below a total tap weight of 1e-3.  hmax: largest hlen among taps
 // with non-zero weight.
 template <class T>
-__device__ __forceinline__ bool hist_sample(const TemporalArgs& a, float ux, float uy, const T* plane, T& out,
-                                            int* hmax) {
-    float x0 = floorf(ux), y0 = floorf(uy), fx = ux - x0, fy = uy - y0;
+__device__ __forceinline__ bool hist_sample(const HistTaps& h, const T (&v)[4], float ux, float uy, T& out, int* hmax) {
+    const float x0 = floorf(ux), y0 = floorf(uy), fx = ux - x0, fy = uy - y0;
     float ws = 0.f;
     zero(out);
     if (hmax) *hmax = 0;
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            float x = x0 + c, y = y0 + b;
-            if (x < 0.f || y < 0.f || x >= (float)a.W || y >= (float)a.H) continue;
-            size_t q = (size_t)y * a.W + (size_t)x;
-            int hl = __ldg(&a.hl[q]);
-            if (hl == 0) continue;
-            float w = (c ? fx : 1.f - fx) * (b ? fy : 1.f - fy);
-            ws += w;
-            acc(out, w, __ldg(&plane[q]));
-            if (hmax && w > 0.f && hl > *hmax) *hmax = hl;
-        }
+    for (int k = 0; k < 4; ++k) {
+        if (h.hl[k] == 0) continue;
+        float w = ((k & 1) ? fx : 1.f - fx) * ((k >> 1) ? fy : 1.f - fy);
+        ws += w;
+        acc(out, w, v[k]);
+        if (hmax && w > 0.f && h.hl[k] > *hmax) *hmax = h.hl[k];
+    }
     if (!(ws >= HDOF_HIST_MIN_W)) return false;
     scale(out, 1.f / ws);
     return true;
@@ -113,11 +135,14 @@ __device__ __forceinline__ void temporal_body(const TemporalArgs& a, const ND* _
     // near reprojection
     float2 m = __ldg(&a.mv[q]);
     float un = (float)i - m.x, vn = (float)j - m.y;
+    const HistTaps tn = hist_taps(a, true, un, vn, q);
+    float4 vnear[4];
+    float2 vmom[4];
+    hist_load(tn, a.hn, vnear);
+    hist_load(tn, a.hm, vmom);
     float4 hn;
     float2 hm = make_float2(0.f, 0.f);
     int hl = 0;
-    bool vn_ok = hist_sample(a, un, vn, a.hn, hn, &hl);
-    if (vn_ok) hist_sample(a, un, vn, a.hm, hm, (int*)nullptr);
     // far world position
     float3 P;
     if (fok) {
@@ -125,18 +150,26 @@ __device__ __forceinline__ void temporal_body(const TemporalArgs& a, const ND* _
     } else {
         float3 s = f3(0.f, 0.f, 0.f);
         int cnt = 0;
-        for (int b = -1; b <= 1; ++b)
-            for (int c = -1; c <= 1; ++c) {
-                if (!b && !c) continue;
-                int x = i + c, y = j + b;
-                if (x < 0 || y < 0 || x >= a.W || y >= a.H) continue;
-                size_t qq = (size_t)y * a.W + x;
-                if (a.spp[qq] == 0) continue;
-                float4 p2 = __ldg(&a.rt[3 * qq + 2]);
-                if (p2.w < 0.f) continue;
-                s = s + f3(p2.x, p2.y, p2.z);
-                ++cnt;
+#pragma unroll
+        for (int b = -1; b <= 1; ++b) {
+            // a row's loads together; rt of an untraced neighbour is not used
+            bool on[3];
+            float4 p2[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int x = i + c - 1, y = j + b;
+                on[c] = (b != 0 || c != 1) && x >= 0 && y >= 0 && x < a.W && y < a.H;
+                const size_t qq = on[c] ? (size_t)y * a.W + x : q;
+                on[c] = on[c] && __ldg(&a.spp[qq]) != 0;
+                p2[c] = __ldg(&a.rt[3 * qq + 2]);
             }
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (on[c] && p2[c].w >= 0.f) {
+                    s = s + f3(p2[c].x, p2[c].y, p2[c].z);
+                    ++cnt;
+                }
+        }
         if (cnt > 0) {
             P = (1.f / (float)cnt) * s;
         } else {
@@ -146,7 +179,13 @@ __device__ __forceinline__ void temporal_body(const TemporalArgs& a, const ND* _
     }
     float uf, vf;
     float4 hf;
-    bool vf_ok = project(a.prev, P, uf, vf) && hist_sample(a, uf, vf, a.hf, hf, (int*)nullptr);
+    const bool seen = project(a.prev, P, uf, vf);
+    const HistTaps tf = hist_taps(a, seen, seen ? uf : 0.f, seen ? vf : 0.f, q);
+    float4 vfar[4];
+    hist_load(tf, a.hf, vfar);
+    const bool vn_ok = hist_sample(tn, vnear, un, vn, hn, &hl);
+    if (vn_ok) hist_sample(tn, vmom, un, vn, hm, (int*)nullptr);
+    const bool vf_ok = seen && hist_sample(tf, vfar, uf, vf, hf, (int*)nullptr);
     // EMA weight: fixed, or per pixel from the temporal gradient (the paper's
     // per-pixel blend factors against ghosting): the larger of this frame's
     // luminance change against the reprojected history beyond alpha_k of its
@@ -189,8 +228,9 @@ __device__ __forceinline__ void temporal_body(const TemporalArgs& a, const ND* _
     a.hacc[q] = Hacc;
 }
 
+// 3 resident blocks (80 registers): with 2 or 5 the loads in flight of hist_taps gain nothing
 template <class ND>
-__global__ void __launch_bounds__(256) k_temporal(TemporalArgs a, const ND* __restrict__ nd) {
+__global__ void __launch_bounds__(256, 3) k_temporal(TemporalArgs a, const ND* __restrict__ nd) {
     temporal_body(a, nd, blockIdx.x, blockIdx.y);
 }
 
@@ -233,70 +273,41 @@ __device__ __forceinline__ void spatial_finish(const SpatialArgs& a, size_t q, c
                             0.f);
 }
 
-// the spatial gather of one traced pixel (i, j)
-__device__ __forceinline__ void spatial_pixel(const SpatialArgs& a, int i, int j) {
-    const float4* __restrict__ crt = a.crt;
-    const int W = a.W, H = a.H;
-    const float r_s = a.r_s;
-    const size_t q = (size_t)j * W + i;
-    const float4 cp = __ldg(&crt[q]);
-    const float rp = fminf(cp.w * 0.5f, r_s);
-    // a tap weighs only if d < R = rp + 1/2: per row, the columns of that
-    // disk (the bounds lean outwards by 1e-3 pixel; the taps they add weigh 0)
-    const float R = rp + 0.5f, R2 = R * R;
-    const int K = (int)floorf(R + 1e-3f);
-    // s(r - d) = clamp(r + 1/2 - d, 0, 1): the half folded into the radii
-    // (R here; for the neighbour min(c/2 + 1/2, r_s + 1/2))
-    const float Rq = r_s + 0.5f;
-    float3 S = f3(0, 0, 0);
-    float Ws = 0.f;
-    const int y0 = max(j - K, 0), y1 = min(j + K, H - 1);
-    for (int y = y0; y <= y1; ++y) {
-        const float dy = (float)(y - j), dy2 = dy * dy;
-        const int wr = (int)floorf(sqrtf(fmaxf(R2 - dy2, 0.f)) + 1e-3f);
-        const int x0 = max(i - wr, 0), x1 = min(i + wr, W - 1);
-        const float4* row = crt + (size_t)y * W;
-        float dx = (float)(x0 - i);
-#pragma unroll SP_UNROLL
-        for (int x = x0; x <= x1; ++x, dx += 1.f) {
-            const float4 c = __ldg(&row[x]);
-            const float d = sqrt_approx(fmaf(dx, dx, dy2));
-            // an untraced neighbour (written as (0, 0, 0, -1)) weighs
-            // clamp(-d, 0, 1) = 0 times colour 0: it adds nothing
-            const float wq = clamp01(R - d) * clamp01(fminf(fmaf(c.w, 0.5f, 0.5f), Rq) - d);
-            S.x = fmaf(wq, c.x, S.x);
-            S.y = fmaf(wq, c.y, S.y);
-            S.z = fmaf(wq, c.z, S.z);
-            Ws += wq;
-        }
-    }
-    spatial_finish(a, q, cp, S, Ws);
-}
+// A tile's traced pixels are few or many and their windows 1 to 33 rows, so
+// each pixel's rows are shared by SP_G threads: group g takes the source rows
+// y with y mod SP_G = g (absolute, so a pixel's sums do not depend on the
+// window of the pixel beside it), and the groups are added in order.
+constexpr int SP_G = 4;
 
-// One thread gathers the horizontally adjacent pixels (i, j) and (i + 1, j)
-// (tl, tr: which of them is traced) over the union of their windows: each
-// tap is loaded once, and the right pixel's distance to a tap is the left
-// pixel's distance to the previous tap (the same float operations), so both
-// sums equal spatial_pixel's bit for bit (the union only adds taps of weight
-// exactly 0).  An untraced pixel of the pair gets reach 0 and is not written.
-__device__ __forceinline__ void spatial_pair(const SpatialArgs& a, int i, int j, bool tl, bool tr) {
+struct PairSums {
+    float4 l, r;  // (S rgb, W) of the left and the right pixel
+};
+
+// One thread gathers group g's rows for the horizontally adjacent pixels
+// (i, j) and (i + 1, j) (tl, tr: which of them is traced) over the union of
+// their windows: each tap is loaded once, and the right pixel's distance to a
+// tap is the left pixel's distance to the previous tap (the same float
+// operations); the union only adds taps of weight exactly 0.  An untraced
+// pixel of the pair gets reach 0.
+__device__ __forceinline__ PairSums spatial_pair(const SpatialArgs& a, int i, int j, bool tl, bool tr, int g) {
     const float4* __restrict__ crt = a.crt;
     const int W = a.W, H = a.H;
     const float r_s = a.r_s, Rq = r_s + 0.5f;
     const size_t q = (size_t)j * W + i;
-    const float4 cl = tl ? __ldg(&crt[q]) : make_float4(0.f, 0.f, 0.f, -1.f);
-    const float4 cr = tr ? __ldg(&crt[q + 1]) : make_float4(0.f, 0.f, 0.f, -1.f);
-    const float Rl = tl ? fminf(cl.w * 0.5f, r_s) + 0.5f : 0.f;
-    const float Rr = tr ? fminf(cr.w * 0.5f, r_s) + 0.5f : 0.f;
+    // a tap weighs only if d < R = min(c/2, r_s) + 1/2: per row, the columns of
+    // that disk (the bounds lean outwards by 1e-3 pixel; the taps they add
+    // weigh 0).  s(r - d) = clamp(r + 1/2 - d, 0, 1): the half folded into the
+    // radii (R here; for the neighbour min(c/2 + 1/2, r_s + 1/2))
+    const float Rl = tl ? fminf(__ldg(&crt[q].w) * 0.5f, r_s) + 0.5f : 0.f;
+    const float Rr = tr ? fminf(__ldg(&crt[q + 1].w) * 0.5f, r_s) + 0.5f : 0.f;
     const float Rl2 = Rl * Rl, Rr2 = Rr * Rr;
     const int K = (int)floorf(fmaxf(Rl, Rr) + 1e-3f);
-    float3 Sl = f3(0, 0, 0), Sr = f3(0, 0, 0);
-    float Wl = 0.f, Wr = 0.f;
+    f32x2 lxy = 0ull, lzw = 0ull, rxy = 0ull, rzw = 0ull;  // (S.x, S.y), (S.z, W)
     const int y0 = max(j - K, 0), y1 = min(j + K, H - 1);
-    for (int y = y0; y <= y1; ++y) {
+    for (int y = y0 + ((g - y0) & (SP_G - 1)); y <= y1; y += SP_G) {
         const float dy = (float)(y - j), dy2 = dy * dy;
-        const int wl = (int)floorf(sqrtf(fmaxf(Rl2 - dy2, 0.f)) + 1e-3f);
-        const int wr = (int)floorf(sqrtf(fmaxf(Rr2 - dy2, 0.f)) + 1e-3f);
+        const int wl = (int)(sqrt_approx(fmaxf(Rl2 - dy2, 0.f)) + 1e-3f);
+        const int wr = (int)(sqrt_approx(fmaxf(Rr2 - dy2, 0.f)) + 1e-3f);
         const int x0 = max(min(i - wl, i + 1 - wr), 0), x1 = min(max(i + wl, i + 1 + wr), W - 1);
         const float4* row = crt + (size_t)y * W;
         float dx = (float)(x0 - i);
@@ -305,70 +316,56 @@ __device__ __forceinline__ void spatial_pair(const SpatialArgs& a, int i, int j,
         for (int x = x0; x <= x1; ++x, dx += 1.f) {
             const float4 c = __ldg(&row[x]);
             const float dl = sqrt_approx(fmaf(dx, dx, dy2)), dr = dprev;
+            // an untraced neighbour (written as (0, 0, 0, -1)) weighs
+            // clamp(-d, 0, 1) = 0 times colour 0: it adds nothing
             const float rq = fminf(fmaf(c.w, 0.5f, 0.5f), Rq);
-            const float ql = clamp01(Rl - dl) * clamp01(rq - dl);
-            const float qr = clamp01(Rr - dr) * clamp01(rq - dr);
-            Sl.x = fmaf(ql, c.x, Sl.x);
-            Sl.y = fmaf(ql, c.y, Sl.y);
-            Sl.z = fmaf(ql, c.z, Sl.z);
-            Wl += ql;
-            Sr.x = fmaf(qr, c.x, Sr.x);
-            Sr.y = fmaf(qr, c.y, Sr.y);
-            Sr.z = fmaf(qr, c.z, Sr.z);
-            Wr += qr;
+            const float ql = __saturatef(Rl - dl) * __saturatef(rq - dl);
+            const float qr = __saturatef(Rr - dr) * __saturatef(rq - dr);
+            const f32x2 cxy = pk2(c.x, c.y), czw = pk2(c.z, 1.f), qql = pk2(ql, ql), qqr = pk2(qr, qr);
+            lxy = ffma2(qql, cxy, lxy);
+            lzw = ffma2(qql, czw, lzw);
+            rxy = ffma2(qqr, cxy, rxy);
+            rzw = ffma2(qqr, czw, rzw);
             dprev = dl;
         }
     }
-    if (tl) spatial_finish(a, q, cl, Sl, Wl);
-    if (tr) spatial_finish(a, q + 1, cr, Sr, Wr);
+    const float2 l0 = unpk2(lxy), l1 = unpk2(lzw), r0 = unpk2(rxy), r1 = unpk2(rzw);
+    PairSums o;
+    o.l = make_float4(l0.x, l0.y, l1.x, l1.y);
+    o.r = make_float4(r0.x, r0.y, r1.x, r1.y);
+    return o;
 }
 
-// block = one T x T tile (T = 8 or 16), one thread per pixel: the tile's
-// traced pixels are compacted (row-major) so the threads that run all gather
-// for traced pixels, in one round; small blocks keep many tiles resident
-// where few of their pixels are traced
-constexpr int SP_TILE = 8, SP_THREADS = SP_TILE * SP_TILE;
-template <int T>
+// Block = one 16 x TH tile as 8 x TH horizontal pixel pairs, SP_G threads per
+// pair: the n pairs holding a traced pixel are compacted, thread t takes
+// group t / n of pair t mod n, so the threads that run fill whole warps and
+// all gather.  Bound by the latency of the taps (L1 hits): with one thread
+// per pair the widest windows (1089 serial taps) outlasted the rest of the
+// grid at 8-17% of the warps active.  75 -> 37 us at 1024x1024 (the fitting
+// step's frame), 194 -> 186 us at 1080p with half the pixels traced at random
+// CoCs (bound by issue there: lanes of unlike windows).
+constexpr int SP_TW = 16;
+template <int TH>
+constexpr int sp_threads() {
+    return SP_G * SP_TW * TH / 2;
+}
+template <int TH>
 __device__ __forceinline__ void spatial_body(const SpatialArgs& a, int bx, int by) {
-    constexpr int NT = T * T;
-    __shared__ unsigned char s_list[NT];
-    __shared__ int s_cnt[NT / 32];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int i0 = bx * T + (t % T), j0 = by * T + (t / T);
-    const bool traced = i0 < a.W && j0 < a.H && __ldg(&a.crt[(size_t)j0 * a.W + i0].w) >= 0.f;
-    const unsigned tm = __ballot_sync(0xffffffffu, traced);
-    if (lane == 0) s_cnt[w] = __popc(tm);
-    __syncthreads();
-    int off = 0, n = 0;
-#pragma unroll
-    for (int c = 0; c < NT / 32; ++c) {
-        off += c < w ? s_cnt[c] : 0;
-        n += s_cnt[c];
-    }
-    if (traced) s_list[off + __popc(tm & ((1u << lane) - 1u))] = (unsigned char)t;
-    __syncthreads();
-    if (t < n) {
-        const int li = s_list[t];
-        spatial_pixel(a, bx * T + (li % T), by * T + (li / T));
-    }
-}
-
-// block = one 16x8 tile as 8x8 horizontal pixel pairs, one thread per pair:
-// the pairs holding a traced pixel are compacted so the threads that run
-// all gather, in one round
-constexpr int SPP_TW = 16, SPP_TH = 8, SPP_THREADS = SPP_TW * SPP_TH / 2;
-__global__ void __launch_bounds__(SPP_THREADS) k_spatial(SpatialArgs a) {
-    constexpr int NP = SPP_THREADS, PW = SPP_TW / 2;
-    __shared__ unsigned char s_list[NP];
+    constexpr int PW = SP_TW / 2, NP = PW * TH;
+    __shared__ unsigned short s_list[NP];
     __shared__ int s_cnt[NP / 32];
+    __shared__ float4 s_part[2][sp_threads<TH>()];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int i0 = blockIdx.x * SPP_TW + 2 * (t % PW), j0 = blockIdx.y * SPP_TH + t / PW;
-    const bool row_in = j0 < a.H;
-    const bool tl = row_in && i0 < a.W && __ldg(&a.crt[(size_t)j0 * a.W + i0].w) >= 0.f;
-    const bool tr = row_in && i0 + 1 < a.W && __ldg(&a.crt[(size_t)j0 * a.W + i0 + 1].w) >= 0.f;
-    const bool act = tl || tr;
-    const unsigned tm = __ballot_sync(0xffffffffu, act);
-    if (lane == 0) s_cnt[w] = __popc(tm);
+    bool tl = false, tr = false;
+    unsigned tm = 0;
+    if (t < NP) {  // whole warps
+        const int i0 = bx * SP_TW + 2 * (t % PW), j0 = by * TH + t / PW;
+        const bool row_in = j0 < a.H;
+        tl = row_in && i0 < a.W && __ldg(&a.crt[(size_t)j0 * a.W + i0].w) >= 0.f;
+        tr = row_in && i0 + 1 < a.W && __ldg(&a.crt[(size_t)j0 * a.W + i0 + 1].w) >= 0.f;
+        tm = __ballot_sync(0xffffffffu, tl || tr);
+        if (lane == 0) s_cnt[w] = __popc(tm);
+    }
     __syncthreads();
     int off = 0, n = 0;
 #pragma unroll
@@ -376,20 +373,39 @@ __global__ void __launch_bounds__(SPP_THREADS) k_spatial(SpatialArgs a) {
         off += c < w ? s_cnt[c] : 0;
         n += s_cnt[c];
     }
+    if (n == 0) return;  // the whole block
     // the pair's slot and which of its pixels are traced
-    if (act) s_list[off + __popc(tm & ((1u << lane) - 1u))] = (unsigned char)(t | (tl ? 0x80 : 0) | (tr ? 0x40 : 0));
+    if (tl || tr)
+        s_list[off + __popc(tm & ((1u << lane) - 1u))] = (unsigned short)(t | (tl ? 0x8000 : 0) | (tr ? 0x4000 : 0));
     __syncthreads();
-    if (t < n) {
-        const int e = s_list[t], p = e & 0x3f;
-        spatial_pair(a, blockIdx.x * SPP_TW + 2 * (p % PW), blockIdx.y * SPP_TH + p / PW, (e & 0x80) != 0,
-                     (e & 0x40) != 0);
+    if (t < SP_G * n) {
+        const int g = t / n, e = s_list[t - g * n], p = e & 0x3fff;
+        const PairSums o = spatial_pair(a, bx * SP_TW + 2 * (p % PW), by * TH + p / PW, (e & 0x8000) != 0,
+                                        (e & 0x4000) != 0, g);
+        s_part[0][t] = o.l;
+        s_part[1][t] = o.r;
+    }
+    __syncthreads();
+    for (int k = t; k < 2 * n; k += sp_threads<TH>()) {  // pixel k & 1 of pair k / 2
+        const int e = s_list[k >> 1], p = e & 0x3fff;
+        if (!(e & ((k & 1) ? 0x4000 : 0x8000))) continue;
+        float4 S = s_part[k & 1][k >> 1];
+#pragma unroll
+        for (int g = 1; g < SP_G; ++g) S = add4(S, s_part[k & 1][g * n + (k >> 1)]);
+        const size_t q = (size_t)(by * TH + p / PW) * a.W + bx * SP_TW + 2 * (p % PW) + (k & 1);
+        spatial_finish(a, q, __ldg(&a.crt[q]), f3(S.x, S.y, S.z), S.w);
     }
 }
-template <int T>
-__global__ void __launch_bounds__(T * T) k_spatial_batch(const SpatialArgs* __restrict__ a, BatchGrid g) {
+
+constexpr int SP_TILE = 8;  // tile height
+__global__ void __launch_bounds__(sp_threads<SP_TILE>(), 1024 / sp_threads<SP_TILE>()) k_spatial(SpatialArgs a) {
+    spatial_body<SP_TILE>(a, blockIdx.x, blockIdx.y);
+}
+template <int TH>
+__global__ void __launch_bounds__(sp_threads<TH>(), 1024 / sp_threads<TH>()) k_spatial_batch(const SpatialArgs* __restrict__ a, BatchGrid g) {
     int v, bx, by;
     g.locate(blockIdx.x, v, bx, by);
-    spatial_body<T>(batch_record(a, v), bx, by);
+    spatial_body<TH>(batch_record(a, v), bx, by);
 }
 
 TemporalArgs temporal_args(const float* rt, const hdof_gbuf* in, const uint8_t* spp, const hdof_camera* cam,
@@ -423,9 +439,9 @@ TemporalArgs temporal_args(const float* rt, const hdof_gbuf* in, const uint8_t* 
 
 int launch_spatial(const float4* crt, const float2* mom, const uint8_t* hlen, int W, int H, float r_s, float var_ref,
                    float4* crec, float4* aux, cudaStream_t s) {
-    dim3 g2((W + SPP_TW - 1) / SPP_TW, (H + SPP_TH - 1) / SPP_TH);
+    dim3 g2((W + SP_TW - 1) / SP_TW, (H + SP_TILE - 1) / SP_TILE);
     ProfScope ps_("spatial", s);
-    k_spatial<<<g2, SPP_THREADS, 0, s>>>(SpatialArgs{crt, mom, hlen, W, H, r_s, var_ref, crec, aux});
+    k_spatial<<<g2, sp_threads<SP_TILE>(), 0, s>>>(SpatialArgs{crt, mom, hlen, W, H, r_s, var_ref, crec, aux});
     HDOF_LAUNCHED("spatial reconstruction");
     return HDOF_OK;
 }
@@ -492,7 +508,7 @@ void spatial_fill(const hdof_view& v, const ViewWs& w, unsigned*, void* dst, int
                     v.hist_out.hlen, v.cam.width, v.cam.height, v.params.r_s, v.params.var_ref,
                     reinterpret_cast<float4*>(v.crec), nullptr};
     const int T = w.spatial_tile == 16 ? 16 : SP_TILE;
-    *gx = (v.cam.width + T - 1) / T;
+    *gx = (v.cam.width + SP_TW - 1) / SP_TW;
     *gy = (v.cam.height + T - 1) / T;
 }
 void spatial_launch_batch(const void* args, BatchGrid g, int blocks, cudaStream_t s) {
@@ -500,8 +516,8 @@ void spatial_launch_batch(const void* args, BatchGrid g, int blocks, cudaStream_
 }
 void spatial_launch_batch_tile(const void* args, BatchGrid g, int blocks, int tile, cudaStream_t s) {
     ProfScope ps_("batch_spatial", s);
-    if (tile == 16) k_spatial_batch<16><<<blocks, 256, 0, s>>>(static_cast<const SpatialArgs*>(args), g);
-    else k_spatial_batch<SP_TILE><<<blocks, SP_THREADS, 0, s>>>(static_cast<const SpatialArgs*>(args), g);
+    if (tile == 16) k_spatial_batch<16><<<blocks, sp_threads<16>(), 0, s>>>(static_cast<const SpatialArgs*>(args), g);
+    else k_spatial_batch<SP_TILE><<<blocks, sp_threads<SP_TILE>(), 0, s>>>(static_cast<const SpatialArgs*>(args), g);
 }
 
 }  // namespace hdof

@@ -565,6 +565,32 @@ def test_reconstruct(orc, seed, W, Hh, moved, alpha_k):
     assert np.all(host(crt)[~tr][:, 3] == -1.0)
 
 
+@pytest.mark.parametrize("W,Hh,density", [(1, 40, 1.0), (17, 9, 0.02), (33, 8, 1.0), (50, 21, 0.05), (16, 16, 0.5)])
+def test_spatial_sparse_and_edges(orc, W, Hh, density):
+    """The spatial gather where a tile holds one traced pair, none, or all of
+    them, at image edges and odd widths, with windows wider than the image.
+    Sums of at most 33^2 positive weights: as test_reconstruct."""
+    rng = np.random.default_rng(W * 100 + Hh)
+    spp = (8 * (rng.uniform(size=(Hh, W)) < density)).astype(np.uint8)
+    spp[Hh // 2, W // 2] = 8
+    cam = hi.Camera(width=W, height=Hh).f32()
+    rt, gb, hist = hi.random_rt(W, Hh, spp, seed=1), hi.random_gbuffer(max(W, 8), max(Hh, 8), seed=1), None
+    gb = {k: v[:Hh, :W] for k, v in gb.items()}
+    hist = hi.random_history(W, Hh, seed=1)
+    p = hi.room_params(camera_moved=0, r_s=16.0)
+    hout = H.History(W, Hh)
+    z = lambda *c: torch.zeros((Hh, W) + c, dtype=torch.float32, device="cuda")  # noqa: E731
+    crt, hacc, crec = z(4), z(), z(4)
+    H.hdof_reconstruct(dev(rt), gbuf_from(gb["nd"], gb["col"], gb["mv"]), dev(spp), cam, cam,
+                       hi.Lens(3.0, 0.02, 0.05).f32(), p, history_from(hist), hout, crt, hacc, crec)
+    H.hdof_sync()
+    ref = orc.spatial(p, host(crt).astype(np.float64), spp, host(hout.mom).astype(np.float64), host(hout.hlen))
+    tr = spp > 0
+    got = host(crec)
+    assert frac_close(got[tr][:, :3], ref[tr][:, :3], 1e-4, 1e-4) == 1.0, report("crec", got[tr], ref[tr])
+    assert not got[~tr].any()
+
+
 # --------------------------------------------------------------- composite --
 
 def test_composite(orc):
