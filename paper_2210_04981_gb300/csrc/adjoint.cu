@@ -54,19 +54,33 @@ __device__ __forceinline__ float wn_slope(float c) { return (c > -HDOF_SQRT2 && 
 __device__ __forceinline__ float dot3f(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ __forceinline__ float3 ldf3(const float4& v) { return f3(v.x, v.y, v.z); }
 
-// block sum of a per-thread (float, float) in double, fixed order; lane 0 of
-// warp 0 writes the block's partial
+// A sum carried as an unevaluated pair hi + lo of floats (Knuth's TwoSum; 48
+// bits).  Sums of a block's few hundred floats in it agree with double ones
+// to far below the float result's rounding, at FP32 rates: FP64 adds run at
+// 1/64 of them here, and ten shuffle steps of doubles per thread held up the
+// composite adjoint (37 us at 1024x1024, 30 so) and the replay's (32 and 26).
+struct Pair {
+    float hi, lo;
+};
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+    const float s = __fadd_rn(a.hi, b.hi), bb = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
+    return Pair{s, __fadd_rn(__fadd_rn(a.lo, b.lo), e)};
+}
+
+// block sum of a per-thread (float, float), fixed order: pairs of floats
+// within a warp, double across the warps; thread 0 writes the block's partial
 __device__ __forceinline__ void block_partial(float2 v, double2* partial) {
     __shared__ double red[2][32];
-    double a = v.x, b = v.y;
+    Pair a{v.x, 0.f}, b{v.y, 0.f};
     for (int o = 16; o; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
+        a = pair_add(a, Pair{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)});
+        b = pair_add(b, Pair{__shfl_xor_sync(0xffffffffu, b.hi, o), __shfl_xor_sync(0xffffffffu, b.lo, o)});
     }
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
     if (l == 0) {
-        red[0][w] = a;
-        red[1][w] = b;
+        red[0][w] = (double)a.hi + (double)a.lo;
+        red[1][w] = (double)b.hi + (double)b.lo;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -315,69 +329,107 @@ __global__ void __launch_bounds__(256) k_spatial_bwd_prep(const float4* __restri
 }
 
 // spatial adjoint, part 2 (per traced pixel x over its own window): x as a
-// gathered sample of its neighbours and x as a gatherer
-__global__ void __launch_bounds__(256) k_spatial_bwd(const float4* __restrict__ crt, const float4* __restrict__ spb,
-                                                     int W, int H, float r_s, float4* __restrict__ gcrt) {
-    // block = one 16x16 tile; its traced pixels are compacted (row-major) so
-    // that every warp which runs works on traced pixels only
-    __shared__ unsigned char s_list[256];
-    __shared__ int s_wcnt[8];
-    const int t = threadIdx.x, lane = t & 31;
-    bool traced = false;
-    {
-        const int i0 = blockIdx.x * 16 + (t & 15), j0 = blockIdx.y * 16 + (t >> 4);
-        if (i0 < W && j0 < H) traced = __ldg(&crt[(size_t)j0 * W + i0].w) >= 0.f;
+// gathered sample of its neighbours and x as a gatherer.  Block = one 16x8
+// tile as pixel pairs; its pairs holding a traced pixel are compacted and
+// SBG threads share a pair's rows (y mod SBG), as in the forward gather: one
+// thread per pixel took 131 us at 1024x1024 with 20% of the warps active,
+// this 60 us (few tiles are traced there: the longest still set the time).
+constexpr int SB_TW = 16, SB_TH = 8, SB_NP = SB_TW * SB_TH / 2, SBG = 4, SB_THREADS = SB_NP * SBG;
+
+// one pixel x's share of a tap: gC += sy sx a_y, gcx += sy s'x (x gathered by y + x gathering y)
+__device__ __forceinline__ void spatial_bwd_tap(float4& acc, float R, float d, float rq, const float3& Cx,
+                                                const float4& bx, const float4& cy, const float4& by) {
+    const float ux = R - d, sx = __saturatef(ux), sy = __saturatef(rq - d);
+    const float spx = (ux > 0.f && ux < 1.f) ? sy : 0.f, w = sy * sx;
+    acc.x = fmaf(w, by.x, acc.x);
+    acc.y = fmaf(w, by.y, acc.y);
+    acc.z = fmaf(w, by.z, acc.z);
+    const float v = (dot3f(ldf3(by), Cx) - by.w) + (dot3f(ldf3(bx), ldf3(cy)) - bx.w);
+    acc.w = fmaf(spx, v, acc.w);
+}
+
+__global__ void __launch_bounds__(SB_THREADS, 3) k_spatial_bwd(const float4* __restrict__ crt,
+                                                               const float4* __restrict__ spb, int W, int H, float r_s,
+                                                               float4* __restrict__ gcrt) {
+    constexpr int PW = SB_TW / 2;
+    __shared__ unsigned short s_list[SB_NP];
+    __shared__ int s_cnt[SB_NP / 32];
+    __shared__ float4 s_part[2][SB_THREADS];
+    const int t = threadIdx.x, lane = t & 31, wi = t >> 5, bx0 = blockIdx.x * SB_TW, by0 = blockIdx.y * SB_TH;
+    bool tl = false, tr = false;
+    unsigned tm = 0;
+    if (t < SB_NP) {  // whole warps
+        const int i0 = bx0 + 2 * (t % PW), j0 = by0 + t / PW;
+        tl = j0 < H && i0 < W && __ldg(&crt[(size_t)j0 * W + i0].w) >= 0.f;
+        tr = j0 < H && i0 + 1 < W && __ldg(&crt[(size_t)j0 * W + i0 + 1].w) >= 0.f;
+        tm = __ballot_sync(0xffffffffu, tl || tr);
+        if (lane == 0) s_cnt[wi] = __popc(tm);
     }
-    const unsigned tm = __ballot_sync(0xffffffffu, traced);
-    if (lane == 0) s_wcnt[t >> 5] = __popc(tm);
     __syncthreads();
     int off = 0, n = 0;
-    for (int k = 0; k < 8; ++k) {
-        off += k < (t >> 5) ? s_wcnt[k] : 0;
-        n += s_wcnt[k];
+#pragma unroll
+    for (int k = 0; k < SB_NP / 32; ++k) {
+        off += k < wi ? s_cnt[k] : 0;
+        n += s_cnt[k];
     }
-    if (traced) s_list[off + __popc(tm & ((1u << lane) - 1u))] = (unsigned char)t;
+    if (n == 0) return;  // the whole block
+    if (tl || tr)
+        s_list[off + __popc(tm & ((1u << lane) - 1u))] = (unsigned short)(t | (tl ? 0x8000 : 0) | (tr ? 0x4000 : 0));
     __syncthreads();
-    if (t >= n) return;
-    const int li = s_list[t];
-    const int i = blockIdx.x * 16 + (li & 15), j = blockIdx.y * 16 + (li >> 4);
-    const size_t q = (size_t)j * W + i;
-    const float4 cx = crt[q];
-    const float rx = fminf(cx.w * 0.5f, r_s);
-    const float rpx = cx.w * 0.5f < r_s ? 0.5f : 0.f;
-    const float4 bx = spb[q];
-    const float3 Cx = ldf3(cx), ax = ldf3(bx);
-    // a neighbour takes part only if d < R = rx + 1/2: per row, the columns
-    // of that disk (bounds lean outwards by 1e-3 pixel; taps they add weigh 0)
-    const float R = rx + 0.5f, R2 = R * R;
-    const int K = (int)floorf(R + 1e-3f);
-    float3 gC = f3(0, 0, 0);
-    float gcx = 0.f;
-    const int y0 = max(j - K, 0), y1 = min(j + K, H - 1);
-    for (int y = y0; y <= y1; ++y) {
-        const float dy = (float)(y - j), dy2 = dy * dy;
-        const int wr = (int)floorf(sqrtf(fmaxf(R2 - dy2, 0.f)) + 1e-3f);
-        const int x0 = max(i - wr, 0), x1 = min(i + wr, W - 1);
-        for (int x = x0; x <= x1; ++x) {
-            float dx = (float)(x - i);
-            size_t qq = (size_t)y * W + x;
-            // branch-free: untraced neighbours (and their unwritten spb) are
-            // selected away, out-of-disk pairs weigh exactly zero
-            const float4 cy = __ldg(&crt[qq]), by = __ldg(&spb[qq]);
-            const bool ty = cy.w >= 0.f;
-            float d = sqrt_approx(fmaf(dx, dx, dy2));
-            float ux = R - d, uy = fminf(fmaf(cy.w, 0.5f, 0.5f), r_s + 0.5f) - d;
-            float sx = clamp01(ux), sy = ty ? clamp01(uy) : 0.f;
-            float spx = (ux > 0.f && ux < 1.f) ? 1.f : 0.f;
-            const float3 ay = ty ? ldf3(by) : f3(0.f, 0.f, 0.f);
-            const float byw = ty ? by.w : 0.f;
-            gC = gC + (sy * sx) * ay;
-            gcx += sy * spx * (dot3f(ay, Cx) - byw);               // x gathered by y
-            gcx += spx * sy * (dot3f(ax, ldf3(cy)) - bx.w);        // x gathering y
+    if (t < SBG * n) {
+        const int g = t / n, e = s_list[t - g * n], p = e & 0x3fff;
+        const int i = bx0 + 2 * (p % PW), j = by0 + p / PW;
+        const size_t q = (size_t)j * W + i;
+        const bool hl = e & 0x8000, hr = e & 0x4000;
+        const float4 none = make_float4(0.f, 0.f, 0.f, -1.f), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 cl = hl ? __ldg(&crt[q]) : none, cr = hr ? __ldg(&crt[q + 1]) : none;
+        const float4 bl = hl ? __ldg(&spb[q]) : zero, br = hr ? __ldg(&spb[q + 1]) : zero;
+        // a neighbour takes part only if d < R = min(c/2, r_s) + 1/2 (0 for an
+        // untraced pixel of the pair): per row, the columns of that disk
+        // (bounds lean outwards by 1e-3 pixel; taps they add weigh 0)
+        const float Rl = hl ? fminf(cl.w * 0.5f, r_s) + 0.5f : 0.f, Rr = hr ? fminf(cr.w * 0.5f, r_s) + 0.5f : 0.f;
+        const float Rl2 = Rl * Rl, Rr2 = Rr * Rr, Rq = r_s + 0.5f;
+        const float3 Cl = ldf3(cl), Cr = ldf3(cr);
+        const int K = (int)floorf(fmaxf(Rl, Rr) + 1e-3f);
+        float4 al = zero, ar = zero;  // (gC, gcx)
+        const int y0 = max(j - K, 0), y1 = min(j + K, H - 1);
+        for (int y = y0 + ((g - y0) & (SBG - 1)); y <= y1; y += SBG) {
+            const float dy = (float)(y - j), dy2 = dy * dy;
+            const int wl = (int)floorf(sqrtf(fmaxf(Rl2 - dy2, 0.f)) + 1e-3f);
+            const int wr = (int)floorf(sqrtf(fmaxf(Rr2 - dy2, 0.f)) + 1e-3f);
+            const int x0 = max(min(i - wl, i + 1 - wr), 0), x1 = min(max(i + wl, i + 1 + wr), W - 1);
+            float dx = (float)(x0 - i);
+            float dprev = sqrt_approx(fmaf(dx - 1.f, dx - 1.f, dy2));
+            for (int x = x0; x <= x1; ++x, dx += 1.f) {
+                const size_t qq = (size_t)y * W + x;
+                // branch-free: untraced neighbours (and their unwritten spb)
+                // are selected away, out-of-disk pairs weigh exactly zero
+                const float4 cy = __ldg(&crt[qq]);
+                float4 by = __ldg(&spb[qq]);
+                const bool ty = cy.w >= 0.f;
+                by = make_float4(ty ? by.x : 0.f, ty ? by.y : 0.f, ty ? by.z : 0.f, ty ? by.w : 0.f);
+                const float rq = ty ? fminf(fmaf(cy.w, 0.5f, 0.5f), Rq) : -1.f;
+                const float d = sqrt_approx(fmaf(dx, dx, dy2));
+                spatial_bwd_tap(al, Rl, d, rq, Cl, bl, cy, by);
+                spatial_bwd_tap(ar, Rr, dprev, rq, Cr, br, cy, by);
+                dprev = d;
+            }
         }
+        s_part[0][t] = al;
+        s_part[1][t] = ar;
     }
-    float4 g = gcrt[q];
-    gcrt[q] = make_float4(g.x + gC.x, g.y + gC.y, g.z + gC.z, g.w + gcx * rpx);
+    __syncthreads();
+    for (int k = t; k < 2 * n; k += SB_THREADS) {  // pixel k & 1 of pair k / 2
+        const int e = s_list[k >> 1], p = e & 0x3fff;
+        if (!(e & ((k & 1) ? 0x4000 : 0x8000))) continue;
+        float4 S = s_part[k & 1][k >> 1];
+#pragma unroll
+        for (int g = 1; g < SBG; ++g) S = add4(S, s_part[k & 1][g * n + (k >> 1)]);
+        const size_t q = (size_t)(by0 + p / PW) * W + bx0 + 2 * (p % PW) + (k & 1);
+        const float rpx = __ldg(&crt[q].w) * 0.5f < r_s ? 0.5f : 0.f;
+        const float4 g0 = gcrt[q];
+        gcrt[q] = make_float4(g0.x + S.x, g0.y + S.y, g0.z + S.z, g0.w + S.w * rpx);
+    }
 }
 
 // temporal + replay adjoint (per traced pixel, forward recomputed): the
@@ -504,9 +556,11 @@ __device__ __forceinline__ float2 area_and_slope(const float4* tab, int n, float
 // post-filter adjoint, part 1 (per pixel p): factors of dL/d(near weight) =
 // A . C_q - E and dL/d(far weight) = Af . C_q - Ef, and the sharp-colour
 // fallback of an empty far layer
-// Written per pixel q: (A, E) and (Af, Ef) in two planes, each split by
-// pixel-index parity (even pixels, then odd), and kb_q = 1 / (kz_rel z_q) of
-// the forward's depth test, row-major.
+// Written per pixel q, row-major: (A, E) and (Af, Ef) in two planes, and
+// kb_q = 1 / (kz_rel z_q) of the forward's depth test.
+__host__ __device__ inline size_t pfb_plane(int W, int H) {  // an even count: both planes' pairs are 32-byte aligned
+    return ((size_t)W * H + 1) & ~size_t(1);
+}
 __global__ void __launch_bounds__(256) k_pf_bwd_prep(const float4* __restrict__ aux, const float4* __restrict__ gpp,
                                                      const float4* __restrict__ nd, float kz_rel, int W, int H,
                                                      float4* __restrict__ pfb, float* __restrict__ kbp,
@@ -514,7 +568,6 @@ __global__ void __launch_bounds__(256) k_pf_bwd_prep(const float4* __restrict__ 
     int i = blockIdx.x * 32 + (threadIdx.x & 31), j = blockIdx.y * 8 + (threadIdx.x >> 5);
     if (i >= W || j >= H) return;
     size_t q = (size_t)j * W + i;
-    const size_t px = (size_t)W * H, qs = (q >> 1) + (q & 1) * ((px + 1) >> 1);
     kbp[q] = 1.f / (kz_rel * __ldg(&nd[q].w));
     float4 an = aux[2 * q], af = aux[2 * q + 1];
     float3 g = ldf3(gpp[q]), N = ldf3(an), F = ldf3(af);
@@ -532,8 +585,8 @@ __global__ void __launch_bounds__(256) k_pf_bwd_prep(const float4* __restrict__ 
         float4 gc = gcol[q];  // F is this pixel's sharp colour
         gcol[q] = make_float4(gc.x + (1.f - alpha) * g.x, gc.y + (1.f - alpha) * g.y, gc.z + (1.f - alpha) * g.z, 0.f);
     }
-    pfb[qs] = make_float4(A.x, A.y, A.z, E);
-    pfb[px + qs] = make_float4(Af.x, Af.y, Af.z, Ef);
+    pfb[q] = make_float4(A.x, A.y, A.z, E);
+    pfb[pfb_plane(W, H) + q] = make_float4(Af.x, Af.y, Af.z, Ef);
 }
 
 // per source pixel: the radius and the layer weights of the forward map and
@@ -560,153 +613,205 @@ __device__ __forceinline__ PfSrc pf_src(float zq, const LensD& L, float rmax, co
     return o;
 }
 
+// One layer's sums over the targets of the four sources of a thread, two
+// sources (a row's left and right pixel) to a register pair so that one
+// packed FMA serves both: per row k, sum s A (gx, gy, gz), sum t s and
+// sum t s' with t = A . C_q - E (times the depth test in the far layer),
+// s = clamp(R - d, 0, 1) and s' its slope.
 struct PfBwdAcc {
-    float3 gC;
-    float S1, S2, S3, S4;
+    f32x2 gx[2], gy[2], gz[2], S1[2], S2[2];
+};
+struct PfBwdSrc {
+    float R[4], zq[4];
+    f32x2 Cx[2], Cy[2], Cz[2];
 };
 
-// the four sources of a thread against one target: sources (i, j) and
-// (i, j + 1) get fresh distances, sources (i + 1, j) and (i + 1, j + 1) the
-// previous target's (the same offsets, so the same floats), carried in c
-struct PfBwdSrc {
-    float zq[4], R[4], wnia[4], fia[4];
-    float3 Cq[4];
-};
-__device__ __forceinline__ void pf_bwd_tap(PfBwdAcc (&acc)[4], float (&c)[2], const PfBwdSrc& src, float dx,
-                                           float dy0, float dy1, float ka, float kb, const float4& bn,
-                                           const float4& bf) {
-    const float3 An = ldf3(bn), Af = ldf3(bf);
+// the four sources of a thread against one target: row k's left source gets a
+// fresh distance, its right source the previous target's (the same offsets,
+// so the same floats), carried in c
+template <bool FAR>
+__device__ __forceinline__ void pf_bwd_tap(PfBwdAcc& acc, float (&c)[2], const PfBwdSrc& src, float dx, float dy0,
+                                           float dy1, float ka, float kb, const float4& b) {
+    const f32x2 Ax = pk2(b.x, b.x), Ay = pk2(b.y, b.y), Az = pk2(b.z, b.z), E = pk2(-b.w, -b.w);
     const float dx2 = dx * dx;
-    const float e0 = sqrt_approx(dx2 + dy0), e2 = sqrt_approx(dx2 + dy1);
-    const float d[4] = {e0, c[0], e2, c[1]};
-    c[0] = e0;
-    c[1] = e2;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float u = src.R[k] - d[k];
-        const float sw = __saturatef(u), sp = (u > 0.f && u < 1.f) ? 1.f : 0.f;
-        const float kz = __saturatef(fmaf(-src.zq[k], kb, ka));
-        const float an = sw * src.wnia[k], af = sw * src.fia[k] * kz;
-        acc[k].gC.x = fmaf(an, An.x, fmaf(af, Af.x, acc[k].gC.x));
-        acc[k].gC.y = fmaf(an, An.y, fmaf(af, Af.y, acc[k].gC.y));
-        acc[k].gC.z = fmaf(an, An.z, fmaf(af, Af.z, acc[k].gC.z));
-        const float tn = dot3f(An, src.Cq[k]) - bn.w, tf = (dot3f(Af, src.Cq[k]) - bf.w) * kz;
-        acc[k].S1 = fmaf(tn, sw, acc[k].S1);
-        acc[k].S2 = fmaf(tn, sp, acc[k].S2);
-        acc[k].S3 = fmaf(tf, sw, acc[k].S3);
-        acc[k].S4 = fmaf(tf, sp, acc[k].S4);
+    for (int k = 0; k < 2; ++k) {
+        const float d = sqrt_approx(dx2 + (k ? dy1 : dy0));
+        const float ul = src.R[2 * k] - d, ur = src.R[2 * k + 1] - c[k];
+        c[k] = d;
+        const float sl = __saturatef(ul), sr = __saturatef(ur);
+        float kl = 1.f, kr = 1.f;
+        if (FAR) {
+            kl = __saturatef(fmaf(-src.zq[2 * k], kb, ka));
+            kr = __saturatef(fmaf(-src.zq[2 * k + 1], kb, ka));
+        }
+        // on the rim, 0 < u < 1, the clamp is the identity (and its slope 1)
+        const f32x2 s = pk2(FAR ? sl * kl : sl, FAR ? sr * kr : sr), sp = pk2(sl == ul ? kl : 0.f, sr == ur ? kr : 0.f);
+        const f32x2 t = ffma2(Az, src.Cz[k], ffma2(Ay, src.Cy[k], ffma2(Ax, src.Cx[k], E)));
+        acc.gx[k] = ffma2(s, Ax, acc.gx[k]);
+        acc.gy[k] = ffma2(s, Ay, acc.gy[k]);
+        acc.gz[k] = ffma2(s, Az, acc.gz[k]);
+        acc.S1[k] = ffma2(t, s, acc.S1[k]);
+        acc.S2[k] = ffma2(t, sp, acc.S2[k]);
+    }
+}
+
+constexpr int PBT = 16, PBG = 4;  // source tile edge, thread groups over the target rows
+
+// One layer's sums of the 2x2 source block at (i, j) over the rows g, g + PBG,
+// ... of its window: per target row, the columns closer than the layer's
+// reach R to one of the four (bounds lean outwards by 1e-3 pixel; other
+// pairs weigh zero, and so do their slopes)
+template <bool FAR>
+__device__ __forceinline__ void pf_bwd_layer(PfBwdAcc& acc, const PfBwdSrc& src, float R, int g, int i, int j, int W,
+                                             int H, float ka, const float4* __restrict__ rec,
+                                             const float* __restrict__ kbp) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) acc.gx[k] = acc.gy[k] = acc.gz[k] = acc.S1[k] = acc.S2[k] = 0ull;
+    const float R2 = R * R;
+    const int G = (int)floorf(R + 1e-3f);
+    const float2* __restrict__ kb2 = reinterpret_cast<const float2*>(kbp);
+    const int y0 = max(j - G, 0), y1 = min(j + 1 + G, H - 1);
+    for (int y = y0 + g; y <= y1; y += PBG) {
+        const float dy = (float)(y - j);
+        const float dy0 = dy * dy, dy1 = (dy - 1.f) * (dy - 1.f);
+        const float dmin = dy >= 0.f && dy <= 1.f ? 0.f : fminf(dy0, dy1);
+        const int w = (int)(sqrt_approx(fmaxf(R2 - dmin, 0.f)) + 1e-3f);
+        const int x0 = max(i - w, 0), x1 = min(i + 1 + w, W - 1);
+        float dx = (float)(x0 - i);
+        const float dm = (dx - 1.f) * (dx - 1.f);
+        float c[2] = {sqrt_approx(dm + dy0), sqrt_approx(dm + dy1)};
+        // targets in (even, odd) index pairs; a lone odd first and even last on their own
+        unsigned q = (unsigned)y * W + x0;
+        const unsigned qend = (unsigned)y * W + x1 + 1;
+        if (q & 1) {
+            pf_bwd_tap<FAR>(acc, c, src, dx, dy0, dy1, ka, FAR ? __ldg(&kbp[q]) : 0.f, __ldg(&rec[q]));
+            ++q;
+            dx += 1.f;
+        }
+        const unsigned mend = qend >> 1;
+#pragma unroll 1
+        for (unsigned m = q >> 1; m < mend; ++m, dx += 2.f) {
+            const float2 kb = FAR ? __ldg(&kb2[m]) : make_float2(0.f, 0.f);
+            float4 b0, b1;
+            ld_rec_pair(rec + 2 * (size_t)m, b0, b1);
+            pf_bwd_tap<FAR>(acc, c, src, dx, dy0, dy1, ka, kb.x, b0);
+            pf_bwd_tap<FAR>(acc, c, src, dx + 1.f, dy0, dy1, ka, kb.y, b1);
+        }
+        if (qend & 1)
+            pf_bwd_tap<FAR>(acc, c, src, dx, dy0, dy1, ka, FAR ? __ldg(&kbp[qend - 1]) : 0.f,
+                            __ldg(&rec[qend - 1]));
     }
 }
 
 // post-filter adjoint, part 2: per source pixel q over the target pixels its
 // soft disk reaches, the colour gradient and the gradient of q's CoC.  One
-// block per 16x16 tile of sources, 64 threads; thread t takes the 2x2 source
-// block at (2 (t & 7), 2 (t >> 3)), so every target it loads serves four
-// sources.  The loop covers, per target row, the columns closer than the
-// tile's largest radius to one of the four (other pairs have zero weight) and
-// is branch-free; the depth test is the forward's clamp(ka - z_q kb_p).
+// block per 16x16 tile of sources, PBG groups of 64 threads; thread t of a
+// group takes the 2x2 source block at (2 (t & 7), 2 (t >> 3)) over the
+// group's target rows, so every target it loads serves four sources.  The
+// near and the far layer run one after the other, each only where a source
+// of the tile feeds it (a source outside the focus zone feeds one) and as far
+// as the largest radius that does; the depth test is the forward's
+// clamp(ka - z_q kb_p).  The layer weights w/a and (1-w)/a of a source are
+// factored out of its sums.  Thread p finishes source p of the tile.  Bound
+// by issue (about 11 instructions per source and target, 58% busy) and the
+// latency of the target loads.  Both layers in one loop over every target
+// with scalar FMAs took 383 us at 1024x1024 (radii to 10 px, all far); this
+// 219 us.
 #ifndef HDOF_PFB_MINB
-#define HDOF_PFB_MINB 8  // resident blocks per SM the post-filter adjoint's register budget targets (128 registers)
+#define HDOF_PFB_MINB 3  // resident blocks per SM the register budget targets (80 registers)
 #endif
-__global__ void __launch_bounds__(64, HDOF_PFB_MINB) k_pf_bwd(const float4* __restrict__ nd, const float4* __restrict__ col,
+__global__ void __launch_bounds__(64 * PBG, HDOF_PFB_MINB) k_pf_bwd(const float4* __restrict__ nd, const float4* __restrict__ col,
                                                const float4* __restrict__ pfb, const float* __restrict__ kbp,
                                                const float4* __restrict__ tab, int ntab, int W, int H, LensD L,
                                                float rmax, float kz_rel, float4* __restrict__ gcol,
                                                double2* partial) {
     L = lens_at(L, H);
-    __shared__ int s_win;
-    if (threadIdx.x == 0) s_win = 0;
+    __shared__ int s_win[2];                // bit patterns of the layers' reach, -1: not fed
+    __shared__ float4 s_src[PBT * PBT];     // (C_q, R)
+    __shared__ float s_z[PBT * PBT];
+    __shared__ float s_part[PBG][5][PBT * PBT];  // one layer's (gx, gy, gz, S1, S2) per group
+    const int p = threadIdx.x;
+    if (p < 2) s_win[p] = -1;
     __syncthreads();
-    const int i = blockIdx.x * 16 + 2 * (threadIdx.x & 7), j = blockIdx.y * 16 + 2 * (threadIdx.x >> 3);
-    const bool in0 = i < W && j < H;
-    const bool ok[4] = {in0, in0 && i + 1 < W, in0 && j + 1 < H, in0 && i + 1 < W && j + 1 < H};
-    const int ox[4] = {0, 1, 0, 1}, oy[4] = {0, 0, 1, 1};
-    PfBwdSrc src;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        src.zq[k] = 1.f;
-        src.R[k] = 0.f;  // an absent source weighs nothing
-        src.wnia[k] = src.fia[k] = 0.f;
-        src.Cq[k] = f3(0, 0, 0);
-        if (ok[k]) {
-            const size_t q = (size_t)(j + oy[k]) * W + (i + ox[k]);
-            src.zq[k] = __ldg(&nd[q].w);
-            const PfSrc sr = pf_src(src.zq[k], L, rmax, tab, ntab);
-            src.R[k] = sr.R;
-            src.wnia[k] = sr.wnia;
-            src.fia[k] = sr.fia;
-            src.Cq[k] = ldf3(__ldg(&col[q]));
-            atomicMax(&s_win, __float_as_int(sr.R));  // positive floats order as their bits
+    const int pi = blockIdx.x * PBT + (p & 15), pj = blockIdx.y * PBT + (p >> 4);
+    const bool ok = pi < W && pj < H;
+    const size_t pq = (size_t)pj * W + pi;
+    float z = 1.f;
+    PfSrc sr{};
+    {
+        float4 cr = make_float4(0.f, 0.f, 0.f, 0.f);  // R = 0: an absent source weighs nothing
+        if (ok) {
+            z = __ldg(&nd[pq].w);
+            sr = pf_src(z, L, rmax, tab, ntab);
+            const float3 C = ldf3(__ldg(&col[pq]));
+            cr = make_float4(C.x, C.y, C.z, sr.R);
+            // positive floats order as their bits; NaN radii (a lens that is not finite) take the whole cap
+            const int rb = __float_as_int(sr.R <= rmax + 0.5f ? sr.R : rmax + 0.5f);
+            if (!(sr.wnia == 0.f && sr.dwnia == 0.f)) atomicMax(&s_win[0], rb);
+            if (!(sr.fia == 0.f && sr.dfia == 0.f)) atomicMax(&s_win[1], rb);
         }
+        s_src[p] = cr;
+        s_z[p] = z;
     }
     __syncthreads();
+    const int g = threadIdx.x >> 6, t = threadIdx.x & 63;
+    const int li = 2 * (t & 7), lj = 2 * (t >> 3), i = blockIdx.x * PBT + li, j = blockIdx.y * PBT + lj;
+    const float ka = 1.f + 1.f / kz_rel;
+    PfBwdSrc src;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int e = (lj + k) * PBT + li;
+        const float4 a = s_src[e], b = s_src[e + 1];
+        src.R[2 * k] = a.w;
+        src.R[2 * k + 1] = b.w;
+        src.zq[2 * k] = s_z[e];
+        src.zq[2 * k + 1] = s_z[e + 1];
+        src.Cx[k] = pk2(a.x, b.x);
+        src.Cy[k] = pk2(a.y, b.y);
+        src.Cz[k] = pk2(a.z, b.z);
+    }
+    float3 gC = f3(0.f, 0.f, 0.f);
+    float gc = 0.f;  // gradient of source p's CoC
+#pragma unroll
+    for (int layer = 0; layer < 2; ++layer) {
+        const int rb = s_win[layer];
+        if (rb < 0) continue;  // block-uniform
+        if (i < W && j < H) {
+            PfBwdAcc acc;
+            const float reach = __int_as_float(rb);
+            if (layer) pf_bwd_layer<true>(acc, src, reach, g, i, j, W, H, ka, pfb + pfb_plane(W, H), kbp);
+            else pf_bwd_layer<false>(acc, src, reach, g, i, j, W, H, ka, pfb, kbp);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int e = (lj + k) * PBT + li;
+                const float2 v[5] = {unpk2(acc.gx[k]), unpk2(acc.gy[k]), unpk2(acc.gz[k]), unpk2(acc.S1[k]),
+                                     unpk2(acc.S2[k])};
+#pragma unroll
+                for (int m = 0; m < 5; ++m) *reinterpret_cast<float2*>(&s_part[g][m][e]) = v[m];
+            }
+        }
+        __syncthreads();
+        if (ok) {
+            float v[5];
+#pragma unroll
+            for (int m = 0; m < 5; ++m) {
+                v[m] = s_part[0][m][p];
+#pragma unroll
+                for (int b = 1; b < PBG; ++b) v[m] += s_part[b][m][p];
+            }
+            const float wa = layer ? sr.fia : sr.wnia, da = layer ? sr.dfia : sr.dwnia;
+            gC = gC + wa * f3(v[0], v[1], v[2]);
+            gc += v[3] * da + v[4] * wa * sr.rp;
+        }
+        __syncthreads();
+    }
     float2 dth = make_float2(0.f, 0.f);
-    if (in0) {
-        // the block's reach R = max(r) + 1/2: a pair weighs (and its rim term
-        // counts) only closer than that; bounds lean outwards by 1e-3 pixel
-        const float Rw = __int_as_float(s_win), R2w = Rw * Rw;
-        const int G = (int)floorf(Rw + 1e-3f);
-        const float ka = 1.f + 1.f / kz_rel;
-        const size_t px = (size_t)W * H, half = (px + 1) >> 1;
-        const float4* __restrict__ pn_e = pfb;
-        const float4* __restrict__ pn_o = pfb + half;
-        const float4* __restrict__ pf_e = pfb + px;
-        const float4* __restrict__ pf_o = pfb + px + half;
-        const float2* __restrict__ kb2 = reinterpret_cast<const float2*>(kbp);
-        PfBwdAcc acc[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            acc[k].gC = f3(0, 0, 0);
-            acc[k].S1 = acc[k].S2 = acc[k].S3 = acc[k].S4 = 0.f;
-        }
-        const int y0 = max(j - G, 0), y1 = min(j + 1 + G, H - 1);
-        for (int y = y0; y <= y1; ++y) {
-            const float dy = (float)(y - j);
-            const float dy0 = dy * dy, dy1 = (dy - 1.f) * (dy - 1.f);
-            const float dmin = dy >= 0.f && dy <= 1.f ? 0.f : fminf(dy0, dy1);
-            const int w = (int)floorf(sqrtf(fmaxf(R2w - dmin, 0.f)) + 1e-3f);
-            const int x0 = max(i - w, 0), x1 = min(i + 1 + w, W - 1);
-            float dx = (float)(x0 - i);
-            float c[2];
-            {
-                const float dm = (dx - 1.f) * (dx - 1.f);
-                c[0] = sqrt_approx(dm + dy0);
-                c[1] = sqrt_approx(dm + dy1);
-            }
-            // targets in (even, odd) index pairs; a lone odd first and even last on their own
-            size_t g = (size_t)y * W + x0;
-            const size_t gend = (size_t)y * W + x1 + 1;
-            if (g & 1) {
-                pf_bwd_tap(acc, c, src, dx, dy0, dy1, ka, __ldg(&kbp[g]), __ldg(&pn_o[g >> 1]), __ldg(&pf_o[g >> 1]));
-                ++g;
-                dx += 1.f;
-            }
-            const size_t mend = gend >> 1;
-#pragma unroll 1
-            for (size_t m = g >> 1; m < mend; ++m, dx += 2.f) {
-                const float2 kb = __ldg(&kb2[m]);
-                pf_bwd_tap(acc, c, src, dx, dy0, dy1, ka, kb.x, __ldg(&pn_e[m]), __ldg(&pf_e[m]));
-                pf_bwd_tap(acc, c, src, dx + 1.f, dy0, dy1, ka, kb.y, __ldg(&pn_o[m]), __ldg(&pf_o[m]));
-            }
-            if (gend & 1) {
-                const size_t gl = gend - 1;
-                pf_bwd_tap(acc, c, src, dx, dy0, dy1, ka, __ldg(&kbp[gl]), __ldg(&pn_e[gl >> 1]),
-                           __ldg(&pf_e[gl >> 1]));
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (!ok[k]) continue;
-            const size_t q = (size_t)(j + oy[k]) * W + (i + ox[k]);
-            const float4 g0 = gcol[q];
-            gcol[q] = make_float4(g0.x + acc[k].gC.x, g0.y + acc[k].gC.y, g0.z + acc[k].gC.z, 0.f);
-            const PfSrc sr = pf_src(src.zq[k], L, rmax, tab, ntab);
-            const float gc = acc[k].S1 * sr.dwnia + acc[k].S2 * sr.wnia * sr.rp + acc[k].S3 * sr.dfia +
-                             acc[k].S4 * sr.fia * sr.rp;
-            const float2 dc = dcoc(src.zq[k], L);
-            dth.x = fmaf(gc, dc.x, dth.x);
-            dth.y = fmaf(gc, dc.y, dth.y);
-        }
+    if (ok) {
+        const float4 g0 = gcol[pq];
+        gcol[pq] = make_float4(g0.x + gC.x, g0.y + gC.y, g0.z + gC.z, 0.f);
+        const float2 dc = dcoc(z, L);
+        dth = make_float2(gc * dc.x, gc * dc.y);
     }
     block_partial(dth, partial);
 }
@@ -714,6 +819,7 @@ __global__ void __launch_bounds__(64, HDOF_PFB_MINB) k_pf_bwd(const float4* __re
 __global__ void __launch_bounds__(1024) k_reduce(const double2* __restrict__ partial, int n, float* out) {
     __shared__ double red[2][1024];
     double a = 0.0, b = 0.0;
+#pragma unroll 4
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         a += partial[k].x;
         b += partial[k].y;
@@ -774,7 +880,7 @@ BwdWs bwd_layout(int W, int H, char* base) {
     b.gcrec = reinterpret_cast<float4*>(take(16 * px));
     b.gcrt = reinterpret_cast<float4*>(take(16 * px));
     b.spb = reinterpret_cast<float4*>(take(16 * px));
-    b.pfb = reinterpret_cast<float4*>(take(32 * px));
+    b.pfb = reinterpret_cast<float4*>(take(32 * pfb_plane(W, H)));
     b.kbp = reinterpret_cast<float*>(take(4 * px));
     b.ghacc = reinterpret_cast<float*>(take(4 * px));
     b.gmom = reinterpret_cast<float2*>(take(8 * px));
@@ -891,13 +997,14 @@ int post_backward(const hdof_gbuf* in, const uint8_t* spp, const float* rec, con
                                           reinterpret_cast<const float2*>(st->mom), st->hlen,
                                           reinterpret_cast<const float4*>(st->sp_aux), b.gcrec, W, H, p->var_ref, b.spb,
                                           b.gcrt, b.gmom);
-    k_spatial_bwd<<<g2, 256, 0, s>>>(reinterpret_cast<const float4*>(st->crt), b.spb, W, H, p->r_s, b.gcrt);
+    const dim3 gs((W + SB_TW - 1) / SB_TW, (H + SB_TH - 1) / SB_TH);
+    k_spatial_bwd<<<gs, SB_THREADS, 0, s>>>(reinterpret_cast<const float4*>(st->crt), b.spb, W, H, p->r_s, b.gcrt);
     k_temporal_replay_bwd<<<g1, 256, 0, s>>>(reinterpret_cast<const float4*>(rec), ray_off, spp,
                                              reinterpret_cast<const float4*>(hist_samples), b.gcrt, b.ghacc, b.gmom, W,
                                              H, L, p->ema_alpha, p->camera_moved, b.partial + n1);
     k_pf_bwd_prep<<<g1, 256, 0, s>>>(reinterpret_cast<const float4*>(st->pp_aux), b.gpp, nd, p->kz_rel, W, H, b.pfb,
                                      b.kbp, gcol);
-    k_pf_bwd<<<g2, 64, 0, s>>>(nd, col, b.pfb, b.kbp, tab, ntab, W, H, L, p->r_max, p->kz_rel, gcol,
+    k_pf_bwd<<<g2, 64 * PBG, 0, s>>>(nd, col, b.pfb, b.kbp, tab, ntab, W, H, L, p->r_max, p->kz_rel, gcol,
                                b.partial + 2 * n1);
     k_reduce<<<1, 1024, 0, s>>>(b.partial, b.n_partial, grad_lens);
     HDOF_LAUNCHED("post-path backward");

@@ -150,6 +150,44 @@ def test_colour_gradient_equals_the_oracle_vjp(orc):
     assert np.abs(ref - g).max() > 1e-2 * scale  # blur: J is not the identity
 
 
+@pytest.mark.parametrize("W,Hh,zlo,zhi", [(33, 19, 0.8, 1.2), (17, 35, 4.0, 8.0), (31, 16, 1.2, 5.0)])
+def test_post_filter_adjoint_by_layer(orc, W, Hh, zlo, zhi):
+    """The post-filter's adjoint with every source near, every source far and
+    both, at odd sizes (pairs of targets straddling rows), nothing traced:
+    grad_col against the oracle's J^T g, the lens gradient against the
+    oracle's central differences (2%; h = 1e-6: the map is piecewise smooth
+    and at 1e-4 the oracle's own difference straddles a kink, 34.300 where
+    1e-5 to 1e-7 give 35.4933).  Each entry sums at most (2 x 11)^2 products in FP32: 484 x 2^-24 =
+    3e-5 of the largest."""
+    rng = np.random.default_rng(W)
+    cam = hi.Camera(width=W, height=Hh).f32()
+    p = hi.room_params(r_max=10.0, camera_moved=0, kz_rel=0.5)
+    col = rng.uniform(0.0, 1.0, (Hh, W, 3)).astype(np.float32)
+    z = rng.uniform(zlo, zhi, (Hh, W)).astype(np.float32)
+    spp = np.zeros((Hh, W), np.uint8)
+    zf, A = 2.2, 0.15
+    g = rng.normal(size=(Hh, W, 3)).astype(np.float32)
+    rec = torch.zeros((1, 4), dtype=torch.float32, device="cuda")
+    off = torch.zeros((Hh, W), dtype=torch.int32, device="cuda")
+    path = H.PostPath(torch.from_numpy(z).cuda(), torch.from_numpy(spp).cuda(), rec, off, None, cam, p)
+    path.forward(torch.from_numpy(col).cuda(), zf, A)
+    gcol, glens = path.backward(torch.from_numpy(g).cuda(), zf, A)
+    H.hdof_sync()
+    orec, ooff = np.zeros((1, 4)), np.zeros((Hh, W), np.int32)
+    f64 = lambda a: a.astype(np.float64)  # noqa: E731
+    hs = np.zeros((Hh, W, 12))
+    ref = orc.post_colour_vjp(f64(col), f64(z), spp, orec, ooff, hs, cam, hi.Lens(zf, A, 0.05).f32(), p, f64(g))
+    assert np.abs(host(gcol) - ref).max() <= 3e-5 * np.abs(ref).max(), report("grad_col", host(gcol), ref)
+
+    def loss(zf_, A_):
+        o = orc.post_forward(f64(col), f64(z), spp, orec, ooff, hs, cam, hi.Lens(zf_, A_, 0.05), p)
+        return float((o["out"][..., :3] * f64(g)).sum())
+
+    h = 1e-6
+    fd = np.array([(loss(zf + h, A) - loss(zf - h, A)) / (2 * h), (loss(zf, A + h) - loss(zf, A - h)) / (2 * h)])
+    assert np.all(np.abs(host(glens) - fd) <= 2e-2 * np.abs(fd)), (host(glens), fd)
+
+
 def _loss_gpu(path, C, Y, zf, A):
     return float((path.forward(C, zf, A).double() * Y.double()).sum())
 
