@@ -645,8 +645,10 @@ __device__ __forceinline__ void pf_bwd_tap(PfBwdAcc& acc, float (&c)[2], const P
             kl = __saturatef(fmaf(-src.zq[2 * k], kb, ka));
             kr = __saturatef(fmaf(-src.zq[2 * k + 1], kb, ka));
         }
-        // on the rim, 0 < u < 1, the clamp is the identity (and its slope 1)
-        const f32x2 s = pk2(FAR ? sl * kl : sl, FAR ? sr * kr : sr), sp = pk2(sl == ul ? kl : 0.f, sr == ur ? kr : 0.f);
+        // the clamp's slope: 1 where 0 < u < 1, that is u - u^2 > 0 (the fused
+        // form's sign is exact; u of exactly 0 or 1 is met tens of times a frame)
+        const f32x2 s = pk2(FAR ? sl * kl : sl, FAR ? sr * kr : sr);
+        const f32x2 sp = pk2(fmaf(-ul, ul, ul) > 0.f ? kl : 0.f, fmaf(-ur, ur, ur) > 0.f ? kr : 0.f);
         const f32x2 t = ffma2(Az, src.Cz[k], ffma2(Ay, src.Cy[k], ffma2(Ax, src.Cx[k], E)));
         acc.gx[k] = ffma2(s, Ax, acc.gx[k]);
         acc.gy[k] = ffma2(s, Ay, acc.gy[k]);
