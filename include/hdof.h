@@ -307,8 +307,8 @@ int hdof_mask_noalloc(const hdof_gbuf* in, const hdof_history* prev_hist, const 
  *   close, i.e. for small lens apertures); 1..32 = ray level (one ray per
  *   lane; a warp fetches new rays for its idle lanes once fewer than this
  *   many of its 32 lanes still trace); -1 = each view in its default form:
- *   warp packets when the view's CoC scale K = A H / (zf tan(fovy/2)) is
- *   below 20 pixels, ray level with refill 4 otherwise (a batch traces the
+ *   warp packets when the lens's width against the view's, A / (zf
+ *   tan(fovy/2)), is below 0.1, ray level with refill 4 otherwise (a batch traces the
  *   two groups of views in two persistent launches, both of trace_block
  *   threads).
  * trace_chunk, spatial_tile: launch granularity of the trace's work queue and
@@ -352,10 +352,11 @@ typedef struct hdof_tuning {
  * rec holds stats[1] float4 entries (at most spp_max x W x H).
  * tune (host, may be NULL): the trace's form and block size (out-of-range
  * values are rejected with HDOF_EINVAL); NULL takes 128 threads and the
- * default form (trace_refill -1): warp packets when the lens's CoC scale
- * K = A H / (zf tan(fovy/2)) is below 20 pixels (|c(z)| = K |zf/z - 1|: the
- * lens rays of neighbouring pixels stay close), ray level with refill 4
- * otherwise. */
+ * default form (trace_refill -1): warp packets when A / (zf tan(fovy/2)), the
+ * lens's width against the view's, is below 0.1 (the lens rays of
+ * neighbouring pixels stay close), ray level with refill 4 otherwise.  Where
+ * the CoC scale K = A H / (zf tan(fovy/2)) reaches 8 pixels, a tile's rays
+ * are listed by the part of the lens they leave, in either form. */
 int hdof_trace(const hdof_bvh* bvh, const hdof_camera* cam, const hdof_lens* lens,
                const hdof_params* p, const uint8_t* spp, const int32_t* hint_tri, float* rt,
                uint32_t* stats, float* rec, uint32_t* ray_off, void* workspace,

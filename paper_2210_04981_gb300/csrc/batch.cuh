@@ -60,7 +60,7 @@ struct ViewWs {
     unsigned* roffsets;  // [ntiles]
     unsigned* totals;    // [4] queue length, -, ray count, ray head
     unsigned* queue;     // [W * H] traced pixels
-    unsigned* qoff;      // [W * H] first ray of each queue entry
+    unsigned* qoff;      // [W * H] first record of each traced pixel
     unsigned* ray_pix;   // [W * H * spp_max] pixel of each ray
     uint8_t* ray_s;      // [W * H * spp_max] sample index of each ray
     float2* rec;         // [W * H * spp_max] (hit distance, triangle) of each ray

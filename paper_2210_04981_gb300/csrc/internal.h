@@ -72,7 +72,7 @@ struct WsLayout {
     size_t mask_tile_r;     // float per mask tile: largest CoC radius of its pixels (CoC-scaled mask)
     size_t trace_counts;    // uint32 per 16x16 tile: traced pixels, rays; + scan output
     size_t trace_queue;     // uint32 per pixel: traced pixels in queue order
-    size_t trace_qoff;      // uint32 per pixel: first ray of each queue entry
+    size_t trace_qoff;      // uint32 per pixel: its first ray's record
     size_t trace_ray_pix;   // uint32 per possible ray (pixels x spp_max): its pixel
     size_t trace_ray_s;     // uint8 per possible ray: its sample index
     size_t trace_rec;       // float2 per possible ray: hit distance, triangle

@@ -7,7 +7,7 @@
 // Compaction (deterministic, tile order): k_count counts traced pixels and
 // rays per 16x16 tile, k_scan turns the counts into queue and ray offsets,
 // k_scatter writes the traced pixels in Z order within each tile and lists
-// every ray as (pixel, sample).
+// every ray as (pixel, sample), for wide lenses in order of lens bins.
 //
 // Trace: two persistent forms over the ray list, each writing a (hit
 // distance, triangle slot) record per ray.  k_trace_packets: a warp takes 32
@@ -23,18 +23,37 @@
 
 namespace hdof {
 
-// default form of a view's trace: warp packets below this CoC scale K =
-// A H / (zf tan(fovy/2)) (pixels of CoC per unit of zf/z - 1), ray level with
-// refill 4 above
-constexpr float PACKET_K_MAX = 20.f;
-static bool packet_view(const hdof_lens& l, const hdof_camera& c) {
-    const float K = l.aperture_radius * (float)c.height / (l.focus_dist * c.tan_half_fovy);
-    return K < PACKET_K_MAX;
+// What a view's trace depends on is how far apart the rays that run together
+// are.  K = A H / (zf tan(fovy/2)) is the CoC scale (pixels of CoC per unit
+// of zf/z - 1), K / H = A / (zf tan(fovy/2)) the lens's width against the
+// view's.  Both only choose an order or a form: every ray's hit is the same.
+//
+// From K = 8 pixels on, where the lens spreads a pixel's rays farther than
+// the 8x4 pixels of 32 one-ray neighbours lie apart, a tile's rays are listed
+// by lens bin (scatter_binned).  Rooms of about 165k triangles, trace and
+// compaction, unsorted / sorted: 1080p K = 4.6 242 / 265 us, 7 312 / 318,
+// 10 359 / 345, 25 521 / 381, 60 638 / 458 (the better form of each); 480x270
+// K = 2 162 / 179, 4.6 216 / 198, 10 314 / 246, 25 351 / 316.
+//
+// Below K / H = 0.1 warp packets are the default form, ray level with refill
+// 4 above: sorted packets / rays at 1080p K = 60 458 / 528 us, 100 545 / 568,
+// 140 630 / 600; at 480x270 K = 18 283 / 320, 25 316 / 328, 60 422 / 344.
+// (Unsorted, the line lay at K = 20 pixels.)
+constexpr float BIN_K_MIN = 8.f;
+constexpr float PACKET_KH_MAX = 0.1f;
+static float coc_scale(const hdof_lens& l, const hdof_camera& c) {
+    return l.aperture_radius * (float)c.height / (l.focus_dist * c.tan_half_fovy);
 }
+static bool packet_view(const hdof_lens& l, const hdof_camera& c) {
+    return coc_scale(l, c) < PACKET_KH_MAX * (float)c.height;
+}
+static bool binned_view(const hdof_lens& l, const hdof_camera& c) { return coc_scale(l, c) >= BIN_K_MIN; }
 
 namespace {
 
 constexpr int TB = 16;  // compaction tile edge
+
+uint2 trace_key(const hdof_params& p) { return make_uint2(p.seed, (unsigned)p.view * 65536u + (unsigned)p.frame); }
 
 // a pixel traces min(spp, spp_max) rays (the ray lists are sized for spp_max)
 struct CountArgs {
@@ -197,6 +216,8 @@ __global__ void __launch_bounds__(1024) k_scan(ScanArgs a) { scan_body(a); }
 struct ScatterArgs {
     const uint8_t* spp;
     int W, H, ntx, smax;
+    int binned;  // a tile's rays in order of their lens samples' bins (binned_view)
+    uint2 key;   // the samples' Philox key
     const unsigned* offsets;
     const unsigned* roffsets;
     unsigned* queue;
@@ -205,6 +226,98 @@ struct ScatterArgs {
     uint8_t* ray_s;
     unsigned* ray_off;
 };
+
+// a tile pixel's column and row from its Z-order index (even bits, odd bits)
+__device__ __forceinline__ int zx(int t) { return (t & 1) | ((t >> 1) & 2) | ((t >> 2) & 4) | ((t >> 3) & 8); }
+__device__ __forceinline__ int zy(int t) { return zx(t >> 1); }
+
+// Lens bin of sample `smp` of pixel q: 16 bins of equal area, 4 sectors of the
+// inner half radius and 12 of the ring around it (on a polygon the same parts
+// of its sampling).
+constexpr int LENS_BINS = 16;
+__device__ __forceinline__ unsigned lens_bin(uint2 key, unsigned q, unsigned smp) {
+    const uint4 x = philox4x32_10(make_uint4(q, smp, 0u, 0u), key);
+    return (x.x >> 30) == 0u ? x.y >> 30 : 4u + (((x.y >> 16) * 12u) >> 16);
+}
+
+// The tile's ray list grouped by lens bin, within a bin in the tile's Z order:
+// 32 consecutive rays leave one part of the lens from one small block of
+// pixels.  A counting sort over (bin, pixel): counts per thread and bin,
+// their prefix, then every ray to its place; with at most 16 samples a pixel
+// through shared memory (SORT_STAGE entries), so that the list is written in
+// whole lines.  Bound by the samples' Philox rounds (compaction of 15M rays:
+// 52 us unsorted, 110 so; 141 with warp matches and direct stores).
+constexpr int SORT_STAGE = 16 * 256;
+__device__ __forceinline__ void scatter_binned(const ScatterArgs& a, unsigned q, unsigned n, unsigned rbase, int bx,
+                                               int by) {
+    __shared__ __align__(16) uint8_t s_cnt[LENS_BINS][256];
+    __shared__ __align__(16) uint16_t s_off[LENS_BINS][256];
+    __shared__ uint16_t s_list[SORT_STAGE];
+    __shared__ unsigned s_bin[LENS_BINS + 1];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+#pragma unroll
+    for (int b = 0; b < LENS_BINS; ++b) s_cnt[b][t] = 0;
+    unsigned long long bins = 0ull;  // the first 16 samples' bins, 4 bits each
+    for (unsigned smp = 0; smp < n; ++smp) {
+        const unsigned b = lens_bin(a.key, q, smp);
+        if (smp < 16) bins |= (unsigned long long)b << (4 * smp);
+        ++s_cnt[b][t];
+    }
+    __syncthreads();
+    for (int b = w; b < LENS_BINS; b += 8) {  // a warp per bin, eight threads' counts a lane
+        const uint2 c = *reinterpret_cast<const uint2*>(&s_cnt[b][8 * lane]);
+        unsigned v[8], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = sum;
+            sum += ((k < 4 ? c.x : c.y) >> (8 * (k & 3))) & 255u;
+        }
+        unsigned x = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_bin[b] = x;
+        x -= sum;
+        uint4 pk;
+        pk.x = (x + v[0]) | (x + v[1]) << 16;
+        pk.y = (x + v[2]) | (x + v[3]) << 16;
+        pk.z = (x + v[4]) | (x + v[5]) << 16;
+        pk.w = (x + v[6]) | (x + v[7]) << 16;
+        *reinterpret_cast<uint4*>(&s_off[b][8 * lane]) = pk;
+    }
+    __syncthreads();
+    if (w == 0) {
+        const unsigned v = lane < LENS_BINS ? s_bin[lane] : 0u;
+        unsigned x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane <= LENS_BINS) s_bin[lane] = x - v;  // [LENS_BINS]: the total
+    }
+    __syncthreads();
+    const bool stage = a.smax <= 16;
+    for (unsigned smp = 0; smp < n; ++smp) {
+        const unsigned b = smp < 16 ? (unsigned)(bins >> (4 * smp)) & 15u : lens_bin(a.key, q, smp);
+        const unsigned e = s_bin[b] + s_off[b][t]++;
+        if (stage) {
+            s_list[e] = (uint16_t)(t << 8 | smp);
+        } else {
+            a.ray_pix[rbase + e] = q;
+            a.ray_s[rbase + e] = (uint8_t)smp;
+        }
+    }
+    if (!stage) return;
+    __syncthreads();
+    const unsigned total = s_bin[LENS_BINS];
+    for (unsigned e = t; e < total; e += 256) {
+        const unsigned v = s_list[e], z = v >> 8;
+        const int i = bx * TB + zx(z), j = by * TB + zy(z);
+        a.ray_pix[rbase + e] = (unsigned)(j * a.W + i);
+        a.ray_s[rbase + e] = (uint8_t)v;
+    }
+}
 
 __device__ __forceinline__ void scatter_body(const ScatterArgs& a, int bx, int by) {
     const uint8_t* __restrict__ spp = a.spp;
@@ -216,10 +329,8 @@ __device__ __forceinline__ void scatter_body(const ScatterArgs& a, int bx, int b
     unsigned* __restrict__ ray_pix = a.ray_pix;
     uint8_t* __restrict__ ray_s = a.ray_s;
     unsigned* __restrict__ ray_off = a.ray_off;
-    const int t = threadIdx.x;  // Z-order index: x from the even bits, y from the odd bits
-    const int mx = (t & 1) | ((t >> 1) & 2) | ((t >> 2) & 4) | ((t >> 3) & 8);
-    const int my = ((t >> 1) & 1) | ((t >> 2) & 2) | ((t >> 3) & 4) | ((t >> 4) & 8);
-    int i = bx * TB + mx, j = by * TB + my;
+    const int t = threadIdx.x;  // Z-order index
+    int i = bx * TB + zx(t), j = by * TB + zy(t);
     unsigned n = (i < W && j < H) ? min((unsigned)spp[(size_t)j * W + i], (unsigned)a.smax) : 0u;
     bool on = n > 0;
     unsigned m = __ballot_sync(0xffffffffu, on);
@@ -243,8 +354,12 @@ __device__ __forceinline__ void scatter_body(const ScatterArgs& a, int bx, int b
     if (on) {
         const unsigned k = base + __popc(m & ((1u << lane) - 1u)), ro = rbase + r - n;
         queue[k] = q;
-        qoff[k] = ro;
+        qoff[q] = ro;
         if (ray_off) ray_off[q] = ro;
+    }
+    if (a.binned) {  // uniform per view
+        scatter_binned(a, q, n, roffsets[tile], bx, by);
+        return;
     }
     // the warp's rays are contiguous from rbase: lanes write them together,
     // entry e going to the lane whose inclusive spp prefix first exceeds e
@@ -279,6 +394,7 @@ struct TraceArgs {
     uint2 key;
     int cap, smax;
     int packets;  // the view's default form is warp packets (packet_view)
+    int binned;   // the ray list is in lens-bin order (binned_view)
     unsigned* status;
     const uint8_t* spp;
     const int* hint;   // optional per-pixel original id of the primary hit (< 0: none)
@@ -522,6 +638,7 @@ __device__ __forceinline__ void trace_rays_body(const Src& src, unsigned total, 
                     }
                     L.sp = 0;
                     L.steps = 0;
+                    if (a.binned) L.r = __ldg(&a.qoff[qp]) + __ldg(&a.ray_s[L.r]);  // its record
                     L.live = true;
                 } else {
                     L.done = true;
@@ -590,8 +707,9 @@ __device__ __forceinline__ void trace_packets_body(const Src& src, unsigned tota
             h.b0 = h.b1 = h.b2 = 0.f;
             float3 O = f3(0.f, 0.f, 0.f), dir = f3(0.f, 0.f, 1.f);
             if (act) {
-                const unsigned qp = __ldg(&a.ray_pix[r]);
-                lens_ray(a, qp, __ldg(&a.ray_s[r]), O, dir);
+                const unsigned qp = __ldg(&a.ray_pix[r]), smp = __ldg(&a.ray_s[r]);
+                lens_ray(a, qp, smp, O, dir);
+                if (a.binned) r = __ldg(&a.qoff[qp]) + smp;  // its record
                 if (a.hint) {  // the pixel's primary hit first (see trace_rays_body)
                     sh = make_shear(dir);
                     const int id = __ldg(&a.hint[qp]);
@@ -621,8 +739,9 @@ __global__ void __launch_bounds__(BS, 1280 / BS) k_trace_packets(TraceArgs a, in
     trace_packets_body(OneView{a}, __ldcg(&a.totals[2]), &a.totals[3], chunk);
 }
 
+// 36 resident warps (56 registers): a 12-view batch frame 45.8 ms a pair, 46.6 with 40, 46.2 with 32
 template <int BS>
-__global__ void __launch_bounds__(BS) k_trace_packets_batch(const TraceArgs* __restrict__ tab,
+__global__ void __launch_bounds__(BS, 1152 / BS) k_trace_packets_batch(const TraceArgs* __restrict__ tab,
                                                             const unsigned* __restrict__ gq, int n, unsigned* head,
                                                             int chunk) {
     trace_packets_body(ManyViews{tab, gq, n}, __ldcg(&gq[n]), head, chunk);
@@ -647,7 +766,7 @@ __global__ void __launch_bounds__(BS) k_trace_rays_batch(const TraceArgs* __rest
 __device__ __forceinline__ void resolve_body(const TraceArgs& a, int bx) {
     const unsigned k = (unsigned)bx * 256u + threadIdx.x;
     if (k >= __ldcg(&a.totals[0])) return;
-    const unsigned q = __ldg(&a.queue[k]), ro = __ldg(&a.qoff[k]);
+    const unsigned q = __ldg(&a.queue[k]), ro = __ldg(&a.qoff[q]);
     const int n = min((int)a.spp[q], a.smax);
     float3 SwL = f3(0, 0, 0), SfL = f3(0, 0, 0), SfP = f3(0, 0, 0);
     float Sw = 0.f, Sf = 0.f, Swc = 0.f, Sfc = 0.f, Ss = 0.f;
@@ -704,8 +823,8 @@ __device__ __forceinline__ void resolve_body(const TraceArgs& a, int bx) {
 __global__ void __launch_bounds__(256) k_resolve(TraceArgs a) { resolve_body(a, blockIdx.x); }
 
 // Per-ray closest hits of the last trace on this workspace, in the order of
-// its hit records: ids[qoff[k] + s] = original id of sample s of queue entry
-// k (-1 for a miss), ts[...] = ray parameter of the hit (+inf for a miss).
+// its hit records: ids[qoff[q] + s] = original id of sample s of pixel q, queue
+// entry k (-1 for a miss), ts[...] = ray parameter of the hit (+inf for a miss).
 struct HitsArgs {
     const Tri* tris;
     const uint8_t* spp;
@@ -720,7 +839,7 @@ struct HitsArgs {
 __global__ void __launch_bounds__(256) k_hits(HitsArgs a) {
     const unsigned k = blockIdx.x * 256u + threadIdx.x;
     if (k >= __ldg(&a.totals[0])) return;
-    const unsigned q = __ldg(&a.queue[k]), ro = __ldg(&a.qoff[k]);
+    const unsigned q = __ldg(&a.queue[k]), ro = __ldg(&a.qoff[q]);
     const int n = min((int)__ldg(&a.spp[q]), a.smax);
     for (int smp = 0; smp < n; ++smp) {
         const float2 rc = a.recs[ro + smp];
@@ -744,10 +863,11 @@ TraceArgs trace_args(const hdof_bvh* b, const hdof_camera* cam, const hdof_lens*
     a.blades = p->blades;
     a.blade_rot = p->blade_rot;
     a.aberration = p->aberration;
-    a.key = make_uint2(p->seed, (unsigned)p->view * 65536u + (unsigned)p->frame);
+    a.key = trace_key(*p);
     a.cap = p->trav_cap > 0 ? p->trav_cap : 64 * (b->n_nodes + b->n_tris) + 64;
     a.smax = p->spp_max;
     a.packets = packet_view(*lens, *cam) ? 1 : 0;
+    a.binned = binned_view(*lens, *cam) ? 1 : 0;
     a.status = st;
     a.spp = spp;
     a.hint = hint;
@@ -886,7 +1006,7 @@ size_t scatter_args_size() { return sizeof(ScatterArgs); }
 void scatter_fill(const hdof_view& v, const ViewWs& w, unsigned*, void* dst, int* gx, int* gy) {
     const int W = v.cam.width, H = v.cam.height, ntx = (W + TB - 1) / TB;
     *reinterpret_cast<ScatterArgs*>(dst) =
-        ScatterArgs{v.spp, W, H, ntx, v.params.spp_max, w.offsets, w.roffsets, w.queue, w.qoff, w.ray_pix, w.ray_s,
+        ScatterArgs{v.spp, W, H, ntx, v.params.spp_max, binned_view(v.lens, v.cam) ? 1 : 0, trace_key(v.params), w.offsets, w.roffsets, w.queue, w.qoff, w.ray_pix, w.ray_s,
                     nullptr};
     *gx = ntx;
     *gy = (H + TB - 1) / TB;
@@ -1019,7 +1139,7 @@ extern "C" int hdof_trace(const hdof_bvh* b, const hdof_camera* cam, const hdof_
         k_count<<<tg, 256, 0, s>>>(CountArgs{spp, W, H, ntx, p->spp_max, w.counts});
         k_scan<<<1, 1024, 0, s>>>(ScanArgs{w.counts, ntiles, w.offsets, w.roffsets, w.totals, stats});
         k_scatter<<<tg, 256, 0, s>>>(
-            ScatterArgs{spp, W, H, ntx, p->spp_max, w.offsets, w.roffsets, w.queue, w.qoff, w.ray_pix, w.ray_s, ray_off});
+            ScatterArgs{spp, W, H, ntx, p->spp_max, binned_view(*lens, *cam) ? 1 : 0, trace_key(*p), w.offsets, w.roffsets, w.queue, w.qoff, w.ray_pix, w.ray_s, ray_off});
         HDOF_LAUNCHED("hdof_trace: compaction");
     }
 

@@ -403,6 +403,44 @@ def test_trace_forms_agree(aperture):
         assert torch.equal(outs[0].view(torch.int32), o.view(torch.int32))
 
 
+@pytest.mark.parametrize("W,Hh,spp_max,K", [(33, 17, 16, 8.0), (50, 40, 17, 30.0), (16, 16, 1, 60.0), (97, 31, 5, 7.9),
+                                            (40, 40, 255, 12.0)])
+def test_trace_lens_sorted_list(orc, W, Hh, spp_max, K):
+    """Views on both sides of the line from which a tile's rays are listed by
+    lens bin: ray counts from 0 to spp_max a pixel (beyond 16 the list is
+    written unstaged), partial tiles; both forms give the same bits, the hit
+    records sit at each pixel's own place and every ray's closest hit is that
+    of a brute query of the same ray (the trace's radiance against the
+    oracle's, as for the other forms)."""
+    scene = hi.room_scene(seed=3, n_boxes=24, n_spheres=6, subdiv=2, aspect=W / Hh)
+    cam = hi.Camera(width=W, height=Hh).f32()
+    lens = hi.Lens(3.0, K * 3.0 * cam.tan_half_fovy / Hh, 0.05).f32()
+    p = hi.room_params(spp_max=spp_max)
+    bvh = bvh_of(scene)
+    rng = np.random.default_rng(W)
+    spp = rng.integers(0, spp_max + 1, (Hh, W)).astype(np.uint8)
+    n = int(spp.astype(np.int64).sum())
+    outs = []
+    for refill in (0, 4):
+        rt = torch.zeros((Hh, W, 12), dtype=torch.float32, device="cuda")
+        rec = torch.zeros((n, 4), dtype=torch.float32, device="cuda")
+        off = torch.zeros((Hh, W), dtype=torch.int32, device="cuda")
+        stats = torch.zeros(2, dtype=torch.int32, device="cuda")
+        ws = workspace(W, Hh, p)
+        H.hdof_trace(bvh, cam, lens, p, dev(spp), rt, stats, ws, rec=rec, ray_off=off, tune=H.tuning(128, refill))
+        ids = torch.full((n,), -7, dtype=torch.int32, device="cuda")
+        H.hdof_trace_hits(bvh, cam, p, dev(spp), ws, ids)
+        H.hdof_sync()
+        assert host(stats).tolist() == [int((spp > 0).sum()), n]
+        outs.append((rt, rec, ids))
+    for a, b in zip(*outs):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+    assert (outs[0][2] >= -1).all()
+    ref = orc.trace(orc.OScene(scene), cam, lens, p, spp)
+    ok = rt_close(host(outs[0][0]), ref, spp > 0)
+    assert ok.mean() >= 0.998, report("rt", host(outs[0][0])[spp > 0], ref[spp > 0])
+
+
 @pytest.mark.parametrize("refill", [0, 4])
 def test_trace_watchdog_reports_timeout(refill):
     """A traversal step cap of 1 stops every lens ray after one step (the
