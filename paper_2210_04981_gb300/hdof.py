@@ -202,7 +202,12 @@ def _stream(stream):
 
 # ------------------------------------------------------------ records ----
 
+# Each of these takes its C record as it is: a caller that makes several calls
+# with the same records (a frame) marshals them once.
+
 def camera(c) -> hdof_camera:
+    if isinstance(c, hdof_camera):
+        return c
     o = hdof_camera()
     o.pos[:] = list(c.pos)
     o.right[:] = list(c.right)
@@ -215,6 +220,8 @@ def camera(c) -> hdof_camera:
 
 
 def lens(l) -> hdof_lens:
+    if isinstance(l, hdof_lens):
+        return l
     return hdof_lens(l.focus_dist, l.aperture_radius, l.focal_length)
 
 
@@ -227,6 +234,8 @@ _PARAM_NAMES = ("gauss_sigma", "edge_tau", "tile", "dilate", "spp_max", "varianc
 def params(p=None) -> hdof_params:
     """Marshal a parameter record (attributes named as the C fields; light
     directions are normalised here); None gives the library defaults."""
+    if isinstance(p, hdof_params):
+        return p
     o = hdof_params()
     load().hdof_default_params(C.byref(o))
     if p is None:
@@ -288,6 +297,14 @@ class History:
 
     def reset(self):
         self.hlen.zero_()
+
+
+def _gbuf(g) -> hdof_gbuf:
+    return g if isinstance(g, hdof_gbuf) else g.struct()
+
+
+def _hist(h) -> hdof_history:
+    return h if isinstance(h, hdof_history) else h.struct()
 
 
 class Bvh:
@@ -364,18 +381,18 @@ def hdof_gbuffer(bvh: Bvh, cam, prev, p, gbuf: GBuffer, stream=None, hint=None):
     """hint (int32 [H][W], e.g. the previous frame's tri plane, possibly
     gbuf.tri itself) optionally seeds each primary ray with a likely hit."""
     _check(load().hdof_gbuffer(bvh.handle, C.byref(camera(cam)), C.byref(camera(prev)), C.byref(params(p)),
-                               _ptr(hint), C.byref(gbuf.struct()), _stream(stream)))
+                               _ptr(hint), C.byref(_gbuf(gbuf)), _stream(stream)))
 
 
 def hdof_mask(gbuf: GBuffer, prev_hist, p, edge, spp, workspace, stream=None):
-    hs = C.byref(prev_hist.struct()) if prev_hist is not None else None
-    _check(load().hdof_mask(C.byref(gbuf.struct()), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
+    hs = C.byref(_hist(prev_hist)) if prev_hist is not None else None
+    _check(load().hdof_mask(C.byref(_gbuf(gbuf)), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
                             _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def hdof_mask_coc(gbuf: GBuffer, prev_hist, cam, lns, p, edge, spp, workspace, stream=None):
     """hdof_mask whose edge tiles reach their pixels' largest CoC radius when p.mask_coc = 1."""
-    _check(load().hdof_mask_coc(C.byref(gbuf.struct()), C.byref(prev_hist.struct()) if prev_hist is not None else None,
+    _check(load().hdof_mask_coc(C.byref(_gbuf(gbuf)), C.byref(_hist(prev_hist)) if prev_hist is not None else None,
                                 C.byref(camera(cam)), C.byref(lens(lns)), C.byref(params(p)), _ptr(edge), _ptr(spp),
                                 _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)))
 
@@ -383,8 +400,8 @@ def hdof_mask_coc(gbuf: GBuffer, prev_hist, cam, lns, p, edge, spp, workspace, s
 def hdof_mask_noalloc(gbuf: GBuffer, prev_hist, p, edge, spp, stream=None):
     """hdof_mask for callers that cannot give the library device memory: the
     tile flags live in a fixed array inside the library (see include/hdof.h)."""
-    hs = C.byref(prev_hist.struct()) if prev_hist is not None else None
-    _check(load().hdof_mask_noalloc(C.byref(gbuf.struct()), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
+    hs = C.byref(_hist(prev_hist)) if prev_hist is not None else None
+    _check(load().hdof_mask_noalloc(C.byref(_gbuf(gbuf)), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
                                     _stream(stream)))
 
 
@@ -443,34 +460,34 @@ def error_summary(stats) -> dict:
 
 
 def hdof_postfilter(gbuf: GBuffer, cam, lns, p, pp, workspace, stream=None):
-    _check(load().hdof_postfilter(C.byref(gbuf.struct()), C.byref(camera(cam)), C.byref(lens(lns)),
+    _check(load().hdof_postfilter(C.byref(_gbuf(gbuf)), C.byref(camera(cam)), C.byref(lens(lns)),
                                   C.byref(params(p)), _ptr(pp), _ptr(workspace),
                                   workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def hdof_reconstruct(rt, gbuf: GBuffer, spp, cam, prev, lns, p, hist_in: History, hist_out: History, crt, hacc,
                      crec, stream=None):
-    _check(load().hdof_reconstruct(_ptr(rt), C.byref(gbuf.struct()), _ptr(spp), C.byref(camera(cam)),
+    _check(load().hdof_reconstruct(_ptr(rt), C.byref(_gbuf(gbuf)), _ptr(spp), C.byref(camera(cam)),
                                    C.byref(camera(prev)), C.byref(lens(lns)), C.byref(params(p)),
-                                   C.byref(hist_in.struct()), C.byref(hist_out.struct()), _ptr(crt), _ptr(hacc),
+                                   C.byref(_hist(hist_in)), C.byref(_hist(hist_out)), _ptr(crt), _ptr(hacc),
                                    _ptr(crec), _stream(stream)))
 
 
 def hdof_composite(gbuf: GBuffer, spp, pp, crt, crec, hacc, cam, lns, p, out, stream=None):
-    _check(load().hdof_composite(C.byref(gbuf.struct()), _ptr(spp), _ptr(pp), _ptr(crt), _ptr(crec), _ptr(hacc),
+    _check(load().hdof_composite(C.byref(_gbuf(gbuf)), _ptr(spp), _ptr(pp), _ptr(crt), _ptr(crec), _ptr(hacc),
                                  C.byref(camera(cam)), C.byref(lens(lns)), C.byref(params(p)), _ptr(out),
                                  _stream(stream)))
 
 
 def hdof_postfilter_spec(gbuf: GBuffer, cam, lns, p, pp_spec, workspace, stream=None):
     """Post-filter of the specular plane col.w: pp_spec [H,W,4] = (S_pp x3, alpha)."""
-    _check(load().hdof_postfilter_spec(C.byref(gbuf.struct()), C.byref(camera(cam)), C.byref(lens(lns)),
+    _check(load().hdof_postfilter_spec(C.byref(_gbuf(gbuf)), C.byref(camera(cam)), C.byref(lens(lns)),
                                        C.byref(params(p)), _ptr(pp_spec), _ptr(workspace),
                                        workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def hdof_composite_spec(gbuf: GBuffer, spp, pp, pp_spec, crt, crec, hacc, cam, lns, p, out, stream=None):
-    _check(load().hdof_composite_spec(C.byref(gbuf.struct()), _ptr(spp), _ptr(pp),
+    _check(load().hdof_composite_spec(C.byref(_gbuf(gbuf)), _ptr(spp), _ptr(pp),
                                       _ptr(pp_spec) if pp_spec is not None else None, _ptr(crt), _ptr(crec),
                                       _ptr(hacc), C.byref(camera(cam)), C.byref(lens(lns)), C.byref(params(p)),
                                       _ptr(out), _stream(stream)))
@@ -539,29 +556,31 @@ class Renderer:
         main = self.crit
         self._start.record(caller)
         main.wait_event(self._start)
-        hin = self.hist[self.cur]
-        hout = self.hist[1 - self.cur]
-        hdof_gbuffer(self.bvh, cam, prev, p, self.g, main, hint=self.g.tri)
+        # the frame's records, marshalled once for its six calls: a 128x128 frame, whose kernels are
+        # shorter than the host's work on it, takes 121 us so and 156 with each call marshalling its own
+        cam, prev, lns, p, g = camera(cam), camera(prev), lens(lns), params(p), self.g.struct()
+        hin, hout = self.hist[self.cur].struct(), self.hist[1 - self.cur].struct()
+        hdof_gbuffer(self.bvh, cam, prev, p, g, main, hint=self.g.tri)
         # the post-filter on the side stream, after the G-buffer (it touches only
         # the workspace's post-filter region)
         self._gbuf_done.record(main)
         self.side.wait_event(self._gbuf_done)
-        hdof_postfilter(self.g, cam, lns, p, self.pp, self.ws, self.side)
+        hdof_postfilter(g, cam, lns, p, self.pp, self.ws, self.side)
         self._pf_done.record(self.side)
-        hdof_mask_coc(self.g, hin if with_history else None, cam, lns, p, self.edge, self.spp, self.ws, main)
+        hdof_mask_coc(g, hin if with_history else None, cam, lns, p, self.edge, self.spp, self.ws, main)
         hdof_trace(self.bvh, cam, lns, p, self.spp, self.rt, self.stats, self.ws, main, hint=self.g.tri)
-        hdof_reconstruct(self.rt, self.g, self.spp, cam, prev, lns, p, hin, hout, self.crt, self.hacc,
+        hdof_reconstruct(self.rt, g, self.spp, cam, prev, lns, p, hin, hout, self.crt, self.hacc,
                          self.crec, main)
         main.wait_event(self._pf_done)
         if p.spec_pref > 0:
             # the specular plane's post-filter uses the whole workspace: after the trace and the post-filter
             if self.pp_spec is None:
                 self.pp_spec = torch.empty_like(self.pp)
-            hdof_postfilter_spec(self.g, cam, lns, p, self.pp_spec, self.ws, main)
-            hdof_composite_spec(self.g, self.spp, self.pp, self.pp_spec, self.crt, self.crec, self.hacc, cam, lns,
+            hdof_postfilter_spec(g, cam, lns, p, self.pp_spec, self.ws, main)
+            hdof_composite_spec(g, self.spp, self.pp, self.pp_spec, self.crt, self.crec, self.hacc, cam, lns,
                                 p, self.out, main)
         else:
-            hdof_composite(self.g, self.spp, self.pp, self.crt, self.crec, self.hacc, cam, lns, p, self.out, main)
+            hdof_composite(g, self.spp, self.pp, self.crt, self.crec, self.hacc, cam, lns, p, self.out, main)
         self._done.record(main)
         caller.wait_event(self._done)
         self.cur = 1 - self.cur
