@@ -354,9 +354,9 @@ typedef struct hdof_tuning {
  * values are rejected with HDOF_EINVAL); NULL takes 128 threads and the
  * default form (trace_refill -1): warp packets when A / (zf tan(fovy/2)), the
  * lens's width against the view's, is below 0.1 (the lens rays of
- * neighbouring pixels stay close), ray level with refill 4 otherwise.  Where
- * the CoC scale K = A H / (zf tan(fovy/2)) reaches 8 pixels, a tile's rays
- * are listed by the part of the lens they leave, in either form. */
+ * neighbouring pixels stay close), ray level with refill 4 otherwise.  From
+ * 0.01 on a tile's rays are listed by the part of the lens they leave, in
+ * either form. */
 int hdof_trace(const hdof_bvh* bvh, const hdof_camera* cam, const hdof_lens* lens,
                const hdof_params* p, const uint8_t* spp, const int32_t* hint_tri, float* rt,
                uint32_t* stats, float* rec, uint32_t* ray_off, void* workspace,

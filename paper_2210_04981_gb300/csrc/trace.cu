@@ -24,30 +24,28 @@
 namespace hdof {
 
 // What a view's trace depends on is how far apart the rays that run together
-// are.  K = A H / (zf tan(fovy/2)) is the CoC scale (pixels of CoC per unit
-// of zf/z - 1), K / H = A / (zf tan(fovy/2)) the lens's width against the
-// view's.  Both only choose an order or a form: every ray's hit is the same.
+// are against the scene's triangles, so on the lens's width against the
+// view's, K / H = A / (zf tan(fovy/2)) (K the CoC scale in pixels: pixels of
+// CoC per unit of zf/z - 1).  Both lines only choose an order or a form: every
+// ray's hit is the same.
 //
-// From K = 8 pixels on, where the lens spreads a pixel's rays farther than
-// the 8x4 pixels of 32 one-ray neighbours lie apart, a tile's rays are listed
-// by lens bin (scatter_binned).  Rooms of about 165k triangles, trace and
-// compaction, unsorted / sorted: 1080p K = 4.6 242 / 265 us, 7 312 / 318,
-// 10 359 / 345, 25 521 / 381, 60 638 / 458 (the better form of each); 480x270
-// K = 2 162 / 179, 4.6 216 / 198, 10 314 / 246, 25 351 / 316.
+// From K / H = 0.01 on a tile's rays are listed by lens bin (scatter_binned).
+// Rooms of about 165k triangles, trace and compaction, unsorted / sorted:
+// 1080p K = 4.6 242 / 265 us, 7 312 / 318, 10 359 / 345, 14 409 / 360, 25
+// 521 / 381, 60 638 / 458 (the better form of each); 480x270 K = 2 162 / 179,
+// 4.6 216 / 198, 10 314 / 246, 25 351 / 316; 4K K = 9.3 390 / 495.
 //
 // Below K / H = 0.1 warp packets are the default form, ray level with refill
 // 4 above: sorted packets / rays at 1080p K = 60 458 / 528 us, 100 545 / 568,
 // 140 630 / 600; at 480x270 K = 18 283 / 320, 25 316 / 328, 60 422 / 344.
 // (Unsorted, the line lay at K = 20 pixels.)
-constexpr float BIN_K_MIN = 8.f;
+constexpr float BIN_KH_MIN = 0.01f;
 constexpr float PACKET_KH_MAX = 0.1f;
-static float coc_scale(const hdof_lens& l, const hdof_camera& c) {
-    return l.aperture_radius * (float)c.height / (l.focus_dist * c.tan_half_fovy);
+static float lens_width(const hdof_lens& l, const hdof_camera& c) {
+    return l.aperture_radius / (l.focus_dist * c.tan_half_fovy);
 }
-static bool packet_view(const hdof_lens& l, const hdof_camera& c) {
-    return coc_scale(l, c) < PACKET_KH_MAX * (float)c.height;
-}
-static bool binned_view(const hdof_lens& l, const hdof_camera& c) { return coc_scale(l, c) >= BIN_K_MIN; }
+static bool packet_view(const hdof_lens& l, const hdof_camera& c) { return lens_width(l, c) < PACKET_KH_MAX; }
+static bool binned_view(const hdof_lens& l, const hdof_camera& c) { return lens_width(l, c) >= BIN_KH_MIN; }
 
 namespace {
 
