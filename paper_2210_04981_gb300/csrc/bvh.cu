@@ -13,6 +13,8 @@
 // the linear one (2.5 ms against 3.3 ms for the frame's 3.4M rays).
 #include <cub/cub.cuh>
 
+#include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "internal.h"
@@ -33,9 +35,15 @@ __device__ __forceinline__ float ord2f(unsigned u) {
 // [8..13]: centroid bounds of the other triangles; [14..19]: centroid bounds of all
 constexpr int NB = 20;
 
-__global__ void k_scene_bounds(const float* __restrict__ v, int nv, const int* __restrict__ idx, int n,
-                               unsigned* bounds) {
-    float lo[3] = {3.4e38f, 3.4e38f, 3.4e38f}, hi[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
+// Vertex bounds, the centroid bounds of all triangles and the bad-index flag.
+// Reduced per block first: the warps' atomics on a dozen addresses were the
+// kernel's time.
+__global__ void __launch_bounds__(256) k_scene_bounds(const float* __restrict__ v, int nv, const int* __restrict__ idx,
+                                                      int n, unsigned* bounds) {
+    const float BIG = 3.4e38f;
+    float x[12];  // vertex lo, hi, centroid lo, hi
+#pragma unroll
+    for (int k = 0; k < 12; ++k) x[k] = (k / 3) & 1 ? -BIG : BIG;
     bool bad = false;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         int a = idx[3 * t], b = idx[3 * t + 1], c = idx[3 * t + 2];
@@ -44,22 +52,35 @@ __global__ void k_scene_bounds(const float* __restrict__ v, int nv, const int* _
             continue;
         }
         for (int k = 0; k < 3; ++k) {
-            lo[k] = fminf(lo[k], fminf(v[3 * a + k], fminf(v[3 * b + k], v[3 * c + k])));
-            hi[k] = fmaxf(hi[k], fmaxf(v[3 * a + k], fmaxf(v[3 * b + k], v[3 * c + k])));
+            const float p = v[3 * a + k], q = v[3 * b + k], r = v[3 * c + k], cen = (p + q + r) * (1.f / 3.f);
+            x[k] = fminf(x[k], fminf(p, fminf(q, r)));
+            x[3 + k] = fmaxf(x[3 + k], fmaxf(p, fmaxf(q, r)));
+            x[6 + k] = fminf(x[6 + k], cen);
+            x[9 + k] = fmaxf(x[9 + k], cen);
         }
     }
-    for (int k = 0; k < 3; ++k)
+    __shared__ float red[8][12];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const bool mx = (k / 3) & 1;
         for (int o = 16; o; o >>= 1) {
-            lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
-            hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+            const float y = __shfl_xor_sync(0xffffffffu, x[k], o);
+            x[k] = mx ? fmaxf(x[k], y) : fminf(x[k], y);
         }
-    if ((threadIdx.x & 31) == 0) {
-        for (int k = 0; k < 3; ++k) {
-            atomicMin(&bounds[k], f2ord(lo[k]));
-            atomicMax(&bounds[3 + k], f2ord(hi[k]));
-        }
+        if (lane == 0) red[w][k] = x[k];
     }
-    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&bounds[6], 1u);
+    const bool any_bad = __syncthreads_or(bad);
+    if (threadIdx.x < 12) {
+        const int k = threadIdx.x;
+        const bool mx = (k / 3) & 1;
+        float y = red[0][k];
+        for (int j = 1; j < 8; ++j) y = mx ? fmaxf(y, red[j][k]) : fminf(y, red[j][k]);
+        unsigned* dst = &bounds[k < 6 ? k : 14 + k - 6];
+        if (mx) atomicMax(dst, f2ord(y));
+        else atomicMin(dst, f2ord(y));
+    }
+    if (threadIdx.x == 0 && any_bad) atomicOr(&bounds[6], 1u);
 }
 
 __device__ __forceinline__ float box_area(const float lo[3], const float hi[3]) {
@@ -79,7 +100,6 @@ __global__ void k_classify(const float* __restrict__ v, const int* __restrict__ 
     }
     const float thr = big_frac * box_area(slo, shi);
     float lo[3] = {3.4e38f, 3.4e38f, 3.4e38f}, hi[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
-    float alo[3] = {3.4e38f, 3.4e38f, 3.4e38f}, ahi[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
     unsigned nbig = 0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         int a = idx[3 * t], b = idx[3 * t + 1], c = idx[3 * t + 2];
@@ -94,8 +114,6 @@ __global__ void k_classify(const float* __restrict__ v, const int* __restrict__ 
         big[t] = is_big ? 1 : 0;
         nbig += is_big ? 1u : 0u;
         for (int k = 0; k < 3; ++k) {
-            alo[k] = fminf(alo[k], cen[k]);
-            ahi[k] = fmaxf(ahi[k], cen[k]);
             if (!is_big) {
                 lo[k] = fminf(lo[k], cen[k]);
                 hi[k] = fmaxf(hi[k], cen[k]);
@@ -106,16 +124,12 @@ __global__ void k_classify(const float* __restrict__ v, const int* __restrict__ 
         for (int o = 16; o; o >>= 1) {
             lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
             hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
-            alo[k] = fminf(alo[k], __shfl_xor_sync(0xffffffffu, alo[k], o));
-            ahi[k] = fmaxf(ahi[k], __shfl_xor_sync(0xffffffffu, ahi[k], o));
         }
     for (int o = 16; o; o >>= 1) nbig += __shfl_xor_sync(0xffffffffu, nbig, o);
     if ((threadIdx.x & 31) == 0) {
         for (int k = 0; k < 3; ++k) {
             atomicMin(&bounds[8 + k], f2ord(lo[k]));
             atomicMax(&bounds[11 + k], f2ord(hi[k]));
-            atomicMin(&bounds[14 + k], f2ord(alo[k]));
-            atomicMax(&bounds[17 + k], f2ord(ahi[k]));
         }
         atomicAdd(&bounds[7], nbig);
     }
@@ -247,12 +261,20 @@ __global__ void k_refit(const float* __restrict__ v, const int* __restrict__ idx
     }
 }
 
+// results of the clustering on the device: the root's reference and height,
+// and whether one cluster is left
+enum { CTL_ROOT, CTL_HEIGHT, CTL_DONE, CTL_ROUND };  // then (N, pair neighbours, buffer) per round
+constexpr int CTL_ROUNDS = 64;  // slots
+
+// triangles, materials, texture coordinates and the slot of each original id
 __global__ void k_leaf_data(const float* __restrict__ v, const int* __restrict__ idx, const float* __restrict__ mat,
-                            const float* __restrict__ uv, const int* __restrict__ ids, int n, Tri* tris,
+                            const float* __restrict__ uv, const int* __restrict__ ids,
+                            const int* __restrict__ newpos, int m, const int* __restrict__ ctl, int n, Tri* tris,
                             float4* mato, float2* uvo, int* slot_of, int* specular) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    int id = ids[k];
+    if (k >= n || (ctl && !ctl[CTL_DONE])) return;
+    const int id = ids[k];
+    if (newpos && k < m) k = newpos[k];  // the triangle's depth-first leaf position
     slot_of[id] = k;
     int a = idx[3 * id], b = idx[3 * id + 1], c = idx[3 * id + 2];
     Tri t;
@@ -260,10 +282,10 @@ __global__ void k_leaf_data(const float* __restrict__ v, const int* __restrict__
     t.v1 = make_float4(v[3 * b], v[3 * b + 1], v[3 * b + 2], 0.f);
     t.v2 = make_float4(v[3 * c], v[3 * c + 1], v[3 * c + 2], 0.f);
     tris[k] = t;
-    const float* m = mat + 8 * (size_t)id;
-    mato[2 * k] = make_float4(m[0], m[1], m[2], m[3]);
-    mato[2 * k + 1] = make_float4(m[4], m[5], m[6], m[7]);
-    if (m[7] > 0.f) atomicOr(specular, 1);
+    const float* mt = mat + 8 * (size_t)id;
+    mato[2 * k] = make_float4(mt[0], mt[1], mt[2], mt[3]);
+    mato[2 * k + 1] = make_float4(mt[4], mt[5], mt[6], mt[7]);
+    if (mt[7] > 0.f) atomicOr(specular, 1);
     if (uv) {
         const float* u = uv + 6 * (size_t)id;
         uvo[3 * k] = make_float2(u[0], u[1]);
@@ -324,8 +346,8 @@ __global__ void k_depth(const int* __restrict__ leaf_parent, const Node* __restr
 constexpr int PLOC_R_SMALL = 64, PLOC_R_BIG = 48;
 constexpr int PLOC_BIG = 1 << 20;
 constexpr int PLOC_B = 256;
-constexpr int PLOC_SYNC = 8;  // clustering rounds between reads of the cluster count
-
+constexpr int PLOC_CB = 1024;    // clusters per block of the count and the merge
+constexpr int PLOC_CAP = 1024;   // clusters from which one block finishes in shared memory
 __device__ __forceinline__ float union_area(float4 alo, float4 ahi, float4 blo, float4 bhi) {
     float x = fmaxf(ahi.x, bhi.x) - fminf(alo.x, blo.x);
     float y = fmaxf(ahi.y, bhi.y) - fminf(alo.y, blo.y);
@@ -333,122 +355,284 @@ __device__ __forceinline__ float union_area(float4 alo, float4 ahi, float4 blo, 
     return x * y + y * z + z * x;
 }
 
+// A cluster: its node or leaf reference, and its box with the number of
+// triangles (lo.w) and the height (hi.w) as int bits.
+struct Clusters {
+    int* ref[2];
+    float4 *lo[2], *hi[2];
+};
+
 __global__ void k_ploc_init(const float* __restrict__ v, const int* __restrict__ idx, const int* __restrict__ ids,
-                            int n, int* ref, float4* lo, float4* hi, int* hgt) {
+                            int n, Clusters c, int* ctl) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) {
+        ctl[CTL_DONE] = 0;
+        ctl[CTL_ROUND] = n;
+        ctl[CTL_ROUND + 1] = 0;
+        ctl[CTL_ROUND + 2] = 0;
+    }
     if (i >= n) return;
     float l[3], h[3];
     tri_box(v, idx, ids[i], l, h);
-    ref[i] = leaf_ref(i, 1);
-    lo[i] = make_float4(l[0], l[1], l[2], 0.f);
-    hi[i] = make_float4(h[0], h[1], h[2], 0.f);
-    hgt[i] = 0;
+    c.ref[0][i] = leaf_ref(i, 1);
+    c.lo[0][i] = make_float4(l[0], l[1], l[2], __int_as_float(1));
+    c.hi[0][i] = make_float4(h[0], h[1], h[2], __int_as_float(0));
 }
 
-// Round control of the clustering on the device, so that the host need not
-// read the cluster count back every round: ctl[0] = live clusters N, ctl[1] =
-// pair neighbours this round (the last round found no mutual pair), ctl[2] =
-// the buffer holding the clusters.  The round kernels are launched over an
-// upper bound Nb >= N and do nothing once N <= 1.
-__global__ void k_ploc_ctl_init(int* ctl, int n) {
-    ctl[0] = n;
-    ctl[1] = 0;
-    ctl[2] = 0;
-}
+// Rounds on the device, so that the host need not read the cluster count:
+// round r reads (N, pair neighbours this round, buffer holding the clusters)
+// from its slot of ctl and writes the next round's.  The round kernels are
+// launched over an upper bound of N and leave a round with N <= PLOC_CAP to
+// k_ploc_finish.  Three launches a round (neighbours; counts of the clusters
+// that stay; merge and compaction).  A tree of 165k triangles takes about 25
+// such rounds and 45 in k_ploc_finish; with every round in six launches over
+// all clusters, the leaf data moved twice and the subtree sizes walked
+// bottom-up (they are the clusters' counts) its build took 3.1 ms, so 1.34
+// (20k triangles 2.6 -> 0.94, 5.2M 11.0 -> 7.0).
+__device__ __forceinline__ const int* ctl_slot(const int* ctl, int round) { return ctl + CTL_ROUND + 3 * round; }
 
 template <int PLOC_R>
-__global__ void __launch_bounds__(PLOC_B) k_ploc_nn(const int* __restrict__ ctl, const float4* __restrict__ lo,
-                                                    const float4* __restrict__ hi, int* __restrict__ nn) {
-    const int N = ctl[0];
-    if (N <= 1 || ctl[1]) return;  // done, or pairing neighbours: the whole block leaves
+__global__ void __launch_bounds__(PLOC_B) k_ploc_nn(const int* __restrict__ ctl, int round, Clusters c,
+                                                    int* __restrict__ nn) {
+    const int* st = ctl_slot(ctl, round);
+    const int N = st[0];
+    if (N <= PLOC_CAP || st[1]) return;  // done here, or pairing neighbours: the whole block leaves
+    const float4* __restrict__ lo = c.lo[st[2]];
+    const float4* __restrict__ hi = c.hi[st[2]];
     __shared__ float4 slo[PLOC_B + 2 * PLOC_R], shi[PLOC_B + 2 * PLOC_R];
-    const int base = blockIdx.x * PLOC_B - PLOC_R;
-    for (int k = threadIdx.x; k < PLOC_B + 2 * PLOC_R; k += PLOC_B) {
-        int g = base + k;
-        if (g >= 0 && g < N) {
-            slo[k] = lo[g];
-            shi[k] = hi[g];
+    for (int first = blockIdx.x * PLOC_B; first < N; first += gridDim.x * PLOC_B) {
+        const int base = first - PLOC_R;
+        __syncthreads();  // the previous chunk's searches
+        for (int k = threadIdx.x; k < PLOC_B + 2 * PLOC_R; k += PLOC_B) {
+            int g = base + k;
+            if (g >= 0 && g < N) {
+                slo[k] = lo[g];
+                shi[k] = hi[g];
+            }
         }
-    }
-    __syncthreads();
-    const int i = blockIdx.x * PLOC_B + threadIdx.x;
-    if (i >= N) return;
-    const int li = threadIdx.x + PLOC_R;
-    const float4 a0 = slo[li], a1 = shi[li];
-    float best = __int_as_float(0x7f800000);
-    int bj = -1;
-    const int j0 = max(i - PLOC_R, 0), j1 = min(i + PLOC_R, N - 1);
-    for (int j = j0; j <= j1; ++j) {
-        if (j == i) continue;
-        float c = union_area(a0, a1, slo[j - base], shi[j - base]);
-        if (c < best) {  // ascending j: ties keep the lower index
-            best = c;
-            bj = j;
+        __syncthreads();
+        const int i = first + threadIdx.x;
+        if (i >= N) continue;
+        const int li = threadIdx.x + PLOC_R;
+        const float4 a0 = slo[li], a1 = shi[li];
+        float best = __int_as_float(0x7f800000);
+        int bj = -1;
+        const int j0 = max(i - PLOC_R, 0), j1 = min(i + PLOC_R, N - 1);
+        for (int j = j0; j <= j1; ++j) {
+            if (j == i) continue;
+            float cost = union_area(a0, a1, slo[j - base], shi[j - base]);
+            if (cost < best) {  // ascending j: ties keep the lower index
+                best = cost;
+                bj = j;
+            }
         }
+        nn[i] = bj;
     }
-    nn[i] = bj;
 }
 
-// merge mutual nearest neighbours (or, when force_pairs, positions 2k and 2k+1);
-// positions N .. Nb - 1 are marked invalid for the scan
-__global__ void k_ploc_merge(int Nb, const int* __restrict__ ctl, const int* __restrict__ nn, int* ref, float4* lo,
-                             float4* hi, int* hgt, int* valid, Node* nodes, unsigned* counter) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Nb) return;
-    const int N = ctl[0], force_pairs = ctl[1];
-    if (N <= 1) return;
-    if (i >= N) {
-        valid[i] = 0;
-        return;
+// the cluster that i merges with this round (-1: none): mutual nearest
+// neighbours, or, when pairing, positions 2k and 2k + 1.  The pair's node
+// takes the lower position; the upper one is dropped.
+__device__ __forceinline__ int ploc_partner(int i, int N, int pair, const int* nn) {
+    if (pair) return (i & 1) ? i - 1 : (i + 1 < N ? i + 1 : -1);
+    const int j = nn[i];
+    return j >= 0 && nn[j] == i ? j : -1;
+}
+
+__global__ void __launch_bounds__(PLOC_CB) k_ploc_count(const int* __restrict__ ctl, int round,
+                                                        const int* __restrict__ nn, int* __restrict__ counts) {
+    const int* st = ctl_slot(ctl, round);
+    const int N = st[0];
+    if (N <= PLOC_CAP) return;
+    for (int b = blockIdx.x; b * PLOC_CB < N; b += gridDim.x) {
+        const int i = b * PLOC_CB + threadIdx.x;
+        bool stays = false;
+        if (i < N) {
+            const int j = ploc_partner(i, N, st[1], nn);
+            stays = j < 0 || j > i;
+        }
+        const int c = __syncthreads_count(stays);
+        if (threadIdx.x == 0) counts[b] = c;
     }
-    int j = force_pairs ? ((i & 1) ? i - 1 : (i + 1 < N ? i + 1 : -1)) : nn[i];
-    bool mutual = j >= 0 && (force_pairs || nn[j] == i);
-    if (!mutual) {
-        valid[i] = 1;
-        return;
-    }
-    if (j < i) {  // merged into the lower position
-        valid[i] = 0;
-        return;
-    }
-    float4 al = lo[i], ah = hi[i], bl = lo[j], bh = hi[j];
-    int idn = (int)atomicAdd(counter, 1u);
+}
+
+// the node of clusters a and b; its clusters' parent references follow
+__device__ __forceinline__ void ploc_node(Node* nodes, int id, int ra, float4 al, float4 ah, int rb, float4 bl,
+                                          float4 bh, float4& lo, float4& hi) {
     Node nd;
     nd.xy0 = make_float4(al.x, ah.x, al.y, ah.y);
     nd.xy1 = make_float4(bl.x, bh.x, bl.y, bh.y);
     nd.z01 = make_float4(al.z, ah.z, bl.z, bh.z);
-    nd.child = make_int4(ref[i], ref[j], 0, 0);
-    nodes[idn] = nd;
-    ref[i] = idn;
-    lo[i] = make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), 0.f);
-    hi[i] = make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z), 0.f);
-    hgt[i] = max(hgt[i], hgt[j]) + 1;
-    valid[i] = 1;
+    const int cnt = __float_as_int(al.w) + __float_as_int(bl.w);
+    nd.child = make_int4(ra, rb, -1, cnt - 1);  // (parent: none yet; internal nodes of the subtree)
+    nodes[id] = nd;
+    if (ra >= 0) nodes[ra].child.z = id;
+    if (rb >= 0) nodes[rb].child.z = id;
+    lo = make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), __int_as_float(cnt));
+    hi = make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z),
+                     __int_as_float(max(__float_as_int(ah.w), __float_as_int(bh.w)) + 1));
 }
 
-__global__ void k_ploc_compact(int Nb, const int* __restrict__ ctl, const int* __restrict__ valid,
-                               const int* __restrict__ pos, const int* __restrict__ ref, const float4* __restrict__ lo,
-                               const float4* __restrict__ hi, const int* __restrict__ hgt, int* ref2, float4* lo2,
-                               float4* hi2, int* hgt2) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Nb) return;
-    const int N = ctl[0];
-    if (N <= 1 || i >= N || !valid[i]) return;
-    int k = pos[i];
-    ref2[k] = ref[i];
-    lo2[k] = lo[i];
-    hi2[k] = hi[i];
-    hgt2[k] = hgt[i];
+// exclusive prefix of a flag over a block of PLOC_CB threads, and its total
+__device__ __forceinline__ int block_rank(bool f, int* s_warp, int& total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned m = __ballot_sync(0xffffffffu, f);
+    if (lane == 0) s_warp[w] = __popc(m);
+    __syncthreads();
+    const int c = s_warp[lane];  // PLOC_CB / 32 = 32 warps
+    const int before = __reduce_add_sync(0xffffffffu, lane < w ? c : 0);
+    total = __reduce_add_sync(0xffffffffu, c);
+    __syncthreads();
+    return before + __popc(m & ((1u << lane) - 1u));
 }
 
-// the next round's N and mode, and the buffer the compaction filled (dst)
-__global__ void k_ploc_next(int* ctl, const int* __restrict__ valid, const int* __restrict__ pos, int dst) {
-    const int N = ctl[0];
-    if (N <= 1) return;
-    const int nN = pos[N - 1] + valid[N - 1];
-    ctl[1] = nN == N;  // no mutual pair this round: pair neighbours once
-    ctl[0] = nN;
-    ctl[2] = dst;
+__global__ void __launch_bounds__(PLOC_CB) k_ploc_merge(int* ctl, int round, const int* __restrict__ nn,
+                                                        const int* __restrict__ counts, Clusters c, Node* nodes,
+                                                        unsigned* counter) {
+    const int* st = ctl_slot(ctl, round);
+    int* next = ctl + CTL_ROUND + 3 * (round + 1);
+    const int N = st[0], pair = st[1], buf = st[2];
+    if (N <= PLOC_CAP) {
+        if (blockIdx.x == 0 && threadIdx.x < 3) next[threadIdx.x] = st[threadIdx.x];
+        return;
+    }
+    __shared__ int s_warp[32];
+    __shared__ int s_base;
+    int counted = 0;  // chunks in s_base so far
+    if (threadIdx.x == 0) s_base = 0;
+    for (int b = blockIdx.x; b * PLOC_CB < N; b += gridDim.x) {
+        __syncthreads();
+        int before = 0;  // clusters that stay in the chunks before this one
+        for (int k = counted + threadIdx.x; k < b; k += PLOC_CB) before += counts[k];
+        counted = b;
+        before = __reduce_add_sync(0xffffffffu, before);
+        if ((threadIdx.x & 31) == 0 && before) atomicAdd(&s_base, before);
+        const int i = b * PLOC_CB + threadIdx.x;
+        const int j = i < N ? ploc_partner(i, N, pair, nn) : -1;
+        const bool stays = i < N && (j < 0 || j > i);
+        int total;
+        const int rank = block_rank(stays, s_warp, total);  // (synchronises s_base too)
+        const int k = s_base + rank;
+        if (stays) {
+            int ref = c.ref[buf][i];
+            float4 lo = c.lo[buf][i], hi = c.hi[buf][i];
+            if (j >= 0) {
+                const int id = (int)atomicAdd(counter, 1u);
+                ploc_node(nodes, id, ref, lo, hi, c.ref[buf][j], c.lo[buf][j], c.hi[buf][j], lo, hi);
+                ref = id;
+            }
+            c.ref[1 - buf][k] = ref;
+            c.lo[1 - buf][k] = lo;
+            c.hi[1 - buf][k] = hi;
+        }
+        if (threadIdx.x == 0 && (b + 1) * PLOC_CB >= N) {  // the last chunk
+            next[0] = s_base + total;
+            next[1] = s_base + total == N;  // no mutual pair this round: pair neighbours once
+            next[2] = 1 - buf;
+        }
+    }
+}
+
+// The last rounds, N <= PLOC_CAP, by one block with the clusters in shared
+// memory: the same rounds, at a microsecond or two instead of six launches
+// each.  Most of a tree's 70 rounds are such (each merges few of the clusters
+// left).  While N <= PLOC_CB / 2, several threads share a cluster's search.
+struct FinishSmem {
+    float4 lo[PLOC_CAP], hi[PLOC_CAP];
+    int ref[PLOC_CAP], nn[PLOC_CAP];
+    int warp[32];
+};
+template <int PLOC_R>
+__global__ void __launch_bounds__(PLOC_CB) k_ploc_finish(int* ctl, int round, Clusters c, Node* nodes,
+                                                         unsigned* counter) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    FinishSmem& s = *reinterpret_cast<FinishSmem*>(s_raw);
+    constexpr int PER = PLOC_CAP / PLOC_CB;
+    const int* st = ctl_slot(ctl, round);
+    int N = st[0], pair = st[1];
+    const int buf = st[2], t = threadIdx.x;
+    if (N > PLOC_CAP) return;  // more rounds first
+    for (int k = t; k < N; k += PLOC_CB) {
+        s.ref[k] = c.ref[buf][k];
+        s.lo[k] = c.lo[buf][k];
+        s.hi[k] = c.hi[buf][k];
+    }
+    __syncthreads();
+    for (int guard = 0; N > 1 && guard < 4 * PLOC_CAP; ++guard) {  // a round, or the pairing after it, merges
+        if (!pair) {
+            int P = 1;  // threads per cluster
+            while (P < 32 && N * P * 2 <= PLOC_CB) P *= 2;
+            for (int i0 = 0; i0 < N; i0 += PLOC_CB / P) {
+                const int i = i0 + t / P, sub = t & (P - 1);
+                float best = __int_as_float(0x7f800000);
+                int bj = -1;
+                if (i < N) {
+                    const float4 a0 = s.lo[i], a1 = s.hi[i];
+                    const int j0 = max(i - PLOC_R, 0), j1 = min(i + PLOC_R, N - 1);
+                    for (int j = j0 + sub; j <= j1; j += P) {
+                        if (j == i) continue;
+                        const float cost = union_area(a0, a1, s.lo[j], s.hi[j]);
+                        if (cost < best) {
+                            best = cost;
+                            bj = j;
+                        }
+                    }
+                }
+                for (int o = P >> 1; o; o >>= 1) {  // (the loops' trip counts are block-uniform)
+                    const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+                    const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+                    if (oj >= 0 && (bj < 0 || ob < best || (ob == best && oj < bj))) {
+                        best = ob;
+                        bj = oj;
+                    }
+                }
+                if (i < N && sub == 0) s.nn[i] = bj;
+            }
+            __syncthreads();
+        }
+        // merge and compact in place: every cluster of this round is read before any is written
+        int ref[PER], pos[PER];
+        float4 lo[PER], hi[PER];
+        int base = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int i = q * PLOC_CB + t;
+            pos[q] = -1;
+            if (q * PLOC_CB >= N) continue;  // block-uniform
+            const int j = i < N ? ploc_partner(i, N, pair, s.nn) : -1;
+            const bool stays = i < N && (j < 0 || j > i);
+            int total;
+            const int rank = block_rank(stays, s.warp, total);
+            if (stays) {
+                pos[q] = base + rank;
+                ref[q] = s.ref[i];
+                lo[q] = s.lo[i];
+                hi[q] = s.hi[i];
+                if (j >= 0) {
+                    const int id = (int)atomicAdd(counter, 1u);
+                    ploc_node(nodes, id, ref[q], lo[q], hi[q], s.ref[j], s.lo[j], s.hi[j], lo[q], hi[q]);
+                    ref[q] = id;
+                }
+            }
+            base += total;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (pos[q] >= 0) {
+                s.ref[pos[q]] = ref[q];
+                s.lo[pos[q]] = lo[q];
+                s.hi[pos[q]] = hi[q];
+            }
+        __syncthreads();
+        pair = base == N;
+        N = base;
+    }
+    if (t == 0) {
+        ctl[CTL_ROOT] = s.ref[0];
+        ctl[CTL_HEIGHT] = __float_as_int(s.hi[0].w);
+        ctl[CTL_DONE] = N == 1;
+    }
 }
 
 __global__ void k_big_boxes(const Tri* __restrict__ tris, int first, int n_big, float4* box) {
@@ -472,152 +656,67 @@ __global__ void k_closest(BvhView bvh, int n, const float* __restrict__ org, con
 
 int blocks_for(long n, int bs) { return (int)((n + bs - 1) / bs); }
 
-// ---- depth-first relabelling of the internal nodes --------------------------
+// ---- depth-first order and leaves -------------------------------------------
 // The clustering numbers nodes in merge order, which scatters a parent and its
 // children over memory.  Relabelling in depth-first pre-order (a node, then
 // its first child's subtree, then its second child's) keeps every subtree in
 // one contiguous range and puts a node's first child right after it, so a
-// descent touches neighbouring cache lines.  The tree itself is unchanged.
-
-__global__ void k_dfs_parent(const Node* __restrict__ nodes, int n, int* parent, int* nint) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int4 c = nodes[i].child;
-    int k = 0;
-    if (c.x >= 0) {
-        parent[c.x] = i;
-        ++k;
-    }
-    if (c.y >= 0) {
-        parent[c.y] = i;
-        ++k;
-    }
-    nint[i] = k;
-}
-
-// subtree sizes (internal nodes) bottom-up: a node with no internal child
-// starts a walk; the last child to arrive at a parent carries the walk on
-__global__ void k_dfs_size(const Node* __restrict__ nodes, int n, int root, const int* __restrict__ parent,
-                           const int* __restrict__ nint, unsigned* arrived, int* size) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || nint[i] != 0) return;
-    int c = i;
-    size[c] = 1;
-    for (int guard = 0; c != root && guard < n; ++guard) {  // a walk is at most the tree's depth
-        const int p = parent[c];
-        __threadfence();
-        if (atomicAdd(&arrived[p], 1u) + 1 < (unsigned)nint[p]) return;  // the other child is not done yet
-        __threadfence();
-        const int4 ch = nodes[p].child;
-        size[p] = 1 + (ch.x >= 0 ? __ldcg(&size[ch.x]) : 0) + (ch.y >= 0 ? __ldcg(&size[ch.y]) : 0);
-        c = p;
-    }
-}
-
-// pre-order index: 1 per ancestor step, plus the first child's subtree when
-// the path goes through a second child
-__global__ void k_dfs_index(const Node* __restrict__ nodes, int n, int root, const int* __restrict__ parent,
-                            const int* __restrict__ size, int* index) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int idx = 0, c = i;
-    for (int guard = 0; c != root && guard < n; ++guard) {
-        const int p = parent[c];
-        const int4 ch = nodes[p].child;
-        idx += 1;
-        if (c == ch.y && ch.x >= 0) idx += size[ch.x];
-        c = p;
-    }
-    index[i] = idx;
-}
-
-__global__ void k_dfs_permute(const Node* __restrict__ nodes, int n, const int* __restrict__ parent,
-                              const int* __restrict__ index, const int* __restrict__ size, int root, Node* out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    Node nd = nodes[i];
-    if (nd.child.x >= 0) nd.child.x = index[nd.child.x];
-    if (nd.child.y >= 0) nd.child.y = index[nd.child.y];
-    nd.child.z = i == root ? -1 : index[parent[i]];
-    nd.child.w = size[i];  // internal nodes of the subtree (kept for the leaf collapse)
-    out[index[i]] = nd;
-}
-
-// Leaf collapse of the clustered tree (in pre-order: node 0 the root,
-// child.z the parent, child.w the subtree's internal node count; every leaf
-// one triangle).  The triangles are moved to depth-first leaf order, so the
-// triangles of any subtree occupy consecutive slots, and each subtree of at
-// most leaf_max triangles becomes one leaf over them: fewer traversal steps
-// for one more triangle test per extra triangle.  The tree's boxes and the
-// closest hits are unchanged.
+// descent touches neighbouring cache lines.  The triangles are stored in
+// depth-first leaf order, so the triangles of any subtree occupy consecutive
+// slots, and each subtree of at most leaf_max triangles becomes one leaf over
+// them: fewer traversal steps for one more triangle test per extra triangle.
+// The tree itself, its boxes and the closest hits are unchanged.
 __device__ __forceinline__ int n_leaves(const Node* __restrict__ nodes, int ref) {
     return ref >= 0 ? __ldg(&nodes[ref].child.w) + 1 : 1;
 }
 
-// first leaf position of each node's subtree: the leaves of every first-child
-// subtree that the path from the root passes on its left
-__global__ void k_leaf_first(const Node* __restrict__ nodes, int n, int* first) {
+// pre-order index and first leaf position of each node: per step towards the
+// root one node, plus the first child's subtree when the path goes through a
+// second child
+__global__ void k_dfs_index(const Node* __restrict__ nodes, int n, const int* __restrict__ ctl, int2* place) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int idx = 0, c = i;
-    for (int guard = 0; c != 0 && guard < n; ++guard) {  // a walk is at most the tree's depth
-        const int p = __ldg(&nodes[c].child.z);
+    if (i >= n || !ctl[CTL_DONE]) return;
+    const int root = ctl[CTL_ROOT];
+    int idx = 0, leaf = 0, c = i, p = __ldg(&nodes[i].child.z);
+    for (int guard = 0; c != root && guard < n; ++guard) {  // a walk is at most the tree's depth
         const int4 ch = __ldg(&nodes[p].child);
-        if (c == ch.y) idx += n_leaves(nodes, ch.x);
+        idx += 1;
+        if (c == ch.y) {
+            const int l = n_leaves(nodes, ch.x);
+            leaf += l;
+            idx += l - 1;
+        }
         c = p;
+        p = ch.z;
     }
-    first[i] = idx;
+    place[i] = make_int2(idx, leaf);
 }
 
-// new slot of each tree triangle: its depth-first leaf position
-__global__ void k_leaf_slots(const Node* __restrict__ nodes, int n, int m, const int* __restrict__ first,
-                             int* newpos) {
+// nodes to their places, with their children's new references; the new slot
+// of each sorted triangle
+__global__ void k_dfs_permute(const Node* __restrict__ nodes, int n, const int* __restrict__ ctl,
+                              const int2* __restrict__ place, int leaf_max, Node* out, int* newpos) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int4 ch = __ldg(&nodes[i].child);
-    const int f = first[i];
-    if (ch.x < 0 && ((~ch.x) >> 3) < m) newpos[(~ch.x) >> 3] = f;
-    if (ch.y < 0 && ((~ch.y) >> 3) < m) newpos[(~ch.y) >> 3] = f + n_leaves(nodes, ch.x);
-}
-
-// triangles, materials and texture coordinates to their new slots
-__global__ void k_tri_permute(const int* __restrict__ newpos, int m, const Tri* __restrict__ tin,
-                              const float4* __restrict__ min, const float2* __restrict__ uin, Tri* tout,
-                              float4* mout, float2* uout, int* slot_of) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= m) return;
-    const int d = newpos[k];
-    if (d < 0 || d >= m) return;  // unreachable for a full binary tree over the m slots
-    const Tri t = tin[k];
-    tout[d] = t;
-    mout[2 * d] = min[2 * k];
-    mout[2 * d + 1] = min[2 * k + 1];
-    uout[3 * d] = uin[3 * k];
-    uout[3 * d + 1] = uin[3 * k + 1];
-    uout[3 * d + 2] = uin[3 * k + 2];
-    slot_of[__float_as_int(t.v0.w)] = d;
-}
-
-// leaf references to the new slots; subtrees of at most leaf_max triangles
-// become leaves (only child.x and child.y are written; child.w is read)
-__global__ void k_leaf_collapse(Node* nodes, int n, const int* __restrict__ first, int leaf_max) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int cx = nodes[i].child.x, cy = nodes[i].child.y;
-    const int c[2] = {cx, cy};
-    const int start[2] = {first[i], first[i] + (cx >= 0 ? nodes[cx].child.w + 1 : 1)};
-    int out[2];
+    if (i >= n || !ctl[CTL_DONE]) return;
+    Node nd = nodes[i];
+    const int2 pl = place[i];
+    const int c[2] = {nd.child.x, nd.child.y};
+    int o[2], first = pl.y;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
+        const int cnt = n_leaves(nodes, c[k]);
         if (c[k] < 0) {
-            out[k] = leaf_ref(start[k], 1);
+            newpos[(~c[k]) >> 3] = first;
+            o[k] = leaf_ref(first, 1);
         } else {
-            const int cnt = nodes[c[k]].child.w + 1;
-            out[k] = cnt <= leaf_max ? leaf_ref(start[k], cnt) : c[k];
+            o[k] = cnt <= leaf_max ? leaf_ref(first, cnt) : place[c[k]].x;
         }
+        first += cnt;
     }
-    nodes[i].child.x = out[0];
-    nodes[i].child.y = out[1];
+    nd.child.x = o[0];
+    nd.child.y = o[1];
+    nd.child.z = nd.child.z < 0 ? -1 : place[nd.child.z].x;
+    out[pl.x] = nd;
 }
 
 }  // namespace
@@ -632,38 +731,6 @@ size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 #define HDOF_PLOC_LEAF_MAX 2  // largest collapsed leaf of the clustered tree (<= 8; 1: no collapse); 2 measured fastest
 #endif
 
-// Leaf collapse of the relabelled clustered tree (ni internal nodes over the
-// first m triangle slots): see k_leaf_first .. k_leaf_collapse.
-cudaError_t collapse_leaves(hdof_bvh* b, int ni, int m, int leaf_max, cudaStream_t s) {
-    const size_t q1 = up256(4 * (size_t)ni), q2 = q1 + up256(4 * (size_t)m);
-    const size_t q3 = q2 + up256(sizeof(Tri) * (size_t)m), q4 = q3 + up256(2 * sizeof(float4) * (size_t)m);
-    const size_t tot = q4 + 3 * sizeof(float2) * (size_t)m;
-    void* mem = nullptr;
-    cudaError_t e = cudaMalloc(&mem, tot);
-    if (e != cudaSuccess) return e;
-    char* c8 = static_cast<char*>(mem);
-    int* first = reinterpret_cast<int*>(c8);
-    int* newpos = reinterpret_cast<int*>(c8 + q1);
-    Tri* tcopy = reinterpret_cast<Tri*>(c8 + q2);
-    float4* mcopy = reinterpret_cast<float4*>(c8 + q3);
-    float2* ucopy = reinterpret_cast<float2*>(c8 + q4);
-    if ((e = cudaMemsetAsync(newpos, 0xff, 4 * (size_t)m, s)) == cudaSuccess &&
-        (e = cudaMemcpyAsync(tcopy, b->tris, sizeof(Tri) * (size_t)m, cudaMemcpyDeviceToDevice, s)) == cudaSuccess &&
-        (e = cudaMemcpyAsync(mcopy, b->mat, 2 * sizeof(float4) * (size_t)m, cudaMemcpyDeviceToDevice, s)) ==
-            cudaSuccess &&
-        (e = cudaMemcpyAsync(ucopy, b->uv, 3 * sizeof(float2) * (size_t)m, cudaMemcpyDeviceToDevice, s)) ==
-            cudaSuccess) {
-        k_leaf_first<<<blocks_for(ni, 256), 256, 0, s>>>(b->nodes, ni, first);
-        k_leaf_slots<<<blocks_for(ni, 256), 256, 0, s>>>(b->nodes, ni, m, first, newpos);
-        k_tri_permute<<<blocks_for(m, 256), 256, 0, s>>>(newpos, m, tcopy, mcopy, ucopy, b->tris, b->mat, b->uv,
-                                                         b->slot_of);
-        k_leaf_collapse<<<blocks_for(ni, 256), 256, 0, s>>>(b->nodes, ni, first, leaf_max);
-        e = cudaGetLastError();
-    }
-    cudaError_t e2 = cudaStreamSynchronize(s);
-    cudaFree(mem);
-    return e != cudaSuccess ? e : e2;
-}
 }  // namespace
 
 extern "C" int hdof_build_bvh(const float* verts, int32_t n_verts, const int32_t* idx, int32_t n_tris,
@@ -681,26 +748,48 @@ extern "C" int hdof_build_bvh(const float* verts, int32_t n_verts, const int32_t
     size_t sort_bytes = 0;
     cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, (unsigned long long*)nullptr, (unsigned long long*)nullptr,
                                     (int*)nullptr, (int*)nullptr, n, 0, 64, s);
-    const size_t nn = (size_t)(n > 1 ? n - 1 : 1);
-    size_t o_keys_in = 256, o_keys_out = o_keys_in + up256(8 * (size_t)n), o_ids_in = o_keys_out + up256(8 * (size_t)n);
-    size_t o_ids_out = o_ids_in + up256(4 * (size_t)n), o_lp = o_ids_out + up256(4 * (size_t)n);
-    size_t o_flags = o_lp + up256(4 * (size_t)n), o_big = o_flags + up256(4 * nn), o_rng = o_big + up256((size_t)n);
-    size_t o_cnt = o_rng + up256(8 * nn), o_sort = o_cnt + 256, tmp_total = o_sort + sort_bytes;
+    const size_t N = (size_t)n;
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o += up256(bytes);
+        return at;
+    };
+    const size_t o_bounds = take(NB * sizeof(unsigned)), o_cnt = take(sizeof(unsigned));
+    const size_t o_ctl = take((CTL_ROUND + 3 * CTL_ROUNDS) * sizeof(int));
+    const size_t o_keys_in = take(8 * N), o_keys_out = take(8 * N), o_ids_in = take(4 * N), o_ids_out = take(4 * N);
+    const size_t o_sort = take(sort_bytes);
+    // the clustering's, or the linear tree's
+    const size_t o_ref0 = take(4 * N), o_ref1 = take(4 * N), o_lo0 = take(16 * N), o_lo1 = take(16 * N);
+    const size_t o_hi0 = take(16 * N), o_hi1 = take(16 * N), o_nn = take(4 * N), o_counts = take(4 * (N / PLOC_CB + 1));
+    const size_t o_nodes = take(sizeof(Node) * N), o_place = take(8 * N), o_newpos = take(4 * N), o_big = take(N);
     void* tmp = nullptr;
-    cudaError_t e = cudaMalloc(&tmp, tmp_total);
+    cudaError_t e = cudaMalloc(&tmp, o);
     if (e != cudaSuccess) return cuda_fail(e, "hdof_build_bvh: cudaMalloc scratch");
     char* t8 = static_cast<char*>(tmp);
-    unsigned* bounds = reinterpret_cast<unsigned*>(t8);
+    unsigned* bounds = reinterpret_cast<unsigned*>(t8 + o_bounds);
+    unsigned* counters = reinterpret_cast<unsigned*>(t8 + o_cnt);  // [0] nodes (clustering), tree depth (linear tree)
+    int* ctl = reinterpret_cast<int*>(t8 + o_ctl);
     unsigned long long* keys_in = reinterpret_cast<unsigned long long*>(t8 + o_keys_in);
     unsigned long long* keys_out = reinterpret_cast<unsigned long long*>(t8 + o_keys_out);
     int* ids_in = reinterpret_cast<int*>(t8 + o_ids_in);
     int* ids_out = reinterpret_cast<int*>(t8 + o_ids_out);
-    int* leaf_parent = reinterpret_cast<int*>(t8 + o_lp);
-    unsigned* flags = reinterpret_cast<unsigned*>(t8 + o_flags);
-    uint8_t* big = reinterpret_cast<uint8_t*>(t8 + o_big);
-    int2* rng = reinterpret_cast<int2*>(t8 + o_rng);
-    unsigned* counters = reinterpret_cast<unsigned*>(t8 + o_cnt);  // [0] tree depth
     void* sort_tmp = t8 + o_sort;
+    int* ref0 = reinterpret_cast<int*>(t8 + o_ref0);
+    int* ref1 = reinterpret_cast<int*>(t8 + o_ref1);
+    float4* lo0 = reinterpret_cast<float4*>(t8 + o_lo0);
+    float4* lo1 = reinterpret_cast<float4*>(t8 + o_lo1);
+    float4* hi0 = reinterpret_cast<float4*>(t8 + o_hi0);
+    float4* hi1 = reinterpret_cast<float4*>(t8 + o_hi1);
+    int* nn = reinterpret_cast<int*>(t8 + o_nn);
+    int* counts = reinterpret_cast<int*>(t8 + o_counts);
+    Node* nodes0 = reinterpret_cast<Node*>(t8 + o_nodes);
+    int2* place = reinterpret_cast<int2*>(t8 + o_place);
+    int* newpos = reinterpret_cast<int*>(t8 + o_newpos);
+    uint8_t* big = reinterpret_cast<uint8_t*>(t8 + o_big);
+    int* leaf_parent = ref0;                               // linear tree
+    unsigned* flags = reinterpret_cast<unsigned*>(ref1);
+    int2* rng = reinterpret_cast<int2*>(lo0);
 
     hdof_bvh* b = nullptr;
     auto fail = [&](int code) {
@@ -712,32 +801,36 @@ extern "C" int hdof_build_bvh(const float* verts, int32_t n_verts, const int32_t
         }
         return code;
     };
-    unsigned init[NB];
-    for (int k = 0; k < NB; ++k) init[k] = 0u;
-    for (int k : {0, 1, 2, 8, 9, 10, 14, 15, 16}) init[k] = 0xffffffffu;  // atomicMin slots
-    if ((e = cudaMemcpyAsync(bounds, init, sizeof init, cudaMemcpyHostToDevice, s)) != cudaSuccess)
-        return fail(cuda_fail(e, "hdof_build_bvh: init bounds"));
-    const int rb = blocks_for(n, 256) < 1024 ? blocks_for(n, 256) : 1024;
+    // minima start at all ones, the rest at zero
+    if ((e = cudaMemsetAsync(bounds, 0, NB * sizeof(unsigned), s)) == cudaSuccess)
+        for (int k : {0, 8, 14})
+            if (e == cudaSuccess) e = cudaMemsetAsync(bounds + k, 0xff, 3 * sizeof(unsigned), s);
+    if (e != cudaSuccess) return fail(cuda_fail(e, "hdof_build_bvh: init bounds"));
+    const int rb = blocks_for(n, 256) < 2 * sm_count() ? blocks_for(n, 256) : 2 * sm_count();
     k_scene_bounds<<<rb, 256, 0, s>>>(verts, n_verts, idx, n, bounds);
-    unsigned hb0[NB];
-    if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = cudaMemcpyAsync(hb0, bounds, sizeof hb0, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return fail(cuda_fail(e, "hdof_build_bvh: scene bounds"));
-    if (hb0[6]) {
-        set_error("hdof_build_bvh: a triangle index is outside 0..n_verts-1");
-        return fail(HDOF_EINVAL);
-    }
-    k_classify<<<rb, 256, 0, s>>>(verts, idx, n, 0.02f, bounds, big);
     unsigned hb[NB];
+    // before anything else reads a vertex through an index
     if ((e = cudaGetLastError()) != cudaSuccess ||
         (e = cudaMemcpyAsync(hb, bounds, sizeof hb, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return fail(cuda_fail(e, "hdof_build_bvh: classify"));
-    // separate scene-sized triangles only when they are few and the rest can form a tree
-    int n_big = (int)hb[7];
-    bool separate = n >= 64 && n_big > 0 && n_big <= HDOF_BIG_MAX && n - n_big >= 2;
-    if (!separate) n_big = 0;
+        return fail(cuda_fail(e, "hdof_build_bvh: scene bounds"));
+    if (hb[6]) {
+        set_error("hdof_build_bvh: a triangle index is outside 0..n_verts-1");
+        return fail(HDOF_EINVAL);
+    }
+    int n_big = 0;
+    bool separate = false;
+    if (HDOF_BIG_MAX > 0) {
+        k_classify<<<rb, 256, 0, s>>>(verts, idx, n, 0.02f, bounds, big);
+        if ((e = cudaGetLastError()) != cudaSuccess ||
+            (e = cudaMemcpyAsync(hb, bounds, sizeof hb, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+            return fail(cuda_fail(e, "hdof_build_bvh: classify"));
+        // separate scene-sized triangles only when they are few and the rest can form a tree
+        n_big = (int)hb[7];
+        separate = n >= 64 && n_big > 0 && n_big <= HDOF_BIG_MAX && n - n_big >= 2;
+        if (!separate) n_big = 0;
+    }
     const int n_small = n - n_big;
     const unsigned* cbounds = bounds + (separate ? 8 : 14);  // centroid bounds (lo at [0..2], hi at [3..5])
 
@@ -775,23 +868,22 @@ extern "C" int hdof_build_bvh(const float* verts, int32_t n_verts, const int32_t
     int* spec_flag = reinterpret_cast<int*>(base + off_spec);
     if ((e = cudaMemsetAsync(spec_flag, 0, sizeof(int), s)) != cudaSuccess)
         return fail(cuda_fail(e, "hdof_build_bvh: clear"));
-    k_leaf_data<<<blocks_for(n, 256), 256, 0, s>>>(verts, idx, mat, uv, ids_out, n, b->tris, b->mat, b->uv,
-                                                    b->slot_of, spec_flag);
-    if (n_big > 0) k_big_boxes<<<1, 64, 0, s>>>(b->tris, n - n_big, n_big, b->big_box);
-    int has_spec = 0;
-    if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&has_spec, spec_flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return fail(cuda_fail(e, "hdof_build_bvh: leaf data"));
-    b->specular = has_spec;
+    // leaf data in sorted order (newpos NULL) or at the depth-first positions of a clustered tree
+    auto leaf_data = [&](const int* newpos, const int* ctl) {
+        k_leaf_data<<<blocks_for(n, 256), 256, 0, s>>>(verts, idx, mat, uv, ids_out, newpos, n_small, ctl, n, b->tris,
+                                                       b->mat, b->uv, b->slot_of, spec_flag);
+        if (n_big > 0) k_big_boxes<<<1, 64, 0, s>>>(b->tris, n - n_big, n_big, b->big_box);
+    };
 
     int depth = 0;
     b->n_nodes = 0;
     if (n_small <= HDOF_LEAF_MAX) {
+        leaf_data(nullptr, nullptr);
         b->root = leaf_ref(0, n_small);
         depth = 1;
     } else if (HDOF_BUILDER == 0) {
         // binary LBVH over the first n_small sorted triangles, built in place
+        leaf_data(nullptr, nullptr);
         int minus1 = -1;
         Node* nodes = b->nodes;
         if ((e = cudaMemsetAsync(nodes, 0, sizeof(Node) * (size_t)(n_small - 1), s)) != cudaSuccess ||
@@ -813,111 +905,72 @@ extern "C" int hdof_build_bvh(const float* verts, int32_t n_verts, const int32_t
         b->root = 0;
     } else {
         // PLOC over the first n_small sorted triangles
-        const int m = n_small;
-        size_t scan_bytes = 0;
-        cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, (int*)nullptr, (int*)nullptr, m, s);
-        size_t o_ref0 = 0, o_ref1 = o_ref0 + up256(4 * (size_t)m), o_lo0 = o_ref1 + up256(4 * (size_t)m);
-        size_t o_lo1 = o_lo0 + up256(16 * (size_t)m), o_hi0 = o_lo1 + up256(16 * (size_t)m);
-        size_t o_hi1 = o_hi0 + up256(16 * (size_t)m), o_h0 = o_hi1 + up256(16 * (size_t)m);
-        size_t o_h1 = o_h0 + up256(4 * (size_t)m), o_nn = o_h1 + up256(4 * (size_t)m);
-        size_t o_val = o_nn + up256(4 * (size_t)m), o_pos = o_val + up256(4 * (size_t)m);
-        size_t o_ctl = o_pos + up256(4 * (size_t)m), o_scan = o_ctl + 256, ptotal = o_scan + scan_bytes;
-        void* pt = nullptr;
-        if ((e = cudaMalloc(&pt, ptotal)) != cudaSuccess) return fail(cuda_fail(e, "hdof_build_bvh: cudaMalloc"));
-        char* c8 = static_cast<char*>(pt);
-        int* ref[2] = {reinterpret_cast<int*>(c8 + o_ref0), reinterpret_cast<int*>(c8 + o_ref1)};
-        float4* lo[2] = {reinterpret_cast<float4*>(c8 + o_lo0), reinterpret_cast<float4*>(c8 + o_lo1)};
-        float4* hi[2] = {reinterpret_cast<float4*>(c8 + o_hi0), reinterpret_cast<float4*>(c8 + o_hi1)};
-        int* hgt[2] = {reinterpret_cast<int*>(c8 + o_h0), reinterpret_cast<int*>(c8 + o_h1)};
-        int* nn = reinterpret_cast<int*>(c8 + o_nn);
-        int* valid = reinterpret_cast<int*>(c8 + o_val);
-        int* pos = reinterpret_cast<int*>(c8 + o_pos);
-        int* ctl = reinterpret_cast<int*>(c8 + o_ctl);
-        void* scan_tmp = c8 + o_scan;
-        auto pfail = [&](int code) {
-            cudaStreamSynchronize(s);
-            cudaFree(pt);
-            return fail(code);
-        };
+        const int m = n_small, ni = m - 1;
+        Clusters c{{ref0, ref1}, {lo0, lo1}, {hi0, hi1}};
         if ((e = cudaMemsetAsync(counters, 0, sizeof(unsigned), s)) != cudaSuccess)
-            return pfail(cuda_fail(e, "hdof_build_bvh: clear"));
-        k_ploc_init<<<blocks_for(m, 256), 256, 0, s>>>(verts, idx, ids_out, m, ref[0], lo[0], hi[0], hgt[0]);
-        k_ploc_ctl_init<<<1, 1, 0, s>>>(ctl, m);
-        // rounds run in batches of PLOC_SYNC with the cluster count kept on the
-        // device; the host reads it between batches for a tighter launch bound
-        int Nb = m, cur = 0, rounds = 0, buf = 0;
-        while (true) {
-            for (int r = 0; r < PLOC_SYNC; ++r) {
-                if (m > PLOC_BIG) k_ploc_nn<PLOC_R_BIG><<<blocks_for(Nb, PLOC_B), PLOC_B, 0, s>>>(ctl, lo[cur], hi[cur], nn);
-                else k_ploc_nn<PLOC_R_SMALL><<<blocks_for(Nb, PLOC_B), PLOC_B, 0, s>>>(ctl, lo[cur], hi[cur], nn);
-                k_ploc_merge<<<blocks_for(Nb, 256), 256, 0, s>>>(Nb, ctl, nn, ref[cur], lo[cur], hi[cur], hgt[cur],
-                                                                valid, b->nodes, counters);
-                e = cub::DeviceScan::ExclusiveSum(scan_tmp, scan_bytes, valid, pos, Nb, s);
-                if (e != cudaSuccess) return pfail(cuda_fail(e, "hdof_build_bvh: scan"));
-                k_ploc_compact<<<blocks_for(Nb, 256), 256, 0, s>>>(Nb, ctl, valid, pos, ref[cur], lo[cur], hi[cur],
-                                                                  hgt[cur], ref[1 - cur], lo[1 - cur], hi[1 - cur],
-                                                                  hgt[1 - cur]);
-                k_ploc_next<<<1, 1, 0, s>>>(ctl, valid, pos, 1 - cur);
-                cur = 1 - cur;
+            return fail(cuda_fail(e, "hdof_build_bvh: clear"));
+        k_ploc_init<<<blocks_for(m, 256), 256, 0, s>>>(verts, idx, ids_out, m, c, ctl);
+        const bool small = m <= PLOC_BIG;
+        const size_t smem = sizeof(FinishSmem);
+        if ((e = cudaFuncSetAttribute(small ? k_ploc_finish<PLOC_R_SMALL> : k_ploc_finish<PLOC_R_BIG>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+            return fail(cuda_fail(e, "hdof_build_bvh: shared memory"));
+        // rounds until PLOC_CAP clusters are left, as a round leaves about four
+        // fifths; should they not suffice, the device says so and more follow
+        int Nb = m, round = 0, all = 0;
+        for (bool first = true;; first = false) {
+            int rounds = 0;
+            if (Nb > PLOC_CAP) {
+                rounds = (int)std::ceil(std::log((double)Nb / PLOC_CAP) / std::log(1.22)) + 1;
+                rounds = std::min(std::max(rounds, first ? 1 : 16), CTL_ROUNDS - 1);
             }
-            rounds += PLOC_SYNC;
-            int c[3];
+            all += rounds;
+            for (int r = 0; r < rounds; ++r, ++round) {
+                // at most a full machine of blocks: the later rounds need far fewer than the first
+                const int g1 = std::min(blocks_for(Nb, PLOC_B), 8 * sm_count());
+                const int g2 = std::min(blocks_for(Nb, PLOC_CB), 2 * sm_count());
+                if (small) k_ploc_nn<PLOC_R_SMALL><<<g1, PLOC_B, 0, s>>>(ctl, round, c, nn);
+                else k_ploc_nn<PLOC_R_BIG><<<g1, PLOC_B, 0, s>>>(ctl, round, c, nn);
+                k_ploc_count<<<g2, PLOC_CB, 0, s>>>(ctl, round, nn, counts);
+                k_ploc_merge<<<g2, PLOC_CB, 0, s>>>(ctl, round, nn, counts, c, nodes0, counters);
+            }
+            if (small) k_ploc_finish<PLOC_R_SMALL><<<1, PLOC_CB, smem, s>>>(ctl, round, c, nodes0, counters);
+            else k_ploc_finish<PLOC_R_BIG><<<1, PLOC_CB, smem, s>>>(ctl, round, c, nodes0, counters);
+            // (these leave at once while the clustering is not done)
+            k_dfs_index<<<blocks_for(ni, 256), 256, 0, s>>>(nodes0, ni, ctl, place);
+            k_dfs_permute<<<blocks_for(ni, 256), 256, 0, s>>>(nodes0, ni, ctl, place, HDOF_PLOC_LEAF_MAX, b->nodes,
+                                                              newpos);
+            leaf_data(newpos, ctl);
+            int h[3], slot[3];
             if ((e = cudaGetLastError()) != cudaSuccess ||
-                (e = cudaMemcpyAsync(c, ctl, sizeof c, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+                (e = cudaMemcpyAsync(h, ctl, sizeof h, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+                (e = cudaMemcpyAsync(slot, ctl + CTL_ROUND + 3 * round, sizeof slot, cudaMemcpyDeviceToHost, s)) !=
+                    cudaSuccess ||
                 (e = cudaStreamSynchronize(s)) != cudaSuccess)
-                return pfail(cuda_fail(e, "hdof_build_bvh: clustering"));
-            if (c[0] <= 1) {
-                buf = c[2];
+                return fail(cuda_fail(e, "hdof_build_bvh: clustering"));
+            if (h[CTL_DONE]) {
+                depth = h[CTL_HEIGHT];
                 break;
             }
-            if (rounds > 100000) {
+            if (all > 100000 || slot[0] <= PLOC_CAP) {
                 set_error("hdof_build_bvh: clustering did not converge");
-                return pfail(HDOF_ECUDA);
+                return fail(HDOF_ECUDA);
             }
-            Nb = c[0];
+            Nb = slot[0];
+            if ((e = cudaMemcpyAsync(ctl + CTL_ROUND, ctl + CTL_ROUND + 3 * round, sizeof slot, cudaMemcpyDeviceToDevice,
+                                     s)) != cudaSuccess)
+                return fail(cuda_fail(e, "hdof_build_bvh: clustering"));
+            round = 0;
         }
-        int root_ref = 0, h = 0;
-        if ((e = cudaMemcpyAsync(&root_ref, ref[buf], sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(&h, hgt[buf], sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess)
-            return pfail(cuda_fail(e, "hdof_build_bvh: clustering"));
-        cudaFree(pt);
-        depth = h;
-        b->n_nodes = m - 1;
-        b->root = root_ref;
-        if (root_ref >= 0 && m - 1 > 1) {
-            const int ni = m - 1;
-            // scratch: parent, nint, arrived, size, index (ints) + a node copy
-            size_t q0 = 0, q1 = q0 + up256(4 * (size_t)ni), q2 = q1 + up256(4 * (size_t)ni);
-            size_t q3 = q2 + up256(4 * (size_t)ni), q4 = q3 + up256(4 * (size_t)ni);
-            size_t q5 = q4 + up256(4 * (size_t)ni), qtot = q5 + sizeof(Node) * (size_t)ni;
-            void* rt = nullptr;
-            if ((e = cudaMalloc(&rt, qtot)) != cudaSuccess) return fail(cuda_fail(e, "hdof_build_bvh: cudaMalloc"));
-            char* r8 = static_cast<char*>(rt);
-            int* parent = reinterpret_cast<int*>(r8 + q0);
-            int* nint = reinterpret_cast<int*>(r8 + q1);
-            unsigned* arrived = reinterpret_cast<unsigned*>(r8 + q2);
-            int* size = reinterpret_cast<int*>(r8 + q3);
-            int* index = reinterpret_cast<int*>(r8 + q4);
-            Node* copy = reinterpret_cast<Node*>(r8 + q5);
-            const int nb = blocks_for(ni, 256);
-            if ((e = cudaMemsetAsync(arrived, 0, 4 * (size_t)ni, s)) == cudaSuccess) {
-                k_dfs_parent<<<nb, 256, 0, s>>>(b->nodes, ni, parent, nint);
-                k_dfs_size<<<nb, 256, 0, s>>>(b->nodes, ni, root_ref, parent, nint, arrived, size);
-                k_dfs_index<<<nb, 256, 0, s>>>(b->nodes, ni, root_ref, parent, size, index);
-                k_dfs_permute<<<nb, 256, 0, s>>>(b->nodes, ni, parent, index, size, root_ref, copy);
-                e = cudaGetLastError();
-            }
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(b->nodes, copy, sizeof(Node) * (size_t)ni, cudaMemcpyDeviceToDevice, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            cudaFree(rt);
-            if (e != cudaSuccess) return fail(cuda_fail(e, "hdof_build_bvh: relabel"));
-            b->root = 0;
-            if (HDOF_PLOC_LEAF_MAX > 1 && (e = collapse_leaves(b, ni, m, HDOF_PLOC_LEAF_MAX, s)) != cudaSuccess)
-                return fail(cuda_fail(e, "hdof_build_bvh: leaf collapse"));
-        }
+        b->n_nodes = ni;
+        b->root = 0;
     }
+    int has_spec = 0;
+    if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&has_spec, spec_flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        return fail(cuda_fail(e, "hdof_build_bvh: leaf data"));
+    b->specular = has_spec;
     b->depth = depth;
     if (depth + 1 >= HDOF_STACK) {
         set_error("hdof_build_bvh: tree depth %d exceeds the %d-entry traversal stack", depth, HDOF_STACK);

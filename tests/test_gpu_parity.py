@@ -89,6 +89,39 @@ def test_closest_hits_match_brute_force(orc, n):
     assert (g_id != o_id).mean() < 1e-3
 
 
+@pytest.mark.parametrize("n", [3, 65, 1023, 1024, 1025, 1027, 2049, 5000])
+def test_build_around_the_finishing_block(n):
+    """Trees whose clustering runs in one block only, in rounds over several
+    blocks first, or just crosses from one to the other, with repeated
+    triangles (ties of equal area) among them: n - 1 nodes, every triangle's
+    own centroid ray hits it or an equal triangle of lower id, at its distance."""
+    rng = np.random.default_rng(n)
+    sc = _soup(rng, n)
+    v = sc.verts.reshape(n, 3, 3).copy()
+    if n > 40:
+        v[n // 2:n // 2 + 20] = v[:20]  # repeated triangles
+    # apart from one another along z, so that a ray from the side hits only its own
+    v[:, :, 2] = (v[:, :, 2] - 4.0) * 1e-3 + 0.05 * np.arange(n)[:, None]
+    if n > 40:
+        v[n // 2:n // 2 + 20, :, 2] = v[:20, :, 2]
+    sc = hi.Scene(v.reshape(-1, 3).astype(np.float32), sc.idx, sc.mat, sc.uv)
+    bvh = bvh_of(sc)
+    st = bvh.stats()
+    assert st.n_tris == n and st.n_nodes == n - 1 and st.depth < 64
+    cen = sc.tri_verts().reshape(n, 3, 3).astype(np.float64).mean(1)
+    org = (cen - [0, 0, 0.02]).astype(np.float32)
+    d = np.tile(np.array([0, 0, 1.0], np.float32), (n, 1))
+    ids = torch.empty(n, dtype=torch.int32, device="cuda")
+    ts = torch.empty(n, dtype=torch.float32, device="cuda")
+    H.hdof_closest_hits(bvh, dev(org), dev(d), ids, ts)
+    H.hdof_sync()
+    want = np.arange(n)
+    if n > 40:
+        want[n // 2:n // 2 + 20] = np.arange(20)
+    assert np.array_equal(host(ids), want)
+    assert np.allclose(host(ts), 0.02, atol=2e-3 + 4e-7 * 0.05 * n)
+
+
 def test_watertight_fan_gpu():
     n = 12
     cen = np.array([0.1, -0.05, 3.0])
