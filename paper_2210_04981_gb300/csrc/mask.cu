@@ -32,6 +32,7 @@ struct EdgeArgs {
     GaussW g;
     float tau;
     int tile, ntx;
+    int rows;       // output rows per warp
     uint8_t* edge;
     uint8_t* tiles;
     Coc coc;        // CoC-scaled mask: the lens's CoC in pixels
@@ -40,7 +41,7 @@ struct EdgeArgs {
 };
 
 // ---- register sweep form of the edge pass ----------------------------------
-// A warp owns a strip of 32 input columns (x0 - 3 .. x0 + 28) and SW_ROWS
+// A warp owns a strip of 32 input columns (x0 - 3 .. x0 + 28) and up to SW_ROWS
 // output rows; it walks down the strip one input row at a time, lane = column:
 //   horizontal Gaussian of the new row from its +-1, +-2 neighbours (shuffles),
 //   vertical Gaussian from a ring of the last five horizontally filtered rows,
@@ -52,7 +53,7 @@ struct EdgeArgs {
 //   once per strip (plus the 3-pixel halos).  Edge flags and CoC radii are
 //   reduced per mask tile in registers and written once per tile row.
 constexpr int SW_OUT = 26;   // output columns per warp
-constexpr int SW_ROWS = 32;  // output rows per warp
+constexpr int SW_ROWS = 32;  // output rows per warp, fewer on small images (sweep_rows)
 constexpr int SW_WARPS = 4;  // warps per block (side by side)
 
 // float4 arithmetic as two packed two-lane FP32 operations (Blackwell's
@@ -117,7 +118,7 @@ __device__ __forceinline__ void mask_sweep_body(const EdgeArgs<ND>& ar, int bx, 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int x0 = (bx * SW_WARPS + warp) * SW_OUT;  // first output column of the strip
     if (x0 >= W) return;                                // a whole warp leaves together
-    const int y0 = by * SW_ROWS, y1 = min(y0 + SW_ROWS, H);
+    const int y0 = by * ar.rows, y1 = min(y0 + ar.rows, H);
     const int x = x0 - 3 + lane;                      // this lane's column (may lie outside the image)
     const int xc = min(max(x, 0), W - 1);
     const bool out_lane = lane >= 3 && lane < 3 + SW_OUT && x < W;
@@ -237,9 +238,21 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) k_mask_sweep_batch(const Edg
     g.locate(blockIdx.x, v, bx, by);
     mask_sweep_body(batch_record(a, v), bx, by);
 }
+// Output rows per warp of the sweep: a warp walks its rows one after another
+// (6 more for the halo), so a small image, whose few strips leave the machine
+// empty (below 8 warps an SM), is cut into shorter ones: the 128x128 mask 35
+// -> 23 us.  The filtered values do not depend on it.  At 1080p (2516 warps)
+// 8 or 16 rows shorten the mask by 5% and the frame not at all.
+inline int sweep_rows(int W, int H) {
+    const int strips = (W + SW_OUT - 1) / SW_OUT;
+    int rows = SW_ROWS;
+    while (rows > 8 && strips * ((H + rows - 1) / rows) < 1216) rows /= 2;
+    return rows;
+}
 // grid of the sweep for a W x H frame
 inline dim3 sweep_grid(int W, int H) {
-    return dim3((W + SW_OUT * SW_WARPS - 1) / (SW_OUT * SW_WARPS), (H + SW_ROWS - 1) / SW_ROWS);
+    const int rows = sweep_rows(W, H);
+    return dim3((W + SW_OUT * SW_WARPS - 1) / (SW_OUT * SW_WARPS), (H + rows - 1) / rows);
 }
 
 struct SppArgs {
@@ -384,6 +397,7 @@ EdgeArgs<ND> edge_args(const hdof_gbuf* in, const hdof_params* p, uint8_t* edge,
     a.tau = p->edge_tau;
     a.tile = p->tile;
     a.ntx = (in->width + p->tile - 1) / p->tile;
+    a.rows = sweep_rows(in->width, in->height);
     a.edge = edge;
     a.tiles = tiles;
     a.coc = coc ? *coc : Coc{0.f, 0.f};
