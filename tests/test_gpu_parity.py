@@ -474,6 +474,35 @@ def test_trace_lens_sorted_list(orc, W, Hh, spp_max, K):
     assert ok.mean() >= 0.998, report("rt", host(outs[0][0])[spp > 0], ref[spp > 0])
 
 
+@pytest.mark.parametrize("W,Hh", [(181, 181), (182, 181), (1, 1), (3, 7)])
+def test_resolve_around_its_small_form(orc, W, Hh):
+    """Images just below and just above the 32768 pixels up to which several
+    threads resolve a pixel, and single pixels; 0 to 7 samples a pixel (uneven
+    against the threads sharing it): the trace output as the oracle's.  The
+    lens is focused on the checker: all rays of a pixel meet it in one point,
+    and at odd sizes the middle column's and row's points lie exactly on the
+    line between two cells (u or v = 1/2), a tie of floor() that is left out."""
+    scene, _, lens, p = hi.tiny_config()
+    p = p.replace(spp_max=7)
+    cam = hi.Camera(width=W, height=Hh).f32()
+    spp = (np.arange(W * Hh) % 8).astype(np.uint8).reshape(Hh, W)
+    rt = torch.zeros((Hh, W, 12), dtype=torch.float32, device="cuda")
+    stats = torch.zeros(2, dtype=torch.int32, device="cuda")
+    H.hdof_trace(bvh_of(scene), cam, lens, p, dev(spp), rt, stats, workspace(W, Hh, p))
+    H.hdof_sync()
+    assert host(stats).tolist() == [int((spp > 0).sum()), int(spp.sum())]
+    tr = spp > 0
+    if tr.any():
+        ref = orc.trace(orc.OScene(scene), cam, lens, p, spp)
+        sel = tr.copy()
+        if W % 2:
+            sel[:, W // 2] = False
+        if Hh % 2:
+            sel[Hh // 2] = False
+        assert not sel.any() or rt_close(host(rt), ref, sel).mean() >= 0.999, report("rt", host(rt)[sel], ref[sel])
+    assert not host(rt)[~tr].any()
+
+
 @pytest.mark.parametrize("refill", [0, 4])
 def test_trace_watchdog_reports_timeout(refill):
     """A traversal step cap of 1 stops every lens ray after one step (the
