@@ -50,54 +50,94 @@ __global__ void __launch_bounds__(256) k_rt_accum(const float4* __restrict__ rt,
     out[q] = o;
 }
 
+// A sum carried as an unevaluated pair of floats (Knuth's TwoSum): 48 bits, at
+// FP32 rates (FP64 adds run at 1/64 of them here).
+struct Pair {
+    float hi, lo;
+};
+__device__ __forceinline__ Pair two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ void pair_add(Pair& s, float x, float x_lo = 0.f) {
+    const Pair t = two_sum(s.hi, x);
+    s = two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(s.lo, x_lo)));
+}
+
 // per pixel: err = mean over rgb of |a - b|; per block: [count, sum |d|,
-// sum d^2, max |d|] over all pixels, then the same over the region
+// sum d^2, max |d|] over all pixels, then the same over the region.  A thread
+// sums its few pixels as float pairs (each d^2 exactly, with its rounding
+// error), the block in double precision: 160 us in double throughout at
+// 1280x720 (with the final block), 29 so.
 __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ a, const float4* __restrict__ b,
                                                      const uint8_t* __restrict__ region, int n_px,
                                                      float* __restrict__ err, double* __restrict__ part) {
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    int cnt[2] = {0, 0};
+    Pair s1[2] = {{0.f, 0.f}, {0.f, 0.f}}, s2[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    float mx[2] = {0.f, 0.f};
     for (int q = blockIdx.x * ERR_THREADS + threadIdx.x; q < n_px; q += ERR_BLOCKS * ERR_THREADS) {
         const float4 x = a[q], y = b[q];
-        const float dx = fabsf(x.x - y.x), dy = fabsf(x.y - y.y), dz = fabsf(x.z - y.z);
-        const float e = (dx + dy + dz) * (1.f / 3.f);
-        if (err) err[q] = e;
-        const double s1 = (double)dx + dy + dz, s2 = (double)dx * dx + (double)dy * dy + (double)dz * dz;
-        const double mx = fmax(fmax((double)dx, (double)dy), (double)dz);
-        acc[0] += 1.0;
-        acc[1] += s1;
-        acc[2] += s2;
-        acc[3] = fmax(acc[3], mx);
-        if (region && region[q]) {
-            acc[4] += 1.0;
-            acc[5] += s1;
-            acc[6] += s2;
-            acc[7] = fmax(acc[7], mx);
+        const float d[3] = {fabsf(x.x - y.x), fabsf(x.y - y.y), fabsf(x.z - y.z)};
+        if (err) err[q] = (d[0] + d[1] + d[2]) * (1.f / 3.f);
+        const bool in[2] = {true, region && region[q]};
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            if (!in[r]) continue;
+            ++cnt[r];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float p = __fmul_rn(d[k], d[k]);
+                pair_add(s1[r], d[k]);
+                pair_add(s2[r], p, fmaf(d[k], d[k], -p));
+                mx[r] = fmaxf(mx[r], d[k]);
+            }
         }
     }
-    __shared__ double sh[8][ERR_THREADS];
-    for (int k = 0; k < 8; ++k) sh[k][threadIdx.x] = acc[k];
-    __syncthreads();
-    for (int w = ERR_THREADS / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int k = 0; k < 8; ++k) {
-                const double o = sh[k][threadIdx.x + w];
-                sh[k][threadIdx.x] = (k & 3) == 3 ? fmax(sh[k][threadIdx.x], o) : sh[k][threadIdx.x] + o;
-            }
-        __syncthreads();
+    // a warp in pairs of floats, then the eight warps in double, in a fixed order
+    __shared__ double sh[8][ERR_THREADS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        cnt[r] = __reduce_add_sync(0xffffffffu, cnt[r]);
+        for (int o = 16; o; o >>= 1) {
+            const Pair u{__shfl_xor_sync(0xffffffffu, s1[r].hi, o), __shfl_xor_sync(0xffffffffu, s1[r].lo, o)};
+            const Pair v{__shfl_xor_sync(0xffffffffu, s2[r].hi, o), __shfl_xor_sync(0xffffffffu, s2[r].lo, o)};
+            pair_add(s1[r], u.hi, u.lo);
+            pair_add(s2[r], v.hi, v.lo);
+            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], o));
+        }
+        if (lane == 0) {
+            sh[4 * r][w] = (double)cnt[r];
+            sh[4 * r + 1][w] = (double)s1[r].hi + (double)s1[r].lo;
+            sh[4 * r + 2][w] = (double)s2[r].hi + (double)s2[r].lo;
+            sh[4 * r + 3][w] = (double)mx[r];
+        }
     }
-    if (threadIdx.x < 8) part[(size_t)blockIdx.x * 8 + threadIdx.x] = sh[threadIdx.x][0];
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        const int k = threadIdx.x;
+        double v = sh[k][0];
+        for (int j = 1; j < ERR_THREADS / 32; ++j) v = (k & 3) == 3 ? fmax(v, sh[k][j]) : v + sh[k][j];
+        part[(size_t)blockIdx.x * 8 + k] = v;
+    }
 }
 
-// one block: the blocks' partials in block order
-__global__ void __launch_bounds__(32) k_err_final(const double* __restrict__ part, double* __restrict__ stats) {
-    if (threadIdx.x >= 8) return;
-    const int k = threadIdx.x;
+// one block, a warp per summary: lane l adds the partials l, l + 32, ... in
+// block order, the lanes' sums then pairwise (a fixed order).  One thread per
+// summary over all 1024 partials was a chain of 1024 double additions.
+__global__ void __launch_bounds__(256) k_err_final(const double* __restrict__ part, double* __restrict__ stats) {
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double v = 0.0;
-    for (int b = 0; b < ERR_BLOCKS; ++b) {
+#pragma unroll 8
+    for (int b = lane; b < ERR_BLOCKS; b += 32) {
         const double o = part[(size_t)b * 8 + k];
         v = (k & 3) == 3 ? fmax(v, o) : v + o;
     }
-    stats[k] = v;
+    for (int o = 16; o; o >>= 1) {
+        const double u = __shfl_xor_sync(0xffffffffu, v, o);
+        v = (k & 3) == 3 ? fmax(v, u) : v + u;
+    }
+    if (lane == 0) stats[k] = v;
 }
 
 }  // namespace
@@ -158,7 +198,7 @@ extern "C" int hdof_error_map(const float* a, const float* b, const uint8_t* reg
     k_err<<<ERR_BLOCKS, ERR_THREADS, 0, s>>>(reinterpret_cast<const float4*>(a), reinterpret_cast<const float4*>(b),
                                             region, width * height, err, stats + HDOF_ERR_STATS);
     HDOF_LAUNCHED("hdof_error_map");
-    k_err_final<<<1, 32, 0, s>>>(stats + HDOF_ERR_STATS, stats);
+    k_err_final<<<1, 256, 0, s>>>(stats + HDOF_ERR_STATS, stats);
     HDOF_LAUNCHED("hdof_error_map: reduce");
     return HDOF_OK;
 }
