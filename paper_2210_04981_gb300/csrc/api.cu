@@ -132,12 +132,13 @@ WsLayout ws_layout(int W, int H, const hdof_params* p) {
     l.trace_ray_s = align256(nray);
     l.trace_rec = align256(nray * sizeof(float2));
     l.trace = l.trace_counts + l.trace_queue + l.trace_qoff + l.trace_ray_pix + l.trace_ray_s + l.trace_rec;
-    l.pf_nrec = align256(npx * sizeof(float4));
-    l.pf_frec = align256(npx * sizeof(float4));
-    l.pf_rh = align256(npx * sizeof(float));
-    l.pf_zq = align256(npx * sizeof(float));
+    const size_t npp = (size_t)((W + 1) & ~1) * H;  // the post-filter's planes have an even pitch
+    l.pf_nrec = align256(npp * sizeof(float4));
+    l.pf_frec = align256(npp * sizeof(float4));
+    l.pf_rh = align256(npp * sizeof(float));
+    l.pf_zq = align256(npp * sizeof(float));
     l.pf_tiles = align256(ptiles * sizeof(float4));
-    l.pf_pre = align256(npx * sizeof(float4));
+    l.pf_pre = align256(npp * sizeof(float4));
     l.pf_bokeh = bokeh_scratch_bytes(p);
     l.pf = l.pf_nrec + l.pf_frec + l.pf_rh + l.pf_zq + l.pf_tiles + l.pf_pre + l.pf_bokeh;
     const size_t mask = l.mask_tiles + l.mask_tile_r;

@@ -24,12 +24,14 @@
 //   summed as one difference of the row prefix and only the ring around them
 //   is tapped.  Each thread gathers
 //   a 2x2 pixel block so every tap it loads serves four pixels; the per-tap
-//   arithmetic is branch-free (saturating adds).  Four thread groups share a
-//   tile's window rows.  Bound by the latency of the tap and prefix loads and
-//   by issue.  One common interior per thread (no per-pixel masks, a quarter
-//   of the prefix loads) and the row split took the gather alone from 308 to
-//   240 us (1080p room), 3270 to 2436 us (4K room, FP16/BF16 planes), 455 to
-//   255 us (1080p, mixed depths) and 43 to 17.5 us (128x128).
+//   arithmetic is branch-free (saturating adds).  The rows above and below the
+//   block are walked in pairs: they share bounds and distances, and their
+//   loads are in flight together.  Two thread groups share a tile's window.
+//   Bound by the latency of the tap and prefix loads and by issue (57% busy).
+//   One common interior per thread (no per-pixel masks, a quarter of the
+//   prefix loads), the row pairs and the split took the gather alone from 308
+//   to 218 us (1080p room), 3270 to 2116 us (4K room, FP16/BF16 planes), 455
+//   to 252 us (1080p, mixed depths) and 43 to 18.5 us (128x128).
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -42,31 +44,18 @@ namespace hdof {
 namespace {
 
 constexpr int TP = HDOF_TILE_PF;
-#ifndef HDOF_PF_RY
-#define HDOF_PF_RY 2  // pixel rows per gather thread (each thread gathers 2 x RY pixels; 4 slower by 5-30%)
-#endif
-constexpr int PF_RY = HDOF_PF_RY;
-constexpr int PF_NPX = 2 * PF_RY;
-constexpr int PF_GROUP = 8 * (16 / PF_RY);  // threads that cover a 16x16 tile once
-// Thread groups per tile, group g taking the source rows g, g + PF_G, ... of
-// each pixel's window.  A tile's work runs from nothing to (2 r_max)^2 taps a
-// pixel, so with one group the widest windows were the kernel's tail (32 of
+constexpr int PF_GROUP = 64;  // threads that cover a 16x16 tile once (2x2 pixels each; 2x4 slower by 5-30%)
+// Thread groups per tile, group g taking the source row pairs g, g + PF_G, ...
+// of each pixel's window.  A tile's work runs from nothing to (2 r_max)^2 taps
+// a pixel, so with one group the widest windows were the kernel's tail (32 of
 // them on one SM outlast the rest of the grid), and a small image had one
-// long serial loop a thread.  Gather alone, 1 / 2 / 4 / 8 groups: mixed
-// depths at 1080p 421 / 283 / 239 / 320 us, the 128x128 frame 43 / 25 / 17.5
-// us, the 1080p room 246 / 222 / 227 us, 4K 2461 / 2425 / 2421 / 2600 us.
-#ifndef HDOF_PF_G
-#define HDOF_PF_G 4
-#endif
-constexpr int PF_G = HDOF_PF_G;
+// long serial loop a thread.  Gather alone, 1 / 2 / 4 groups: mixed depths at
+// 1080p 355 / 252 / 258 us, the 128x128 frame 29 / 18.5 / 14-16 us, the
+// 1080p room 224 / 218 / 240 us, 4K 2187 / 2116 / 2148 us.
+constexpr int PF_G = 2;
 constexpr int GATHER_THREADS = PF_G * PF_GROUP;
-#ifndef HDOF_PF_MINB
-#define HDOF_PF_MINB 4  // resident gather blocks per SM the register budget targets (64 registers; 3: 5-10% slower)
-#endif
-#ifndef HDOF_PF_UNROLL
-#define HDOF_PF_UNROLL 1  // unroll of the gather's tap-pair loop (1, 2, 4, 8 swept: 1 fastest)
-#endif
-constexpr int PF_UNROLL = HDOF_PF_UNROLL;
+constexpr int PF_MINB = 6;    // resident blocks per SM: 80 registers (7, 72 registers: 5-15% slower but for 4K)
+constexpr int PF_UNROLL = 2;  // of the tap-pair loop: a pair's four record loads beside the next one's (1: 3% slower)
 // A near tile's interior path runs above this share of its reach, and a row
 // takes the prefix only for at least PF_MIN_IN columns (two 16-byte loads
 // cost about as much as two tap pairs): 0.2 to 0.5, and 2 to 8 columns, are
@@ -74,13 +63,10 @@ constexpr int PF_UNROLL = HDOF_PF_UNROLL;
 constexpr float PF_IN_SHARE = 0.5f;
 constexpr int PF_MIN_IN = 4;
 constexpr float PF_ROW_W = 8.f;  // entries round to 2^-22 at most: 160 of them to below 1e-5 of a pixel's weight
-// Shared-memory carve-out (percent of the maximum) for the gather: four
-// resident blocks hold 16 KB of partial sums each, and the taps are served
-// from L1, so no more than that (50%: the same time).
-#ifndef HDOF_PF_CARVEOUT
-#define HDOF_PF_CARVEOUT 30
-#endif
-constexpr int GATHER_CARVEOUT = HDOF_PF_CARVEOUT;
+// Shared-memory carve-out (percent of the maximum) for the gather: six
+// resident blocks hold 8 KB of partial sums each, and the taps are served
+// from L1, so no more than that (20 to 45%: within 2%).
+constexpr int GATHER_CARVEOUT = 30;
 constexpr int AREA_MAX = 16384;  // breakpoints for radii up to 127.5
 
 // (x_m, a(x_m), slope on [x_m, x_{m+1}], 0)
@@ -97,6 +83,10 @@ __device__ __forceinline__ float disk_area(float r) {
     float4 e = __ldg(&g_area[lo]);
     return fmaf(e.z, r - e.x, e.y);
 }
+
+// The gather's planes have an even pitch, so that a pair of pixels (2m, 2m + 1)
+// of any row is aligned (records to 32 bytes).
+__host__ __device__ inline int pf_pitch(int W) { return (W + 1) & ~1; }
 
 // Per source pixel q the gather reads r_q + 1/2, z_q and two premultiplied
 // layer records (c_q w/a, w/a) with w = w_near(q) for the near layer and
@@ -148,10 +138,18 @@ __device__ __forceinline__ void pf_prep_body(const PrepArgs<ND, COL>& a, int bx,
         float ia = 1.f / disk_area(r);
         float wn = w_near(c), an = wn * ia, af = (1.f - wn) * ia;
         float4 col = ld4(a.col + q);
-        a.rh[q] = r + 0.5f;
-        a.zq[q] = z;
-        st4(a.nrec + q, make_float4(col.x * an, col.y * an, col.z * an, an));
-        st4(a.frec + q, make_float4(col.x * af, col.y * af, col.z * af, af));
+        const size_t o = (size_t)j * pf_pitch(W) + i;
+        a.rh[o] = r + 0.5f;
+        a.zq[o] = z;
+        st4(a.nrec + o, make_float4(col.x * an, col.y * an, col.z * an, an));
+        st4(a.frec + o, make_float4(col.x * af, col.y * af, col.z * af, af));
+        if (i == W - 1 && (W & 1)) {  // the padding column of an odd width: a source of no weight
+            const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+            a.rh[o + 1] = 0.f;
+            a.zq[o + 1] = 1.f;
+            st4(a.nrec + o + 1, none);
+            st4(a.frec + o + 1, none);
+        }
         rn = wn > 0.f ? r : -1.f;
         rf = wn < 1.f ? r : -1.f;
         rnmin = wn > 0.f ? r : INF;
@@ -190,7 +188,7 @@ using RowScanArgs = RowScanArgsT<float4>;
 
 template <class REC>
 __device__ __forceinline__ void pf_rowscan_body(const RowScanArgsT<REC>& a, int y) {
-    const int W = a.W, t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int W = pf_pitch(a.W), t = threadIdx.x, lane = t & 31, w = t >> 5;
     const size_t row = (size_t)y * W;
     __shared__ float4 s_warp[8];
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -283,155 +281,149 @@ __device__ __forceinline__ void acc(FarAcc& a, float d, float rh, float zq, cons
     a.zw = fma2(t, f.z, f.w, a.zw);
 }
 
-// One (source, thread) tap: the thread's left pixels get fresh distances,
-// its right pixels the left pixels' distances of the previous tap (the same
-// offsets, so the same floats), carried in c (and the squared column offset
-// in pdx2).  MASK: a pixel takes the tap only if its column offset exceeds
-// its interior half-width for that row (squared: win2).
+// Two taps of one column, one in each of the rows ya = j - s and yb = j + 1 + s
+// around a thread's 2x2 block of rows j, j + 1.  Row ya lies s above the upper
+// pixels and s + 1 above the lower ones, row yb the reverse, so the two rows
+// share their distances: dn (s rows away) and df (s + 1).  The left pixels see
+// the column at fresh distances, the right ones at the previous column's (the
+// same offsets, so the same floats), carried in cn and cf (and the squared
+// column offset in pdx2).  MASK: a pixel takes the tap only if its column
+// offset exceeds its interior half-width for that row distance (squared: wn,
+// wf).
+struct TapCarry {
+    float cn, cf, pdx2;
+};
 template <bool MASK, class A>
-__device__ __forceinline__ void pf_tap(A (&a)[PF_NPX], float (&c)[PF_RY], float& pdx2, const float (&dyk)[PF_RY],
-                                       const float (&win2)[PF_RY], float dx, float r, float z, const float4& e) {
+__device__ __forceinline__ void pf_tap(A (&a)[4], TapCarry& c, float sn2, float sf2, float wn, float wf, float dx,
+                                       float ra, float za, const float4& ea, float rb, float zb, const float4& eb) {
     const float dx2 = dx * dx;
-#pragma unroll
-    for (int k = 0; k < PF_RY; ++k) {
-        const float d0 = sqrt_approx(dx2 + dyk[k]);
-        acc(a[2 * k], d0, r, z, e, !MASK || dx2 > win2[k]);
-        acc(a[2 * k + 1], c[k], r, z, e, !MASK || pdx2 > win2[k]);
-        c[k] = d0;
-    }
-    pdx2 = dx2;
+    const float dn = sqrt_approx(dx2 + sn2), df = sqrt_approx(dx2 + sf2);
+    acc(a[0], dn, ra, za, ea, !MASK || dx2 > wn);
+    acc(a[1], c.cn, ra, za, ea, !MASK || c.pdx2 > wn);
+    acc(a[2], df, ra, za, ea, !MASK || dx2 > wf);
+    acc(a[3], c.cf, ra, za, ea, !MASK || c.pdx2 > wf);
+    acc(a[0], df, rb, zb, eb, !MASK || dx2 > wf);
+    acc(a[1], c.cf, rb, zb, eb, !MASK || c.pdx2 > wf);
+    acc(a[2], dn, rb, zb, eb, !MASK || dx2 > wn);
+    acc(a[3], c.cn, rb, zb, eb, !MASK || c.pdx2 > wn);
+    c.cn = dn;
+    c.cf = df;
+    c.pdx2 = dx2;
 }
 
-// The taps of source row y from column xs to xe (inclusive) for the 2 x RY
-// block at (i, j).  Taps go in pairs (even, odd pixel index): one 256-bit
-// load of the two records and one float2 load of r + 1/2 (and z) per pair;
-// the threads of a row, two columns apart, read consecutive pairs.  (Loading
-// the next pair ahead of the sums wants 80 registers: with 12 instead of 16
-// warps' worth of blocks the 4K gather is 20% slower.)
+// The taps of the columns xs .. xe (xs even, xe odd: whole pairs) of the rows
+// at plane offsets oa and ob: one 256-bit load of a pair's two records and one
+// float2 load of r + 1/2 (and z) per row; the threads of a row, two columns
+// apart, read consecutive pairs.  A row outside the image (on_a, on_b false:
+// its offset is the other row's) gets radii that reach nothing.
 template <bool NEAR, bool MASK, class A, class REC>
-__device__ __forceinline__ void pf_segment(A (&a)[PF_NPX], const float (&dyk)[PF_RY], const float (&win2)[PF_RY],
-                                           int xs, int xe, int i, int y, int W, const float* __restrict__ rh,
-                                           const float* __restrict__ zq, const REC* __restrict__ rec) {
+__device__ __forceinline__ void pf_segment(A (&a)[4], float sn2, float sf2, float wn, float wf, int xs, int xe, int i,
+                                           unsigned oa, unsigned ob, bool on_a, bool on_b,
+                                           const float* __restrict__ rh, const float* __restrict__ zq,
+                                           const REC* __restrict__ rec) {
     const float2* __restrict__ rh2 = reinterpret_cast<const float2*>(rh);
     const float2* __restrict__ zq2 = reinterpret_cast<const float2*>(zq);
+    const float2 none = make_float2(-1e30f, -1e30f), zero = make_float2(0.f, 0.f);
     float dx = (float)(xs - i);
-    float c[PF_RY], pdx2 = (dx - 1.f) * (dx - 1.f);
-#pragma unroll
-    for (int k = 0; k < PF_RY; ++k) c[k] = sqrt_approx(pdx2 + dyk[k]);
-    unsigned g = (unsigned)y * W + xs;  // pixel index of the next tap
-    const unsigned gend = (unsigned)y * W + xe + 1;
-    if (g & 1) {  // an odd first tap on its own
-        const float z = NEAR ? 0.f : __ldg(&zq[g]);
-        pf_tap<MASK>(a, c, pdx2, dyk, win2, dx, __ldg(&rh[g]), z, ld4(rec + g));
-        ++g;
-        dx += 1.f;
-    }
-    unsigned m = g >> 1;
-    const unsigned mend = gend >> 1;  // pairs (2m, 2m + 1) with 2m + 1 < gend
+    TapCarry c;
+    c.pdx2 = (dx - 1.f) * (dx - 1.f);
+    c.cn = sqrt_approx(c.pdx2 + sn2);
+    c.cf = sqrt_approx(c.pdx2 + sf2);
+    unsigned ma = (oa + xs) >> 1, mb = (ob + xs) >> 1;
 #pragma unroll PF_UNROLL
-    for (; m < mend; ++m, dx += 2.f) {
-        const float2 r2 = __ldg(&rh2[m]);
-        float4 e0, e1;
-        ld_rec_pair(rec + 2 * (size_t)m, e0, e1);
-        const float2 z2 = NEAR ? make_float2(0.f, 0.f) : __ldg(&zq2[m]);
-        pf_tap<MASK>(a, c, pdx2, dyk, win2, dx, r2.x, z2.x, e0);
-        pf_tap<MASK>(a, c, pdx2, dyk, win2, dx + 1.f, r2.y, z2.y, e1);
-    }
-    if (gend & 1) {  // an even last tap on its own
-        const unsigned gl = gend - 1;
-        const float z = NEAR ? 0.f : __ldg(&zq[gl]);
-        pf_tap<MASK>(a, c, pdx2, dyk, win2, dx, __ldg(&rh[gl]), z, ld4(rec + gl));
+    for (int x = xs; x < xe; x += 2, ++ma, ++mb, dx += 2.f) {
+        const float2 ra = on_a ? __ldg(&rh2[ma]) : none, rb = on_b ? __ldg(&rh2[mb]) : none;
+        float4 ea0, ea1, eb0, eb1;
+        ld_rec_pair(rec + 2 * (size_t)ma, ea0, ea1);
+        ld_rec_pair(rec + 2 * (size_t)mb, eb0, eb1);
+        const float2 za = NEAR ? zero : __ldg(&zq2[ma]), zb = NEAR ? zero : __ldg(&zq2[mb]);
+        pf_tap<MASK>(a, c, sn2, sf2, wn, wf, dx, ra.x, za.x, ea0, rb.x, zb.x, eb0);
+        pf_tap<MASK>(a, c, sn2, sf2, wn, wf, dx + 1.f, ra.y, za.y, ea1, rb.y, zb.y, eb1);
     }
 }
 
-// One layer's loop over a disk-shaped window of radius R around the 2x2
-// block at (i, j): every source feeding the layer within reach has
-// r + 1/2 <= R, so only taps closer than R to one of the four pixels can
-// weigh; per source row, the columns of that disk (squared distances are
-// exact integers in float).
+template <class A>
+__device__ __forceinline__ void add_sum(A& t, const float4& s) {
+    t.xy = make_float2(t.xy.x + s.x, t.xy.y + s.y);
+    t.zw = make_float2(t.zw.x + s.z, t.zw.y + s.w);
+}
+// pre[hi] - pre[lo - 1] of one row of the prefix
+__device__ __forceinline__ float4 prefix_sum(const float4* __restrict__ row, int lo, int hi) {
+    float4 s = __ldg(&row[hi]);
+    if (lo > 0) {
+        const float4 l = __ldg(&row[lo - 1]);
+        s = make_float4(s.x - l.x, s.y - l.y, s.z - l.z, s.w - l.w);
+    }
+    return s;
+}
+
+// One layer's loop over a disk-shaped window of radius R around the 2x2 block
+// at (i, j): every source feeding the layer within reach has r + 1/2 <= R, so
+// only taps closer than R to one of the four pixels can weigh; per pair of
+// source rows (j - s, j + 1 + s), the columns of that disk, in whole pairs of
+// pixels (squared distances are exact integers in float).  The two rows share
+// their bounds and their distances.
 // Near layer with Rin >= 0: every source that feeds the near layer and lies
 // within Rin of the block has r - 1/2 >= Rin, so a tap closer than Rin
 // weighs exactly 1 and is summed from the row prefix `pre`.  PERPX false: per
-// row, the columns closer than Rin to all 2 x RY pixels are summed once (two
+// row, the columns closer than Rin to all four pixels are summed once (two
 // loads, the same sum for every pixel) and the rest are tapped.  PERPX true:
 // each pixel sums its own interior columns (two loads a pixel); the columns
 // inside every pixel's interior are skipped, the rest are tapped with each
 // pixel's interior masked out.
 template <bool NEAR, bool PERPX, class A, class REC>
-__device__ __forceinline__ void pf_layer(A (&a)[PF_NPX], float R, float Rin, int g, int i, int j, int W, int H,
+__device__ __forceinline__ void pf_layer(A (&a)[4], float R, float Rin, int g, int i, int j, int W, int H,
                                          const float* __restrict__ rh, const float* __restrict__ zq,
                                          const REC* __restrict__ rec, const float4* __restrict__ pre) {
     if (R < 0.f) return;  // nothing within reach feeds this layer
     // bounds lean outwards by 1e-3 pixel (float rounding); taps they add weigh 0
-    const int G = (int)floorf(R + 1e-3f);
-    const int y0 = max(j - G, 0), y1 = min(j + PF_RY - 1 + G, H - 1);
+    const int G = (int)floorf(R + 1e-3f), Wp = pf_pitch(W);
     const float R2 = R * R, Rin2 = Rin * Rin;
-    for (int y = y0 + g; y <= y1; y += PF_G) {
-        const float dy = (float)(y - j);
-        float dyk[PF_RY], win2[PF_RY];
-#pragma unroll
-        for (int k = 0; k < PF_RY; ++k) dyk[k] = (dy - (float)k) * (dy - (float)k);
-        // nearest and farthest of the thread's rows to this source row
-        const float dmin = dy >= 0.f && dy <= (float)(PF_RY - 1) ? 0.f : fminf(dyk[0], dyk[PF_RY - 1]);
-        const float dmax = fmaxf(dyk[0], dyk[PF_RY - 1]);
-        const int w = (int)(sqrt_approx(fmaxf(R2 - dmin, 0.f)) + 1e-3f);
-        const int x0 = max(i - w, 0), x1 = min(i + 1 + w, W - 1);
+    for (int s = g; s <= G; s += PF_G) {
+        const int ya = j - s, yb = j + 1 + s;
+        const bool on_a = ya >= 0, on_b = yb < H;
+        if (!on_a && !on_b) break;
+        const unsigned oa = (unsigned)(on_a ? ya : yb) * Wp, ob = (unsigned)(on_b ? yb : ya) * Wp;
+        const float sn2 = (float)(s * s), sf2 = (float)((s + 1) * (s + 1));
+        const int w = (int)(sqrt_approx(fmaxf(R2 - sn2, 0.f)) + 1e-3f);
+        const int x0 = max(i - w, 0) & ~1, x1 = min(i + 1 + w, W - 1) | 1;
         int ls = x1 + 1, rs = x1;  // [ls, rs]: the columns that are not tapped (none)
+        float wn = -1.f, wf = -1.f;
         if (PERPX) {
-            const float4* prow = pre + (size_t)y * W;
-            int wmin = 1 << 30;  // interior half-width common to the thread's rows (-1: none)
+            // inward: no outward lean here (Rin already has its margin)
+            const int in = sn2 <= Rin2 ? (int)floorf(sqrtf(Rin2 - sn2)) : -1;
+            const int jf = sf2 <= Rin2 ? (int)floorf(sqrtf(Rin2 - sf2)) : -1;
+            wn = in >= 0 ? (float)(in * in) : -1.f;
+            wf = jf >= 0 ? (float)(jf * jf) : -1.f;
 #pragma unroll
-            for (int k = 0; k < PF_RY; ++k) {
-                // inward: no outward lean here (Rin already has its margin)
-                const int wi = dyk[k] <= Rin2 ? (int)floorf(sqrtf(Rin2 - dyk[k])) : -1;
-                win2[k] = wi >= 0 ? (float)(wi * wi) : -1.f;
-                wmin = min(wmin, wi);
-                if (wi >= 0) {
-#pragma unroll
-                    for (int b = 0; b < 2; ++b) {
-                        const int xa = i + b;
-                        if (xa < W) {
-                            const int lo = max(xa - wi, 0), hi = min(xa + wi, W - 1);
-                            float4 sum = __ldg(&prow[hi]);
-                            if (lo > 0) {
-                                const float4 l = __ldg(&prow[lo - 1]);
-                                sum = make_float4(sum.x - l.x, sum.y - l.y, sum.z - l.z, sum.w - l.w);
-                            }
-                            A& t = a[2 * k + b];
-                            t.xy = make_float2(t.xy.x + sum.x, t.xy.y + sum.y);
-                            t.zw = make_float2(t.zw.x + sum.z, t.zw.y + sum.w);
-                        }
-                    }
-                }
+            for (int k = 0; k < 4; ++k) {
+                const int xa = i + (k & 1), wa = k < 2 ? in : jf, wb = k < 2 ? jf : in;
+                if (xa >= W) continue;
+                if (on_a && wa >= 0) add_sum(a[k], prefix_sum(pre + oa, max(xa - wa, 0), min(xa + wa, W - 1)));
+                if (on_b && wb >= 0) add_sum(a[k], prefix_sum(pre + ob, max(xa - wb, 0), min(xa + wb, W - 1)));
             }
-            if (wmin >= 1) {
-                // columns [i + 1 - wmin, i + wmin] lie in every pixel's interior
-                ls = min(x1 + 1, i + 1 - wmin);
-                rs = max(x0 - 1, i + wmin);
+            if (jf >= 2) {
+                // columns [i + 1 - jf, i + jf] lie in every pixel's interior
+                ls = max(min(x1 + 1, (i + 2 - jf) & ~1), x0);
+                rs = min(((i + jf + 1) & ~1) - 1, x1);
             }
-        } else if (NEAR && dmax < Rin2) {
+        } else if (NEAR && sf2 < Rin2) {
             // columns [i + 1 - wi, i + wi] lie in every pixel's interior
             // (Rin's margin covers the root's rounding); rounded inwards to
             // whole pairs, so that the taps around them are whole pairs too
-            const int wi = (int)sqrt_approx(Rin2 - dmax), odd = (y & W) & 1;  // parity of the row's first index
-            const int l = max(i + 1 - wi, 0), r = min(i + wi, W - 1);
-            const int la = l + ((l + odd) & 1), ra = r - ((r + odd + 1) & 1);
+            const int wi = (int)sqrt_approx(Rin2 - sf2);
+            const int la = (max(i + 1 - wi, 0) + 1) & ~1, ra = i + wi >= W - 1 ? Wp - 1 : ((i + wi + 1) & ~1) - 1;
             if (ra - la + 1 >= PF_MIN_IN) {
-                const float4* prow = pre + (size_t)y * W;
-                const float4 s = __ldg(&prow[ra]);
-                const float4 l4 = la > 0 ? __ldg(&prow[la - 1]) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float2 sxy = make_float2(s.x - l4.x, s.y - l4.y), szw = make_float2(s.z - l4.z, s.w - l4.w);
+                float4 sum = on_a ? prefix_sum(pre + oa, la, ra) : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (on_b) sum = add4(sum, prefix_sum(pre + ob, la, ra));
 #pragma unroll
-                for (int k = 0; k < PF_NPX; ++k) {
-                    a[k].xy = make_float2(a[k].xy.x + sxy.x, a[k].xy.y + sxy.y);
-                    a[k].zw = make_float2(a[k].zw.x + szw.x, a[k].zw.y + szw.y);
-                }
+                for (int k = 0; k < 4; ++k) add_sum(a[k], sum);
                 ls = la;
                 rs = ra;
             }
         }
-        if (x0 < ls) pf_segment<NEAR, PERPX>(a, dyk, win2, x0, ls - 1, i, y, W, rh, zq, rec);
-        if (rs < x1) pf_segment<NEAR, PERPX>(a, dyk, win2, rs + 1, x1, i, y, W, rh, zq, rec);
+        if (x0 < ls) pf_segment<NEAR, PERPX>(a, sn2, sf2, wn, wf, x0, ls - 1, i, oa, ob, on_a, on_b, rh, zq, rec);
+        if (rs < x1) pf_segment<NEAR, PERPX>(a, sn2, sf2, wn, wf, rs + 1, x1, i, oa, ob, on_a, on_b, rh, zq, rec);
     }
 }
 
@@ -443,10 +435,10 @@ __device__ __forceinline__ float4 pf_group_sum(const float4 (&part)[PF_G][TP * T
     return s;
 }
 
-// PF_G groups of 8 x (16 / RY) threads per 16x16 tile; thread t of a group
-// gathers the 2 x RY pixel block at (2 (t & 7), RY (t >> 3)) over the group's
-// source rows, so each loaded tap serves 2 RY pixels; the groups' sums are
-// added in group order.
+// PF_G groups of 64 threads per 16x16 tile; thread t of a group gathers the
+// 2x2 pixel block at (2 (t & 7), 2 (t >> 3)) over the group's source rows, so
+// each loaded tap serves four pixels; the groups' sums are added in group
+// order.
 template <class COL>
 __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx, int ty) {
     const COL* __restrict__ col = ar.col;
@@ -511,7 +503,7 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
         const int G = (int)floorf(Gn + 1e-3f), y0 = max(ty * TP - G, 0), y1 = min(ty * TP + TP - 1 + G, H - 1);
         bool big = false;
         for (int y = y0 + threadIdx.x; y <= y1; y += GATHER_THREADS)
-            big |= !(__ldg(&ar.pre[(size_t)y * W + W - 1].w) <= PF_ROW_W);
+            big |= !(__ldg(&ar.pre[(size_t)y * pf_pitch(W) + W - 1].w) <= PF_ROW_W);
         per_px = __syncthreads_or(big);
     }
     // group g of the block's PF_G takes every PF_G-th source row; t is the
@@ -519,27 +511,28 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
     // thread p < 256 adds and finishes pixel p of the tile.
     __shared__ float4 s_part[PF_G][TP * TP];
     const int g = threadIdx.x / PF_GROUP, t = threadIdx.x % PF_GROUP;
-    const int li = 2 * (t & 7), lj = PF_RY * (t >> 3);
+    const int li = 2 * (t & 7), lj = 2 * (t >> 3);
     const int i = tx * TP + li, j = ty * TP + lj;
     const bool in = i < W && j < H;
     // far layer first; its sums wait in the pixels' own pp slots (each pixel
     // is one thread's alone) so they hold no registers during the near loop
     if (Gf >= 0.f) {
-        FarAcc f[PF_NPX];  // pixel (i + (k & 1), j + (k >> 1))
+        FarAcc f[4];  // pixel (i + (k & 1), j + (k >> 1))
         if (in) {
             const float ka = 1.f + 1.f / ar.kz_rel;  // k_z = clamp(ka - z_q kb), kb = 1 / (kz_rel z_p)
-            const float z00 = __ldg(&ar.zq[(size_t)j * W + i]);
+            const size_t zo = (size_t)j * pf_pitch(W) + i;
+            const float z00 = __ldg(&ar.zq[zo]);
 #pragma unroll
-            for (int k = 0; k < PF_NPX; ++k) {
+            for (int k = 0; k < 4; ++k) {
                 const int x = i + (k & 1), y = j + (k >> 1);
-                const float zp = x < W && y < H ? __ldg(&ar.zq[(size_t)y * W + x]) : z00;
+                const float zp = x < W && y < H ? __ldg(&ar.zq[zo + (size_t)(k >> 1) * pf_pitch(W) + (k & 1)]) : z00;
                 f[k].ka = ka;
                 f[k].kb = 1.f / (ar.kz_rel * zp);
                 f[k].xy = f[k].zw = make_float2(0.f, 0.f);
             }
             pf_layer<false, false>(f, Gf, -1.f, g, i, j, W, H, ar.rh, ar.zq, ar.frec, nullptr);
 #pragma unroll
-            for (int k = 0; k < PF_NPX; ++k)
+            for (int k = 0; k < 4; ++k)
                 s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = make_float4(f[k].xy.x, f[k].xy.y, f[k].zw.x, f[k].zw.y);
         }
         __syncthreads();
@@ -550,13 +543,13 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
         __syncthreads();
     }
     if (in) {
-        NearAcc a[PF_NPX];
+        NearAcc a[4];
 #pragma unroll
-        for (int k = 0; k < PF_NPX; ++k) a[k].xy = a[k].zw = make_float2(0.f, 0.f);
+        for (int k = 0; k < 4; ++k) a[k].xy = a[k].zw = make_float2(0.f, 0.f);
         if (per_px) pf_layer<true, true>(a, Gn, Rin, g, i, j, W, H, ar.rh, ar.zq, ar.nrec, ar.pre);
         else pf_layer<true, false>(a, Gn, Rin, g, i, j, W, H, ar.rh, ar.zq, ar.nrec, ar.pre);
 #pragma unroll
-        for (int k = 0; k < PF_NPX; ++k)
+        for (int k = 0; k < 4; ++k)
             s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = make_float4(a[k].xy.x, a[k].xy.y, a[k].zw.x, a[k].zw.y);
     }
     __syncthreads();
@@ -571,7 +564,7 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
 }
 
 template <class COL>
-__global__ void __launch_bounds__(GATHER_THREADS, HDOF_PF_MINB) k_pf_gather(GatherArgs<COL> a) {
+__global__ void __launch_bounds__(GATHER_THREADS, PF_MINB) k_pf_gather(GatherArgs<COL> a) {
     pf_gather_body(a, blockIdx.x, blockIdx.y);
 }
 
@@ -586,7 +579,7 @@ __global__ void __launch_bounds__(256) k_pf_prep_batch(const PrepF32* __restrict
     g.locate(blockIdx.x, v, bx, by);
     pf_prep_body(batch_record(a, v), bx, by);
 }
-__global__ void __launch_bounds__(GATHER_THREADS, HDOF_PF_MINB)
+__global__ void __launch_bounds__(GATHER_THREADS, PF_MINB)
     k_pf_gather_batch(const GatherArgs<float4>* __restrict__ a, BatchGrid g) {
     int v, bx, by;
     g.locate(blockIdx.x, v, bx, by);
