@@ -282,6 +282,14 @@ __global__ void k_leaf_data(const float* __restrict__ v, const int* __restrict__
     t.v1 = make_float4(v[3 * b], v[3 * b + 1], v[3 * b + 2], 0.f);
     t.v2 = make_float4(v[3 * c], v[3 * c + 1], v[3 * c + 2], 0.f);
     tris[k] = t;
+    Tri* r1 = tris + (size_t)n + k;  // the same triangle with its axes rotated (RayTri)
+    r1->v0 = make_float4(t.v0.y, t.v0.z, t.v0.x, t.v0.w);
+    r1->v1 = make_float4(t.v1.y, t.v1.z, t.v1.x, 0.f);
+    r1->v2 = make_float4(t.v2.y, t.v2.z, t.v2.x, 0.f);
+    Tri* r2 = r1 + n;
+    r2->v0 = make_float4(t.v0.z, t.v0.x, t.v0.y, t.v0.w);
+    r2->v1 = make_float4(t.v1.z, t.v1.x, t.v1.y, 0.f);
+    r2->v2 = make_float4(t.v2.z, t.v2.x, t.v2.y, 0.f);
     const float* mt = mat + 8 * (size_t)id;
     mato[2 * k] = make_float4(mt[0], mt[1], mt[2], mt[3]);
     mato[2 * k + 1] = make_float4(mt[4], mt[5], mt[6], mt[7]);
@@ -650,7 +658,7 @@ __global__ void k_closest(BvhView bvh, int n, const float* __restrict__ org, con
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     Hit h = closest_hit(bvh, ld3(org + 3 * (size_t)i), ld3(dir + 3 * (size_t)i), cap, status);
-    ids[i] = h.id;
+    ids[i] = h.slot >= 0 ? __float_as_int(__ldg(&bvh.tris[h.slot].v0.w)) : -1;
     ts[i] = h.t;
 }
 
@@ -844,7 +852,7 @@ extern "C" int hdof_build_bvh(const float* verts, int32_t n_verts, const int32_t
     b->n_big = n_big;
     const int n_int = n_small > 1 ? n_small - 1 : 1;
     size_t off_tris = up256(sizeof(Node) * (size_t)n_int);
-    size_t off_mat = off_tris + up256(sizeof(Tri) * (size_t)n);
+    size_t off_mat = off_tris + up256(sizeof(Tri) * 3 * (size_t)n);
     size_t off_uv = off_mat + up256(sizeof(float4) * 2 * (size_t)n);
     size_t off_big = off_uv + up256(sizeof(float2) * 3 * (size_t)n);
     size_t off_slot = off_big + up256(sizeof(float4) * 2 * (size_t)(n_big > 0 ? n_big : 1));

@@ -216,14 +216,15 @@ struct __align__(64) Node {
 };
 __host__ __device__ inline int leaf_ref(int first, int count) { return ~((first << 3) | (count - 1)); }
 
-// triangle in leaf order: (v0, original id), (v1, 0), (v2, 0)
+// triangle in leaf order: (v0, original id), (v1, 0), (v2, 0); with the axes
+// rotated in the second and third copy of the array (RayTri)
 struct __align__(16) Tri {
     float4 v0, v1, v2;
 };
 
 struct BvhView {
     const Node* nodes;
-    const Tri* tris;
+    const Tri* tris;    // [3][n_tris], axes (x, y, z), (y, z, x), (z, x, y)
     const float4* mat;  // sorted order: [2] per triangle (albedo_a rgb + checker_n, albedo_b rgb + k_s)
     const float2* uv;   // sorted order: [3] per triangle
     int n_tris;
@@ -344,10 +345,9 @@ __device__ __forceinline__ float slab(const Ray& r, float lx, float hx, float ly
     return slab_hit(r, pk2(lx, hx), pk2(ly, hy), pk2(lz, hz), tmax, tn) ? tn : __int_as_float(0x7f800000);
 }
 
-// Watertight ray/triangle test (Woop, Benthin, Wald, JCGT 2013).  Edge
-// functions are evaluated without contraction so a shared edge gives exactly
-// negated values in its two triangles; exact zeros are re-evaluated in double.
-// Returns true for a hit with 0 < t; writes t and barycentrics (b0 at v0).
+// Shear of the watertight ray/triangle test (Woop, Benthin, Wald, JCGT 2013):
+// kz the direction's largest component, kx and ky the others, in an order that
+// keeps the winding.
 struct Shear {
     int kx, ky, kz;
     float Sx, Sy, Sz;
@@ -373,40 +373,8 @@ __device__ __forceinline__ Shear make_shear(float3 d) {
 }
 __device__ __forceinline__ float comp(float3 v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : v.z); }
 
-__device__ __forceinline__ bool intersect_tri(float3 o, const Shear& s, float3 v0, float3 v1, float3 v2,
-                                              float& t, float& b0, float& b1, float& b2) {
-    float3 A = v0 - o, B = v1 - o, C = v2 - o;
-    float Akz = comp(A, s.kz), Bkz = comp(B, s.kz), Ckz = comp(C, s.kz);
-    float Ax = __fsub_rn(comp(A, s.kx), __fmul_rn(s.Sx, Akz));
-    float Ay = __fsub_rn(comp(A, s.ky), __fmul_rn(s.Sy, Akz));
-    float Bx = __fsub_rn(comp(B, s.kx), __fmul_rn(s.Sx, Bkz));
-    float By = __fsub_rn(comp(B, s.ky), __fmul_rn(s.Sy, Bkz));
-    float Cx = __fsub_rn(comp(C, s.kx), __fmul_rn(s.Sx, Ckz));
-    float Cy = __fsub_rn(comp(C, s.ky), __fmul_rn(s.Sy, Ckz));
-    float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
-    float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
-    float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-    if (U == 0.f || V == 0.f || W == 0.f) {
-        U = (float)((double)Cx * (double)By - (double)Cy * (double)Bx);
-        V = (float)((double)Ax * (double)Cy - (double)Ay * (double)Cx);
-        W = (float)((double)Bx * (double)Ay - (double)By * (double)Ax);
-    }
-    if ((U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f)) return false;
-    const float det = __fadd_rn(__fadd_rn(U, V), W);
-    if (det == 0.f) return false;
-    const float T = __fadd_rn(__fadd_rn(__fmul_rn(U, __fmul_rn(s.Sz, Akz)), __fmul_rn(V, __fmul_rn(s.Sz, Bkz))),
-                              __fmul_rn(W, __fmul_rn(s.Sz, Ckz)));
-    if (det > 0.f ? !(T > 0.f) : !(T < 0.f)) return false;
-    const float inv = __frcp_rn(det);
-    t = __fmul_rn(T, inv);
-    b0 = __fmul_rn(U, inv);
-    b1 = __fmul_rn(V, inv);
-    b2 = __fmul_rn(W, inv);
-    return true;
-}
-
 // Barycentrics of a known hit, recomputed with the arithmetic of
-// intersect_tri (same inputs give the same values) but without its rejection
+// hit_tri (same inputs give the same values) but without its rejection
 // tests, so a hit found by the traversal is always reproduced.
 __device__ __forceinline__ void tri_bary(float3 o, const Shear& s, float3 v0, float3 v1, float3 v2, float& b0,
                                          float& b1, float& b2) {
@@ -433,26 +401,87 @@ __device__ __forceinline__ void tri_bary(float3 o, const Shear& s, float3 v0, fl
     b2 = __fmul_rn(W, inv);
 }
 
+// The closest hit so far.  Its original id and its barycentrics are read and
+// recomputed where they are wanted: four registers fewer over the traversal.
 struct Hit {
-    float t, b0, b1, b2;
+    float t;
     int slot;  // sorted triangle slot, -1 = miss
-    int id;    // original triangle id
 };
 
-__device__ __forceinline__ void hit_tri(const BvhView& bvh, int slot, float3 o, const Shear& sh, Hit& h) {
-    const Tri* tr = bvh.tris + slot;
-    float4 p0 = __ldg(&tr->v0), p1 = __ldg(&tr->v1), p2 = __ldg(&tr->v2);
-    float t, b0, b1, b2;
-    if (intersect_tri(o, sh, f3(p0.x, p0.y, p0.z), f3(p1.x, p1.y, p1.z), f3(p2.x, p2.y, p2.z), t, b0, b1, b2)) {
-        int id = __float_as_int(p0.w);
-        if (t < h.t || (t == h.t && id < h.id)) {
-            h.t = t;
-            h.b0 = b0;
-            h.b1 = b1;
-            h.b2 = b2;
-            h.slot = slot;
-            h.id = id;
-        }
+// A ray's constants of the triangle test.  The test works in the axes (kx, ky,
+// kz) of the ray's shear.  Picking them from (x, y, z) there cost 18 selects of
+// some 75 instructions a triangle, in kernels bound by issue.  The triangles are
+// stored in the three rotations of the axes instead (96 bytes more each), and a
+// ray reads the one that ends in its kz: (x, y, z), (y, z, x) or (z, x, y).
+// With the id and barycentrics out of Hit: 1080p room primary rays 188 to
+// 179 us, lens rays 188 to 179 us; 8.4M lens rays of the wide aperture 817 to
+// 749 us; 4K primary rays 806 to 775 us; reference pass 550 to 532 us; the
+// build's leaf data costs no more than its runs differ.  kx and ky are not swapped for a negative d[kz]: that negates
+// the three edge functions, their sum and T exactly, and t and the barycentrics,
+// their quotients, stay the same.
+struct RayTri {
+    const Tri* tris;
+    f32x2 no;  // -(o[kx], o[ky])
+    float oz, nSx, nSy, Sz;
+};
+__device__ __forceinline__ RayTri make_ray_tri(const BvhView& bvh, float3 o, float3 d) {
+    const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
+    int rot = 1;  // kz = 0, 1, 2: rotation 1, 2, 0
+    if (ay > ax && ay >= az) rot = 2;
+    else if (az > ax && az > ay) rot = 0;
+    const float3 dr = rot == 0 ? d : rot == 1 ? f3(d.y, d.z, d.x) : f3(d.z, d.x, d.y);
+    const float3 orr = rot == 0 ? o : rot == 1 ? f3(o.y, o.z, o.x) : f3(o.z, o.x, o.y);
+    RayTri r;
+    r.tris = bvh.tris + (size_t)rot * bvh.n_tris;
+    r.no = pk2(-orr.x, -orr.y);
+    r.oz = orr.z;
+    r.nSx = -(dr.x / dr.z);
+    r.nSy = -(dr.y / dr.z);
+    r.Sz = 1.f / dr.z;
+    return r;
+}
+
+// A vertex moved to the ray's origin and sheared: (x, y) in the ray's plane,
+// z along it.  No contraction (the products are scalar: a packed product and
+// sum were fused): a vertex gives the same values in all its triangles.
+__device__ __forceinline__ float2 shear_vertex(const float4* p, const RayTri& r, float& z, float& w) {
+    f32x2 xy, q;
+    asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(xy), "=l"(q) : "l"(p));
+    const float2 zw = unpk2(q);
+    z = __fsub_rn(zw.x, r.oz);
+    w = zw.y;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(xy) : "l"(xy), "l"(r.no));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(xy) : "l"(xy), "l"(pk2(__fmul_rn(r.nSx, z), __fmul_rn(r.nSy, z))));
+    return unpk2(xy);
+}
+
+// Watertight ray/triangle test.  Edge functions are evaluated without
+// contraction so a shared edge gives exactly negated values in its two
+// triangles; exact zeros are re-evaluated in double.  A hit with 0 < t replaces
+// h if it is nearer, or as near with a lower original id.
+__device__ __forceinline__ void hit_tri(const RayTri& r, int slot, Hit& h) {
+    const Tri* tr = r.tris + slot;
+    float az, bz, cz, id, pad;
+    const float2 A = shear_vertex(&tr->v0, r, az, id), B = shear_vertex(&tr->v1, r, bz, pad),
+                 C = shear_vertex(&tr->v2, r, cz, pad);
+    float U = __fsub_rn(__fmul_rn(C.x, B.y), __fmul_rn(C.y, B.x));
+    float V = __fsub_rn(__fmul_rn(A.x, C.y), __fmul_rn(A.y, C.x));
+    float W = __fsub_rn(__fmul_rn(B.x, A.y), __fmul_rn(B.y, A.x));
+    if (U == 0.f || V == 0.f || W == 0.f) {
+        U = (float)((double)C.x * (double)B.y - (double)C.y * (double)B.x);
+        V = (float)((double)A.x * (double)C.y - (double)A.y * (double)C.x);
+        W = (float)((double)B.x * (double)A.y - (double)B.y * (double)A.x);
+    }
+    if ((U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f)) return;
+    const float det = __fadd_rn(__fadd_rn(U, V), W);
+    if (det == 0.f) return;
+    const float T = __fadd_rn(__fadd_rn(__fmul_rn(U, __fmul_rn(r.Sz, az)), __fmul_rn(V, __fmul_rn(r.Sz, bz))),
+                              __fmul_rn(W, __fmul_rn(r.Sz, cz)));
+    if (det > 0.f ? !(T > 0.f) : !(T < 0.f)) return;
+    const float t = __fmul_rn(T, __frcp_rn(det));
+    if (t < h.t || (t == h.t && (h.slot < 0 || __float_as_int(id) < __float_as_int(__ldg(&r.tris[h.slot].v0.w))))) {
+        h.t = t;
+        h.slot = slot;
     }
 }
 
@@ -531,13 +560,11 @@ __device__ __forceinline__ Hit closest_hit_oct(const BvhView& bvh, float3 o, flo
                                                int hint_slot) {
     const float INF = __int_as_float(0x7f800000);
     Ray r = make_ray(o, d);
-    Shear sh = make_shear(d);
+    const RayTri rt = make_ray_tri(bvh, o, d);
     Hit h;
     h.t = INF;
     h.slot = -1;
-    h.id = 0x7fffffff;
-    h.b0 = h.b1 = h.b2 = 0.f;
-    if (hint_slot >= 0) hit_tri(bvh, hint_slot, o, sh, h);
+    if (hint_slot >= 0) hit_tri(rt, hint_slot, h);
     int stack[HDOF_STACK];
     int sp = 0;
     int cur = bvh.root;
@@ -570,7 +597,7 @@ __device__ __forceinline__ Hit closest_hit_oct(const BvhView& bvh, float3 o, flo
             }
         } else {
             int e = ~cur, first = e >> 3, count = (e & 7) + 1;
-            for (int k = 0; k < count; ++k) hit_tri(bvh, first + k, o, sh, h);
+            for (int k = 0; k < count; ++k) hit_tri(rt, first + k, h);
 #if HDOF_TRAV_STATS
             nt += count;
 #endif
@@ -584,14 +611,13 @@ __device__ __forceinline__ Hit closest_hit_oct(const BvhView& bvh, float3 o, flo
     }
     for (int k = 0; k < bvh.big_count; ++k) {
         float4 lo = __ldg(&bvh.big_box[2 * k]), hi = __ldg(&bvh.big_box[2 * k + 1]);
-        if (slab(r, lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, h.t) < INF) hit_tri(bvh, bvh.big_first + k, o, sh, h);
+        if (slab(r, lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, h.t) < INF) hit_tri(rt, bvh.big_first + k, h);
     }
 #if HDOF_TRAV_STATS
     trav_stat(status, 0, 1ull);
     trav_stat(status, 1, nv);
     trav_stat(status, 2, nt);
 #endif
-    if (h.slot < 0) h.id = -1;
     return h;
 }
 
@@ -634,8 +660,8 @@ __device__ __forceinline__ Hit closest_hit(const BvhView& bvh, float3 o, float3 
 // or a miss); scene-sized triangles are left to the caller.  Returns false
 // when the step cap was reached (the warp stops; status is flagged).
 template <int OCT>
-__device__ __forceinline__ bool closest_hit_warp_oct(const BvhView& bvh, bool act, const Ray& r, float3 o,
-                                                     const Shear& sh, Hit& h, int cap, unsigned* status) {
+__device__ __forceinline__ bool closest_hit_warp_oct(const BvhView& bvh, bool act, const Ray& r,
+                                                     const RayTri& rt, Hit& h, int cap, unsigned* status) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     int cur = bvh.root, sp = 0, steps = 0;
@@ -682,7 +708,7 @@ __device__ __forceinline__ bool closest_hit_warp_oct(const BvhView& bvh, bool ac
         } else {
             const int e = ~cur, first = e >> 3, count = (e & 7) + 1;
             if (act)
-                for (int k = 0; k < count; ++k) hit_tri(bvh, first + k, o, sh, h);
+                for (int k = 0; k < count; ++k) hit_tri(rt, first + k, h);
 #if HDOF_TRAV_STATS
             nt += count;
 #endif
@@ -710,23 +736,23 @@ __device__ __forceinline__ bool closest_hit_warp_oct(const BvhView& bvh, bool ac
 
 // the traversal specialised to the packet's octant when all its active rays
 // share one (the usual case for coherent rays), the general one otherwise
-__device__ __forceinline__ bool closest_hit_warp(const BvhView& bvh, bool act, const Ray& r, float3 o,
-                                                 const Shear& sh, Hit& h, int cap, unsigned* status) {
+__device__ __forceinline__ bool closest_hit_warp(const BvhView& bvh, bool act, const Ray& r,
+                                                 const RayTri& rt, Hit& h, int cap, unsigned* status) {
     const unsigned FULL = 0xffffffffu;
     const int oct = ray_octant(r);
     const unsigned am = __ballot_sync(FULL, act);
     const int o0 = __shfl_sync(FULL, oct, am ? __ffs(am) - 1 : 0);
     const int u = __all_sync(FULL, !act || oct == o0) ? o0 : -1;
     switch (u) {
-        case 0: return closest_hit_warp_oct<0>(bvh, act, r, o, sh, h, cap, status);
-        case 1: return closest_hit_warp_oct<1>(bvh, act, r, o, sh, h, cap, status);
-        case 2: return closest_hit_warp_oct<2>(bvh, act, r, o, sh, h, cap, status);
-        case 3: return closest_hit_warp_oct<3>(bvh, act, r, o, sh, h, cap, status);
-        case 4: return closest_hit_warp_oct<4>(bvh, act, r, o, sh, h, cap, status);
-        case 5: return closest_hit_warp_oct<5>(bvh, act, r, o, sh, h, cap, status);
-        case 6: return closest_hit_warp_oct<6>(bvh, act, r, o, sh, h, cap, status);
-        case 7: return closest_hit_warp_oct<7>(bvh, act, r, o, sh, h, cap, status);
-        default: return closest_hit_warp_oct<-1>(bvh, act, r, o, sh, h, cap, status);
+        case 0: return closest_hit_warp_oct<0>(bvh, act, r, rt, h, cap, status);
+        case 1: return closest_hit_warp_oct<1>(bvh, act, r, rt, h, cap, status);
+        case 2: return closest_hit_warp_oct<2>(bvh, act, r, rt, h, cap, status);
+        case 3: return closest_hit_warp_oct<3>(bvh, act, r, rt, h, cap, status);
+        case 4: return closest_hit_warp_oct<4>(bvh, act, r, rt, h, cap, status);
+        case 5: return closest_hit_warp_oct<5>(bvh, act, r, rt, h, cap, status);
+        case 6: return closest_hit_warp_oct<6>(bvh, act, r, rt, h, cap, status);
+        case 7: return closest_hit_warp_oct<7>(bvh, act, r, rt, h, cap, status);
+        default: return closest_hit_warp_oct<-1>(bvh, act, r, rt, h, cap, status);
     }
 }
 
@@ -749,26 +775,27 @@ __host__ __device__ inline Lights make_lights(const hdof_params& p) {
     return l;
 }
 
-// Shading of a hit seen along the unit direction d: Lambert diffuse under
+// Shading of a hit of the ray from o in the unit direction d: Lambert diffuse under
 // directional lights, plus a white Blinn-Phong highlight (exponent 32) for
 // materials with k_s > 0, whose luminance is returned in spec.
-__device__ __forceinline__ void shade(const BvhView& bvh, const Lights& L, const Hit& h, float3 d, float3& n,
+__device__ __forceinline__ void shade(const BvhView& bvh, const Lights& L, int slot, float3 o, float3 d, float3& n,
                                       float3& rad, float& spec) {
-    const Tri* tr = bvh.tris + h.slot;
+    const Tri* tr = bvh.tris + slot;
     float4 p0 = __ldg(&tr->v0), p1 = __ldg(&tr->v1), p2 = __ldg(&tr->v2);
     float3 v0 = f3(p0.x, p0.y, p0.z);
     n = normalize(cross(f3(p1.x, p1.y, p1.z) - v0, f3(p2.x, p2.y, p2.z) - v0));
     if (dot(n, d) > 0.f) n = -1.f * n;
-    float4 ma = __ldg(&bvh.mat[2 * h.slot]);
+    float4 ma = __ldg(&bvh.mat[2 * slot]);
     float3 alb = f3(ma.x, ma.y, ma.z);
     if (ma.w > 0.f) {
-        float2 u0 = __ldg(&bvh.uv[3 * h.slot]), u1 = __ldg(&bvh.uv[3 * h.slot + 1]),
-               u2 = __ldg(&bvh.uv[3 * h.slot + 2]);
-        float uu = h.b0 * u0.x + h.b1 * u1.x + h.b2 * u2.x;
-        float vv = h.b0 * u0.y + h.b1 * u1.y + h.b2 * u2.y;
+        float2 u0 = __ldg(&bvh.uv[3 * slot]), u1 = __ldg(&bvh.uv[3 * slot + 1]), u2 = __ldg(&bvh.uv[3 * slot + 2]);
+        float b0, b1, b2;
+        tri_bary(o, make_shear(d), v0, f3(p1.x, p1.y, p1.z), f3(p2.x, p2.y, p2.z), b0, b1, b2);
+        float uu = b0 * u0.x + b1 * u1.x + b2 * u2.x;
+        float vv = b0 * u0.y + b1 * u1.y + b2 * u2.y;
         int cell = (int)floorf(ma.w * uu) + (int)floorf(ma.w * vv);
         if (cell & 1) {
-            float4 mb = __ldg(&bvh.mat[2 * h.slot + 1]);
+            float4 mb = __ldg(&bvh.mat[2 * slot + 1]);
             alb = f3(mb.x, mb.y, mb.z);
         }
     }
@@ -777,7 +804,7 @@ __device__ __forceinline__ void shade(const BvhView& bvh, const Lights& L, const
     rad = irr * alb;
     spec = 0.f;
     if (bvh.specular) {
-        const float ks = __ldg(&bvh.mat[2 * h.slot + 1].w);
+        const float ks = __ldg(&bvh.mat[2 * slot + 1].w);
         if (ks > 0.f) {
             float s = 0.f;
             for (int k = 0; k < L.n; ++k) {

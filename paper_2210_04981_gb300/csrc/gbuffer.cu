@@ -37,30 +37,27 @@ __device__ __forceinline__ void gbuffer_body(const GbufArgs<ND, COL>& a, int bx,
     float3 d = pinhole_dir(cam, i + 0.5f + cam.jx, j + 0.5f + cam.jy);
     float3 dn = normalize(d);
     const Ray ray = make_ray(cam.pos, dn);
-    const Shear sh = make_shear(dn);
+    const RayTri rt = make_ray_tri(a.bvh, cam.pos, dn);
     Hit h;
     h.t = INF;
     h.slot = -1;
-    h.id = 0x7fffffff;
-    h.b0 = h.b1 = h.b2 = 0.f;
     if (act && a.hint) {  // the previous frame's primary hit bounds the search
         const int id = a.hint[q];
-        if (id >= 0 && id < a.bvh.n_tris) hit_tri(a.bvh, __ldg(&a.bvh.slot_of[id]), cam.pos, sh, h);
+        if (id >= 0 && id < a.bvh.n_tris) hit_tri(rt, __ldg(&a.bvh.slot_of[id]), h);
     }
-    closest_hit_warp(a.bvh, act, ray, cam.pos, sh, h, a.cap, a.status);
+    closest_hit_warp(a.bvh, act, ray, rt, h, a.cap, a.status);
     if (!act) return;
     for (int k = 0; k < a.bvh.big_count; ++k) {
         const float4 lo = __ldg(&a.bvh.big_box[2 * k]), hi = __ldg(&a.bvh.big_box[2 * k + 1]);
         if (slab(ray, lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, h.t) < INF)
-            hit_tri(a.bvh, a.bvh.big_first + k, cam.pos, sh, h);
+            hit_tri(rt, a.bvh.big_first + k, h);
     }
-    if (h.slot < 0) h.id = -1;
     float3 n, rad, P;
     float z, spec = 0.f;
     if (h.slot >= 0) {
         P = cam.pos + h.t * dn;
         z = dot(P - cam.pos, cam.fwd);
-        shade(a.bvh, a.L, h, dn, n, rad, spec);
+        shade(a.bvh, a.L, h.slot, cam.pos, dn, n, rad, spec);
     } else {
         z = a.miss_dist;
         P = cam.pos + z * d;
@@ -69,7 +66,7 @@ __device__ __forceinline__ void gbuffer_body(const GbufArgs<ND, COL>& a, int bx,
     }
     st4(a.nd + q, make_float4(n.x, n.y, n.z, z));
     st4(a.col + q, make_float4(rad.x, rad.y, rad.z, spec));
-    if (a.tri) a.tri[q] = h.id;
+    if (a.tri) a.tri[q] = h.slot >= 0 ? __float_as_int(__ldg(&a.bvh.tris[h.slot].v0.w)) : -1;
     if (a.mv) {
         float ux, uy;
         a.mv[q] = project(a.prev, P, ux, uy) ? make_float2(i - ux, j - uy)

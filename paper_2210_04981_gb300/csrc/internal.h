@@ -124,7 +124,7 @@ struct hdof_bvh {
     int root;
     size_t bytes;
     hdof::Node* nodes;
-    hdof::Tri* tris;
+    hdof::Tri* tris;  // [3][n_tris]: the axes rotated in the second and third copy
     float4* mat;
     float2* uv;
     float4* big_box;  // [2 * n_big]

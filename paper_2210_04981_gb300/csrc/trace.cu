@@ -486,7 +486,7 @@ struct RayLane {
     int v, cur, leaf, sp, steps;
     unsigned r;
     Ray ray;
-    Shear sh;
+    RayTri rt;
     Hit h;
 };
 
@@ -536,7 +536,7 @@ __device__ __forceinline__ void trace_rays_steps(const Src& src, RayLane& L, int
         if (L.live && L.leaf != NO_LEAF) {
             const TraceArgs& a = src.at(L.v);
             int e = ~L.leaf, first = e >> 3, count = (e & 7) + 1;
-            for (int k = 0; k < count; ++k) hit_tri(a.bvh, first + k, L.ray.o, L.sh, L.h);
+            for (int k = 0; k < count; ++k) hit_tri(L.rt, first + k, L.h);
             L.leaf = NO_LEAF;
             if (L.cur < 0) {
                 L.leaf = L.cur;
@@ -556,7 +556,7 @@ __device__ __forceinline__ void trace_rays_steps(const Src& src, RayLane& L, int
                 for (int k = 0; k < bvh.big_count; ++k) {
                     float4 lo = __ldg(&bvh.big_box[2 * k]), hi = __ldg(&bvh.big_box[2 * k + 1]);
                     if (slab(L.ray, lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, L.h.t) < INF)
-                        hit_tri(bvh, bvh.big_first + k, L.ray.o, L.sh, L.h);
+                        hit_tri(L.rt, bvh.big_first + k, L.h);
                 }
                 // shading happens per pixel in the resolve, not here where
                 // few lanes of the warp finish at a time
@@ -615,18 +615,16 @@ __device__ __forceinline__ void trace_rays_body(const Src& src, unsigned total, 
                     float3 O, dir;
                     lens_ray(a, qp, __ldg(&a.ray_s[L.r]), O, dir);
                     L.ray = make_ray(O, dir);
-                    L.sh = make_shear(dir);
+                    L.rt = make_ray_tri(a.bvh, O, dir);
                     L.h.t = INF;
                     L.h.slot = -1;
-                    L.h.id = 0x7fffffff;
-                    L.h.b0 = L.h.b1 = L.h.b2 = 0.f;
                     if (a.hint) {
                         // the pixel's primary hit first: a lens ray often hits the same
                         // triangle, and the tight distance culls what lies behind it (the
                         // closest hit, the minimum of (t, id) over all hits, is unchanged)
                         const int id = __ldg(&a.hint[qp]);
                         if (id >= 0 && id < a.bvh.n_tris)
-                            hit_tri(a.bvh, __ldg(&a.bvh.slot_of[id]), L.ray.o, L.sh, L.h);
+                            hit_tri(L.rt, __ldg(&a.bvh.slot_of[id]), L.h);
                     }
                     L.cur = a.bvh.root;
                     L.leaf = NO_LEAF;
@@ -697,32 +695,29 @@ __device__ __forceinline__ void trace_packets_body(const Src& src, unsigned tota
             const bool act = pending && v == v0;
             const TraceArgs& a = src.at(v0);
             Ray ray;
-            Shear sh;
             Hit h;
             h.t = INF;
             h.slot = -1;
-            h.id = 0x7fffffff;
-            h.b0 = h.b1 = h.b2 = 0.f;
             float3 O = f3(0.f, 0.f, 0.f), dir = f3(0.f, 0.f, 1.f);
             if (act) {
                 const unsigned qp = __ldg(&a.ray_pix[r]), smp = __ldg(&a.ray_s[r]);
                 lens_ray(a, qp, smp, O, dir);
                 if (a.binned) r = __ldg(&a.qoff[qp]) + smp;  // its record
                 if (a.hint) {  // the pixel's primary hit first (see trace_rays_body)
-                    sh = make_shear(dir);
+                    const RayTri rt = make_ray_tri(a.bvh, O, dir);
                     const int id = __ldg(&a.hint[qp]);
-                    if (id >= 0 && id < a.bvh.n_tris) hit_tri(a.bvh, __ldg(&a.bvh.slot_of[id]), O, sh, h);
+                    if (id >= 0 && id < a.bvh.n_tris) hit_tri(rt, __ldg(&a.bvh.slot_of[id]), h);
                 }
             }
             ray = make_ray(O, dir);
-            sh = make_shear(dir);
-            closest_hit_warp(a.bvh, act, ray, O, sh, h, a.cap, a.status);
+            const RayTri rt = make_ray_tri(a.bvh, O, dir);
+            closest_hit_warp(a.bvh, act, ray, rt, h, a.cap, a.status);
             if (act) {
                 const BvhView& bvh = a.bvh;
                 for (int k = 0; k < bvh.big_count; ++k) {
                     float4 lo = __ldg(&bvh.big_box[2 * k]), hi = __ldg(&bvh.big_box[2 * k + 1]);
                     if (slab(ray, lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, h.t) < INF)
-                        hit_tri(bvh, bvh.big_first + k, O, sh, h);
+                        hit_tri(rt, bvh.big_first + k, h);
                 }
                 a.recs[r] = make_float2(h.slot >= 0 ? h.t : INF, __int_as_float(h.slot));
             }
@@ -777,17 +772,9 @@ __device__ __forceinline__ SampleTerm resolve_sample(const TraceArgs& a, unsigne
     o.L = f3(0.f, 0.f, 0.f);
     float c;
     if (hit) {
-        Hit h;
-        h.t = rc.x;
-        h.slot = slot;
-        const Tri* tr = a.bvh.tris + slot;
-        const float4 p0 = __ldg(&tr->v0), p1 = __ldg(&tr->v1), p2 = __ldg(&tr->v2);
-        h.id = __float_as_int(p0.w);
-        tri_bary(O, make_shear(dir), f3(p0.x, p0.y, p0.z), f3(p1.x, p1.y, p1.z), f3(p2.x, p2.y, p2.z), h.b0, h.b1,
-                 h.b2);
         float3 nrm;
         float spec;
-        shade(a.bvh, a.L, h, dir, nrm, o.L, spec);
+        shade(a.bvh, a.L, slot, O, dir, nrm, o.L, spec);
         o.P = O + rc.x * dir;
         c = a.coc(dot(o.P - a.cam.pos, a.cam.fwd));
     } else {

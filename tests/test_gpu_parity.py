@@ -89,6 +89,55 @@ def test_closest_hits_match_brute_force(orc, n):
     assert (g_id != o_id).mean() < 1e-3
 
 
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("sign", [-1.0, 1.0])
+def test_closest_hits_by_main_axis(orc, axis, sign):
+    """Rays whose largest direction component is each axis, either way (the
+    rotated triangle copies and the negated edge functions), the two largest
+    components equal, and rays along the axis itself, through triangles of
+    which some are repeated (equal distances: the lower id).  Sheared
+    coordinates are off by up to 1e-6, edge functions by up to 2.2e-6, and the
+    distance, their mean of depths at most 0.8 apart over their sum (0.2 at
+    least here), by 3 x 2.2e-6 x 0.8 / 0.2 = 2.6e-5 of at least 2.6: within
+    1e-5."""
+    rng = np.random.default_rng(10 * axis + (sign > 0))
+    n, m = 300, 6000
+    c = rng.uniform(-1, 1, (n, 1, 3))
+    v = c + rng.uniform(-0.4, 0.4, (n, 3, 3))
+    v[n - 20:] = v[:20]
+    sc0 = _soup(rng, n)
+    sc = hi.Scene(v.reshape(-1, 3).astype(np.float32), sc0.idx, sc0.mat, sc0.uv)
+    bvh = bvh_of(sc)
+    org = rng.uniform(-0.8, 0.8, (m, 3))
+    org[:, axis] = -4.0 * sign
+    d = rng.uniform(-0.3, 0.3, (m, 3))
+    d[:, axis] = sign
+    d[:1000] = 0.0
+    d[:1000, axis] = sign
+    d[1000:1500, (axis + 1) % 3] = sign  # two largest components equal
+    org[1000:1500, (axis + 1) % 3] = -4.0 * sign
+    org, d = org.astype(np.float32), d.astype(np.float32)
+    ids = torch.empty(m, dtype=torch.int32, device="cuda")
+    ts = torch.empty(m, dtype=torch.float32, device="cuda")
+    H.hdof_closest_hits(bvh, dev(org), dev(d), ids, ts)
+    H.hdof_sync()
+    g_id, g_t = host(ids), host(ts)
+    o_id, o_t = orc.OScene(sc).closest_hits(org.astype(np.float64), d.astype(np.float64), use_bvh=False)
+    tv = sc.tri_verts().astype(np.float64)
+    assert (g_id >= n - 20).sum() == 0  # a repeated triangle never wins over its twin
+    for k in np.nonzero(g_id != o_id)[0]:
+        o, dd = org[k].astype(np.float64), d[k].astype(np.float64)
+        margins = [abs(_bary_margin(tv[t], o, dd)) for t in (g_id[k], o_id[k]) if t >= 0]
+        tie_t = g_id[k] >= 0 and o_id[k] >= 0 and abs(g_t[k] - o_t[k]) <= 1e-5 * o_t[k]
+        assert tie_t or min(margins) < 1e-5, f"ray {k}"
+    hit = (g_id >= 0) & (g_id == o_id)
+    t9 = tv[np.maximum(g_id, 0)]
+    nrm = np.cross(t9[:, 3:6] - t9[:, 0:3], t9[:, 6:9] - t9[:, 0:3])
+    hit &= np.abs((nrm * d).sum(1)) > 0.2  # the largest component of d is 1
+    assert hit.sum() > 200
+    assert np.allclose(g_t[hit], o_t[hit], rtol=1e-5)
+
+
 @pytest.mark.parametrize("n", [3, 65, 1023, 1024, 1025, 1027, 2049, 5000])
 def test_build_around_the_finishing_block(n):
     """Trees whose clustering runs in one block only, in rounds over several
