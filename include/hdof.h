@@ -469,10 +469,11 @@ int hdof_composite(const hdof_gbuf* in, const uint8_t* spp, const float* pp, con
  * hdof_postfilter applied to the plane (S, S, S) of the G-buffer's col.w in
  * place of the colour (the filter is linear in the colour, so this is
  * exactly the share of S in pp).  pp_spec: float [H][W][4] = (S_pp, S_pp,
- * S_pp, alpha).  workspace as for hdof_postfilter, whose first 16 bytes per
- * pixel (the mask's and the trace's region) hold the grey plane: unlike
- * hdof_postfilter it must not run concurrently with hdof_mask, hdof_trace or
- * hdof_postfilter on the same workspace.
+ * S_pp, alpha).  workspace as for hdof_postfilter: it must not run
+ * concurrently with hdof_postfilter on the same workspace.  With a shaped
+ * bokeh (blades or aberration) the first 16 bytes per pixel (the mask's and
+ * the trace's region) also hold the grey plane: then not concurrently with
+ * hdof_mask or hdof_trace either.
  * hdof_composite_spec: hdof_composite whose near branch where traced is
  * lerp(C_rec, C_pp, clamp(spec_pref S_pp, 0, 1)); pp_spec may be NULL and
  * is ignored when spec_pref = 0 (then it equals hdof_composite).  Neither

@@ -43,6 +43,10 @@
 namespace hdof {
 namespace {
 
+using hdof::ld4;  // beside the overloads below
+using hdof::ld_rec_pair;
+using hdof::st4;
+
 constexpr int TP = HDOF_TILE_PF;
 constexpr int PF_GROUP = 64;  // threads that cover a 16x16 tile once (2x2 pixels each; 2x4 slower by 5-30%)
 // Thread groups per tile, group g taking the source row pairs g, g + PF_G, ...
@@ -109,11 +113,43 @@ __host__ __device__ inline int pf_pitch(int W) { return (W + 1) & ~1; }
 template <class COL>
 struct RecOf {
     using T = float4;
+    using P = float4;  // an entry of the row prefix
 };
 template <>
 struct RecOf<bf164s> {
     using T = bf164s;
+    using P = float4;
 };
+// The specular plane col.w as an opaque grey colour: FP32 records (s w/a, w/a)
+// and as many sums, half the loads and FMAs of a colour's, with the same
+// results as the plane filtered as a colour.  That took a pass to write the
+// plane and, alone, 245 us at 1279x717 (wide aperture) and 2197 us at 4K in the
+// gather; this takes 178 and 1525 us.
+template <class COL>
+struct Grey {
+    COL c;
+};
+template <class COL>
+__device__ __forceinline__ float4 ld4(const Grey<COL>* p) {
+    const float s = ld4(&p->c).w;
+    return make_float4(s, s, s, s);
+}
+template <class COL>
+struct RecOf<Grey<COL>> {
+    using T = float2;
+    using P = float2;
+};
+// a record or prefix entry of two channels stands for the last two of four
+__device__ __forceinline__ void st4(float2* p, const float4& v) { *p = make_float2(v.z, v.w); }
+__device__ __forceinline__ float4 ld4(const float2* p) {
+    const float2 v = __ldg(p);
+    return make_float4(0.f, 0.f, v.x, v.y);
+}
+__device__ __forceinline__ void ld_rec_pair(const float2* p, float2& a, float2& b) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    a = make_float2(v.x, v.y);
+    b = make_float2(v.z, v.w);
+}
 
 template <class ND, class COL>
 struct PrepArgs {
@@ -186,16 +222,16 @@ __global__ void __launch_bounds__(256) k_pf_prep(PrepArgs<ND, COL> a) { pf_prep_
 // taps (all of weight exactly 1) as differences of it.  One block per row,
 // in rounds of 256 consecutive pixels (a block scan per round plus the
 // running total): the summation order is fixed.
-template <class REC>
+template <class REC, class PRE = float4>
 struct RowScanArgsT {
     const REC* nrec;  // row-major
     int W, H;
-    float4* pre;
+    PRE* pre;
 };
 using RowScanArgs = RowScanArgsT<float4>;
 
-template <class REC>
-__device__ __forceinline__ void pf_rowscan_body(const RowScanArgsT<REC>& a, int y) {
+template <class REC, class PRE>
+__device__ __forceinline__ void pf_rowscan_body(const RowScanArgsT<REC, PRE>& a, int y) {
     const int W = pf_pitch(a.W), t = threadIdx.x, lane = t & 31, w = t >> 5;
     const size_t row = (size_t)y * W;
     __shared__ float4 s_warp[8];
@@ -215,7 +251,7 @@ __device__ __forceinline__ void pf_rowscan_body(const RowScanArgsT<REC>& a, int 
         __syncthreads();
         float4 before = carry;
         for (int k = 0; k < w; ++k) before = add4(before, s_warp[k]);
-        if (x < W) a.pre[row + x] = add4(before, v);
+        if (x < W) st4(a.pre + row + x, add4(before, v));
         float4 total = carry;
         for (int k = 0; k < 8; ++k) total = add4(total, s_warp[k]);
         carry = total;
@@ -223,8 +259,8 @@ __device__ __forceinline__ void pf_rowscan_body(const RowScanArgsT<REC>& a, int 
     }
 }
 
-template <class REC>
-__global__ void __launch_bounds__(256) k_pf_rowscan(RowScanArgsT<REC> a) { pf_rowscan_body(a, blockIdx.x); }
+template <class REC, class PRE>
+__global__ void __launch_bounds__(256) k_pf_rowscan(RowScanArgsT<REC, PRE> a) { pf_rowscan_body(a, blockIdx.x); }
 
 // Per target pixel: a layer's sums (S.x, S.y) and (S.z, W) as register
 // pairs so one packed FMA updates two of them; the far layer also holds its
@@ -236,6 +272,32 @@ struct FarAcc {
     float2 xy, zw;
     float ka, kb;
 };
+struct GreyNearAcc {  // (S, W)
+    float2 zw;
+};
+struct GreyFarAcc {
+    float2 zw;
+    float ka, kb;
+};
+template <class REC>
+struct AccOf {
+    using Near = NearAcc;
+    using Far = FarAcc;
+};
+template <>
+struct AccOf<float2> {
+    using Near = GreyNearAcc;
+    using Far = GreyFarAcc;
+};
+template <class A>
+__device__ __forceinline__ void acc_clear(A& a) { a.xy = a.zw = make_float2(0.f, 0.f); }
+__device__ __forceinline__ void acc_clear(GreyNearAcc& a) { a.zw = make_float2(0.f, 0.f); }
+__device__ __forceinline__ void acc_clear(GreyFarAcc& a) { a.zw = make_float2(0.f, 0.f); }
+// the sums as (S.x, S.y, S.z, W)
+template <class A>
+__device__ __forceinline__ float4 acc_sum(const A& a) { return make_float4(a.xy.x, a.xy.y, a.zw.x, a.zw.y); }
+__device__ __forceinline__ float4 acc_sum(const GreyNearAcc& a) { return make_float4(a.zw.x, a.zw.x, a.zw.x, a.zw.y); }
+__device__ __forceinline__ float4 acc_sum(const GreyFarAcc& a) { return make_float4(a.zw.x, a.zw.x, a.zw.x, a.zw.y); }
 
 // far = (S.x, S.y, S.z, W) of the far layer
 template <class COL>
@@ -267,7 +329,7 @@ struct GatherArgs {
     const typename RecOf<COL>::T* frec;
     const COL* col;  // sharp colour (empty far layer)
     const float4* tmax;
-    const float4* pre;  // row prefix of the near records
+    const typename RecOf<COL>::P* pre;  // row prefix of the near records
     int W, H, ntx, nty, kt;
     float kz_rel;
     float4* pp;
@@ -287,6 +349,12 @@ __device__ __forceinline__ void acc(FarAcc& a, float d, float rh, float zq, cons
     a.xy = fma2(t, f.x, f.y, a.xy);
     a.zw = fma2(t, f.z, f.w, a.zw);
 }
+__device__ __forceinline__ void acc(GreyNearAcc& a, float d, float rh, float, const float2& n, bool in) {
+    a.zw = fma2(in ? __saturatef(rh - d) : 0.f, n.x, n.y, a.zw);
+}
+__device__ __forceinline__ void acc(GreyFarAcc& a, float d, float rh, float zq, const float2& f, bool) {
+    a.zw = fma2(__saturatef(rh - d) * __saturatef(fmaf(-zq, a.kb, a.ka)), f.x, f.y, a.zw);
+}
 
 // Two taps of one column, one in each of the rows ya = j - s and yb = j + 1 + s
 // around a thread's 2x2 block of rows j, j + 1.  Row ya lies s above the upper
@@ -300,9 +368,9 @@ __device__ __forceinline__ void acc(FarAcc& a, float d, float rh, float zq, cons
 struct TapCarry {
     float cn, cf, pdx2;
 };
-template <bool MASK, class A>
+template <bool MASK, class A, class E>
 __device__ __forceinline__ void pf_tap(A (&a)[4], TapCarry& c, float sn2, float sf2, float wn, float wf, float dx,
-                                       float ra, float za, const float4& ea, float rb, float zb, const float4& eb) {
+                                       float ra, float za, const E& ea, float rb, float zb, const E& eb) {
     const float dx2 = dx * dx;
     const float dn = sqrt_approx(dx2 + sn2), df = sqrt_approx(dx2 + sf2);
     acc(a[0], dn, ra, za, ea, !MASK || dx2 > wn);
@@ -317,6 +385,16 @@ __device__ __forceinline__ void pf_tap(A (&a)[4], TapCarry& c, float sn2, float 
     c.cf = df;
     c.pdx2 = dx2;
 }
+
+// a loaded record
+template <class REC>
+struct EntryOf {
+    using T = float4;
+};
+template <>
+struct EntryOf<float2> {
+    using T = float2;
+};
 
 // The taps of the columns xs .. xe (xs even, xe odd: whole pairs) of the rows
 // at plane offsets oa and ob: one 256-bit load of a pair's two records and one
@@ -340,7 +418,7 @@ __device__ __forceinline__ void pf_segment(A (&a)[4], float sn2, float sf2, floa
 #pragma unroll PF_UNROLL
     for (int x = xs; x < xe; x += 2, ++ma, ++mb, dx += 2.f) {
         const float2 ra = on_a ? __ldg(&rh2[ma]) : none, rb = on_b ? __ldg(&rh2[mb]) : none;
-        float4 ea0, ea1, eb0, eb1;
+        typename EntryOf<REC>::T ea0, ea1, eb0, eb1;
         ld_rec_pair(rec + 2 * (size_t)ma, ea0, ea1);
         ld_rec_pair(rec + 2 * (size_t)mb, eb0, eb1);
         const float2 za = NEAR ? zero : __ldg(&zq2[ma]), zb = NEAR ? zero : __ldg(&zq2[mb]);
@@ -354,15 +432,24 @@ __device__ __forceinline__ void add_sum(A& t, const float4& s) {
     t.xy = make_float2(t.xy.x + s.x, t.xy.y + s.y);
     t.zw = make_float2(t.zw.x + s.z, t.zw.y + s.w);
 }
-// pre[hi] - pre[lo - 1] of one row of the prefix
-__device__ __forceinline__ float4 prefix_sum(const float4* __restrict__ row, int lo, int hi) {
-    float4 s = __ldg(&row[hi]);
-    if (lo > 0) {
-        const float4 l = __ldg(&row[lo - 1]);
-        s = make_float4(s.x - l.x, s.y - l.y, s.z - l.z, s.w - l.w);
-    }
-    return s;
+template <class A>
+__device__ __forceinline__ void add_sum(A& t, const float2& s) {
+    t.zw = make_float2(t.zw.x + s.x, t.zw.y + s.y);
 }
+__device__ __forceinline__ float4 sub_sum(const float4& a, const float4& b) {
+    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+__device__ __forceinline__ float2 sub_sum(const float2& a, const float2& b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float4 both_sums(const float4& a, const float4& b) { return add4(a, b); }
+__device__ __forceinline__ float2 both_sums(const float2& a, const float2& b) { return make_float2(a.x + b.x, a.y + b.y); }
+// pre[hi] - pre[lo - 1] of one row of the prefix
+template <class PRE>
+__device__ __forceinline__ PRE prefix_sum(const PRE* __restrict__ row, int lo, int hi) {
+    const PRE s = __ldg(&row[hi]);
+    return lo > 0 ? sub_sum(s, __ldg(&row[lo - 1])) : s;
+}
+__device__ __forceinline__ float prefix_weight(const float4* p) { return __ldg(&p->w); }
+__device__ __forceinline__ float prefix_weight(const float2* p) { return __ldg(&p->y); }
 
 // One layer's loop over a disk-shaped window of radius R around the 2x2 block
 // at (i, j): every source feeding the layer within reach has r + 1/2 <= R, so
@@ -378,10 +465,10 @@ __device__ __forceinline__ float4 prefix_sum(const float4* __restrict__ row, int
 // each pixel sums its own interior columns (two loads a pixel); the columns
 // inside every pixel's interior are skipped, the rest are tapped with each
 // pixel's interior masked out.
-template <bool NEAR, bool PERPX, class A, class REC>
+template <bool NEAR, bool PERPX, class A, class REC, class PRE>
 __device__ __forceinline__ void pf_layer(A (&a)[4], float R, float Rin, int g, int i, int j, int W, int H,
                                          const float* __restrict__ rh, const float* __restrict__ zq,
-                                         const REC* __restrict__ rec, const float4* __restrict__ pre) {
+                                         const REC* __restrict__ rec, const PRE* __restrict__ pre) {
     if (R < 0.f) return;  // nothing within reach feeds this layer
     // bounds lean outwards by 1e-3 pixel (float rounding); taps they add weigh 0
     const int G = (int)floorf(R + 1e-3f), Wp = pf_pitch(W);
@@ -421,8 +508,8 @@ __device__ __forceinline__ void pf_layer(A (&a)[4], float R, float Rin, int g, i
             const int wi = (int)sqrt_approx(Rin2 - sf2);
             const int la = (max(i + 1 - wi, 0) + 1) & ~1, ra = i + wi >= W - 1 ? Wp - 1 : ((i + wi + 1) & ~1) - 1;
             if (ra - la + 1 >= PF_MIN_IN) {
-                float4 sum = on_a ? prefix_sum(pre + oa, la, ra) : make_float4(0.f, 0.f, 0.f, 0.f);
-                if (on_b) sum = add4(sum, prefix_sum(pre + ob, la, ra));
+                PRE sum = on_a ? prefix_sum(pre + oa, la, ra) : PRE{};
+                if (on_b) sum = both_sums(sum, prefix_sum(pre + ob, la, ra));
 #pragma unroll
                 for (int k = 0; k < 4; ++k) add_sum(a[k], sum);
                 ls = la;
@@ -449,6 +536,7 @@ __device__ __forceinline__ float4 pf_group_sum(const float4 (&part)[PF_G][TP * T
 template <class COL>
 __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx, int ty) {
     const COL* __restrict__ col = ar.col;
+    using Acc = AccOf<typename RecOf<COL>::T>;
     const float4* __restrict__ tmax = ar.tmax;
     const int W = ar.W, H = ar.H, ntx = ar.ntx, nty = ar.nty, kt = ar.kt;
     const int nk = (2 * kt + 1) * (2 * kt + 1);
@@ -510,7 +598,7 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
         const int G = (int)floorf(Gn + 1e-3f), y0 = max(ty * TP - G, 0), y1 = min(ty * TP + TP - 1 + G, H - 1);
         bool big = false;
         for (int y = y0 + threadIdx.x; y <= y1; y += GATHER_THREADS)
-            big |= !(__ldg(&ar.pre[(size_t)y * pf_pitch(W) + W - 1].w) <= PF_ROW_W);
+            big |= !(prefix_weight(&ar.pre[(size_t)y * pf_pitch(W) + W - 1]) <= PF_ROW_W);
         per_px = __syncthreads_or(big);
     }
     // group g of the block's PF_G takes every PF_G-th source row; t is the
@@ -524,7 +612,7 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
     // far layer first; its sums wait in the pixels' own pp slots (each pixel
     // is one thread's alone) so they hold no registers during the near loop
     if (Gf >= 0.f) {
-        FarAcc f[4];  // pixel (i + (k & 1), j + (k >> 1))
+        typename Acc::Far f[4];  // pixel (i + (k & 1), j + (k >> 1))
         if (in) {
             const float ka = 1.f + 1.f / ar.kz_rel;  // k_z = clamp(ka - z_q kb), kb = 1 / (kz_rel z_p)
             const size_t zo = (size_t)j * pf_pitch(W) + i;
@@ -535,12 +623,12 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
                 const float zp = x < W && y < H ? __ldg(&ar.zq[zo + (size_t)(k >> 1) * pf_pitch(W) + (k & 1)]) : z00;
                 f[k].ka = ka;
                 f[k].kb = 1.f / (ar.kz_rel * zp);
-                f[k].xy = f[k].zw = make_float2(0.f, 0.f);
+                acc_clear(f[k]);
             }
-            pf_layer<false, false>(f, Gf, -1.f, g, i, j, W, H, ar.rh, ar.zq, ar.frec, nullptr);
+            pf_layer<false, false>(f, Gf, -1.f, g, i, j, W, H, ar.rh, ar.zq, ar.frec, ar.pre);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = make_float4(f[k].xy.x, f[k].xy.y, f[k].zw.x, f[k].zw.y);
+                s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = acc_sum(f[k]);
         }
         __syncthreads();
         for (int p = threadIdx.x; p < TP * TP; p += GATHER_THREADS) {
@@ -550,14 +638,14 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
         __syncthreads();
     }
     if (in) {
-        NearAcc a[4];
+        typename Acc::Near a[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) a[k].xy = a[k].zw = make_float2(0.f, 0.f);
+        for (int k = 0; k < 4; ++k) acc_clear(a[k]);
         if (per_px) pf_layer<true, true>(a, Gn, Rin, g, i, j, W, H, ar.rh, ar.zq, ar.nrec, ar.pre);
         else pf_layer<true, false>(a, Gn, Rin, g, i, j, W, H, ar.rh, ar.zq, ar.nrec, ar.pre);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = make_float4(a[k].xy.x, a[k].xy.y, a[k].zw.x, a[k].zw.y);
+            s_part[g][(lj + (k >> 1)) * TP + li + (k & 1)] = acc_sum(a[k]);
     }
     __syncthreads();
     for (int p = threadIdx.x; p < TP * TP; p += GATHER_THREADS) {
@@ -571,7 +659,15 @@ __device__ __forceinline__ void pf_gather_body(const GatherArgs<COL>& ar, int tx
 }
 
 template <class COL>
-__global__ void __launch_bounds__(GATHER_THREADS, PF_MINB) k_pf_gather(GatherArgs<COL> a) {
+struct GatherBlocks {
+    static constexpr int MIN = PF_MINB;
+};
+template <class COL>
+struct GatherBlocks<Grey<COL>> {
+    static constexpr int MIN = 8;  // 64 registers; 6, 7, 8, 10 blocks at 4K: 1663, 1577, 1525, 1742 us
+};
+template <class COL>
+__global__ void __launch_bounds__(GATHER_THREADS, GatherBlocks<COL>::MIN) k_pf_gather(GatherArgs<COL> a) {
     pf_gather_body(a, blockIdx.x, blockIdx.y);
 }
 
@@ -697,6 +793,43 @@ using namespace hdof;
 
 namespace hdof {
 
+template <class ND, class COL>
+static int run_postfilter(const hdof_gbuf* in, const Coc& coc, const hdof_params* p, float* pp, float4* aux,
+                          void* scratch, cudaStream_t s, const float* lens_dev, float t) {
+    using REC = typename RecOf<COL>::T;
+    using PRE = typename RecOf<COL>::P;
+    int rc;
+    if ((rc = ensure_area_table(s))) return rc;
+    const int W = in->width, H = in->height;
+    ViewWs w = {};
+    pf_regions(w, static_cast<char*>(scratch), ws_layout(W, H, p));
+    REC* nrec = reinterpret_cast<REC*>(w.nrec);
+    REC* frec = reinterpret_cast<REC*>(w.frec);
+    PRE* pre = reinterpret_cast<PRE*>(w.pre);
+    const COL* col = static_cast<const COL*>(in->col);
+    const int ntx = (W + TP - 1) / TP, nty = (H + TP - 1) / TP;
+    dim3 grid(ntx, nty);
+    {
+        ProfScope ps_("pf_prep", s);
+        k_pf_prep<<<grid, 256, 0, s>>>(PrepArgs<ND, COL>{static_cast<const ND*>(in->nd), col, W, H, coc, p->r_max, ntx,
+                                                         w.rh, w.zq, nrec, frec, w.tmax, lens_dev, t});
+        HDOF_LAUNCHED("post-filter prep");
+    }
+    {
+        ProfScope ps_("pf_rowscan", s);
+        k_pf_rowscan<<<H, 256, 0, s>>>(RowScanArgsT<REC, PRE>{nrec, W, H, pre});
+        HDOF_LAUNCHED("post-filter row prefix");
+    }
+    // the taps are served from L1: a small shared-memory carve-out
+    ProfScope ps_("pf_gather", s);
+    cudaFuncSetAttribute(k_pf_gather<COL>, cudaFuncAttributePreferredSharedMemoryCarveout, GATHER_CARVEOUT);
+    k_pf_gather<COL><<<grid, GATHER_THREADS, 0, s>>>(GatherArgs<COL>{w.rh, w.zq, nrec, frec, col, w.tmax, pre, W, H, ntx,
+                                                                     nty, gather_tiles(p->r_max), p->kz_rel,
+                                                                     reinterpret_cast<float4*>(pp), aux});
+    HDOF_LAUNCHED("post-filter gather");
+    return HDOF_OK;
+}
+
 int launch_postfilter(const hdof_gbuf* in, const Coc& coc, const hdof_params* p, float* pp, float4* aux,
                       void* scratch, cudaStream_t s, const float* lens_dev, float t) {
     if (bokeh_shaped(p)) {
@@ -706,65 +839,11 @@ int launch_postfilter(const hdof_gbuf* in, const Coc& coc, const hdof_params* p,
         }
         return launch_bokeh(in, coc, p, pp, scratch, s);
     }
-    int rc;
-    if ((rc = ensure_area_table(s))) return rc;
-    const int W = in->width, H = in->height;
-    ViewWs w = {};
-    pf_regions(w, static_cast<char*>(scratch), ws_layout(W, H, p));
-    const int ntx = (W + TP - 1) / TP, nty = (H + TP - 1) / TP;
-    dim3 grid(ntx, nty);
     const bool f32n = in->dtype_nd == HDOF_F32, f32c = in->dtype_col == HDOF_F32;
-    const float4* nd4 = static_cast<const float4*>(in->nd);
-    const half4s* ndh = static_cast<const half4s*>(in->nd);
-    const float4* col4 = static_cast<const float4*>(in->col);
-    const bf164s* colb = static_cast<const bf164s*>(in->col);
-    const float rm = p->r_max;
-    {
-        ProfScope ps_("pf_prep", s);
-        if (f32n && f32c)
-            k_pf_prep<<<grid, 256, 0, s>>>(
-                PrepArgs<float4, float4>{nd4, col4, W, H, coc, rm, ntx, w.rh, w.zq, w.nrec, w.frec, w.tmax, lens_dev, t});
-        else if (f32n)
-            k_pf_prep<<<grid, 256, 0, s>>>(
-                PrepArgs<float4, bf164s>{nd4, colb, W, H, coc, rm, ntx, w.rh, w.zq, reinterpret_cast<bf164s*>(w.nrec),
-                                              reinterpret_cast<bf164s*>(w.frec), w.tmax, lens_dev, t});
-        else if (f32c)
-            k_pf_prep<<<grid, 256, 0, s>>>(
-                PrepArgs<half4s, float4>{ndh, col4, W, H, coc, rm, ntx, w.rh, w.zq, w.nrec, w.frec, w.tmax, lens_dev, t});
-        else
-            k_pf_prep<<<grid, 256, 0, s>>>(
-                PrepArgs<half4s, bf164s>{ndh, colb, W, H, coc, rm, ntx, w.rh, w.zq, reinterpret_cast<bf164s*>(w.nrec),
-                                              reinterpret_cast<bf164s*>(w.frec), w.tmax, lens_dev, t});
-        HDOF_LAUNCHED("post-filter prep");
-    }
-    {
-        ProfScope ps_("pf_rowscan", s);
-        if (f32c)
-            k_pf_rowscan<float4><<<H, 256, 0, s>>>(RowScanArgsT<float4>{w.nrec, W, H, w.pre});
-        else
-            k_pf_rowscan<bf164s><<<H, 256, 0, s>>>(
-                RowScanArgsT<bf164s>{reinterpret_cast<const bf164s*>(w.nrec), W, H, w.pre});
-        HDOF_LAUNCHED("post-filter row prefix");
-    }
-    const int kt = gather_tiles(p->r_max);
-    float4* out = reinterpret_cast<float4*>(pp);
-    // the taps are served from L1: a small shared-memory carve-out
-    ProfScope ps_("pf_gather", s);
-    if (f32c) {
-        cudaFuncSetAttribute(k_pf_gather<float4>, cudaFuncAttributePreferredSharedMemoryCarveout, GATHER_CARVEOUT);
-        k_pf_gather<float4><<<grid, GATHER_THREADS, 0, s>>>(
-            GatherArgs<float4>{w.rh, w.zq, w.nrec, w.frec, col4, w.tmax, w.pre, W, H, ntx, nty, kt, p->kz_rel, out,
-                               aux});
-    } else {
-        cudaFuncSetAttribute(k_pf_gather<bf164s>, cudaFuncAttributePreferredSharedMemoryCarveout, GATHER_CARVEOUT);
-        k_pf_gather<bf164s><<<grid, GATHER_THREADS, 0, s>>>(
-            GatherArgs<bf164s>{w.rh, w.zq, reinterpret_cast<const bf164s*>(w.nrec),
-                               reinterpret_cast<const bf164s*>(w.frec), colb, w.tmax, w.pre, W, H, ntx, nty, kt,
-                               p->kz_rel, out,
-                               aux});
-    }
-    HDOF_LAUNCHED("post-filter gather");
-    return HDOF_OK;
+    if (f32n && f32c) return run_postfilter<float4, float4>(in, coc, p, pp, aux, scratch, s, lens_dev, t);
+    if (f32n) return run_postfilter<float4, bf164s>(in, coc, p, pp, aux, scratch, s, lens_dev, t);
+    if (f32c) return run_postfilter<half4s, float4>(in, coc, p, pp, aux, scratch, s, lens_dev, t);
+    return run_postfilter<half4s, bf164s>(in, coc, p, pp, aux, scratch, s, lens_dev, t);
 }
 
 }  // namespace hdof
@@ -815,12 +894,22 @@ extern "C" int hdof_postfilter_spec(const hdof_gbuf* in, const hdof_camera* cam,
     WsLayout L = ws_layout(in->width, in->height, p);
     HDOF_CHECK_ARG(workspace && workspace_bytes >= L.total, "hdof_postfilter_spec: workspace of %zu bytes < %zu",
                    workspace_bytes, L.total);
-    // the grey plane sits below the post-filter's region (the mask and trace
+    // the shaped post-filter's grey plane sits below the post-filter's region (the mask and trace
     // scratch, at least 16 bytes per pixel since spp_max >= 1)
     const size_t n = (size_t)in->width * in->height;
     HDOF_CHECK_ARG(n * sizeof(float4) <= L.pf_off, "hdof_postfilter_spec: no room for the specular plane");
-    float4* plane = static_cast<float4*>(workspace);
     cudaStream_t s = as_stream(stream);
+    const Coc coc = make_coc(*lens, in->height, cam->tan_half_fovy);
+    void* scratch = static_cast<char*>(workspace) + L.pf_off;
+    if (!bokeh_shaped(p)) {
+        const bool f32n = in->dtype_nd == HDOF_F32, f32c = in->dtype_col == HDOF_F32;
+        if (f32n && f32c)
+            return run_postfilter<float4, Grey<float4>>(in, coc, p, pp_spec, nullptr, scratch, s, nullptr, 0.f);
+        if (f32n) return run_postfilter<float4, Grey<bf164s>>(in, coc, p, pp_spec, nullptr, scratch, s, nullptr, 0.f);
+        if (f32c) return run_postfilter<half4s, Grey<float4>>(in, coc, p, pp_spec, nullptr, scratch, s, nullptr, 0.f);
+        return run_postfilter<half4s, Grey<bf164s>>(in, coc, p, pp_spec, nullptr, scratch, s, nullptr, 0.f);
+    }
+    float4* plane = static_cast<float4*>(workspace);
     {
         ProfScope ps_("pf_spec_plane", s);
         const unsigned blocks = (unsigned)((n + 255) / 256);
@@ -833,8 +922,7 @@ extern "C" int hdof_postfilter_spec(const hdof_gbuf* in, const hdof_camera* cam,
     hdof_gbuf g = *in;
     g.dtype_col = HDOF_F32;
     g.col = plane;
-    return launch_postfilter(&g, make_coc(*lens, in->height, cam->tan_half_fovy), p, pp_spec, nullptr,
-                             static_cast<char*>(workspace) + L.pf_off, s);
+    return launch_bokeh(&g, coc, p, pp_spec, scratch, s);
 }
 
 namespace hdof {

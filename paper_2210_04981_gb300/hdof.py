@@ -573,7 +573,8 @@ class Renderer:
                          self.crec, main)
         main.wait_event(self._pf_done)
         if p.spec_pref > 0:
-            # the specular plane's post-filter uses the whole workspace: after the trace and the post-filter
+            # the specular plane's post-filter: after the post-filter, whose region it uses, and the trace (beside
+            # the trace on the side stream it saves 1%, as the trace leaves few registers for other blocks)
             if self.pp_spec is None:
                 self.pp_spec = torch.empty_like(self.pp)
             hdof_postfilter_spec(g, cam, lns, p, self.pp_spec, self.ws, main)

@@ -87,6 +87,33 @@ def test_postfilter_spec(orc, W, Hh, rmax, col_dtype):
     assert ref[..., 0].max() > 0.1
 
 
+@pytest.mark.parametrize("W,Hh", [(61, 47), (33, 18), (17, 130), (64, 5), (1, 9), (157, 33)])
+@pytest.mark.parametrize("nd_dtype,col_dtype", [(torch.float32, torch.float32), (torch.float32, torch.bfloat16),
+                                                (torch.float16, torch.float32), (torch.float16, torch.bfloat16)])
+@pytest.mark.parametrize("z0,slope", [(0.8, 0.002), (2.2, 0.012)])
+def test_postfilter_spec_equals_the_grey_plane(W, Hh, nd_dtype, col_dtype, z0, slope):
+    """The two-channel kernels against the plane (S, S, S) filtered as an FP32
+    colour: the same sums in the same order, so the same bits.  Near field
+    with an interior; a slant through the focus distance (both layers, and
+    each pixel's own prefix columns)."""
+    yy, xx = np.mgrid[0:Hh, 0:W].astype(np.float64)
+    nd = np.zeros((Hh, W, 4))
+    nd[..., 2], nd[..., 3] = -1.0, z0 + slope * xx + 0.001 * yy
+    col = np.random.default_rng(W).uniform(0.0, 3.0, (Hh, W, 4))
+    cam = hi.Camera(width=W, height=Hh).f32()
+    lens = hi.Lens(3.0, 18.0 * 2 * 0.57735 / (Hh * (1 / 0.8 - 1 / 3.0)), 0.05).f32()
+    p = hi.Params(r_max=32.0)
+    g = gbuf_from(nd, col, nd_dtype=nd_dtype, col_dtype=col_dtype)
+    grey = gbuf_from(nd, np.repeat(host(g.col.float())[..., 3:], 4, -1), nd_dtype=nd_dtype)
+    got = torch.empty((Hh, W, 4), dtype=torch.float32, device="cuda")
+    ref = torch.empty_like(got)
+    ws = workspace(W, Hh, p)
+    H.hdof_postfilter_spec(g, cam, lens, p, got, ws)
+    H.hdof_postfilter(grey, cam, lens, p, ref, ws)
+    H.hdof_sync()
+    assert torch.equal(got, ref), report("pp_spec", host(got), host(ref))
+
+
 def test_composite_spec(orc):
     W, Hh = 97, 61
     gb = hi.random_gbuffer(W, Hh, seed=3)
