@@ -823,7 +823,11 @@ __device__ __forceinline__ void resolve_body(const TraceArgs& a, int bx) {
     write_rt(a, q, s);
 }
 
-__global__ void __launch_bounds__(256) k_resolve(TraceArgs a) { resolve_body(a, blockIdx.x); }
+// Bound by the latency of the chain record, triangle, material of each sample,
+// so by the warps in flight: four resident blocks (64 registers) instead of the
+// two that 97 registers leave.  7.4M samples of a reference pass 121 to 92 us
+// (3 blocks 97, 5 with spills 113), a batch of twelve views 1340 to 1249 us.
+__global__ void __launch_bounds__(256, 4) k_resolve(TraceArgs a) { resolve_body(a, blockIdx.x); }
 
 // The same for images of at most RES_SMALL pixels, where a thread's serial
 // samples are the kernel's time: RES_LANES threads share a pixel, each shades
@@ -937,7 +941,7 @@ __global__ void __launch_bounds__(256) k_scatter_batch(const ScatterArgs* __rest
     g.locate(blockIdx.x, v, bx, by);
     scatter_body(batch_record(a, v), bx, by);
 }
-__global__ void __launch_bounds__(256) k_resolve_batch(const TraceArgs* __restrict__ a, BatchGrid g) {
+__global__ void __launch_bounds__(256, 4) k_resolve_batch(const TraceArgs* __restrict__ a, BatchGrid g) {
     int v, bx, by;
     g.locate(blockIdx.x, v, bx, by);
     resolve_body(batch_record(a, v), bx);
