@@ -69,18 +69,30 @@ __device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
 }
 
 // block sum of a per-thread (float, float), fixed order: pairs of floats
-// within a warp, double across the warps; thread 0 writes the block's partial
+// within a warp (doubles in a warp with a value that is not finite or that
+// could overflow the pairs), double across the warps; thread 0 writes the
+// block's partial
 __device__ __forceinline__ void block_partial(float2 v, double2* partial) {
     __shared__ double red[2][32];
-    Pair a{v.x, 0.f}, b{v.y, 0.f};
-    for (int o = 16; o; o >>= 1) {
-        a = pair_add(a, Pair{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)});
-        b = pair_add(b, Pair{__shfl_xor_sync(0xffffffffu, b.hi, o), __shfl_xor_sync(0xffffffffu, b.lo, o)});
-    }
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+    double da = v.x, db = v.y;
+    if (__any_sync(0xffffffffu, !(fabsf(v.x) < 1e36f) || !(fabsf(v.y) < 1e36f))) {
+        for (int o = 16; o; o >>= 1) {
+            da += __shfl_xor_sync(0xffffffffu, da, o);
+            db += __shfl_xor_sync(0xffffffffu, db, o);
+        }
+    } else {
+        Pair a{v.x, 0.f}, b{v.y, 0.f};
+        for (int o = 16; o; o >>= 1) {
+            a = pair_add(a, Pair{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)});
+            b = pair_add(b, Pair{__shfl_xor_sync(0xffffffffu, b.hi, o), __shfl_xor_sync(0xffffffffu, b.lo, o)});
+        }
+        da = (double)a.hi + (double)a.lo;
+        db = (double)b.hi + (double)b.lo;
+    }
     if (l == 0) {
-        red[0][w] = (double)a.hi + (double)a.lo;
-        red[1][w] = (double)b.hi + (double)b.lo;
+        red[0][w] = da;
+        red[1][w] = db;
     }
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -68,13 +68,17 @@ __device__ __forceinline__ void pair_add(Pair& s, float x, float x_lo = 0.f) {
 // sum d^2, max |d|] over all pixels, then the same over the region.  A thread
 // sums its few pixels as float pairs (each d^2 exactly, with its rounding
 // error), the block in double precision: 160 us in double throughout at
-// 1280x720 (with the final block), 29 so.
+// 1280x720 (with the final block), 32 so.  A difference whose square leaves
+// the range of a float pair (tiny, huge, infinite or NaN) is left to a second
+// loop, in double, that runs only where there is one.
 __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ a, const float4* __restrict__ b,
                                                      const uint8_t* __restrict__ region, int n_px,
                                                      float* __restrict__ err, double* __restrict__ part) {
     int cnt[2] = {0, 0};
     Pair s1[2] = {{0.f, 0.f}, {0.f, 0.f}}, s2[2] = {{0.f, 0.f}, {0.f, 0.f}};
     float mx[2] = {0.f, 0.f};
+    bool wide = false;
+    auto in_range = [](float d) { return d == 0.f || (d > 0x1p-50f && d < 0x1p50f); };
     for (int q = blockIdx.x * ERR_THREADS + threadIdx.x; q < n_px; q += ERR_BLOCKS * ERR_THREADS) {
         const float4 x = a[q], y = b[q];
         const float d[3] = {fabsf(x.x - y.x), fabsf(x.y - y.y), fabsf(x.z - y.z)};
@@ -86,9 +90,10 @@ __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ 
             ++cnt[r];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const float p = __fmul_rn(d[k], d[k]);
-                pair_add(s1[r], d[k]);
-                pair_add(s2[r], p, fmaf(d[k], d[k], -p));
+                wide |= !in_range(d[k]);
+                const float v = in_range(d[k]) ? d[k] : 0.f, p = __fmul_rn(v, v);
+                pair_add(s1[r], v);
+                pair_add(s2[r], p, fmaf(v, v, -p));
                 mx[r] = fmaxf(mx[r], d[k]);
             }
         }
@@ -96,6 +101,28 @@ __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ 
     // a warp in pairs of floats, then the eight warps in double, in a fixed order
     __shared__ double sh[8][ERR_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double w1[2] = {0.0, 0.0}, w2[2] = {0.0, 0.0};
+    if (__any_sync(0xffffffffu, wide)) {
+        for (int q = blockIdx.x * ERR_THREADS + threadIdx.x; q < n_px; q += ERR_BLOCKS * ERR_THREADS) {
+            const float4 x = a[q], y = b[q];
+            const float d[3] = {fabsf(x.x - y.x), fabsf(x.y - y.y), fabsf(x.z - y.z)};
+            for (int k = 0; k < 3; ++k) {
+                if (in_range(d[k])) continue;
+                const double v = d[k], vv = v * v;
+                w1[0] += v;
+                w2[0] += vv;
+                if (region && region[q]) {
+                    w1[1] += v;
+                    w2[1] += vv;
+                }
+            }
+        }
+        for (int o = 16; o; o >>= 1)
+            for (int r = 0; r < 2; ++r) {
+                w1[r] += __shfl_xor_sync(0xffffffffu, w1[r], o);
+                w2[r] += __shfl_xor_sync(0xffffffffu, w2[r], o);
+            }
+    }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         cnt[r] = __reduce_add_sync(0xffffffffu, cnt[r]);
@@ -108,8 +135,8 @@ __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ 
         }
         if (lane == 0) {
             sh[4 * r][w] = (double)cnt[r];
-            sh[4 * r + 1][w] = (double)s1[r].hi + (double)s1[r].lo;
-            sh[4 * r + 2][w] = (double)s2[r].hi + (double)s2[r].lo;
+            sh[4 * r + 1][w] = (double)s1[r].hi + (double)s1[r].lo + w1[r];
+            sh[4 * r + 2][w] = (double)s2[r].hi + (double)s2[r].lo + w2[r];
             sh[4 * r + 3][w] = (double)mx[r];
         }
     }

@@ -57,6 +57,35 @@ def test_reference_rt_room(orc):
     assert frac_close(got[..., :3], ref[..., :3], 1e-3) >= 0.999, report("rt", got[..., :3], ref[..., :3])
 
 
+@pytest.mark.parametrize("kind", ["tiny", "huge", "inf", "nan", "mixed"])
+@pytest.mark.parametrize("W,Hh", [(1, 1), (33, 7), (640, 411)])
+def test_error_map_over_the_float_range(kind, W, Hh):
+    """Differences whose squares underflow or overflow a float, infinite and
+    NaN ones, alone or among ordinary ones: the sums are double sums (relative
+    2^-40 for at most 800k positive terms of float pairs; infinities and NaN
+    as in double)."""
+    rng = np.random.default_rng(W)
+    b = np.zeros((Hh, W, 4), np.float32)
+    a = rng.uniform(0.0, 1.0, (Hh, W, 4)).astype(np.float32)
+    scale = {"tiny": 1e-30, "huge": 1e25, "inf": np.inf, "nan": np.nan, "mixed": 1e25}[kind]
+    if kind in ("tiny", "huge"):
+        a = (a * np.float32(scale)).astype(np.float32)
+    else:
+        a[Hh // 2, W // 3, 1] = scale
+        if kind == "mixed":
+            a[0, 0, 0] = 1e-30
+    region = (np.arange(W * Hh).reshape(Hh, W) % 2 == 0).astype(np.uint8)
+    stats = torch.empty(H.ERR_SCRATCH, dtype=torch.float64, device="cuda")
+    H.hdof_error_map(dev(a), dev(b), stats, region=dev(region))
+    H.hdof_sync()
+    got = host(stats)[:8]
+    d = np.abs(a[..., :3].astype(np.float64))
+    for k, x in ((0, d), (4, d[region > 0])):
+        ref = [x.size / 3, x.sum(), (x * x).sum(), np.fmax.reduce(x.ravel())]
+        assert got[k] == ref[0] and (got[k + 3] == ref[3] or kind == "nan")
+        np.testing.assert_allclose(got[k + 1:k + 3], ref[1:3], rtol=2.0 ** -40)
+
+
 def test_error_map_matches_numpy():
     rng = np.random.default_rng(0)
     W, Hh = 333, 77
