@@ -49,19 +49,19 @@ FALLBACK_HBM = 6800.0
 TRACE_VISITS_PER_RAY = 63.9
 TRACE_TESTS_PER_RAY = 6.3
 TRACE_OPS_PER_RAY = 28 * TRACE_VISITS_PER_RAY + 40 * TRACE_TESTS_PER_RAY
-# Post-filter gather, per executed (pixel, tap): squared distance (FMUL +
-# FFMA), soft weight (FADD.SAT), the source's layer (3 colour FFMA + 1 weight
-# FFMA) and, for far sources, the depth test (~1.5 on average); the square
-# root runs on the MUFU pipe and is not counted.  Per interior prefix lookup:
-# a float4 difference and accumulation (8 FADD).
-PF_OPS_PER_TAP = 8.5
-PF_OPS_PER_LOOKUP = 8
+# Post-filter gather, per executed (pixel, tap): its part of the distances (one
+# product and two sums per column and pair of rows, for eight pixel-taps), the
+# soft weight (FADD.SAT) and 3 colour FMAs + 1 weight FMA; the square root runs
+# on the MUFU pipe and is not counted.  Per prefix entry read: its part of the
+# difference and of its addition to the four pixels' sums.
+PF_OPS_PER_TAP = 5.4
+PF_OPS_PER_LOOKUP = 7
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum, one ncu
 # launch-list capture of the 1080p room frame, caches flushed before each launch)
 # of the current kernels; None where the kernel changed since the capture
 MEASURED_TRAFFIC = {
-    ("room", "f32", "trace_packets"): 18719232,
-    ("room", "f32", "pf_gather"): 120400384,
+    ("room", "f32", "trace_packets"): 18699008,
+    ("room", "f32", "pf_gather"): 122034176,
 }
 
 
@@ -199,10 +199,11 @@ def gather_work(z, lens, Hh, t, r_max):
     the kernel's own window rules: per 16x16 tile the reach R (largest r +
     1/2 of the tiles that reach it) and the interior radius R_in (smallest
     max(r_min(T) - 1/2, gap(T)) over the tiles that feed the near layer, used
-    when >= R/2); per 2x2-pixel thread and source row, the columns it taps
-    (interior columns of all four pixels skipped) and its prefix lookups (two
-    per pixel row with an interior).  Returns (tap iterations, each of four
-    pixel-taps, prefix lookups)."""
+    when >= R/2); per 2x2-pixel thread and pair of source rows (s above the
+    block, s below it), the columns it taps, in whole pairs, and the prefix
+    entries it reads: two a row for the columns inside all four pixels'
+    interiors, or two a pixel and row where a row of the window weighs more
+    than 8.  Returns (tap iterations, each of four pixel-taps, prefix reads)."""
     H, W = z.shape
     c = lens.aperture_radius * Hh * (lens.focus_dist - z) / (z * lens.focus_dist * t)
     r = np.minimum(np.abs(c) * 0.5, r_max)
@@ -219,7 +220,16 @@ def gather_work(z, lens, Hh, t, r_max):
     kt = math.ceil((r_max + 0.5) / TP) + 1
     offs = np.arange(-kt, kt + 1)
     gap = np.where(offs == 0, 0.0, (np.abs(offs) - 1) * TP + 1.0)
+    # a row's sum of near weights w / area(r)
+    o = np.arange(-130, 131, dtype=np.float64)
+    rad = np.sort(np.hypot(o[:, None], o[None, :]).ravel())
+    cum = np.concatenate([[0.0], np.cumsum(rad)])
+    grid = np.arange(0.0, 128.0, 1.0 / 64)
+    full, part = np.searchsorted(rad, grid - 0.5, "right"), np.searchsorted(rad, grid + 0.5, "left")
+    area = full + (grid + 0.5) * (part - full) - (cum[part] - cum[full])
+    row_w = (wn / np.interp(r, grid, area)).sum(1)
     th = np.arange(64)
+    Wp = (W + 1) & ~1
     taps = pre = 0
     for ty in range(nty):
         for tx in range(ntx):
@@ -239,21 +249,26 @@ def gather_work(z, lens, Hh, t, r_max):
             i, j = tx * TP + 2 * (th & 7), ty * TP + 2 * (th >> 3)
             ok = (i < W) & (j < H)
             i, j = i[ok][:, None], j[ok][:, None]
-            dy = np.arange(-G, G + 2, dtype=np.float64)[None, :]
-            rows = (j + dy >= 0) & (j + dy < H)
-            d0, d1 = dy ** 2, (dy - 1) ** 2
-            dmin = np.where((dy >= 0) & (dy <= 1), 0.0, np.minimum(d0, d1))
-            w = np.floor(np.sqrt(np.maximum(R * R - dmin, 0.0)) + 1e-3).astype(np.int64)
-            x0, x1 = np.maximum(i - w, 0), np.minimum(i + 1 + w, W - 1)
+            s = np.arange(0, G + 1)[None, :]
+            rows = (j - s >= 0).astype(np.int64) + (j + 1 + s < H)
+            w = np.floor(np.sqrt(np.maximum(R * R - s * s, 0.0)) + 1e-3).astype(np.int64)
+            x0, x1 = np.maximum(i - w, 0) & ~1, np.minimum(i + 1 + w, W - 1) | 1
             span = x1 - x0 + 1
             if Rin >= 0:
-                R2 = Rin * Rin
-                w0 = np.where(d0 <= R2, np.floor(np.sqrt(np.maximum(R2 - d0, 0.0))), -1).astype(np.int64)
-                w1 = np.where(d1 <= R2, np.floor(np.sqrt(np.maximum(R2 - d1, 0.0))), -1).astype(np.int64)
-                wm = np.minimum(w0, w1)
-                ls, rs = np.minimum(x1, i - wm), np.maximum(x0, i + wm + 1)
-                span = np.where(wm >= 1, np.maximum(ls - x0 + 1, 0) + np.maximum(x1 - rs + 1, 0), span)
-                pre += int((((w0 >= 0).astype(np.int64) + (w1 >= 0)) * 2 * rows).sum())
+                wn_ = np.floor(np.sqrt(np.maximum(Rin * Rin - s * s, 0.0))).astype(np.int64)
+                wf_ = np.floor(np.sqrt(np.maximum(Rin * Rin - (s + 1) ** 2, 0.0))).astype(np.int64)
+                n_in, f_in = (s * s <= Rin * Rin).astype(np.int64), ((s + 1) ** 2 <= Rin * Rin).astype(np.int64)
+                if (row_w[max(ty * TP - G, 0):min(ty * TP + TP - 1 + G, H - 1) + 1] > 8.0).any():
+                    ls = np.maximum(np.minimum(x1 + 1, (i + 2 - wf_) & ~1), x0)
+                    rs = np.minimum(((i + wf_ + 1) & ~1) - 1, x1)
+                    use = (f_in > 0) & (wf_ >= 2)
+                    pre += int((4 * (n_in + f_in) * rows).sum())
+                else:
+                    ls = (np.maximum(i + 1 - wf_, 0) + 1) & ~1
+                    rs = np.where(i + wf_ >= W - 1, Wp - 1, ((i + wf_ + 1) & ~1) - 1)
+                    use = (f_in > 0) & (rs - ls + 1 >= 4)
+                    pre += int((2 * use * rows).sum())
+                span = np.where(use, np.maximum(ls - x0, 0) + np.maximum(x1 - rs, 0), span)
             taps += int((span * rows).sum())
     return taps, pre
 
@@ -490,7 +505,8 @@ def quality(H, bvh, r, cam, lens, p, passes, block=8):
         smb = H.error_summary(stats)
         res[name] = {part: {k: (round(v, 6) if isinstance(v, float) else v) for k, v in sm[part].items()}
                      for part in ("all", "region")}
-        res[name][f"block{block}_region_mae"] = round(smb["region"]["mae"], 6)
+        if smb["region"]["pixels"]:  # none where no block is traced by half
+            res[name][f"block{block}_region_mae"] = round(smb["region"]["mae"], 6)
     return res
 
 
@@ -510,9 +526,9 @@ def quality_variants(H, bvh, W, Hh, lens, p0, dev, flush, frames, passes):
                           flush, static=not moving)[0]
         last = frames - 1
         q = quality(H, bvh, r, cams[last], lens, p.replace(frame=last, camera_moved=int(moving)), passes)
-        out[name] = {"hybrid_block8_mae": q["hybrid_vs_rt"]["block8_region_mae"],
-                     "pp_block8_mae": q["pp_vs_rt"]["block8_region_mae"],
-                     "hybrid_mae": q["hybrid_vs_rt"]["region"]["mae"], "pp_mae": q["pp_vs_rt"]["region"]["mae"]}
+        out[name] = {"hybrid_block8_mae": q["hybrid_vs_rt"].get("block8_region_mae"),
+                     "pp_block8_mae": q["pp_vs_rt"].get("block8_region_mae"),
+                     "hybrid_mae": q["hybrid_vs_rt"]["region"].get("mae"), "pp_mae": q["pp_vs_rt"]["region"].get("mae")}
         del r
     return out
 
