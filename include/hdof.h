@@ -247,7 +247,10 @@ int hdof_gbuffer(const hdof_bvh* bvh, const hdof_camera* cam, const hdof_camera*
  * p->spp_max: 13 bytes per possible ray (pixel, sample index, record).  The
  * post-filter's region is disjoint from the mask's and the trace's, so
  * hdof_postfilter may run on another stream concurrently with hdof_mask and
- * hdof_trace once hdof_gbuffer has finished. */
+ * hdof_trace once hdof_gbuffer has finished.  This buffer, like the one of
+ * hdof_post_workspace_bytes below, starts at a multiple of 16 bytes; where a
+ * call needs more, it rounds up inside the buffer (the size returned has room
+ * for that). */
 size_t hdof_workspace_bytes(int32_t width, int32_t height, const hdof_params* p);
 
 /* ----------------------------------------------------------- mask -- */

@@ -882,7 +882,9 @@ struct BwdWs {
     size_t bytes;
 };
 
+// regions from the first multiple of PF_ALIGN at or after base (a null base: the size)
 BwdWs bwd_layout(int W, int H, char* base) {
+    if (base) base = align_up(base, PF_ALIGN);
     BwdWs b{};
     size_t px = (size_t)W * H, o = 0;
     auto take = [&](size_t n) {
@@ -901,7 +903,7 @@ BwdWs bwd_layout(int W, int H, char* base) {
     int n1 = ((W + 31) / 32) * ((H + 7) / 8), n2 = ((W + 15) / 16) * ((H + 15) / 16);
     b.n_partial = 2 * n1 + n2;
     b.partial = reinterpret_cast<double2*>(take(16 * (size_t)b.n_partial));
-    b.bytes = o;
+    b.bytes = o + PF_ALIGN;
     return b;
 }
 

@@ -70,10 +70,13 @@ struct ViewWs {
     float* zq;           // post-filter view depth per pixel
     float4* tmax;        // post-filter per-tile radii (largest near, largest far, smallest near)
     float4* pre;         // post-filter row prefix of the near records (row-major)
+    char* bokeh;         // shaped post-filter: its tables (bokeh_scratch_bytes)
 };
 
-// the post-filter regions, laid out from `pf` (ws_layout(...).pf bytes)
+// the post-filter regions, laid out from the first multiple of PF_ALIGN at or
+// after `pf` (ws_layout(...).pf bytes)
 inline void pf_regions(ViewWs& w, char* pf, const WsLayout& L) {
+    pf = align_up(pf, PF_ALIGN);
     size_t f = 0;
     w.nrec = reinterpret_cast<float4*>(pf + f);
     w.frec = reinterpret_cast<float4*>(pf + (f += L.pf_nrec));
@@ -81,6 +84,7 @@ inline void pf_regions(ViewWs& w, char* pf, const WsLayout& L) {
     w.zq = reinterpret_cast<float*>(pf + (f += L.pf_rh));
     w.tmax = reinterpret_cast<float4*>(pf + (f += L.pf_zq));
     w.pre = reinterpret_cast<float4*>(pf + (f += L.pf_tiles));
+    w.bokeh = pf + (f += L.pf_pre);
 }
 
 inline ViewWs view_ws(const hdof_view& v) {

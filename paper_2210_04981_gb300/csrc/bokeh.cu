@@ -425,12 +425,11 @@ int launch_bokeh(const hdof_gbuf* in, const Coc& coc, const hdof_params* p, floa
     const WsLayout L = ws_layout(W, H, p);
     ViewWs w = {};
     pf_regions(w, static_cast<char*>(scratch), L);
-    char* extra = static_cast<char*>(scratch) + L.pf - L.pf_bokeh;
     const int K = (int)std::ceil(p->r_max + 0.5f) + 1;
     const int n_r = (int)(p->r_max / AREA_STEP) + 2;
-    float* D = reinterpret_cast<float*>(extra);
-    float* area = reinterpret_cast<float*>(extra + (((size_t)(2 * K + 1) * (2 * K + 1) * sizeof(float) + 255) &
-                                                    ~size_t(255)));
+    float* D = reinterpret_cast<float*>(w.bokeh);
+    float* area = reinterpret_cast<float*>(w.bokeh + (((size_t)(2 * K + 1) * (2 * K + 1) * sizeof(float) + 255) &
+                                                      ~size_t(255)));
     float4* pt = reinterpret_cast<float4*>(reinterpret_cast<char*>(area) +
                                            (((size_t)n_r * sizeof(float) + 255) & ~size_t(255)));
     Shape sh{K, D, p->aberration};

@@ -66,6 +66,14 @@ int sm_count();
 // hdof_sync reads and clears it), for the current device.  NULL on error.
 unsigned* status_ptr();
 
+// A caller's workspace may start at any multiple of 16 bytes.  The post-filter
+// and the adjoint load pairs of records of 32 bytes: their regions start at
+// the next multiple of this, and the sizes have room for it.
+constexpr size_t PF_ALIGN = 256;
+inline char* align_up(void* p, size_t a) {
+    return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(p) + a - 1) & ~(uintptr_t)(a - 1));
+}
+
 // workspace layout (bytes) for a width x height frame
 struct WsLayout {
     size_t mask_tiles;      // uint8 per mask tile
@@ -83,8 +91,8 @@ struct WsLayout {
     size_t pf_zq;           // float per pixel: view depth
     size_t pf_tiles;        // float4 per 16x16 tile: largest r near, far; smallest r near
     size_t pf_pre;          // float4 per pixel: row-major inclusive row prefix of the near records
-    size_t pf_bokeh;        // shaped bokeh: aperture-norm and lattice-area tables (at the end of the region)
-    size_t pf;              // sum of the post-filter regions (laid out in this order)
+    size_t pf_bokeh;        // shaped bokeh: aperture-norm and lattice-area tables
+    size_t pf;              // the post-filter regions (laid out in this order) and their alignment
     size_t pf_off;          // where the post-filter regions start: after the mask and trace regions, so
                             // the post-filter can run concurrently with them
     size_t total;

@@ -895,7 +895,7 @@ extern "C" int hdof_postfilter_spec(const hdof_gbuf* in, const hdof_camera* cam,
     HDOF_CHECK_ARG(workspace && workspace_bytes >= L.total, "hdof_postfilter_spec: workspace of %zu bytes < %zu",
                    workspace_bytes, L.total);
     // the shaped post-filter's grey plane sits below the post-filter's region (the mask and trace
-    // scratch, at least 16 bytes per pixel since spp_max >= 1)
+    // scratch, at least 16 bytes per pixel since spp_max >= 1; 16-byte accesses only)
     const size_t n = (size_t)in->width * in->height;
     HDOF_CHECK_ARG(n * sizeof(float4) <= L.pf_off, "hdof_postfilter_spec: no room for the specular plane");
     cudaStream_t s = as_stream(stream);
