@@ -95,7 +95,7 @@ typedef struct hdof_params {
     float light_dir[4][3]; /* unit vectors towards the lights */
     float light_E[4];
     float miss_dist;     /* far position of a ray that hits nothing */
-    int32_t trav_cap;    /* traversal step watchdog; 0 = default (64 x nodes) */
+    int32_t trav_cap;    /* traversal step watchdog; 0 = default (64 x (nodes + triangles), below 2^31) */
     /* temporal reconstruction (Reconstruction section) */
     float ema_alpha;
     int32_t camera_moved; /* compose with this frame's hit ratio */

@@ -1022,7 +1022,7 @@ extern "C" int hdof_closest_hits(const hdof_bvh* b, int32_t n, const float* org,
     HDOF_CHECK_ARG(org && dir && ids && ts, "hdof_closest_hits: NULL buffer");
     unsigned* st = status_ptr();
     HDOF_CHECK_ARG(st, "hdof_closest_hits: no status word on this device");
-    int cap = 64 * (b->n_nodes + b->n_tris) + 64;
+    const int cap = step_cap(0, b->n_nodes, b->n_tris);
     k_closest<<<blocks_for(n, 128), 128, 0, as_stream(stream)>>>(b->view(), n, org, dir, cap, st, ids, ts);
     HDOF_LAUNCHED("hdof_closest_hits");
     return HDOF_OK;

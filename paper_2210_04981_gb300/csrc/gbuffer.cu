@@ -95,7 +95,7 @@ GbufArgs<ND, COL> gbuf_args(const hdof_bvh* b, const hdof_camera* cam, const hdo
     a.prev = make_cam(*prev);
     a.L = make_lights(*p);
     a.miss_dist = p->miss_dist;
-    a.cap = p->trav_cap > 0 ? p->trav_cap : 64 * (b->n_nodes + b->n_tris) + 64;
+    a.cap = step_cap(p->trav_cap, b->n_nodes, b->n_tris);
     a.status = st;
     a.nd = static_cast<ND*>(g->nd);
     a.col = static_cast<COL*>(g->col);

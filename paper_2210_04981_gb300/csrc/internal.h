@@ -10,6 +10,7 @@
 
 #include "../../include/hdof.h"
 #include "common.cuh"
+#include "step_cap.h"
 
 namespace hdof {
 

@@ -909,7 +909,7 @@ TraceArgs trace_args(const hdof_bvh* b, const hdof_camera* cam, const hdof_lens*
     a.blade_rot = p->blade_rot;
     a.aberration = p->aberration;
     a.key = trace_key(*p);
-    a.cap = p->trav_cap > 0 ? p->trav_cap : 64 * (b->n_nodes + b->n_tris) + 64;
+    a.cap = step_cap(p->trav_cap, b->n_nodes, b->n_tris);
     a.smax = p->spp_max;
     a.packets = packet_view(*lens, *cam) ? 1 : 0;
     a.binned = binned_view(*lens, *cam) ? 1 : 0;
