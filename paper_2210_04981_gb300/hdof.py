@@ -202,12 +202,7 @@ def _stream(stream):
 
 # ------------------------------------------------------------ records ----
 
-# Each of these takes its C record as it is: a caller that makes several calls
-# with the same records (a frame) marshals them once.
-
 def camera(c) -> hdof_camera:
-    if isinstance(c, hdof_camera):
-        return c
     o = hdof_camera()
     o.pos[:] = list(c.pos)
     o.right[:] = list(c.right)
@@ -220,8 +215,6 @@ def camera(c) -> hdof_camera:
 
 
 def lens(l) -> hdof_lens:
-    if isinstance(l, hdof_lens):
-        return l
     return hdof_lens(l.focus_dist, l.aperture_radius, l.focal_length)
 
 
@@ -234,8 +227,6 @@ _PARAM_NAMES = ("gauss_sigma", "edge_tau", "tile", "dilate", "spp_max", "varianc
 def params(p=None) -> hdof_params:
     """Marshal a parameter record (attributes named as the C fields; light
     directions are normalised here); None gives the library defaults."""
-    if isinstance(p, hdof_params):
-        return p
     o = hdof_params()
     load().hdof_default_params(C.byref(o))
     if p is None:
@@ -250,6 +241,15 @@ def params(p=None) -> hdof_params:
         o.light_dir[k][:] = [float(x) / n for x in d]
         o.light_E[k] = float(e)
     return o
+
+
+class _Ready:
+    """A C record that is marshalled already, for a caller of its own that
+    makes several calls with it (a frame)."""
+    __slots__ = ("rec",)
+
+    def __init__(self, rec):
+        self.rec = rec
 
 
 # ------------------------------------------------------------- buffers ---
@@ -299,12 +299,24 @@ class History:
         self.hlen.zero_()
 
 
+def _camera(c) -> hdof_camera:
+    return c.rec if type(c) is _Ready else camera(c)
+
+
+def _lens(l) -> hdof_lens:
+    return l.rec if type(l) is _Ready else lens(l)
+
+
+def _params(p) -> hdof_params:
+    return p.rec if type(p) is _Ready else params(p)
+
+
 def _gbuf(g) -> hdof_gbuf:
-    return g if isinstance(g, hdof_gbuf) else g.struct()
+    return g.rec if type(g) is _Ready else g.struct()
 
 
 def _hist(h) -> hdof_history:
-    return h if isinstance(h, hdof_history) else h.struct()
+    return h.rec if type(h) is _Ready else h.struct()
 
 
 class Bvh:
@@ -380,28 +392,28 @@ def hdof_closest_hits(bvh: Bvh, org, dirs, ids, ts, stream=None):
 def hdof_gbuffer(bvh: Bvh, cam, prev, p, gbuf: GBuffer, stream=None, hint=None):
     """hint (int32 [H][W], e.g. the previous frame's tri plane, possibly
     gbuf.tri itself) optionally seeds each primary ray with a likely hit."""
-    _check(load().hdof_gbuffer(bvh.handle, C.byref(camera(cam)), C.byref(camera(prev)), C.byref(params(p)),
+    _check(load().hdof_gbuffer(bvh.handle, C.byref(_camera(cam)), C.byref(_camera(prev)), C.byref(_params(p)),
                                _ptr(hint), C.byref(_gbuf(gbuf)), _stream(stream)))
 
 
 def hdof_mask(gbuf: GBuffer, prev_hist, p, edge, spp, workspace, stream=None):
-    hs = C.byref(_hist(prev_hist)) if prev_hist is not None else None
-    _check(load().hdof_mask(C.byref(_gbuf(gbuf)), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
+    hs = C.byref(prev_hist.struct()) if prev_hist is not None else None
+    _check(load().hdof_mask(C.byref(gbuf.struct()), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
                             _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def hdof_mask_coc(gbuf: GBuffer, prev_hist, cam, lns, p, edge, spp, workspace, stream=None):
     """hdof_mask whose edge tiles reach their pixels' largest CoC radius when p.mask_coc = 1."""
     _check(load().hdof_mask_coc(C.byref(_gbuf(gbuf)), C.byref(_hist(prev_hist)) if prev_hist is not None else None,
-                                C.byref(camera(cam)), C.byref(lens(lns)), C.byref(params(p)), _ptr(edge), _ptr(spp),
+                                C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)), _ptr(edge), _ptr(spp),
                                 _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def hdof_mask_noalloc(gbuf: GBuffer, prev_hist, p, edge, spp, stream=None):
     """hdof_mask for callers that cannot give the library device memory: the
     tile flags live in a fixed array inside the library (see include/hdof.h)."""
-    hs = C.byref(_hist(prev_hist)) if prev_hist is not None else None
-    _check(load().hdof_mask_noalloc(C.byref(_gbuf(gbuf)), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
+    hs = C.byref(prev_hist.struct()) if prev_hist is not None else None
+    _check(load().hdof_mask_noalloc(C.byref(gbuf.struct()), hs, C.byref(params(p)), _ptr(edge), _ptr(spp),
                                     _stream(stream)))
 
 
@@ -412,7 +424,7 @@ def hdof_trace(bvh: Bvh, cam, lns, p, spp, rt, stats, workspace, stream=None, re
     hint (int32 [H][W], the G-buffer's tri plane) optionally seeds each lens
     ray with its pixel's primary hit; tune (hdof_tuning) optionally fixes the
     trace's form and block size (default: chosen from the lens)."""
-    _check(load().hdof_trace(bvh.handle, C.byref(camera(cam)), C.byref(lens(lns)), C.byref(params(p)),
+    _check(load().hdof_trace(bvh.handle, C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)),
                              _ptr(spp), _ptr(hint), _ptr(rt), _ptr(stats), _ptr(rec), _ptr(ray_off), _ptr(workspace),
                              workspace.numel() * workspace.element_size(),
                              C.byref(tune) if tune is not None else None, _stream(stream)))
@@ -460,36 +472,36 @@ def error_summary(stats) -> dict:
 
 
 def hdof_postfilter(gbuf: GBuffer, cam, lns, p, pp, workspace, stream=None):
-    _check(load().hdof_postfilter(C.byref(_gbuf(gbuf)), C.byref(camera(cam)), C.byref(lens(lns)),
-                                  C.byref(params(p)), _ptr(pp), _ptr(workspace),
+    _check(load().hdof_postfilter(C.byref(_gbuf(gbuf)), C.byref(_camera(cam)), C.byref(_lens(lns)),
+                                  C.byref(_params(p)), _ptr(pp), _ptr(workspace),
                                   workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def hdof_reconstruct(rt, gbuf: GBuffer, spp, cam, prev, lns, p, hist_in: History, hist_out: History, crt, hacc,
                      crec, stream=None):
-    _check(load().hdof_reconstruct(_ptr(rt), C.byref(_gbuf(gbuf)), _ptr(spp), C.byref(camera(cam)),
-                                   C.byref(camera(prev)), C.byref(lens(lns)), C.byref(params(p)),
+    _check(load().hdof_reconstruct(_ptr(rt), C.byref(_gbuf(gbuf)), _ptr(spp), C.byref(_camera(cam)),
+                                   C.byref(_camera(prev)), C.byref(_lens(lns)), C.byref(_params(p)),
                                    C.byref(_hist(hist_in)), C.byref(_hist(hist_out)), _ptr(crt), _ptr(hacc),
                                    _ptr(crec), _stream(stream)))
 
 
 def hdof_composite(gbuf: GBuffer, spp, pp, crt, crec, hacc, cam, lns, p, out, stream=None):
     _check(load().hdof_composite(C.byref(_gbuf(gbuf)), _ptr(spp), _ptr(pp), _ptr(crt), _ptr(crec), _ptr(hacc),
-                                 C.byref(camera(cam)), C.byref(lens(lns)), C.byref(params(p)), _ptr(out),
+                                 C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)), _ptr(out),
                                  _stream(stream)))
 
 
 def hdof_postfilter_spec(gbuf: GBuffer, cam, lns, p, pp_spec, workspace, stream=None):
     """Post-filter of the specular plane col.w: pp_spec [H,W,4] = (S_pp x3, alpha)."""
-    _check(load().hdof_postfilter_spec(C.byref(_gbuf(gbuf)), C.byref(camera(cam)), C.byref(lens(lns)),
-                                       C.byref(params(p)), _ptr(pp_spec), _ptr(workspace),
+    _check(load().hdof_postfilter_spec(C.byref(_gbuf(gbuf)), C.byref(_camera(cam)), C.byref(_lens(lns)),
+                                       C.byref(_params(p)), _ptr(pp_spec), _ptr(workspace),
                                        workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def hdof_composite_spec(gbuf: GBuffer, spp, pp, pp_spec, crt, crec, hacc, cam, lns, p, out, stream=None):
     _check(load().hdof_composite_spec(C.byref(_gbuf(gbuf)), _ptr(spp), _ptr(pp),
                                       _ptr(pp_spec) if pp_spec is not None else None, _ptr(crt), _ptr(crec),
-                                      _ptr(hacc), C.byref(camera(cam)), C.byref(lens(lns)), C.byref(params(p)),
+                                      _ptr(hacc), C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)),
                                       _ptr(out), _stream(stream)))
 
 
@@ -558,8 +570,9 @@ class Renderer:
         main.wait_event(self._start)
         # the frame's records, marshalled once for its six calls: a 128x128 frame, whose kernels are
         # shorter than the host's work on it, takes 121 us so and 156 with each call marshalling its own
-        cam, prev, lns, p, g = camera(cam), camera(prev), lens(lns), params(p), self.g.struct()
-        hin, hout = self.hist[self.cur].struct(), self.hist[1 - self.cur].struct()
+        spec_pref = p.spec_pref
+        cam, prev, lns, p, g = map(_Ready, (camera(cam), camera(prev), lens(lns), params(p), self.g.struct()))
+        hin, hout = _Ready(self.hist[self.cur].struct()), _Ready(self.hist[1 - self.cur].struct())
         hdof_gbuffer(self.bvh, cam, prev, p, g, main, hint=self.g.tri)
         # the post-filter on the side stream, after the G-buffer (it touches only
         # the workspace's post-filter region)
@@ -572,7 +585,7 @@ class Renderer:
         hdof_reconstruct(self.rt, g, self.spp, cam, prev, lns, p, hin, hout, self.crt, self.hacc,
                          self.crec, main)
         main.wait_event(self._pf_done)
-        if p.spec_pref > 0:
+        if spec_pref > 0:
             # the specular plane's post-filter: after the post-filter, whose region it uses, and the trace (beside
             # the trace on the side stream it saves 1%, as the trace leaves few registers for other blocks)
             if self.pp_spec is None:
