@@ -16,6 +16,7 @@
 // final block), the pixel count, sum of |d|, sum of d^2 (per channel) and
 // max |d| over all pixels and over a region.
 #include "internal.h"
+#include "sum3.cuh"
 
 namespace hdof {
 namespace {
@@ -50,32 +51,19 @@ __global__ void __launch_bounds__(256) k_rt_accum(const float4* __restrict__ rt,
     out[q] = o;
 }
 
-// A sum carried as an unevaluated pair of floats (Knuth's TwoSum): 48 bits, at
-// FP32 rates (FP64 adds run at 1/64 of them here).
-struct Pair {
-    float hi, lo;
-};
-__device__ __forceinline__ Pair two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-__device__ __forceinline__ void pair_add(Pair& s, float x, float x_lo = 0.f) {
-    const Pair t = two_sum(s.hi, x);
-    s = two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(s.lo, x_lo)));
-}
-
 // per pixel: err = mean over rgb of |a - b|; per block: [count, sum |d|,
 // sum d^2, max |d|] over all pixels, then the same over the region.  A thread
-// sums its few pixels as float pairs (each d^2 exactly, with its rounding
-// error), the block in double precision: 160 us in double throughout at
-// 1280x720 (with the final block), 32 so.  A difference whose square leaves
-// the range of a float pair (tiny, huge, infinite or NaN) is left to a second
-// loop, in double, that runs only where there is one.
+// sums its few pixels, and a warp its threads, in three floats (Sum3: more
+// bits than a double; each d^2 exactly, with its rounding error), the block in
+// double precision: 160 us in double throughout at 1280x720 (with the final
+// block), 34 so.  A difference whose square's rounding error leaves the range
+// of a float (tiny, huge, infinite or NaN) is left to a second loop, in
+// double, that runs only where there is one.
 __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ a, const float4* __restrict__ b,
                                                      const uint8_t* __restrict__ region, int n_px,
                                                      float* __restrict__ err, double* __restrict__ part) {
     int cnt[2] = {0, 0};
-    Pair s1[2] = {{0.f, 0.f}, {0.f, 0.f}}, s2[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    Sum3 s1[2] = {}, s2[2] = {};
     float mx[2] = {0.f, 0.f};
     bool wide = false;
     auto in_range = [](float d) { return d == 0.f || (d > 0x1p-50f && d < 0x1p50f); };
@@ -92,13 +80,13 @@ __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ 
             for (int k = 0; k < 3; ++k) {
                 wide |= !in_range(d[k]);
                 const float v = in_range(d[k]) ? d[k] : 0.f, p = __fmul_rn(v, v);
-                pair_add(s1[r], v);
-                pair_add(s2[r], p, fmaf(v, v, -p));
+                s1[r].add(v);
+                s2[r].add(p, fmaf(v, v, -p));
                 mx[r] = fmaxf(mx[r], d[k]);
             }
         }
     }
-    // a warp in pairs of floats, then the eight warps in double, in a fixed order
+    // a warp in three floats, then the eight warps in double, in a fixed order
     __shared__ double sh[8][ERR_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double w1[2] = {0.0, 0.0}, w2[2] = {0.0, 0.0};
@@ -127,16 +115,14 @@ __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ 
     for (int r = 0; r < 2; ++r) {
         cnt[r] = __reduce_add_sync(0xffffffffu, cnt[r]);
         for (int o = 16; o; o >>= 1) {
-            const Pair u{__shfl_xor_sync(0xffffffffu, s1[r].hi, o), __shfl_xor_sync(0xffffffffu, s1[r].lo, o)};
-            const Pair v{__shfl_xor_sync(0xffffffffu, s2[r].hi, o), __shfl_xor_sync(0xffffffffu, s2[r].lo, o)};
-            pair_add(s1[r], u.hi, u.lo);
-            pair_add(s2[r], v.hi, v.lo);
+            s1[r].add(shfl_xor(s1[r], o));
+            s2[r].add(shfl_xor(s2[r], o));
             mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], o));
         }
         if (lane == 0) {
             sh[4 * r][w] = (double)cnt[r];
-            sh[4 * r + 1][w] = (double)s1[r].hi + (double)s1[r].lo + w1[r];
-            sh[4 * r + 2][w] = (double)s2[r].hi + (double)s2[r].lo + w2[r];
+            sh[4 * r + 1][w] = s1[r].value() + w1[r];
+            sh[4 * r + 2][w] = s2[r].value() + w2[r];
             sh[4 * r + 3][w] = (double)mx[r];
         }
     }

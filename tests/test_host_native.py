@@ -2,6 +2,9 @@
 host compiler alone."""
 import os
 import subprocess
+from fractions import Fraction
+
+import numpy as np
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2210_04981_gb300", "csrc")
@@ -28,3 +31,44 @@ def test_step_cap_of_large_trees(tmp_path):
     # every call takes its cap from there
     for f in ("trace.cu", "gbuffer.cu", "bvh.cu"):
         assert open(os.path.join(CSRC, f)).read().count("step_cap(") == 1
+
+
+def test_three_float_sums(tmp_path):
+    """Sum3 against the exact sum: its value is within one rounding of a double
+    (2^-52 of the sum of magnitudes leaves room for the last addition too),
+    term by term, with rounding errors handed in, and over a tree of partial
+    sums, where a pair of floats would drop what lies 2^-48 below."""
+    rng = np.random.default_rng(0)
+    sets = [np.float32([1.0, 2.0 ** -25, 2.0 ** -49]), np.float32([1.0, 2.0 ** -25, 2.0 ** -28, -1.0, -2.0 ** -25]),
+            rng.uniform(0, 1, 96).astype(np.float32), rng.normal(size=400).astype(np.float32),
+            (rng.normal(size=400) * np.exp2(rng.uniform(-30, 30, 400))).astype(np.float32)]
+    src = """#include <cstdio>
+#include "sum3.cuh"
+int main() {
+    int n;
+    while (scanf("%d", &n) == 1) {
+        hdof::Sum3 s{}, part[32] = {}, sq{};
+        for (int k = 0; k < n; ++k) {
+            float x;
+            scanf("%a", &x);
+            s.add(x);
+            part[k % 32].add(x);
+            const double d = (double)x * x;
+            const float p = (float)d;
+            sq.add(p, (float)(d - p));
+        }
+        for (int o = 16; o; o >>= 1) {
+            hdof::Sum3 t[32];
+            for (int k = 0; k < 32; ++k) { t[k] = part[k]; t[k].add(part[k ^ o]); }
+            for (int k = 0; k < 32; ++k) part[k] = t[k];
+        }
+        printf("%a %a %a\\n", s.value(), part[0].value(), sq.value());
+    }
+}"""
+    got = _run(tmp_path, src, "\n".join(f"{len(x)} " + " ".join(float(v).hex() for v in x) for x in sets))
+    for x, g in zip(sets, np.reshape([float.fromhex(v) for v in got], (-1, 3))):
+        ex = [Fraction(float(v)) for v in x]
+        for k, terms in ((0, ex), (1, ex), (2, [v * v for v in ex])):
+            assert abs(Fraction(float(g[k])) - sum(terms)) <= Fraction(1, 2 ** 52) * sum(map(abs, terms)), (k, len(x))
+    # where a double is exact, so is the sum
+    assert float.fromhex(got[0]) == 1.0 + 2.0 ** -25 + 2.0 ** -49 and float.fromhex(got[4]) == 2.0 ** -28
