@@ -246,23 +246,25 @@ constexpr int BGT = 64;          // threads of a group: 2x2 pixels each
 
 struct BokehAcc {
     float2 xy, zw;  // (S.x, S.y), (S.z, W)
-    float kb;       // far: 1 / (kz_rel z_p)
+    float zp, kb;   // far: the depth z_p and 1 / (kz_rel z_p)
 };
 
 // One source into the thread's 2x2 pixels.  Row k's left pixel sees it at
 // norm D[k] and squared distance d2[k], its right pixel at the previous
-// column's, carried in cD and cd2.
+// column's, carried in cD and cd2.  The far layer's depth test is
+// clamp(1 - (z - z_p) kb): the difference is exact near z_p, where
+// (1 + 1 / kz_rel) - z kb would cancel to 2^-24 / kz_rel.
 template <bool NEAR, bool RAD>
 __device__ __forceinline__ void bk_tap(BokehAcc (&a)[4], float (&cD)[2], float (&cd2)[2], const float (&D)[2],
                                        const float (&d2)[2], float rh, float ir2, float z, float c1, float c0r,
-                                       float ka, const float4& e) {
+                                       const float4& e) {
     const float c0 = RAD ? (ir2 > 0.f ? c0r : 1.f) : 1.f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float Dk = (k & 1) ? cD[k >> 1] : D[k >> 1], dd = (k & 1) ? cd2[k >> 1] : d2[k >> 1];
         float w = __saturatef(rh - Dk);
         if (RAD) w *= fmaf(c1, __saturatef(dd * ir2), c0);
-        if (!NEAR) w *= __saturatef(fmaf(-z, a[k].kb, ka));
+        if (!NEAR) w *= __saturatef(fmaf(a[k].zp - z, a[k].kb, 1.f));
         a[k].xy = fma2(w, e.x, e.y, a[k].xy);
         a[k].zw = fma2(w, e.z, e.w, a[k].zw);
     }
@@ -277,7 +279,7 @@ __device__ __forceinline__ void bk_tap(BokehAcc (&a)[4], float (&cD)[2], float (
 // (i, j), rows g, g + BG, ... (see the round gather's pf_layer)
 template <bool NEAR, bool RAD>
 __device__ __forceinline__ void bk_layer(BokehAcc (&a)[4], float R, int g, int i, int j, int W, int H, const Shape& s,
-                                         float ka, const float* __restrict__ rh, const float* __restrict__ ir2,
+                                         const float* __restrict__ rh, const float* __restrict__ ir2,
                                          const float* __restrict__ zq, const float4* __restrict__ rec) {
     const int G = (int)floorf(R + 1e-3f), n = 2 * s.K + 1;
     const int y0 = max(j - G, 0), y1 = min(j + 1 + G, H - 1);
@@ -305,7 +307,7 @@ __device__ __forceinline__ void bk_layer(BokehAcc (&a)[4], float R, int g, int i
         auto tap = [&](float r, float v, float z, const float4& e) {
             const float D[2] = {__ldg(&D0[SX * dxi]), __ldg(&D1[SX * dxi])}, dx2 = dx * dx;
             const float d2[2] = {dx2 + dy0, dx2 + dy1};
-            bk_tap<NEAR, RAD>(a, cD, cd2, D, d2, r, v, z, c1, c0r, ka, e);
+            bk_tap<NEAR, RAD>(a, cD, cd2, D, d2, r, v, z, c1, c0r, e);
             ++dxi;
             dx += 1.f;
         };
@@ -361,7 +363,6 @@ __global__ void __launch_bounds__(BG* BGT, 3) k_bokeh_gather(BokehGather<COL> a)
     const int p = threadIdx.x, px = tx * BT + (p & 15), py = ty * BT + (p >> 4);  // the pixel this thread finishes
     const bool fin = px < W && py < H;
     const size_t pq = (size_t)py * W + px;
-    const float ka = 1.f + 1.f / a.kz_rel;
     float4 S[2];  // near, far sums of pixel p
 #pragma unroll
     for (int layer = 1; layer >= 0; --layer) {
@@ -373,14 +374,15 @@ __global__ void __launch_bounds__(BG* BGT, 3) k_bokeh_gather(BokehGather<COL> a)
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 acc[k].xy = acc[k].zw = make_float2(0.f, 0.f);
-                acc[k].kb = 0.f;
+                acc[k].zp = acc[k].kb = 0.f;
                 if (layer) {
                     const int x = min(i + (k & 1), W - 1), y = min(j + (k >> 1), H - 1);
-                    acc[k].kb = 1.f / (a.kz_rel * __ldg(&a.zq[(size_t)y * W + x]));
+                    acc[k].zp = __ldg(&a.zq[(size_t)y * W + x]);
+                    acc[k].kb = 1.f / (a.kz_rel * acc[k].zp);
                 }
             }
-            if (layer) bk_layer<false, RAD>(acc, __int_as_float(rb), g, i, j, W, H, a.s, ka, a.rh, a.ir2, a.zq, a.frec);
-            else bk_layer<true, RAD>(acc, __int_as_float(rb), g, i, j, W, H, a.s, ka, a.rh, a.ir2, a.zq, a.nrec);
+            if (layer) bk_layer<false, RAD>(acc, __int_as_float(rb), g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.frec);
+            else bk_layer<true, RAD>(acc, __int_as_float(rb), g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.nrec);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 s_part[g][(lj + (k >> 1)) * BT + li + (k & 1)] =
