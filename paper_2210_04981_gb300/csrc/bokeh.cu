@@ -178,7 +178,7 @@ struct BokehPrep {
     float* ir2;  // 1 / r^2, 0 where r < 1 (no radial weight)
     float4* nrec;
     float4* frec;
-    float2* tmax;  // per tile: largest r feeding the near and the far layer (-1: none)
+    float4* tmax;  // per tile: largest r feeding the near and the far layer (-1: none); 1: a record is not finite
 };
 
 template <class ND, class COL>
@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(256) k_bokeh_prep(BokehPrep<ND, COL> a) {
     __syncthreads();
     const int i = blockIdx.x * BT + (threadIdx.x & 15), j = blockIdx.y * BT + (threadIdx.x >> 4);
     float rn = -1.f, rf = -1.f;
+    bool odd = false;
     if (i < a.W && j < a.H) {
         const size_t q = (size_t)j * a.W + i;
         const float z = ldz(a.nd + q), c = a.coc(z);
@@ -209,6 +210,7 @@ __global__ void __launch_bounds__(256) k_bokeh_prep(BokehPrep<ND, COL> a) {
         a.ir2[q] = ir2;
         a.nrec[q] = make_float4(col.x * an, col.y * an, col.z * an, an);
         a.frec[q] = make_float4(col.x * af, col.y * af, col.z * af, af);
+        odd = !isfinite(col.x) || !isfinite(col.y) || !isfinite(col.z);
         rn = wn > 0.f ? r : -1.f;
         rf = wn < 1.f ? r : -1.f;
     }
@@ -218,11 +220,11 @@ __global__ void __launch_bounds__(256) k_bokeh_prep(BokehPrep<ND, COL> a) {
     }
     __shared__ float2 red[8];
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(rn, rf);
-    __syncthreads();
+    const int any_odd = __syncthreads_or(odd);
     if (threadIdx.x == 0) {
         float2 m = red[0];
         for (int k = 1; k < 8; ++k) m = make_float2(fmaxf(m.x, red[k].x), fmaxf(m.y, red[k].y));
-        a.tmax[blockIdx.y * a.ntx + blockIdx.x] = m;
+        a.tmax[blockIdx.y * a.ntx + blockIdx.x] = make_float4(m.x, m.y, any_odd ? 1.f : 0.f, 0.f);
     }
 }
 
@@ -234,7 +236,7 @@ struct BokehGather {
     const float4* nrec;
     const float4* frec;
     const COL* col;
-    const float2* tmax;
+    const float4* tmax;
     int W, H, ntx, nty, kt;
     float kz_rel;
     Shape s;
@@ -253,8 +255,10 @@ struct BokehAcc {
 // norm D[k] and squared distance d2[k], its right pixel at the previous
 // column's, carried in cD and cd2.  The far layer's depth test is
 // clamp(1 - (z - z_p) kb): the difference is exact near z_p, where
-// (1 + 1 / kz_rel) - z kb would cancel to 2^-24 / kz_rel.
-template <bool NEAR, bool RAD>
+// (1 + 1 / kz_rel) - z kb would cancel to 2^-24 / kz_rel.  ONLY: a source is
+// added only where it weighs (a weight of 0 times an infinite or NaN colour
+// would reach every pixel of the window).
+template <bool NEAR, bool RAD, bool ONLY>
 __device__ __forceinline__ void bk_tap(BokehAcc (&a)[4], float (&cD)[2], float (&cd2)[2], const float (&D)[2],
                                        const float (&d2)[2], float rh, float ir2, float z, float c1, float c0r,
                                        const float4& e) {
@@ -265,8 +269,10 @@ __device__ __forceinline__ void bk_tap(BokehAcc (&a)[4], float (&cD)[2], float (
         float w = __saturatef(rh - Dk);
         if (RAD) w *= fmaf(c1, __saturatef(dd * ir2), c0);
         if (!NEAR) w *= __saturatef(fmaf(a[k].zp - z, a[k].kb, 1.f));
-        a[k].xy = fma2(w, e.x, e.y, a[k].xy);
-        a[k].zw = fma2(w, e.z, e.w, a[k].zw);
+        if (!ONLY || w > 0.f) {
+            a[k].xy = fma2(w, e.x, e.y, a[k].xy);
+            a[k].zw = fma2(w, e.z, e.w, a[k].zw);
+        }
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -277,7 +283,7 @@ __device__ __forceinline__ void bk_tap(BokehAcc (&a)[4], float (&cD)[2], float (
 
 // One layer over the disk-shaped window of radius R around the 2x2 block at
 // (i, j), rows g, g + BG, ... (see the round gather's pf_layer)
-template <bool NEAR, bool RAD>
+template <bool NEAR, bool RAD, bool ONLY>
 __device__ __forceinline__ void bk_layer(BokehAcc (&a)[4], float R, int g, int i, int j, int W, int H, const Shape& s,
                                          const float* __restrict__ rh, const float* __restrict__ ir2,
                                          const float* __restrict__ zq, const float4* __restrict__ rec) {
@@ -307,7 +313,7 @@ __device__ __forceinline__ void bk_layer(BokehAcc (&a)[4], float R, int g, int i
         auto tap = [&](float r, float v, float z, const float4& e) {
             const float D[2] = {__ldg(&D0[SX * dxi]), __ldg(&D1[SX * dxi])}, dx2 = dx * dx;
             const float d2[2] = {dx2 + dy0, dx2 + dy1};
-            bk_tap<NEAR, RAD>(a, cD, cd2, D, d2, r, v, z, c1, c0r, e);
+            bk_tap<NEAR, RAD, ONLY>(a, cD, cd2, D, d2, r, v, z, c1, c0r, e);
             ++dxi;
             dx += 1.f;
         };
@@ -342,12 +348,14 @@ __global__ void __launch_bounds__(BG* BGT, 3) k_bokeh_gather(BokehGather<COL> a)
     __shared__ float4 s_part[BG][BT * BT];
     if (threadIdx.x < 2) s_reach[threadIdx.x] = -1;
     __syncthreads();
+    bool odd = false;  // a tile near enough holds a record that is not finite
     {
         const int n = 2 * a.kt + 1;
         for (int e = threadIdx.x; e < n * n; e += BG * BGT) {
             const int ox = e % n - a.kt, oy = e / n - a.kt, x = tx + ox, y = ty + oy;
             if (x < 0 || y < 0 || x >= a.ntx || y >= a.nty) continue;
-            const float2 r = __ldg(&a.tmax[y * a.ntx + x]);
+            const float4 r = __ldg(&a.tmax[y * a.ntx + x]);
+            odd |= r.z > 0.f;
             const float gx = ox == 0 ? 0.f : (float)((abs(ox) - 1) * BT + 1);
             const float gy = oy == 0 ? 0.f : (float)((abs(oy) - 1) * BT + 1);
             const float g2 = gx * gx + gy * gy;
@@ -356,7 +364,7 @@ __global__ void __launch_bounds__(BG* BGT, 3) k_bokeh_gather(BokehGather<COL> a)
             if (r.y >= 0.f && g2 < (r.y + 0.5f) * (r.y + 0.5f)) atomicMax(&s_reach[1], __float_as_int(r.y + 0.5f));
         }
     }
-    __syncthreads();
+    const bool only = __syncthreads_or(odd);
     const int g = threadIdx.x / BGT, t = threadIdx.x % BGT;
     const int li = 2 * (t & 7), lj = 2 * (t >> 3), i = tx * BT + li, j = ty * BT + lj;
     const bool in = i < W && j < H;
@@ -381,8 +389,11 @@ __global__ void __launch_bounds__(BG* BGT, 3) k_bokeh_gather(BokehGather<COL> a)
                     acc[k].kb = 1.f / (a.kz_rel * acc[k].zp);
                 }
             }
-            if (layer) bk_layer<false, RAD>(acc, __int_as_float(rb), g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.frec);
-            else bk_layer<true, RAD>(acc, __int_as_float(rb), g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.nrec);
+            const float R = __int_as_float(rb);
+            if (layer && only) bk_layer<false, RAD, true>(acc, R, g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.frec);
+            else if (layer) bk_layer<false, RAD, false>(acc, R, g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.frec);
+            else if (only) bk_layer<true, RAD, true>(acc, R, g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.nrec);
+            else bk_layer<true, RAD, false>(acc, R, g, i, j, W, H, a.s, a.rh, a.ir2, a.zq, a.nrec);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 s_part[g][(lj + (k >> 1)) * BT + li + (k & 1)] =
@@ -443,7 +454,7 @@ int launch_bokeh(const hdof_gbuf* in, const Coc& coc, const hdof_params* p, floa
     HDOF_LAUNCHED("post-filter bokeh: area tables");
     const int ntx = (W + BT - 1) / BT, nty = (H + BT - 1) / BT;
     dim3 grid(ntx, nty);
-    float2* tmax = reinterpret_cast<float2*>(w.tmax);
+    float4* tmax = w.tmax;
     float* ir2 = reinterpret_cast<float*>(w.pre);  // the round gather's prefix plane
     const bool f32n = in->dtype_nd == HDOF_F32, f32c = in->dtype_col == HDOF_F32;
     const float4* nd4 = static_cast<const float4*>(in->nd);

@@ -41,3 +41,30 @@ def test_shaped_depth_test_at_a_narrow_range(orc, shape, kz_rel):
     ref = orc.postfilter(nd.astype(np.float64), col.astype(np.float64), lens, cam.tan_half_fovy, p)
     assert ref[..., :3].max() - ref[..., :3].min() > 0.05
     assert frac_close(host(pp), ref, 1e-4) >= 0.999, report("pp", host(pp), ref)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("zf", [0.5, 2.0, 8.0])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_shaped_source_that_is_not_finite(shape, zf, bad):
+    """A source of infinite or NaN colour changes no pixel outside its own disk
+    (those are equal to the image with a finite one there, bit for bit: it
+    adds nothing to them), and is not finite where it weighs."""
+    W, Hh, y, x = 211, 97, 40, 150
+    g = hi.random_gbuffer(W, Hh, seed=3)
+    g["nd"][..., 3] = np.clip(g["nd"][..., 3], 0.4, 12.0)
+    cam, lens = hi.Camera(width=W, height=Hh).f32(), hi.Lens(zf, 0.05, 0.05).f32()
+    p = hi.Params(r_max=20.0, **shape)
+    outs = []
+    for c in (0.5, bad):
+        g["col"][y, x, :3] = c
+        pp = torch.empty((Hh, W, 4), device="cuda")
+        H.hdof_postfilter(gbuf_from(g["nd"], g["col"]), cam, lens, p, pp, workspace(W, Hh, p))
+        H.hdof_sync()
+        outs.append(host(pp))
+    K = lens.aperture_radius * Hh / cam.tan_half_fovy
+    r = min(abs(K * (1.0 / g["nd"][y, x, 3] - 1.0 / zf)) / 2, 20.0)
+    yy, xx = np.mgrid[0:Hh, 0:W]
+    outside = np.hypot(yy - y, xx - x) > r + 0.5 + 1e-3
+    assert outside.any() and np.array_equal(outs[0][outside], outs[1][outside])
+    assert not np.isfinite(outs[1][y, x, :3]).all()
