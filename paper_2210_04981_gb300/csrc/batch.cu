@@ -130,6 +130,7 @@ Layout layout(int n) {
 int fill_image(const hdof_view* views, int n, unsigned* st, const Layout& L, char* img, int* blocks,
                const hdof_tuning& tune) {
     std::memset(img, 0, L.bytes);
+    const int mask_rows = mask_batch_rows(views, n);
     for (int k = 0; k < N_STAGES; ++k) {
         const size_t sz = kStages[k].size();
         int* prefix = reinterpret_cast<int*>(img + L.prefix[k]);
@@ -139,6 +140,7 @@ int fill_image(const hdof_view* views, int n, unsigned* st, const Layout& L, cha
             int gx = 0, gy = 0;
             ViewWs w = view_ws(views[v]);
             w.spatial_tile = tune.spatial_tile;
+            w.mask_rows = mask_rows;
             kStages[k].fill(views[v], w, st, img + L.args[k] + (size_t)v * sz, &gx, &gy);
             prefix[v] = (int)total;
             gxs[v] = gx;

@@ -55,6 +55,7 @@ struct ViewWs {
     uint8_t* tiles;      // mask tile flags
     float* tile_r;       // largest CoC radius per mask tile (CoC-scaled mask)
     int spatial_tile;    // the batch's spatial gather tile (hdof_tuning.spatial_tile), 0 = default
+    int mask_rows;       // the batch's output rows per warp of the mask's sweep (mask_batch_rows)
     unsigned* counts;    // [2 * ntiles] traced pixels, rays per 16x16 tile
     unsigned* offsets;   // [ntiles]
     unsigned* roffsets;  // [ntiles]
@@ -95,6 +96,7 @@ inline ViewWs view_ws(const hdof_view& v) {
     w.tiles = reinterpret_cast<uint8_t*>(base);
     w.tile_r = reinterpret_cast<float*>(base + L.mask_tiles);
     w.spatial_tile = 0;
+    w.mask_rows = 0;
     w.counts = reinterpret_cast<unsigned*>(base);
     w.offsets = w.counts + 2 * ntiles;
     w.roffsets = w.offsets + ntiles;
@@ -126,6 +128,8 @@ HDOF_BATCH_STAGE(temporal)
 HDOF_BATCH_STAGE(spatial)
 HDOF_BATCH_STAGE(composite)
 #undef HDOF_BATCH_STAGE
+
+int mask_batch_rows(const hdof_view* views, int n);
 
 // stages that are not one block grid per view
 size_t scan_args_size();

@@ -16,6 +16,7 @@
 
 #include "batch.cuh"
 #include "internal.h"
+#include "mask_rows.h"
 
 namespace hdof {
 namespace {
@@ -32,12 +33,12 @@ struct EdgeArgs {
     GaussW g;
     float tau;
     int tile, ntx;
-    int rows;       // output rows per warp
     uint8_t* edge;
     uint8_t* tiles;
     Coc coc;        // CoC-scaled mask: the lens's CoC in pixels
     float rmax;     // CoC radius cap (the post-filter's r_max)
     float* tile_r;  // largest CoC radius per mask tile (atomic max of float bits); NULL: fixed dilation
+    int rows;       // output rows per warp (last: before the pointers it cost the batched sweep 16 bytes of spills)
 };
 
 // ---- register sweep form of the edge pass ----------------------------------
@@ -52,8 +53,6 @@ struct EdgeArgs {
 //   columns.  Nothing goes through shared memory; each input pixel is loaded
 //   once per strip (plus the 3-pixel halos).  Edge flags and CoC radii are
 //   reduced per mask tile in registers and written once per tile row.
-constexpr int SW_OUT = 26;   // output columns per warp
-constexpr int SW_ROWS = 32;  // output rows per warp, fewer on small images (sweep_rows)
 constexpr int SW_WARPS = 4;  // warps per block (side by side)
 
 // float4 arithmetic as two packed two-lane FP32 operations (Blackwell's
@@ -239,20 +238,8 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) k_mask_sweep_batch(const Edg
     g.locate(blockIdx.x, v, bx, by);
     mask_sweep_body(batch_record(a, v), bx, by);
 }
-// Output rows per warp of the sweep: a warp walks its rows one after another
-// (6 more for the halo), so a small image, whose few strips leave the machine
-// empty (below 8 warps an SM), is cut into shorter ones: the 128x128 mask 35
-// -> 23 us.  The filtered values do not depend on it.  At 1080p (2516 warps)
-// 8 or 16 rows shorten the mask by 5% and the frame not at all.
-inline int sweep_rows(int W, int H) {
-    const int strips = (W + SW_OUT - 1) / SW_OUT;
-    int rows = SW_ROWS;
-    while (rows > 8 && strips * ((H + rows - 1) / rows) < 1216) rows /= 2;
-    return rows;
-}
 // grid of the sweep for a W x H frame
-inline dim3 sweep_grid(int W, int H) {
-    const int rows = sweep_rows(W, H);
+inline dim3 sweep_grid(int W, int H, int rows) {
     return dim3((W + SW_OUT * SW_WARPS - 1) / (SW_OUT * SW_WARPS), (H + rows - 1) / rows);
 }
 
@@ -388,7 +375,7 @@ GaussW gauss_weights(float sigma) {
 }
 
 template <class ND>
-EdgeArgs<ND> edge_args(const hdof_gbuf* in, const hdof_params* p, uint8_t* edge, uint8_t* tiles,
+EdgeArgs<ND> edge_args(const hdof_gbuf* in, const hdof_params* p, int rows, uint8_t* edge, uint8_t* tiles,
                        const Coc* coc = nullptr, float* tile_r = nullptr) {
     EdgeArgs<ND> a;
     a.nd = static_cast<const ND*>(in->nd);
@@ -398,7 +385,7 @@ EdgeArgs<ND> edge_args(const hdof_gbuf* in, const hdof_params* p, uint8_t* edge,
     a.tau = p->edge_tau;
     a.tile = p->tile;
     a.ntx = (in->width + p->tile - 1) / p->tile;
-    a.rows = sweep_rows(in->width, in->height);
+    a.rows = rows;
     a.edge = edge;
     a.tiles = tiles;
     a.coc = coc ? *coc : Coc{0.f, 0.f};
@@ -436,12 +423,13 @@ SppArgs spp_args(const hdof_gbuf* in, const hdof_history* prev_hist, const hdof_
 int launch_mask(const hdof_gbuf* in, const hdof_history* prev_hist, const hdof_params* p, uint8_t* edge, uint8_t* spp,
                 uint8_t* tiles, cudaStream_t s, const Coc* coc = nullptr, float* tile_r = nullptr) {
     const int W = in->width, H = in->height;
-    const dim3 grid = sweep_grid(W, H);
+    const int rows = sweep_rows([&](int r) { return sweep_warps(W, H, r); }, sm_count());
+    const dim3 grid = sweep_grid(W, H, rows);
     ProfScope ps_("mask", s);
     if (in->dtype_nd == HDOF_F32)
-        k_mask_sweep<float4><<<grid, SW_WARPS * 32, 0, s>>>(edge_args<float4>(in, p, edge, tiles, coc, tile_r));
+        k_mask_sweep<float4><<<grid, SW_WARPS * 32, 0, s>>>(edge_args<float4>(in, p, rows, edge, tiles, coc, tile_r));
     else
-        k_mask_sweep<half4s><<<grid, SW_WARPS * 32, 0, s>>>(edge_args<half4s>(in, p, edge, tiles, coc, tile_r));
+        k_mask_sweep<half4s><<<grid, SW_WARPS * 32, 0, s>>>(edge_args<half4s>(in, p, rows, edge, tiles, coc, tile_r));
     HDOF_LAUNCHED("mask: edge");
     dim3 g2((W + SPP_BX - 1) / SPP_BX, (H + SPP_BY - 1) / SPP_BY);
     k_mask_spp<<<g2, 256, 0, s>>>(spp_args(in, prev_hist, p, tiles, spp, coc ? tile_r : nullptr));
@@ -577,12 +565,21 @@ extern "C" int hdof_mask_noalloc(const hdof_gbuf* in, const hdof_history* prev_h
 
 namespace hdof {
 
+int mask_batch_rows(const hdof_view* views, int n) {
+    return sweep_rows(
+        [&](int r) {
+            long long warps = 0;
+            for (int v = 0; v < n; ++v) warps += sweep_warps(views[v].g.width, views[v].g.height, r);
+            return warps;
+        },
+        sm_count());
+}
 size_t mask_edge_args_size() { return sizeof(EdgeArgs<float4>); }
 void mask_edge_fill(const hdof_view& v, const ViewWs& w, unsigned*, void* dst, int* gx, int* gy) {
     const Coc coc = make_coc(v.lens, v.cam.height, v.cam.tan_half_fovy);
     *reinterpret_cast<EdgeArgs<float4>*>(dst) =
-        edge_args<float4>(&v.g, &v.params, v.edge, w.tiles, v.params.mask_coc ? &coc : nullptr, w.tile_r);
-    const dim3 sg = sweep_grid(v.g.width, v.g.height);
+        edge_args<float4>(&v.g, &v.params, w.mask_rows, v.edge, w.tiles, v.params.mask_coc ? &coc : nullptr, w.tile_r);
+    const dim3 sg = sweep_grid(v.g.width, v.g.height, w.mask_rows);
     *gx = (int)sg.x;
     *gy = (int)sg.y;
 }

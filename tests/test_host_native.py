@@ -50,7 +50,7 @@ int main() {
         hdof::Sum3 s{}, part[32] = {}, sq{};
         for (int k = 0; k < n; ++k) {
             float x;
-            scanf("%a", &x);
+            if (scanf("%a", &x) != 1) return 1;
             s.add(x);
             part[k % 32].add(x);
             const double d = (double)x * x;
@@ -72,3 +72,31 @@ int main() {
             assert abs(Fraction(float(g[k])) - sum(terms)) <= Fraction(1, 2 ** 52) * sum(map(abs, terms)), (k, len(x))
     # where a double is exact, so is the sum
     assert float.fromhex(got[0]) == 1.0 + 2.0 ** -25 + 2.0 ** -49 and float.fromhex(got[4]) == 2.0 ** -28
+
+
+def test_mask_strips_of_an_image_and_of_a_batch(tmp_path):
+    """Strips are cut shorter only while all the warps of a launch are too few:
+    alone, a 256x256 view takes 8 rows, among 64 of them 32."""
+    src = """#include <cstdio>
+#include <vector>
+#include "mask_rows.h"
+int main() {
+    int n, sms;
+    while (scanf("%d %d", &sms, &n) == 2) {
+        std::vector<int> s(2 * n);
+        for (int& v : s) if (scanf("%d", &v) != 1) return 1;
+        printf("%d\\n", hdof::sweep_rows([&](int r) {
+            long long t = 0;
+            for (int k = 0; k < n; ++k) t += hdof::sweep_warps(s[2 * k], s[2 * k + 1], r);
+            return t; }, sms));
+    }
+}"""
+    cases = [(152, [(256, 256)]), (152, [(128, 128)]), (152, [(1920, 1080)]), (152, [(640, 480)]), (152, [(1, 1)]),
+             (152, [(1280, 720)]), (152, [(256, 256)] * 12), (152, [(256, 256)] * 64), (152, [(640, 480)] * 4),
+             (152, [(1920, 1080), (256, 256)]), (8, [(256, 256)]), (1000, [(1920, 1080)]), (152, [(16384, 16384)] * 64)]
+    got = [int(g) for g in _run(tmp_path, src, "\n".join(f"{m} {len(s)} " + " ".join(f"{w} {h}" for w, h in s)
+                                                         for m, s in cases))]
+    for (m, s), g in zip(cases, got):
+        warps = [sum(-(-w // 26) * -(-h // r) for w, h in s) for r in (32, 16, 8)]
+        assert g == next((r for r, t in zip((32, 16, 8), warps) if t >= 8 * m), 8), (m, s[:2], len(s))
+    assert got[0] == 8 and got[7] == 32  # a 256x256 view alone, and 64 of them
