@@ -311,9 +311,9 @@ int hdof_mask_noalloc(const hdof_gbuf* in, const hdof_history* prev_hist, const 
  *   lane; a warp fetches new rays for its idle lanes once fewer than this
  *   many of its 32 lanes still trace); -1 = each view in its default form:
  *   warp packets when the lens's width against the view's, A / (zf
- *   tan(fovy/2)), is below 0.1, ray level with refill 4 otherwise (a batch traces the
- *   two groups of views in two persistent launches, both of trace_block
- *   threads).
+ *   tan(fovy/2)), is below 0.1 (in a batch below 0.1 min(1, H / 400)), ray
+ *   level with refill 4 otherwise (a batch traces the two groups of views in
+ *   two persistent launches, both of trace_block threads).
  * trace_chunk, spatial_tile: launch granularity of the trace's work queue and
  *   of the batched spatial gather (see the fields).  No choice changes a
  *   result: each ray's closest hit and each pixel's gather are computed the
@@ -357,9 +357,10 @@ typedef struct hdof_tuning {
  * values are rejected with HDOF_EINVAL); NULL takes 128 threads and the
  * default form (trace_refill -1): warp packets when A / (zf tan(fovy/2)), the
  * lens's width against the view's, is below 0.1 (the lens rays of
- * neighbouring pixels stay close), ray level with refill 4 otherwise.  From
- * 0.01 on a tile's rays are listed by the part of the lens they leave, in
- * either form. */
+ * neighbouring pixels stay close), ray level with refill 4 otherwise.  A
+ * tile's rays are listed by the part of the lens they leave, in either form,
+ * where that width is at least 0.01 and the CoC scale K = H times it at least
+ * 14 / sqrt(spp_max) pixels (in a batch 36 / sqrt(spp_max)). */
 int hdof_trace(const hdof_bvh* bvh, const hdof_camera* cam, const hdof_lens* lens,
                const hdof_params* p, const uint8_t* spp, const int32_t* hint_tri, float* rt,
                uint32_t* stats, float* rec, uint32_t* ray_off, void* workspace,

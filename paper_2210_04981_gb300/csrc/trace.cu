@@ -20,32 +20,14 @@
 // the output does not depend on scheduling.
 #include "batch.cuh"
 #include "internal.h"
+#include "trace_rule.h"
 
 namespace hdof {
 
-// What a view's trace depends on is how far apart the rays that run together
-// are against the scene's triangles, so on the lens's width against the
-// view's, K / H = A / (zf tan(fovy/2)) (K the CoC scale in pixels: pixels of
-// CoC per unit of zf/z - 1).  Both lines only choose an order or a form: every
-// ray's hit is the same.
-//
-// From K / H = 0.01 on a tile's rays are listed by lens bin (scatter_binned).
-// Rooms of about 165k triangles, trace and compaction, unsorted / sorted:
-// 1080p K = 4.6 242 / 265 us, 7 312 / 318, 10 359 / 345, 14 409 / 360, 25
-// 521 / 381, 60 638 / 458 (the better form of each); 480x270 K = 2 162 / 179,
-// 4.6 216 / 198, 10 314 / 246, 25 351 / 316; 4K K = 9.3 390 / 495.
-//
-// Below K / H = 0.1 warp packets are the default form, ray level with refill
-// 4 above: sorted packets / rays at 1080p K = 60 458 / 528 us, 100 545 / 568,
-// 140 630 / 600; at 480x270 K = 18 283 / 320, 25 316 / 328, 60 422 / 344.
-// (Unsorted, the line lay at K = 20 pixels.)
-constexpr float BIN_KH_MIN = 0.01f;
-constexpr float PACKET_KH_MAX = 0.1f;
-static float lens_width(const hdof_lens& l, const hdof_camera& c) {
-    return l.aperture_radius / (l.focus_dist * c.tan_half_fovy);
+// a view's default form and ray order (batch: as one of several views)
+static TraceRule view_rule(const hdof_lens& l, const hdof_camera& c, const hdof_params& p, bool batch) {
+    return trace_rule(l.aperture_radius / (l.focus_dist * c.tan_half_fovy), c.height, p.spp_max, batch);
 }
-static bool packet_view(const hdof_lens& l, const hdof_camera& c) { return lens_width(l, c) < PACKET_KH_MAX; }
-static bool binned_view(const hdof_lens& l, const hdof_camera& c) { return lens_width(l, c) >= BIN_KH_MIN; }
 
 namespace {
 
@@ -214,7 +196,7 @@ __global__ void __launch_bounds__(1024) k_scan(ScanArgs a) { scan_body(a); }
 struct ScatterArgs {
     const uint8_t* spp;
     int W, H, ntx, smax;
-    int binned;  // a tile's rays in order of their lens samples' bins (binned_view)
+    int binned;  // a tile's rays in order of their lens samples' bins (trace_rule)
     uint2 key;   // the samples' Philox key
     const unsigned* offsets;
     const unsigned* roffsets;
@@ -391,8 +373,8 @@ struct TraceArgs {
     float aberration;        // sample weight 1 + aberration (2 rho^2 / A^2 - 1)
     uint2 key;
     int cap, smax;
-    int packets;  // the view's default form is warp packets (packet_view)
-    int binned;   // the ray list is in lens-bin order (binned_view)
+    int packets;  // the view's default form is warp packets (trace_rule)
+    int binned;   // the ray list is in lens-bin order (trace_rule)
     unsigned* status;
     const uint8_t* spp;
     const int* hint;   // optional per-pixel original id of the primary hit (< 0: none)
@@ -895,7 +877,7 @@ __global__ void __launch_bounds__(256) k_hits(HitsArgs a) {
 }
 
 TraceArgs trace_args(const hdof_bvh* b, const hdof_camera* cam, const hdof_lens* lens, const hdof_params* p,
-                     unsigned* st, const uint8_t* spp, const int* hint, const ViewWs& w, float* rt, float* rec,
+                     TraceRule rule, unsigned* st, const uint8_t* spp, const int* hint, const ViewWs& w, float* rt, float* rec,
                      const unsigned* ray_off) {
     TraceArgs a;
     a.bvh = b->view();
@@ -911,8 +893,8 @@ TraceArgs trace_args(const hdof_bvh* b, const hdof_camera* cam, const hdof_lens*
     a.key = trace_key(*p);
     a.cap = step_cap(p->trav_cap, b->n_nodes, b->n_tris);
     a.smax = p->spp_max;
-    a.packets = packet_view(*lens, *cam) ? 1 : 0;
-    a.binned = binned_view(*lens, *cam) ? 1 : 0;
+    a.packets = rule.packets ? 1 : 0;
+    a.binned = rule.binned ? 1 : 0;
     a.status = st;
     a.spp = spp;
     a.hint = hint;
@@ -1051,8 +1033,8 @@ size_t scatter_args_size() { return sizeof(ScatterArgs); }
 void scatter_fill(const hdof_view& v, const ViewWs& w, unsigned*, void* dst, int* gx, int* gy) {
     const int W = v.cam.width, H = v.cam.height, ntx = (W + TB - 1) / TB;
     *reinterpret_cast<ScatterArgs*>(dst) =
-        ScatterArgs{v.spp, W, H, ntx, v.params.spp_max, binned_view(v.lens, v.cam) ? 1 : 0, trace_key(v.params), w.offsets, w.roffsets, w.queue, w.qoff, w.ray_pix, w.ray_s,
-                    nullptr};
+        ScatterArgs{v.spp, W, H, ntx, v.params.spp_max, view_rule(v.lens, v.cam, v.params, true).binned ? 1 : 0,
+                    trace_key(v.params), w.offsets, w.roffsets, w.queue, w.qoff, w.ray_pix, w.ray_s, nullptr};
     *gx = ntx;
     *gy = (H + TB - 1) / TB;
 }
@@ -1064,7 +1046,7 @@ void scatter_launch_batch(const void* args, BatchGrid g, int blocks, cudaStream_
 size_t trace_args_size() { return sizeof(TraceArgs); }
 void trace_fill(const hdof_view& v, const ViewWs& w, unsigned* st, void* dst, int* gx, int* gy) {
     *reinterpret_cast<TraceArgs*>(dst) =
-        trace_args(v.bvh, &v.cam, &v.lens, &v.params, st, v.spp, v.g.tri, w, v.rt, nullptr, nullptr);
+        trace_args(v.bvh, &v.cam, &v.lens, &v.params, view_rule(v.lens, v.cam, v.params, true), st, v.spp, v.g.tri, w, v.rt, nullptr, nullptr);
     *gx = (v.cam.width * v.cam.height + 255) / 256;  // resolve: one thread per possible queue entry
     *gy = 1;
 }
@@ -1164,7 +1146,8 @@ extern "C" int hdof_trace(const hdof_bvh* b, const hdof_camera* cam, const hdof_
         t.trace_block = 128;
         t.trace_refill = -1;
     }
-    if (t.trace_refill == -1) t.trace_refill = packet_view(*lens, *cam) ? 0 : 4;
+    const TraceRule rule = view_rule(*lens, *cam, *p, false);
+    if (t.trace_refill == -1) t.trace_refill = rule.packets ? 0 : 4;
     const int W = cam->width, H = cam->height;
     WsLayout L = ws_layout(W, H, p);
     HDOF_CHECK_ARG(workspace && workspace_bytes >= L.trace, "hdof_trace: workspace of %zu bytes < %zu",
@@ -1184,11 +1167,12 @@ extern "C" int hdof_trace(const hdof_bvh* b, const hdof_camera* cam, const hdof_
         k_count<<<tg, 256, 0, s>>>(CountArgs{spp, W, H, ntx, p->spp_max, w.counts});
         k_scan<<<1, 1024, 0, s>>>(ScanArgs{w.counts, ntiles, w.offsets, w.roffsets, w.totals, stats});
         k_scatter<<<tg, 256, 0, s>>>(
-            ScatterArgs{spp, W, H, ntx, p->spp_max, binned_view(*lens, *cam) ? 1 : 0, trace_key(*p), w.offsets, w.roffsets, w.queue, w.qoff, w.ray_pix, w.ray_s, ray_off});
+            ScatterArgs{spp, W, H, ntx, p->spp_max, rule.binned ? 1 : 0, trace_key(*p), w.offsets, w.roffsets, w.queue,
+                        w.qoff, w.ray_pix, w.ray_s, ray_off});
         HDOF_LAUNCHED("hdof_trace: compaction");
     }
 
-    TraceArgs a = trace_args(b, cam, lens, p, st, spp, hint_tri, w, rt, rec, ray_off);
+    TraceArgs a = trace_args(b, cam, lens, p, rule, st, spp, hint_tri, w, rt, rec, ray_off);
     int blocks = 0;
     if ((rc = rays_grid(false, t.trace_refill == 0, t.trace_block, &blocks))) return rc;
     {

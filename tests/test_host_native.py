@@ -100,3 +100,29 @@ int main() {
         warps = [sum(-(-w // 26) * -(-h // r) for w, h in s) for r in (32, 16, 8)]
         assert g == next((r for r, t in zip((32, 16, 8), warps) if t >= 8 * m), 8), (m, s[:2], len(s))
     assert got[0] == 8 and got[7] == 32  # a 256x256 view alone, and 64 of them
+
+
+def test_default_trace_rule(tmp_path):
+    """Form and ray order of a view: packets below 0.1 of the view's height,
+    earlier rays for a batch's small views; sorted by lens bin from 0.01 and
+    from a lens that spreads rays over more than a packet's pixel block on
+    (K sqrt(spp) of 14, in a batch 36)."""
+    src = """#include <cstdio>
+#include "trace_rule.h"
+int main() {
+    float kh; int H, spp, batch;
+    while (scanf("%f %d %d %d", &kh, &H, &spp, &batch) == 4) {
+        const hdof::TraceRule r = hdof::trace_rule(kh, H, spp, batch != 0);
+        printf("%d%d\\n", (int)r.packets, (int)r.binned);
+    }
+}"""
+    P, R = "10", "00"  # packets, rays; "11" and "01" sorted
+    cases = [((0.012, 256, 16, 1), P), ((0.025, 256, 16, 1), P), ((0.05, 256, 16, 1), "11"),
+             ((0.08, 256, 16, 1), "01"), ((0.012, 480, 16, 1), P), ((0.08, 480, 16, 1), "11"),
+             ((0.12, 480, 16, 1), "01"), ((0.012, 1080, 16, 1), "11"), ((0.012, 1080, 4, 1), P),
+             ((0.0099, 1080, 16, 1), P), ((0.2, 256, 1, 1), "01"), ((0.2, 64, 1, 1), R),
+             ((0.08, 256, 16, 0), "11"), ((0.0148, 136, 4, 0), P), ((0.0241, 175, 8, 0), P),
+             ((0.0231, 231, 16, 0), "11"), ((0.012, 1080, 8, 0), "11"), ((0.0099, 1080, 255, 0), P),
+             ((0.0043, 2160, 16, 0), P), ((0.2, 128, 16, 0), "01"), ((0.2, 10, 1, 0), R), ((0.0, 1080, 255, 0), P)]
+    got = _run(tmp_path, src, "\n".join(" ".join(map(str, c)) for c, _ in cases))
+    assert got == [w for _, w in cases], [(c, w, g) for (c, w), g in zip(cases, got) if w != g]
