@@ -234,6 +234,7 @@ __device__ __forceinline__ void scatter_binned(const ScatterArgs& a, unsigned q,
     __shared__ __align__(16) uint16_t s_off[LENS_BINS][256];
     __shared__ uint16_t s_list[SORT_STAGE];
     __shared__ unsigned s_bin[LENS_BINS + 1];
+    if (!__syncthreads_or(n > 0)) return;  // no ray here: most tiles of a static view
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
 #pragma unroll
     for (int b = 0; b < LENS_BINS; ++b) s_cnt[b][t] = 0;
