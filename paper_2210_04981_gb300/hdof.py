@@ -243,15 +243,6 @@ def params(p=None) -> hdof_params:
     return o
 
 
-class _Ready:
-    """A C record that is marshalled already, for a caller of its own that
-    makes several calls with it (a frame)."""
-    __slots__ = ("rec",)
-
-    def __init__(self, rec):
-        self.rec = rec
-
-
 # ------------------------------------------------------------- buffers ---
 
 class GBuffer:
@@ -297,26 +288,6 @@ class History:
 
     def reset(self):
         self.hlen.zero_()
-
-
-def _camera(c) -> hdof_camera:
-    return c.rec if type(c) is _Ready else camera(c)
-
-
-def _lens(l) -> hdof_lens:
-    return l.rec if type(l) is _Ready else lens(l)
-
-
-def _params(p) -> hdof_params:
-    return p.rec if type(p) is _Ready else params(p)
-
-
-def _gbuf(g) -> hdof_gbuf:
-    return g.rec if type(g) is _Ready else g.struct()
-
-
-def _hist(h) -> hdof_history:
-    return h.rec if type(h) is _Ready else h.struct()
 
 
 class Bvh:
@@ -392,8 +363,7 @@ def hdof_closest_hits(bvh: Bvh, org, dirs, ids, ts, stream=None):
 def hdof_gbuffer(bvh: Bvh, cam, prev, p, gbuf: GBuffer, stream=None, hint=None):
     """hint (int32 [H][W], e.g. the previous frame's tri plane, possibly
     gbuf.tri itself) optionally seeds each primary ray with a likely hit."""
-    _check(load().hdof_gbuffer(bvh.handle, C.byref(_camera(cam)), C.byref(_camera(prev)), C.byref(_params(p)),
-                               _ptr(hint), C.byref(_gbuf(gbuf)), _stream(stream)))
+    _gbuffer(bvh, camera(cam), camera(prev), params(p), gbuf.struct(), stream, hint)
 
 
 def hdof_mask(gbuf: GBuffer, prev_hist, p, edge, spp, workspace, stream=None):
@@ -404,9 +374,8 @@ def hdof_mask(gbuf: GBuffer, prev_hist, p, edge, spp, workspace, stream=None):
 
 def hdof_mask_coc(gbuf: GBuffer, prev_hist, cam, lns, p, edge, spp, workspace, stream=None):
     """hdof_mask whose edge tiles reach their pixels' largest CoC radius when p.mask_coc = 1."""
-    _check(load().hdof_mask_coc(C.byref(_gbuf(gbuf)), C.byref(_hist(prev_hist)) if prev_hist is not None else None,
-                                C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)), _ptr(edge), _ptr(spp),
-                                _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)))
+    _mask_coc(gbuf.struct(), prev_hist.struct() if prev_hist is not None else None, camera(cam), lens(lns), params(p),
+              edge, spp, workspace, stream)
 
 
 def hdof_mask_noalloc(gbuf: GBuffer, prev_hist, p, edge, spp, stream=None):
@@ -424,10 +393,7 @@ def hdof_trace(bvh: Bvh, cam, lns, p, spp, rt, stats, workspace, stream=None, re
     hint (int32 [H][W], the G-buffer's tri plane) optionally seeds each lens
     ray with its pixel's primary hit; tune (hdof_tuning) optionally fixes the
     trace's form and block size (default: chosen from the lens)."""
-    _check(load().hdof_trace(bvh.handle, C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)),
-                             _ptr(spp), _ptr(hint), _ptr(rt), _ptr(stats), _ptr(rec), _ptr(ray_off), _ptr(workspace),
-                             workspace.numel() * workspace.element_size(),
-                             C.byref(tune) if tune is not None else None, _stream(stream)))
+    _trace(bvh, camera(cam), lens(lns), params(p), spp, rt, stats, workspace, stream, rec, ray_off, hint, tune)
 
 
 def hdof_trace_hits(bvh: Bvh, cam, p, spp, workspace, ids, ts=None, stream=None):
@@ -472,40 +438,78 @@ def error_summary(stats) -> dict:
 
 
 def hdof_postfilter(gbuf: GBuffer, cam, lns, p, pp, workspace, stream=None):
-    _check(load().hdof_postfilter(C.byref(_gbuf(gbuf)), C.byref(_camera(cam)), C.byref(_lens(lns)),
-                                  C.byref(_params(p)), _ptr(pp), _ptr(workspace),
-                                  workspace.numel() * workspace.element_size(), _stream(stream)))
+    _postfilter(gbuf.struct(), camera(cam), lens(lns), params(p), pp, workspace, stream)
 
 
 def hdof_reconstruct(rt, gbuf: GBuffer, spp, cam, prev, lns, p, hist_in: History, hist_out: History, crt, hacc,
                      crec, stream=None):
-    _check(load().hdof_reconstruct(_ptr(rt), C.byref(_gbuf(gbuf)), _ptr(spp), C.byref(_camera(cam)),
-                                   C.byref(_camera(prev)), C.byref(_lens(lns)), C.byref(_params(p)),
-                                   C.byref(_hist(hist_in)), C.byref(_hist(hist_out)), _ptr(crt), _ptr(hacc),
-                                   _ptr(crec), _stream(stream)))
+    _reconstruct(rt, gbuf.struct(), spp, camera(cam), camera(prev), lens(lns), params(p), hist_in.struct(),
+                 hist_out.struct(), crt, hacc, crec, stream)
 
 
 def hdof_composite(gbuf: GBuffer, spp, pp, crt, crec, hacc, cam, lns, p, out, stream=None):
-    _check(load().hdof_composite(C.byref(_gbuf(gbuf)), _ptr(spp), _ptr(pp), _ptr(crt), _ptr(crec), _ptr(hacc),
-                                 C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)), _ptr(out),
-                                 _stream(stream)))
+    _composite(gbuf.struct(), spp, pp, crt, crec, hacc, camera(cam), lens(lns), params(p), out, stream)
 
 
 def hdof_postfilter_spec(gbuf: GBuffer, cam, lns, p, pp_spec, workspace, stream=None):
     """Post-filter of the specular plane col.w: pp_spec [H,W,4] = (S_pp x3, alpha)."""
-    _check(load().hdof_postfilter_spec(C.byref(_gbuf(gbuf)), C.byref(_camera(cam)), C.byref(_lens(lns)),
-                                       C.byref(_params(p)), _ptr(pp_spec), _ptr(workspace),
-                                       workspace.numel() * workspace.element_size(), _stream(stream)))
+    _postfilter_spec(gbuf.struct(), camera(cam), lens(lns), params(p), pp_spec, workspace, stream)
 
 
 def hdof_composite_spec(gbuf: GBuffer, spp, pp, pp_spec, crt, crec, hacc, cam, lns, p, out, stream=None):
-    _check(load().hdof_composite_spec(C.byref(_gbuf(gbuf)), _ptr(spp), _ptr(pp),
-                                      _ptr(pp_spec) if pp_spec is not None else None, _ptr(crt), _ptr(crec),
-                                      _ptr(hacc), C.byref(_camera(cam)), C.byref(_lens(lns)), C.byref(_params(p)),
-                                      _ptr(out), _stream(stream)))
+    _composite_spec(gbuf.struct(), spp, pp, pp_spec, crt, crec, hacc, camera(cam), lens(lns), params(p), out, stream)
 
 
 # ---------------------------------------------------------- frame driver --
+
+# The calls of a frame on C records: Renderer.frame marshals its records once
+# for all of them (the calls above take objects and marshal them each time).
+
+def _gbuffer(bvh, cam, prev, p, g, stream, hint):
+    _check(load().hdof_gbuffer(bvh.handle, C.byref(cam), C.byref(prev), C.byref(p), _ptr(hint), C.byref(g),
+                               _stream(stream)))
+
+
+def _mask_coc(g, prev_hist, cam, lns, p, edge, spp, workspace, stream):
+    _check(load().hdof_mask_coc(C.byref(g), C.byref(prev_hist) if prev_hist is not None else None, C.byref(cam),
+                                C.byref(lns), C.byref(p), _ptr(edge), _ptr(spp), _ptr(workspace),
+                                workspace.numel() * workspace.element_size(), _stream(stream)))
+
+
+def _trace(bvh, cam, lns, p, spp, rt, stats, workspace, stream, rec, ray_off, hint, tune):
+    _check(load().hdof_trace(bvh.handle, C.byref(cam), C.byref(lns), C.byref(p), _ptr(spp), _ptr(hint), _ptr(rt),
+                             _ptr(stats), _ptr(rec), _ptr(ray_off), _ptr(workspace),
+                             workspace.numel() * workspace.element_size(),
+                             C.byref(tune) if tune is not None else None, _stream(stream)))
+
+
+def _postfilter(g, cam, lns, p, pp, workspace, stream):
+    _check(load().hdof_postfilter(C.byref(g), C.byref(cam), C.byref(lns), C.byref(p), _ptr(pp), _ptr(workspace),
+                                  workspace.numel() * workspace.element_size(), _stream(stream)))
+
+
+def _postfilter_spec(g, cam, lns, p, pp_spec, workspace, stream):
+    _check(load().hdof_postfilter_spec(C.byref(g), C.byref(cam), C.byref(lns), C.byref(p), _ptr(pp_spec),
+                                       _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                       _stream(stream)))
+
+
+def _reconstruct(rt, g, spp, cam, prev, lns, p, hist_in, hist_out, crt, hacc, crec, stream):
+    _check(load().hdof_reconstruct(_ptr(rt), C.byref(g), _ptr(spp), C.byref(cam), C.byref(prev), C.byref(lns),
+                                   C.byref(p), C.byref(hist_in), C.byref(hist_out), _ptr(crt), _ptr(hacc), _ptr(crec),
+                                   _stream(stream)))
+
+
+def _composite(g, spp, pp, crt, crec, hacc, cam, lns, p, out, stream):
+    _check(load().hdof_composite(C.byref(g), _ptr(spp), _ptr(pp), _ptr(crt), _ptr(crec), _ptr(hacc), C.byref(cam),
+                                 C.byref(lns), C.byref(p), _ptr(out), _stream(stream)))
+
+
+def _composite_spec(g, spp, pp, pp_spec, crt, crec, hacc, cam, lns, p, out, stream):
+    _check(load().hdof_composite_spec(C.byref(g), _ptr(spp), _ptr(pp), _ptr(pp_spec) if pp_spec is not None else None,
+                                      _ptr(crt), _ptr(crec), _ptr(hacc), C.byref(cam), C.byref(lns), C.byref(p),
+                                      _ptr(out), _stream(stream)))
+
 
 def frame_priorities():
     """(highest, lowest) stream priority of the device: the frame's critical
@@ -571,30 +575,29 @@ class Renderer:
         # the frame's records, marshalled once for its six calls: a 128x128 frame, whose kernels are
         # shorter than the host's work on it, takes 121 us so and 156 with each call marshalling its own
         spec_pref = p.spec_pref
-        cam, prev, lns, p, g = map(_Ready, (camera(cam), camera(prev), lens(lns), params(p), self.g.struct()))
-        hin, hout = _Ready(self.hist[self.cur].struct()), _Ready(self.hist[1 - self.cur].struct())
-        hdof_gbuffer(self.bvh, cam, prev, p, g, main, hint=self.g.tri)
+        cam, prev, lns, p, g = camera(cam), camera(prev), lens(lns), params(p), self.g.struct()
+        hin, hout = self.hist[self.cur].struct(), self.hist[1 - self.cur].struct()
+        _gbuffer(self.bvh, cam, prev, p, g, main, self.g.tri)
         # the post-filter on the side stream, after the G-buffer (it touches only
         # the workspace's post-filter region)
         self._gbuf_done.record(main)
         self.side.wait_event(self._gbuf_done)
-        hdof_postfilter(g, cam, lns, p, self.pp, self.ws, self.side)
+        _postfilter(g, cam, lns, p, self.pp, self.ws, self.side)
         self._pf_done.record(self.side)
-        hdof_mask_coc(g, hin if with_history else None, cam, lns, p, self.edge, self.spp, self.ws, main)
-        hdof_trace(self.bvh, cam, lns, p, self.spp, self.rt, self.stats, self.ws, main, hint=self.g.tri)
-        hdof_reconstruct(self.rt, g, self.spp, cam, prev, lns, p, hin, hout, self.crt, self.hacc,
-                         self.crec, main)
+        _mask_coc(g, hin if with_history else None, cam, lns, p, self.edge, self.spp, self.ws, main)
+        _trace(self.bvh, cam, lns, p, self.spp, self.rt, self.stats, self.ws, main, None, None, self.g.tri, None)
+        _reconstruct(self.rt, g, self.spp, cam, prev, lns, p, hin, hout, self.crt, self.hacc, self.crec, main)
         main.wait_event(self._pf_done)
         if spec_pref > 0:
             # the specular plane's post-filter: after the post-filter, whose region it uses, and the trace (beside
             # the trace on the side stream it saves 1%, as the trace leaves few registers for other blocks)
             if self.pp_spec is None:
                 self.pp_spec = torch.empty_like(self.pp)
-            hdof_postfilter_spec(g, cam, lns, p, self.pp_spec, self.ws, main)
-            hdof_composite_spec(g, self.spp, self.pp, self.pp_spec, self.crt, self.crec, self.hacc, cam, lns,
-                                p, self.out, main)
+            _postfilter_spec(g, cam, lns, p, self.pp_spec, self.ws, main)
+            _composite_spec(g, self.spp, self.pp, self.pp_spec, self.crt, self.crec, self.hacc, cam, lns, p, self.out,
+                            main)
         else:
-            hdof_composite(g, self.spp, self.pp, self.crt, self.crec, self.hacc, cam, lns, p, self.out, main)
+            _composite(g, self.spp, self.pp, self.crt, self.crec, self.hacc, cam, lns, p, self.out, main)
         self._done.record(main)
         caller.wait_event(self._done)
         self.cur = 1 - self.cur
