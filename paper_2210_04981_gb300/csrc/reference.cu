@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(256) k_rt_accum(const float4* __restrict__ rt,
 // sums its few pixels, and a warp its threads, in three floats (Sum3: more
 // bits than a double; each d^2 exactly, with its rounding error), the block in
 // double precision: 160 us in double throughout at 1280x720 (with the final
-// block), 34 so.  A difference whose square's rounding error leaves the range
+// block), 27 so.  A difference whose square's rounding error leaves the range
 // of a float (tiny, huge, infinite or NaN) is left to a second loop, in
 // double, that runs only where there is one.
 __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ a, const float4* __restrict__ b,
@@ -111,18 +111,25 @@ __global__ void __launch_bounds__(ERR_THREADS) k_err(const float4* __restrict__ 
                 w2[r] += __shfl_xor_sync(0xffffffffu, w2[r], o);
             }
     }
+    // a quarter of the warp per sum: the all-pixel sums to the lower half, the
+    // region's to the upper, then |d| and d^2 to the halves of those
+    const bool up = lane & 16, sq = lane & 8;
+    Sum3 u1 = up ? s1[1] : s1[0], u2 = up ? s2[1] : s2[0];
+    u1.add(shfl_xor(up ? s1[0] : s1[1], 16));
+    u2.add(shfl_xor(up ? s2[0] : s2[1], 16));
+    Sum3 s = sq ? u2 : u1;
+    s.add(shfl_xor(sq ? u1 : u2, 8));
+    for (int o = 4; o; o >>= 1) s.add(shfl_xor(s, o));
+    if ((lane & 7) == 0) {
+        const double rest = up ? (sq ? w2[1] : w1[1]) : (sq ? w2[0] : w1[0]);
+        sh[(up ? 4 : 0) + (sq ? 2 : 1)][w] = s.value() + rest;
+    }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         cnt[r] = __reduce_add_sync(0xffffffffu, cnt[r]);
-        for (int o = 16; o; o >>= 1) {
-            s1[r].add(shfl_xor(s1[r], o));
-            s2[r].add(shfl_xor(s2[r], o));
-            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], o));
-        }
+        for (int o = 16; o; o >>= 1) mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], o));
         if (lane == 0) {
             sh[4 * r][w] = (double)cnt[r];
-            sh[4 * r + 1][w] = s1[r].value() + w1[r];
-            sh[4 * r + 2][w] = s2[r].value() + w2[r];
             sh[4 * r + 3][w] = (double)mx[r];
         }
     }
