@@ -19,6 +19,7 @@
 #include <cmath>
 
 #include "internal.h"
+#include "sum3.cuh"
 
 namespace hdof {
 namespace {
@@ -54,24 +55,12 @@ __device__ __forceinline__ float wn_slope(float c) { return (c > -HDOF_SQRT2 && 
 __device__ __forceinline__ float dot3f(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ __forceinline__ float3 ldf3(const float4& v) { return f3(v.x, v.y, v.z); }
 
-// A sum carried as an unevaluated pair hi + lo of floats (Knuth's TwoSum; 48
-// bits).  Sums of a block's few hundred floats in it agree with double ones
-// to far below the float result's rounding, at FP32 rates: FP64 adds run at
-// 1/64 of them here, and ten shuffle steps of doubles per thread held up the
-// composite adjoint (37 us at 1024x1024, 30 so) and the replay's (32 and 26).
-struct Pair {
-    float hi, lo;
-};
-__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
-    const float s = __fadd_rn(a.hi, b.hi), bb = __fsub_rn(s, a.hi);
-    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
-    return Pair{s, __fadd_rn(__fadd_rn(a.lo, b.lo), e)};
-}
-
-// block sum of a per-thread (float, float), fixed order: pairs of floats
-// within a warp (doubles in a warp with a value that is not finite or that
-// could overflow the pairs), double across the warps; thread 0 writes the
-// block's partial
+// block sum of a per-thread (float, float), fixed order: in three floats
+// (Sum3: the terms cancel, and its bits are more than a double's) within a
+// warp, in doubles in a warp with a value that is not finite or that could
+// overflow them, and in double across the warps; thread 0 writes the block's
+// partial.  Ten shuffle steps of doubles per thread held up the composite
+// adjoint (37 us at 1024x1024, 28 so) and the replay's (32 and 25).
 __device__ __forceinline__ void block_partial(float2 v, double2* partial) {
     __shared__ double red[2][32];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
@@ -82,18 +71,15 @@ __device__ __forceinline__ void block_partial(float2 v, double2* partial) {
             db += __shfl_xor_sync(0xffffffffu, db, o);
         }
     } else {
-        Pair a{v.x, 0.f}, b{v.y, 0.f};
-        for (int o = 16; o; o >>= 1) {
-            a = pair_add(a, Pair{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)});
-            b = pair_add(b, Pair{__shfl_xor_sync(0xffffffffu, b.hi, o), __shfl_xor_sync(0xffffffffu, b.lo, o)});
-        }
-        da = (double)a.hi + (double)a.lo;
-        db = (double)b.hi + (double)b.lo;
+        // the lower half of the warp sums x, the upper half y
+        const bool up = l & 16;
+        Sum3 s{up ? v.y : v.x, 0.f, 0.f};
+        s.add(__shfl_xor_sync(0xffffffffu, up ? v.x : v.y, 16));
+        for (int o = 8; o; o >>= 1) s.add(shfl_xor(s, o));
+        da = db = s.value();
     }
-    if (l == 0) {
-        red[0][w] = da;
-        red[1][w] = db;
-    }
+    if (l == 0) red[0][w] = da;
+    if (l == 16) red[1][w] = db;
     __syncthreads();
     if (threadIdx.x == 0) {
         double sa = 0.0, sb = 0.0;

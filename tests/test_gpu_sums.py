@@ -34,3 +34,40 @@ def test_error_map_sums_keep_a_doubles_bits(W, Hh, d, n):
             assert got[k + 1] == v.sum()
         else:
             assert got[k + 2] == (v * v).sum()
+
+
+@pytest.mark.parametrize("zf", [2.9, 3.0, 3.1, 3.3])
+def test_lens_gradient_keeps_a_doubles_bits(zf):
+    """A lens gradient whose terms cancel within a warp.  32x8 traced pixels,
+    all alike: near surfaces (near weight 1, its slope 0), one near hit each
+    inside the composite's focus ramp, no history, no spatial reach.  A
+    pixel's term is then linear in its image gradient, so that gradients 1,
+    2^-25, 2^-28, -1, -2^-25 at five pixels of a row add up to 2^-28 times the
+    term x of one pixel.  Every partial sum of the row fits a double's 53 bits
+    (24 of x, 28 of the scales), so the result is exact; what is 2^-48 below x
+    is lost in a pair of floats, and 4 units in the last place of the result
+    with it."""
+    import hdof_inputs as hi
+    W, Hh, A = 32, 8, 0.5
+    cam = hi.Camera(width=W, height=Hh).f32()
+    K = A * Hh / cam.tan_half_fovy
+    z = np.full((Hh, W), 1.0, np.float32)
+    rec = np.empty((W * Hh, 4), np.float32)
+    rec[:] = [0.7, 0.3, 0.2, 1.0 / (1.6 / K + 1.0 / zf)]  # |c| = 1.6: between sqrt 2 and sqrt 2 + 1/2
+    p = hi.room_params(r_s=0.0, r_max=8.0, variance_on=0)
+    path = H.PostPath(dev(z), torch.ones((Hh, W), dtype=torch.uint8, device="cuda"), dev(rec),
+                      torch.arange(W * Hh, dtype=torch.int32, device="cuda").reshape(Hh, W), None, cam, p)
+    col = torch.full((Hh, W, 3), 0.123, device="cuda")
+
+    def grad(terms):
+        g = torch.zeros((Hh, W, 3), device="cuda")
+        for lane, v in terms.items():
+            g[2, lane, 0] = v
+        path.forward(col, zf, A)
+        return host(path.backward(g, zf, A)[1])
+
+    one = grad({0: 1.0})
+    assert (one != 0).all() and np.isfinite(one).all()
+    assert np.array_equal(grad({0: 2.0 ** -28}), one * np.float32(2.0 ** -28))
+    got = grad({0: 1.0, 16: 2.0 ** -25, 8: 2.0 ** -28, 4: -1.0, 20: -2.0 ** -25})
+    assert np.array_equal(got, one * np.float32(2.0 ** -28)), (got, one)
