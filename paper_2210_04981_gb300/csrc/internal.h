@@ -103,7 +103,6 @@ WsLayout ws_layout(int W, int H, const hdof_params* p);
 // Lattice-area table of the soft disk (post-filter normalisation), uploaded
 // once per device.  Returns HDOF_OK or an error.
 int ensure_area_table(cudaStream_t s);
-int area_table_size();
 // device address of the table ((x, a(x), slope, 0) per breakpoint) and its length
 int area_table(const float4** tab, int* n);
 

@@ -84,7 +84,6 @@ constexpr int AREA_MAX = 16384;  // breakpoints for radii up to 127.5
 
 // (x_m, a(x_m), slope on [x_m, x_{m+1}], 0)
 __device__ float4 g_area[AREA_MAX];
-__device__ int g_area_n;
 // g_area_at[b]: largest m with x_m <= b / 32.  The breakpoints are at most 4
 // to such an interval up to r = 100, so the search within one takes two or
 // three dependent reads instead of the fourteen of the whole table, which
@@ -707,8 +706,6 @@ int g_area_count[64] = {0};
 
 }  // namespace
 
-int area_table_size() { return AREA_MAX; }
-
 int ensure_area_table(cudaStream_t s) {
     int dev = 0;
     HDOF_CUDA(cudaGetDevice(&dev), "area table: device");
@@ -779,7 +776,6 @@ int ensure_area_table(cudaStream_t s) {
               "area table: upload");
     HDOF_CUDA(cudaMemcpyToSymbolAsync(g_area, tab.data(), sizeof(float4) * tab.size(), 0, cudaMemcpyHostToDevice, s),
               "area table: upload");
-    HDOF_CUDA(cudaMemcpyToSymbolAsync(g_area_n, &n, sizeof n, 0, cudaMemcpyHostToDevice, s), "area table: upload");
     HDOF_CUDA(cudaStreamSynchronize(s), "area table: upload");
     g_area_ready[dev] = true;
     g_area_count[dev] = n;
