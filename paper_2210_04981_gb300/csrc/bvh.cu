@@ -984,7 +984,6 @@ extern "C" int hdof_build_bvh(const float* verts, int32_t n_verts, const int32_t
         set_error("hdof_build_bvh: tree depth %d exceeds the %d-entry traversal stack", depth, HDOF_STACK);
         return fail(HDOF_EUNSUPPORTED);
     }
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(cuda_fail(e, "hdof_build_bvh: build"));
     cudaFree(tmp);
     *out = b;
     return HDOF_OK;
