@@ -398,8 +398,9 @@ int hdof_reference_rt(const hdof_bvh* bvh, const hdof_camera* cam, const hdof_le
  * double [HDOF_ERR_SCRATCH], whose first HDOF_ERR_STATS entries receive
  * (pixels, sum |d|, sum d^2, max |d|) over all pixels, then the same over
  * the pixels where region (uint8 [H][W], may be NULL) is non-zero; sums run
- * over the three channels.  The rest is scratch.  Reduced in a fixed order:
- * the same inputs give the same bits. */
+ * over the three channels, with at least a double's bits (a thread's and a
+ * warp's in three floats, then doubles).  The rest is scratch.  Reduced in a
+ * fixed order: the same inputs give the same bits. */
 #define HDOF_ERR_STATS 8
 #define HDOF_ERR_SCRATCH (HDOF_ERR_STATS + 8 * 1024)
 int hdof_error_map(const float* a, const float* b, const uint8_t* region, int32_t width, int32_t height,
@@ -614,8 +615,9 @@ int hdof_post_forward(const hdof_gbuf* in, const uint8_t* spp, const float* rec,
 /* Adjoint of hdof_post_forward (same inputs, its state): from grad_out
  * ([H][W][4], rgb used) writes grad_col ([H][W][4], d/d colour) and
  * grad_lens (device float [2] = d/d focus_dist, d/d aperture_radius).  Gather
- * weights are recomputed, not stored; the lens gradient is reduced per block
- * in double precision and summed in a fixed order (deterministic).  Needs
+ * weights are recomputed, not stored; the lens gradient is reduced with at
+ * least a double's bits (a warp in three floats, then doubles) in a fixed
+ * order (deterministic).  Needs
  * aperture_radius > 0.  Both calls take the fixed EMA weight, the uniform
  * circular lens and no specular preference: alpha_k, blades, aberration and
  * spec_pref other than 0 return HDOF_EUNSUPPORTED. */

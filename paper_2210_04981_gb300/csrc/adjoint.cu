@@ -14,8 +14,8 @@
 // definitions coincide.  Backward: composite -> spatial (transposed gather)
 // -> temporal and replay (per pixel, recomputed) -> post-filter (transposed
 // gather over each source pixel's own disk, gather weights recomputed, not
-// stored).  The lens gradient is reduced per block in double precision and
-// summed in a fixed order: the result is deterministic.
+// stored).  The lens gradient is summed in three floats within a warp and in
+// double precision beyond, in a fixed order: the result is deterministic.
 #include <cmath>
 
 #include "internal.h"

@@ -815,9 +815,12 @@ __global__ void __launch_bounds__(256, 4) k_resolve(TraceArgs a) { resolve_body(
 // The same for images of at most RES_SMALL pixels, where a thread's serial
 // samples are the kernel's time: RES_LANES threads share a pixel, each shades
 // every RES_LANES-th sample, and all of them add every sample in sample order
-// (passed by shuffles), so the sums are the same.  128x128 with 16 samples
-// 28.6 -> 14 us; on full grids the shuffles and repeated additions cost more
-// than the split gains (720p, every pixel: 119 -> 195 us).
+// (passed by shuffles), so the sums are the same.  On full grids the shuffles
+// and repeated additions cost more than the split gains (720p, every pixel:
+// 119 -> 195 us with the earlier k_resolve).  Every pixel traced with 4, 8, 16
+// samples, k_resolve / this: 128x128 10.2/8.1, 14.3/10.1, 20.5/14.2 us,
+// 181x181, at the line, 10.2/10.4, 14.3/14.3, 20.5/20.4, 256x256 12.3/14.3,
+// 16.4/18.5, 24.5/28.6.
 constexpr int RES_SMALL = 1 << 15;
 constexpr int RES_LANES = 4;
 __global__ void __launch_bounds__(256) k_resolve_small(TraceArgs a) {
