@@ -250,7 +250,8 @@ int hdof_gbuffer(const hdof_bvh* bvh, const hdof_camera* cam, const hdof_camera*
  * hdof_trace once hdof_gbuffer has finished.  This buffer, like the one of
  * hdof_post_workspace_bytes below, starts at a multiple of 16 bytes; where a
  * call needs more, it rounds up inside the buffer (the size returned has room
- * for that). */
+ * for that), and a start whose accesses would be misaligned is refused
+ * (HDOF_EINVAL). */
 size_t hdof_workspace_bytes(int32_t width, int32_t height, const hdof_params* p);
 
 /* ----------------------------------------------------------- mask -- */

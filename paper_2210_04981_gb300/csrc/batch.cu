@@ -96,6 +96,7 @@ int check_view(const hdof_view& v, int k, int dev) {
     size_t need = ws_layout(v.cam.width, v.cam.height, &v.params).total;
     HDOF_CHECK_ARG(v.workspace && v.workspace_bytes >= need, "%s: workspace of %zu bytes < %zu", who,
                    v.workspace_bytes, need);
+    HDOF_CHECK_ALIGNED(v.workspace, 8, who);
     return HDOF_OK;
 }
 

@@ -74,6 +74,11 @@ constexpr size_t PF_ALIGN = 256;
 inline char* align_up(void* p, size_t a) {
     return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(p) + a - 1) & ~(uintptr_t)(a - 1));
 }
+// What lies at the workspace's own start keeps its alignment: a call whose
+// accesses there (n bytes each) would be misaligned is refused.
+#define HDOF_CHECK_ALIGNED(ws, n, who)                                                                    \
+    HDOF_CHECK_ARG(!(reinterpret_cast<uintptr_t>(ws) & ((n) - 1)),                                       \
+                   "%s: the workspace has to start at a multiple of 16 bytes", who)
 
 // workspace layout (bytes) for a width x height frame
 struct WsLayout {

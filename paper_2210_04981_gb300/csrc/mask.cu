@@ -486,6 +486,7 @@ extern "C" int hdof_mask_coc(const hdof_gbuf* in, const hdof_history* prev_hist,
     WsLayout L = ws_layout(W, H, p);
     HDOF_CHECK_ARG(workspace && workspace_bytes >= L.mask_tiles + L.mask_tile_r,
                    "hdof_mask_coc: workspace of %zu bytes < %zu", workspace_bytes, L.mask_tiles + L.mask_tile_r);
+    if (p->mask_coc) HDOF_CHECK_ALIGNED(workspace, 4, "hdof_mask_coc");
     cudaStream_t s = as_stream(stream);
     const int T = p->tile, ntx = (W + T - 1) / T, nty = (H + T - 1) / T;
     uint8_t* tiles = static_cast<uint8_t*>(workspace);

@@ -914,6 +914,7 @@ extern "C" int hdof_postfilter_spec(const hdof_gbuf* in, const hdof_camera* cam,
         if (f32c) return run_postfilter<half4s, Grey<float4>>(in, coc, p, pp_spec, nullptr, scratch, s, nullptr, 0.f);
         return run_postfilter<half4s, Grey<bf164s>>(in, coc, p, pp_spec, nullptr, scratch, s, nullptr, 0.f);
     }
+    HDOF_CHECK_ALIGNED(workspace, 16, "hdof_postfilter_spec");
     float4* plane = static_cast<float4*>(workspace);
     {
         ProfScope ps_("pf_spec_plane", s);

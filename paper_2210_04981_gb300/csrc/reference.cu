@@ -181,6 +181,7 @@ extern "C" int hdof_reference_rt(const hdof_bvh* b, const hdof_camera* cam, cons
     WsLayout L = ws_layout(W, H, p);
     HDOF_CHECK_ARG(workspace && workspace_bytes >= L.total, "hdof_reference_rt: workspace of %zu bytes < %zu",
                    workspace_bytes, L.total);
+    HDOF_CHECK_ALIGNED(workspace, 16, "hdof_reference_rt");
     // the post-filter region holds the pass's trace output and the ray-count plane
     char* pf = static_cast<char*>(workspace) + L.pf_off;
     float* rt = reinterpret_cast<float*>(pf);

@@ -1156,6 +1156,7 @@ extern "C" int hdof_trace(const hdof_bvh* b, const hdof_camera* cam, const hdof_
     WsLayout L = ws_layout(W, H, p);
     HDOF_CHECK_ARG(workspace && workspace_bytes >= L.trace, "hdof_trace: workspace of %zu bytes < %zu",
                    workspace_bytes, L.trace);
+    HDOF_CHECK_ALIGNED(workspace, 8, "hdof_trace");
     unsigned* st = status_ptr();
     HDOF_CHECK_ARG(st, "hdof_trace: no status word on this device");
     cudaStream_t s = as_stream(stream);
@@ -1205,6 +1206,7 @@ extern "C" int hdof_trace_hits(const hdof_bvh* b, const hdof_camera* cam, const 
     WsLayout L = ws_layout(W, H, p);
     HDOF_CHECK_ARG(workspace && workspace_bytes >= L.trace, "hdof_trace_hits: workspace of %zu bytes < %zu",
                    workspace_bytes, L.trace);
+    HDOF_CHECK_ALIGNED(workspace, 8, "hdof_trace_hits");
     hdof_view v = {};
     v.cam = *cam;
     v.params = *p;
